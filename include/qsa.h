@@ -149,7 +149,7 @@ typedef struct {
 
 typedef struct {
     double seconds;         /* device time of all launches (timing = 1), else 0 */
-    double apply_seconds;   /* device time of FP32 fused-operator kernels */
+    double apply_seconds;   /* device time of FP32 fused-operator kernels and of group passes */
     double permute_seconds; /* device time of permutation kernels */
     double hbm_bytes;       /* algorithmic HBM bytes: 16 B x 2^N per full-state pass */
     uint64_t blocks;        /* fused blocks applied */
@@ -159,7 +159,7 @@ typedef struct {
     uint64_t launches;      /* kernel launches issued */
     double h2d_bytes;       /* host-to-device bytes copied by the call (fused matrices) */
     double tc_seconds;      /* device time of tensor-core fused-operator kernels */
-    uint64_t diag_blocks;   /* diagonal blocks run on the streaming kernel */
+    uint64_t diag_blocks;   /* diagonal blocks (streaming kernel or group passes) */
     double diag_seconds;    /* device time of diagonal streaming kernels */
     uint64_t prod_blocks;   /* product blocks (one-qubit factors) applied */
     double prod_seconds;    /* device time of product kernels */
@@ -417,6 +417,11 @@ qsa_status qsa_plan_exchanges(qsa_plan p, int rank_bits, const int32_t* layout_i
                               size_t capacity, size_t* n_out, int32_t* layout_out);
 
 /* Apply the plan's blocks to s in order (asynchronous unless opts.timing).
+ * On states of at most 25 qubits whose layout is the plan's, consecutive dense
+ * (k <= 4), diagonal (k <= 8) and product blocks run several to a pass (group
+ * passes: a block may move across blocks on other qubits, or across diagonal
+ * ones where both are diagonal); stats count them as blocks, their passes as
+ * passes.  Per-gate plans and QSA_LOWER_PERMUTE keep one pass per block.
  * The first execution on a device uploads the fused matrices once
  * (stats->h2d_bytes).  Errors: QSA_E_ARG if the plan's N differs from s. */
 qsa_status qsa_plan_execute(qsa_state s, qsa_plan p, qsa_run_stats* stats);
@@ -483,10 +488,10 @@ qsa_status qsa_sample_counts(qsa_state s, uint64_t shots, uint64_t seed, uint64_
  * Many independent small states (noisy trajectories: the per-gate Pauli
  * channels of §IV-A sampled into explicit Pauli branches, so every trajectory
  * is a unitary circuit) evolved in ONE persistent kernel launch: each
- * thread-block cluster of four CTAs pops a trajectory from an atomic queue
- * (longest first), resets it to |0..0> and applies all of its fused blocks,
- * the four CTAs splitting every pass's tiles and meeting at a cluster barrier
- * between blocks; a second kernel samples every state (one CTA per
+ * thread-block cluster (up to four CTAs) pops a trajectory from an atomic queue
+ * (longest first) and applies all of its fused blocks to |0..0> in group
+ * passes (several blocks per pass), the CTAs splitting every pass's tiles and
+ * meeting at a cluster barrier between passes; a second kernel samples every state (one CTA per
  * trajectory, Philox stream id = trajectory index, identity layout), and both
  * can be replayed as one captured CUDA graph. */
 typedef struct qsa_batch_s* qsa_batch;
@@ -506,7 +511,7 @@ qsa_status qsa_batch_info(qsa_batch b, size_t* total_blocks, size_t* total_ops, 
  * (stream id t).  use_graph = 1 captures the launches into a CUDA graph on
  * first use (re-captured when an argument changes) and replays it.
  * budget_cycles > 0 bounds each cluster's run time in SM clock cycles (as seen
- * by its first CTA): a cluster that runs over stops between blocks and the
+ * by its first CTA): a cluster that runs over stops between passes and the
  * call returns QSA_E_TIMEOUT.
  * Synchronises cuda_stream; stats->seconds is the device time of the launch. */
 qsa_status qsa_batch_run(qsa_batch b, void* dev_states, size_t bytes, uint64_t shots, uint64_t seed,

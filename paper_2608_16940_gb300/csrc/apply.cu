@@ -1,5 +1,4 @@
-// FP32 fused dense update, qubit-permutation and batched-trajectory kernels
-// (sm_103a).
+// FP32 fused dense update, product and qubit-permutation kernels (sm_103a).
 //
 // All three share one tile engine: a CTA walks tiles t0, t0 + stride, ...;
 // each tile (2^T amplitudes = 2^nx contiguous runs of 2^m amplitudes) is
@@ -13,12 +12,7 @@
 //           psi'[x|spread(r)] = sum_c G[r][c] psi[x|spread(c)];
 //   permute (§IV-D, Lemma "distributed promotion swap" with the rank bits read
 //           as out-of-block bits): psi'[tau(y)] = psi[y] for a product tau of
-//           disjoint bit transpositions;
-//   batch   many independent states (noisy trajectories, §IV-A channels
-//           sampled as explicit Pauli branches) in one persistent launch: each
-//           CTA pops a trajectory from an atomic queue (longest first), resets
-//           it to |0...0> and applies all of its fused blocks.
-#include <cooperative_groups.h>
+//           disjoint bit transpositions.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -672,126 +666,6 @@ __global__ void __launch_bounds__(kThreads) k_permute(PermArgs a) {
 
 __global__ void k_set_one(float2* psi) { psi[0] = make_float2(1.f, 0.f); }
 
-// ---------------------------------------------------------------------------
-// Batched trajectories: one persistent launch over many small states
-// ---------------------------------------------------------------------------
-constexpr int kBatchT = 11;
-constexpr int kBatchS = 3;
-// A trajectory's blocks run one after another, so the batch ends when its
-// deepest trajectory does: each trajectory is run by a cluster of CTAs that
-// split every pass's tiles (rank r takes tiles r, r + C, ...) and meet at a
-// cluster barrier between blocks.
-constexpr int kBatchCluster = 4;
-
-namespace cg = cooperative_groups;
-
-__global__ void __cluster_dims__(kBatchCluster, 1, 1) __launch_bounds__(kThreads, 4) k_batch_evolve(BatchArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* stage = reinterpret_cast<float2*>(smem_raw);
-    float2* Ms = stage + (kBatchS << kBatchT);
-    uint64_t* runoff = reinterpret_cast<uint64_t*>(Ms + 256);
-    int* loff = reinterpret_cast<int*>(runoff + 64);
-    int* sloff = loff + 64;
-    uint8_t* htab = reinterpret_cast<uint8_t*>(sloff + 64);
-    // Rank 0 of the cluster pops the queue and makes the watchdog's decision;
-    // the others read them from its shared memory after a cluster barrier, so
-    // every CTA of a cluster takes the same path and meets the same barriers
-    // (s_stop alternates by block so a value is never rewritten before all
-    // have read it; s_slot is rewritten only after the trajectory's barriers).
-    __shared__ int s_slot;
-    __shared__ int s_stop[2];
-    cg::cluster_group cluster = cg::this_cluster();
-    const unsigned crank = cluster.block_rank();
-    const long long t_start = clock64();
-    for (;;) {
-        if (crank == 0 && threadIdx.x == 0) s_slot = static_cast<int>(atomicAdd(a.queue, 1u));
-        cluster.sync();
-        const int slot = *cluster.map_shared_rank(&s_slot, 0);
-        if (slot >= a.n_traj) {
-            cluster.sync();   // no CTA leaves while another may still read its shared memory
-            break;
-        }
-        const int traj = a.order[slot];
-        float2* psi = a.states + (static_cast<uint64_t>(traj) << a.n);
-        // |0...0>, a share per CTA
-        float4* p4 = reinterpret_cast<float4*>(psi);
-        const uint64_t npairs = (1ull << a.n) >> 1;
-        for (uint64_t i = crank * blockDim.x + threadIdx.x; i < npairs; i += kBatchCluster * blockDim.x)
-            p4[i] = make_float4(i == 0 ? 1.f : 0.f, 0.f, 0.f, 0.f);
-        __threadfence();
-        cluster.sync();
-        for (uint32_t b = a.bstart[traj]; b < a.bstart[traj + 1]; ++b) {
-            const BatchBlock d = a.blocks[b];
-            ApplyArgs aa{};
-            aa.t.psi = psi;
-            aa.t.T = d.T;
-            aa.t.m = d.m;
-            aa.t.nx = d.nx;
-            aa.t.ntiles = 1ull << (a.n - d.T);
-#pragma unroll
-            for (int e = 0; e < 6; ++e) {
-                aa.t.xpos[e] = d.xpos[e];
-                aa.tl[e] = d.tl[e];
-                aa.tls[e] = d.tls[e];
-            }
-#pragma unroll
-            for (int e = 0; e < 16; ++e) aa.fv[e] = d.fv[e];
-            const int D = 1 << d.k;
-            const float2* gm = reinterpret_cast<const float2*>(a.mats + d.mat_off);
-            for (int i = threadIdx.x; i < D * D; i += blockDim.x) Ms[i] = gm[i];
-            build_runoff(aa.t, runoff);
-            switch (d.k) {
-                case 1: build_loff<1>(aa.tl, loff); break;
-                case 2: build_loff<2>(aa.tl, loff); break;
-                case 3: build_loff<3>(aa.tl, loff); break;
-                default: build_loff<4>(aa.tl, loff); break;
-            }
-            if (d.form) build_htab(aa, htab);
-            __syncthreads();
-            if (d.form) {
-                for (int c = threadIdx.x; c < D; c += blockDim.x)
-                    sloff[c] = loff[c] ^ static_cast<int>(stage_xor(htab, loff[c]));
-                __syncthreads();
-            }
-            // the stage forms of the single-state kernel (k = 4 takes two items
-            // per group here, so no in-place write-back)
-#define QSA_BATCH_FORMS(K, R)                                                                                     \
-    if (d.form == 2)                                                                                              \
-        apply_tiles<K, R, kBatchS, true, true, kBatchT>(aa, stage, Ms, runoff, loff, crank, kBatchCluster, htab,  \
-                                                        sloff);                                                   \
-    else if (d.form == 1)                                                                                         \
-        apply_tiles<K, R, kBatchS, true, false, kBatchT>(aa, stage, Ms, runoff, loff, crank, kBatchCluster, htab, \
-                                                         sloff);                                                  \
-    else                                                                                                          \
-        apply_tiles<K, R, kBatchS>(aa, stage, Ms, runoff, loff, crank, kBatchCluster);
-            switch (d.k) {
-                case 1: QSA_BATCH_FORMS(1, 2) break;
-                case 2: QSA_BATCH_FORMS(2, 4) break;
-                case 3: QSA_BATCH_FORMS(3, 8) break;
-                default:
-                    if (d.form)
-                        apply_tiles<4, 8, kBatchS, true, false, kBatchT>(aa, stage, Ms, runoff, loff, crank,
-                                                                         kBatchCluster, htab, sloff);
-                    else
-                        apply_tiles<4, 8, kBatchS>(aa, stage, Ms, runoff, loff, crank, kBatchCluster);
-                    break;
-            }
-#undef QSA_BATCH_FORMS
-            // the pass's tiles are written before any CTA of the cluster reads
-            // them in the next block; the watchdog's decision travels with it
-            if (crank == 0 && threadIdx.x == 0)
-                s_stop[b & 1] = (a.budget != 0 && static_cast<unsigned long long>(clock64() - t_start) > a.budget) ? 1 : 0;
-            __threadfence();
-            cluster.sync();
-            if (*cluster.map_shared_rank(&s_stop[b & 1], 0)) {
-                if (crank == 0 && threadIdx.x == 0) atomicExch(a.err, 7);
-                cluster.sync();
-                return;
-            }
-        }
-    }
-}
-
 }  // namespace
 
 QSA_BOUNDS_READER(bounds_word_apply)
@@ -852,45 +726,6 @@ bool make_geom(int n, const int* special, int ns, int T_want, TileGeom* g) {
     for (int e = 0; e < 6; ++e) g->xpos[e] = e < nx ? tmp[e] : 0;
     g->ntiles = 1ull << (n - g->T);
     return true;
-}
-
-bool make_batch_block(int n, const int* phys, int k, uint32_t mat_off, BatchBlock* b) {
-    if (k < 1 || k > 4) return false;
-    TileGeom g;
-    if (!make_geom(n, phys, k, kBatchT, &g)) return false;
-    *b = BatchBlock{};
-    b->k = k;
-    b->T = g.T;
-    b->m = g.m;
-    b->nx = g.nx;
-    for (int e = 0; e < 6; ++e) b->xpos[e] = g.xpos[e];
-    local_targets(g, phys, k, b->tl, b->tls);
-    b->mat_off = mat_off;
-    b->form = g.T == kBatchT ? apply_form(g.T, b->tls, k) : 0;
-    if (k == 4 && b->form == 2) b->form = 1;   // two items per group: gathers only
-    if (b->form) stage_slots(g.T, b->tls, k, b->fv);
-    return true;
-}
-
-cudaError_t launch_batch_evolve(const BatchArgs& a, cudaStream_t st, uint64_t* launches) {
-    const size_t smem = sizeof(float2) * (static_cast<size_t>(kBatchS) << kBatchT) + sizeof(float2) * 256 +
-                        sizeof(uint64_t) * 64 + 2 * sizeof(int) * 64 + 256;
-    {
-        cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(k_batch_evolve), static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-    }
-    int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_evolve, kThreads, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) occ = 1;
-    // one cluster per trajectory in flight (clusters that find the queue
-    // empty leave at once)
-    unsigned clusters = static_cast<unsigned>(num_sms() * occ / kBatchCluster);
-    if (clusters > static_cast<unsigned>(a.n_traj)) clusters = static_cast<unsigned>(a.n_traj);
-    if (clusters == 0) clusters = 1;
-    k_batch_evolve<<<clusters * kBatchCluster, kThreads, smem, st>>>(a);
-    ++*launches;
-    return cudaGetLastError();
 }
 
 __global__ void k_fill_one(float4* psi2, uint64_t npairs) {

@@ -241,6 +241,55 @@ void build_next_use(qsa_plan_s* p) {
     }
 }
 
+// Runs of consecutive dense (k <= 4), diagonal and product blocks become group
+// passes (several blocks per pass over the state) for the plan's layout.
+// Per-gate plans keep one pass per op, and permuting plans one layout per block.
+void build_groups(qsa_plan_s* p) {
+    if (p->n > kGroupMaxQubits || p->opts.planner == QSA_PLAN_PER_GATE || p->opts.lowering == QSA_LOWER_PERMUTE) return;
+    auto takes = [](const PlanBlock& b) { return b.layer < 0 && (b.prod || group_takes(b.k, b.diag)); };
+    const size_t nb = p->blocks.size();
+    for (size_t i = 0; i < nb;) {
+        size_t e = i;
+        while (e < nb && takes(p->blocks[e])) ++e;
+        if (e - i >= 2) {
+            std::vector<GroupSrc> src;
+            std::vector<int> whole;   // the block an operator is all of, or -1 (a product's factor)
+            for (size_t x = i; x < e; ++x) {
+                const PlanBlock& b = p->blocks[x];
+                const float* mat = p->host_mat.data() + b.off;
+                if (b.prod) {
+                    for (int j = 0; j < b.k; ++j) {
+                        src.push_back({1, false, {p->L0[b.t[j]]}, mat + 8 * j});
+                        whole.push_back(-1);
+                    }
+                } else {
+                    GroupSrc g{b.k, b.diag, {}, mat};
+                    for (int j = 0; j < b.k; ++j) g.pos[j] = p->L0[b.t[j]];
+                    src.push_back(g);
+                    whole.push_back(static_cast<int>(x));
+                }
+            }
+            PlanGroup gr{i, e, p->gpasses.size(), 0};
+            for (size_t x = i; x < e; ++x) {
+                gr.blocks += 1;
+                gr.diags += p->blocks[x].diag ? 1 : 0;
+                gr.prods += p->blocks[x].prod ? 1 : 0;
+            }
+            for (GroupPass& gp : group_build(p->n, src, &p->host_group)) {
+                if (gp.only >= 0) gp.only = whole[gp.only];
+                if (gp.only >= 0) {   // counted where it runs
+                    gr.blocks -= 1;
+                    gr.diags -= p->blocks[gp.only].diag ? 1 : 0;
+                }
+                p->gpasses.push_back(gp);
+            }
+            gr.p1 = p->gpasses.size();
+            p->groups.push_back(gr);
+        }
+        i = std::max(e, i + 1);
+    }
+}
+
 uint64_t op_mask(const qsa_op& op) {
     uint64_t m = 0;
     for (int j = 0; j < op.k; ++j) m |= 1ull << op.targets[j];
@@ -771,6 +820,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
     for (PlanLayer& pl : p->layers)
         pl.launches = prepare_layer(n_qubits, p->L0.data(), pl.spec, &p->host_layer, &carry);
     build_next_use(p);
+    build_groups(p);
     *out = p;
     return QSA_OK;
 }
@@ -907,90 +957,139 @@ qsa_status qsa_plan_block_kinds(qsa_plan p, int32_t* kinds, int32_t* n_diag, siz
     return QSA_OK;
 }
 
-qsa_status qsa_plan_destroy(qsa_plan p) {
-    if (!p) return fail(QSA_E_ARG, "plan is NULL");
-    if (p->d_mat || p->d_layer) cudaDeviceSynchronize();
+namespace {
+
+void plan_free_device(qsa_plan p) {
     if (p->d_mat) dev_free(p->d_mat);
     if (p->d_layer) dev_free(p->d_layer);
+    if (p->d_group) dev_free(p->d_group);
+    p->d_mat = nullptr;
+    p->d_layer = nullptr;
+    p->d_group = nullptr;
+}
+
+}  // namespace
+
+qsa_status qsa_plan_destroy(qsa_plan p) {
+    if (!p) return fail(QSA_E_ARG, "plan is NULL");
+    if (p->d_mat || p->d_layer || p->d_group) cudaDeviceSynchronize();
+    plan_free_device(p);
     delete p;
     return QSA_OK;
 }
 
-qsa_status qsa_plan_execute(qsa_state s, qsa_plan p, qsa_run_stats* stats) {
+namespace {
+
+// First execution on a device: the fused matrices, the layer payloads and the
+// group programs are uploaded once.
+qsa_status plan_upload(qsa_state s, qsa_plan p, qsa_run_stats* rs) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (p->dev == dev) return QSA_OK;
+    if (p->d_mat || p->d_layer || p->d_group) cudaStreamSynchronize(s->stream);
+    plan_free_device(p);
+    const size_t bytes = p->host_mat.size() * sizeof(float);
+    const size_t lbytes = p->host_layer.size(), gbytes = p->host_group.size();
+    cudaError_t e = bytes ? dev_malloc(&p->d_mat, bytes) : cudaSuccess;
+    if (e == cudaSuccess && lbytes) e = dev_malloc(&p->d_layer, lbytes);
+    if (e == cudaSuccess && gbytes) e = dev_malloc(&p->d_group, gbytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        plan_free_device(p);
+        return fail(QSA_E_NOMEM, "cudaMalloc of plan matrices failed");
+    }
+    if (bytes) {
+        e = cudaMemcpyAsync(p->d_mat, p->host_mat.data(), bytes, cudaMemcpyHostToDevice, s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "plan matrix upload");
+    }
+    if (lbytes) {
+        e = cudaMemcpyAsync(p->d_layer, p->host_layer.data(), lbytes, cudaMemcpyHostToDevice, s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "plan layer upload");
+    }
+    if (gbytes) {
+        e = cudaMemcpyAsync(p->d_group, p->host_group.data(), gbytes, cudaMemcpyHostToDevice, s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "plan group upload");
+    }
+    p->dev = dev;
+    rs->h2d_bytes = static_cast<double>(bytes + lbytes + gbytes);
+    return QSA_OK;
+}
+
+qsa_status run_block(qsa_state s, qsa_plan p, size_t i, qsa_run_stats* rs) {
+    const PlanBlock& b = p->blocks[i];
+    if (b.init && !s->known_zero) return fail(QSA_E_STATE, "a zero_init plan needs the state |0..0>");
+    if (b.layer >= 0) {
+        const PlanLayer& pl = p->layers[b.layer];
+        if (s->n >= QSA_LAYER_TILE_BITS && std::equal(p->L0.begin(), p->L0.end(), s->L))
+            return run_layer_launches(s, pl.launches, p->d_layer, rs);
+        return apply_layer_logical(s, pl.spec, rs);   // another layout: prepare again
+    }
+    if (b.prod) return apply_prod_logical(s, b.t, b.k, p->d_mat + b.off, rs);
+    if (b.diag) return apply_diag_logical(s, b.t, b.k, p->d_mat + b.off, rs);
+    if (p->opts.lowering == QSA_LOWER_PERMUTE) {
+        // promote the targets into the in-block frames, victims per the plan's rule
+        int phys[QSA_MAX_K], pa[QSA_MAX_K], pb[QSA_MAX_K];
+        for (int j = 0; j < b.k; ++j) phys[j] = s->L[b.t[j]];
+        const int np = choose_promotions(s->L, s->n, phys, b.k, std::min(kInBlockBits, s->n), p->opts.victim,
+                                         p->next_use.data() + i * s->n, pa, pb);
+        qsa_status st = np < 0 ? fail(QSA_E_ARG, "block wider than the in-block frames")
+                               : permute_positions(s, pa, pb, np, rs);
+        if (st == QSA_OK) st = apply_physical(s, phys, b.k, p->d_mat + b.off, p->opts.precision, rs);
+        return st;
+    }
+    return apply_logical(s, b.t, b.k, p->d_mat + b.off, p->opts.lowering, p->opts.precision, rs);
+}
+
+// The blocks of a group in its passes; zero: the state is |0...0> and the first
+// pass writes it (nothing is read).
+qsa_status run_group(qsa_state s, qsa_plan p, const PlanGroup& g, bool zero, qsa_run_stats* rs) {
+    for (size_t i = g.p0; i < g.p1; ++i) {
+        const GroupPass& gp = p->gpasses[i];
+        if (gp.only >= 0) {   // one block: its own kernel
+            qsa_status st = run_block(s, p, static_cast<size_t>(gp.only), rs);
+            if (st != QSA_OK) return st;
+            continue;
+        }
+        Timer tm(s, &rs->apply_seconds);
+        cudaError_t e = launch_group(s->psi, s->n, gp, p->d_group, zero && i == g.p0, s->stream, &s->launches);
+        tm.stop();
+        if (e != cudaSuccess) return cuda_fail(s, e, "group kernel");
+        s->known_zero = false;
+        rs->passes += 1;
+        rs->hbm_bytes += 16.0 * static_cast<double>(1ull << s->n);
+    }
+    rs->blocks += g.blocks;
+    rs->diag_blocks += g.diags;
+    rs->prod_blocks += g.prods;
+    return QSA_OK;
+}
+
+// zero: the state is |0...0> in the plan's layout, perhaps not written yet (the
+// first block writes every amplitude).
+qsa_status execute(qsa_state s, qsa_plan p, bool zero, qsa_run_stats* stats) {
     qsa_status st = check_state(s);
     if (st != QSA_OK) return st;
-    if (!p) return fail(QSA_E_ARG, "plan is NULL");
-    if (p->n != s->n) return fail(QSA_E_ARG, "plan and state have different qubit counts");
     qsa_run_stats local{};
     qsa_run_stats* rs = stats ? stats : &local;
     *rs = qsa_run_stats{};
     if (p->blocks.empty()) return QSA_OK;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (p->dev != dev) {
-        // first execution on this device: upload the fused matrices and the
-        // layer payloads once
-        if (p->d_mat || p->d_layer) cudaStreamSynchronize(s->stream);
-        if (p->d_mat) dev_free(p->d_mat);
-        if (p->d_layer) dev_free(p->d_layer);
-        p->d_mat = nullptr;
-        p->d_layer = nullptr;
-        const size_t bytes = p->host_mat.size() * sizeof(float);
-        const size_t lbytes = p->host_layer.size();
-        cudaError_t e = bytes ? dev_malloc(&p->d_mat, bytes) : cudaSuccess;
-        if (e == cudaSuccess && lbytes) e = dev_malloc(&p->d_layer, lbytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            if (p->d_mat) dev_free(p->d_mat);
-            p->d_mat = nullptr;
-            p->d_layer = nullptr;
-            return fail(QSA_E_NOMEM, "cudaMalloc of plan matrices failed");
-        }
-        if (bytes) {
-            e = cudaMemcpyAsync(p->d_mat, p->host_mat.data(), bytes, cudaMemcpyHostToDevice, s->stream);
-            if (e != cudaSuccess) return cuda_fail(s, e, "plan matrix upload");
-        }
-        if (lbytes) {
-            e = cudaMemcpyAsync(p->d_layer, p->host_layer.data(), lbytes, cudaMemcpyHostToDevice, s->stream);
-            if (e != cudaSuccess) return cuda_fail(s, e, "plan layer upload");
-        }
-        p->dev = dev;
-        rs->h2d_bytes = static_cast<double>(bytes + lbytes);
-    }
+    st = plan_upload(s, p, rs);
+    if (st != QSA_OK) return st;
     const uint64_t l0 = s->launches;
     s->timing = p->opts.timing != 0;
-    for (size_t i = 0; i < p->blocks.size(); ++i) {
-        const PlanBlock& b = p->blocks[i];
-        if (b.init && !s->known_zero) {
-            st = fail(QSA_E_STATE, "a zero_init plan needs the state |0..0>");
-        } else if (b.layer >= 0) {
-            const PlanLayer& pl = p->layers[b.layer];
-            if (s->n >= QSA_LAYER_TILE_BITS && std::equal(p->L0.begin(), p->L0.end(), s->L))
-                st = run_layer_launches(s, pl.launches, p->d_layer, rs);
-            else
-                st = apply_layer_logical(s, pl.spec, rs);   // another layout: prepare again
-        } else if (b.prod) {
-            st = apply_prod_logical(s, b.t, b.k, p->d_mat + b.off, rs);
-        } else if (b.diag) {
-            st = apply_diag_logical(s, b.t, b.k, p->d_mat + b.off, rs);
-        } else if (p->opts.lowering == QSA_LOWER_PERMUTE) {
-            // promote the targets into the in-block frames, victims per the plan's rule
-            int phys[QSA_MAX_K], pa[QSA_MAX_K], pb[QSA_MAX_K];
-            for (int j = 0; j < b.k; ++j) phys[j] = s->L[b.t[j]];
-            const int np = choose_promotions(s->L, s->n, phys, b.k, std::min(kInBlockBits, s->n), p->opts.victim,
-                                             p->next_use.data() + i * s->n, pa, pb);
-            st = np < 0 ? fail(QSA_E_ARG, "block wider than the in-block frames")
-                        : permute_positions(s, pa, pb, np, rs);
-            if (st == QSA_OK) st = apply_physical(s, phys, b.k, p->d_mat + b.off, p->opts.precision, rs);
+    const bool grouped = !p->groups.empty() && std::equal(p->L0.begin(), p->L0.end(), s->L);
+    size_t next = 0;
+    for (size_t i = 0; i < p->blocks.size() && st == QSA_OK;) {
+        while (next < p->groups.size() && p->groups[next].b0 < i) ++next;
+        if (grouped && next < p->groups.size() && p->groups[next].b0 == i) {
+            st = run_group(s, p, p->groups[next], zero && i == 0, rs);
+            i = p->groups[next].b1;
         } else {
-            st = apply_logical(s, b.t, b.k, p->d_mat + b.off, p->opts.lowering, p->opts.precision, rs);
-        }
-        if (st != QSA_OK) {
-            s->timing = false;
-            return st;
+            st = run_block(s, p, i++, rs);
         }
     }
     s->timing = false;
+    if (st != QSA_OK) return st;
     rs->launches = s->launches - l0;
     if (p->opts.timing) {
         collect_timers(s, &rs->seconds);
@@ -999,21 +1098,34 @@ qsa_status qsa_plan_execute(qsa_state s, qsa_plan p, qsa_run_stats* stats) {
     return QSA_OK;
 }
 
+}  // namespace
+
+qsa_status qsa_plan_execute(qsa_state s, qsa_plan p, qsa_run_stats* stats) {
+    qsa_status st = check_state(s);
+    if (st != QSA_OK) return st;
+    if (!p) return fail(QSA_E_ARG, "plan is NULL");
+    if (p->n != s->n) return fail(QSA_E_ARG, "plan and state have different qubit counts");
+    return execute(s, p, false, stats);
+}
+
 qsa_status qsa_plan_execute_from_zero(qsa_state s, qsa_plan p, qsa_run_stats* stats) {
     if (!s) return fail(QSA_E_ARG, "state is NULL");
     if (!p) return fail(QSA_E_ARG, "plan is NULL");
     if (p->n != s->n) return fail(QSA_E_ARG, "plan and state have different qubit counts");
-    if (!p->blocks.empty() && p->blocks[0].init && s->n >= QSA_LAYER_TILE_BITS && !s->failed) {
-        // the preparation pass writes every amplitude: |0..0> in the plan's
-        // layout needs no clearing first
-        for (int q = 0; q < s->n; ++q) s->L[q] = p->L0[q];
-        s->known_zero = true;
-    } else {
+    // a plan whose first pass writes every amplitude (the zero_init preparation,
+    // or a group pass) needs no clearing first: |0..0> in the plan's layout is relabelled
+    const bool prep = !p->blocks.empty() && p->blocks[0].init && s->n >= QSA_LAYER_TILE_BITS;
+    const bool group = !p->groups.empty() && p->groups[0].b0 == 0 && p->gpasses[p->groups[0].p0].only < 0;
+    const bool writes = (prep || group) && !s->failed;
+    if (!writes) {
         qsa_status st = qsa_state_reset(s);
         if (st != QSA_OK) return st;
-        for (int q = 0; q < s->n; ++q) s->L[q] = p->L0[q];   // relabelling |0..0> is free
     }
-    return qsa_plan_execute(s, p, stats);
+    for (int q = 0; q < s->n; ++q) s->L[q] = p->L0[q];   // relabelling |0..0> is free
+    s->known_zero = true;
+    const qsa_status st = execute(s, p, writes && group, stats);
+    if (st != QSA_OK && writes) s->known_zero = false;   // the amplitudes may be the old ones
+    return st;
 }
 
 qsa_status qsa_apply_circuit(qsa_state s, const qsa_op* ops, size_t n_ops, const qsa_plan_opts* opts,
@@ -1024,13 +1136,10 @@ qsa_status qsa_apply_circuit(qsa_state s, const qsa_op* ops, size_t n_ops, const
     st = plan_create(ops, n_ops, s->n, opts, s->L, s->cm ? s->cm : costmodel_global(), &p);
     if (st != QSA_OK) return st;
     st = qsa_plan_execute(s, p, stats);
-    if (p->d_mat || p->d_layer) {
+    if (p->d_mat || p->d_layer || p->d_group) {
         // free after the stream has consumed the matrices
         cudaStreamSynchronize(s->stream);
-        if (p->d_mat) dev_free(p->d_mat);
-        if (p->d_layer) dev_free(p->d_layer);
-        p->d_mat = nullptr;
-        p->d_layer = nullptr;
+        plan_free_device(p);
     }
     delete p;
     return st;
@@ -1050,14 +1159,17 @@ qsa_status qsa_state_counters(qsa_state s, uint64_t* launches) {
 struct qsa_batch_s {
     int n = 0, n_traj = 0;
     size_t total_ops = 0;
-    std::vector<qsa::BatchBlock> blocks;
-    std::vector<uint32_t> bstart;
+    size_t total_blocks = 0;
+    std::vector<qsa::GroupPass> passes;
+    std::vector<uint32_t> pstart;
     std::vector<int32_t> order;
-    std::vector<float> mats;
-    qsa::BatchBlock* d_blocks = nullptr;
-    uint32_t* d_bstart = nullptr;
+    std::vector<unsigned char> progs;
+    std::vector<uint64_t> prog_base;   // per trajectory
+    qsa::GroupPass* d_passes = nullptr;
+    uint32_t* d_pstart = nullptr;
     int32_t* d_order = nullptr;
-    float* d_mats = nullptr;
+    unsigned char* d_progs = nullptr;
+    uint64_t* d_prog_base = nullptr;
     unsigned* d_queue = nullptr;   // [0] work counter, [1] error word
     uint32_t* d_out = nullptr;     // keys, counts (n_traj * shots each), n_distinct (n_traj)
     size_t out_cap = 0;
@@ -1073,8 +1185,9 @@ struct qsa_batch_s {
 namespace {
 
 void batch_free_device(qsa_batch b) {
-    for (void* p : {static_cast<void*>(b->d_blocks), static_cast<void*>(b->d_bstart), static_cast<void*>(b->d_order),
-                    static_cast<void*>(b->d_mats), static_cast<void*>(b->d_queue), static_cast<void*>(b->d_out)})
+    for (void* p : {static_cast<void*>(b->d_passes), static_cast<void*>(b->d_pstart), static_cast<void*>(b->d_order),
+                    static_cast<void*>(b->d_progs), static_cast<void*>(b->d_prog_base), static_cast<void*>(b->d_queue),
+                    static_cast<void*>(b->d_out)})
         if (p) dev_free(p);
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->graph) cudaGraphDestroy(b->graph);
@@ -1091,10 +1204,11 @@ cudaError_t batch_enqueue(qsa_batch b, float2* states, uint64_t shots, uint64_t 
     a.states = states;
     a.n = b->n;
     a.n_traj = b->n_traj;
-    a.blocks = b->d_blocks;
-    a.bstart = b->d_bstart;
+    a.passes = b->d_passes;
+    a.pstart = b->d_pstart;
     a.order = b->d_order;
-    a.mats = b->d_mats;
+    a.progs = b->d_progs;
+    a.prog_base = b->d_prog_base;
     a.queue = b->d_queue;
     a.err = reinterpret_cast<int*>(b->d_queue + 1);
     a.budget = budget;
@@ -1131,59 +1245,64 @@ qsa_status qsa_batch_create(int n_qubits, int n_traj, const qsa_op* ops, const s
     b->n = n_qubits;
     b->n_traj = n_traj;
     b->total_ops = op_offsets[n_traj];
-    b->bstart.push_back(0);
+    b->pstart.push_back(0);
     std::vector<double> M;
+    std::vector<uint64_t> cost(n_traj, 0);
     for (int t = 0; t < n_traj; ++t) {
         const qsa_op* tops = ops + op_offsets[t];
         const size_t cnt = op_offsets[t + 1] - op_offsets[t];
         std::vector<size_t> order;   // the identity: batches take no layer units
         auto units = plan(tops, cnt, n_qubits, o, nullptr, &order, costmodel_global());
+        b->total_blocks += units.size();
+        std::vector<float> mats;     // addressed by offset until all are in place
+        std::vector<size_t> off;
+        std::vector<GroupSrc> src;
         for (const Unit& u : units) {
-            int32_t tg[QSA_MAX_K];
-            int k = 0;
-            const uint32_t off = static_cast<uint32_t>(b->mats.size());
-            if (u.e - u.s == 1) {
-                k = tops[u.s].k;
-                for (int j = 0; j < k; ++j) tg[j] = tops[u.s].targets[j];
-                b->mats.resize(off + (2u << (2 * k)));
-                to_float_matrix(tops[u.s].matrix, k, b->mats.data() + off);
+            GroupSrc g{};
+            int32_t tg[QSA_MAX_DIAG];
+            off.push_back(mats.size());
+            g.diag = u.diag;
+            if (u.diag) {
+                st = fuse_diag_range(tops, u.s, u.e, tg, &g.k, &M);
+            } else if (u.e - u.s == 1) {
+                g.k = tops[u.s].k;
+                for (int j = 0; j < g.k; ++j) tg[j] = tops[u.s].targets[j];
+                M.assign(tops[u.s].matrix, tops[u.s].matrix + (2u << (2 * g.k)));
             } else {
-                st = fuse_range(tops, u.s, u.e, tg, &k, &M);
-                if (st != QSA_OK) {
-                    delete b;
-                    return st;
-                }
-                b->mats.resize(off + M.size());
-                for (size_t j = 0; j < M.size(); ++j) b->mats[off + j] = static_cast<float>(M[j]);
+                st = fuse_range(tops, u.s, u.e, tg, &g.k, &M);
             }
-            while (b->mats.size() % 4) b->mats.push_back(0.f);
-            qsa::BatchBlock bb;
-            int phys[QSA_MAX_K];
-            for (int j = 0; j < k; ++j) phys[j] = tg[j];
-            if (!qsa::make_batch_block(n_qubits, phys, k, off, &bb)) {
+            for (double x : M) mats.push_back(static_cast<float>(x));
+            if (st == QSA_OK && !group_takes(g.k, g.diag)) st = fail(QSA_E_ARG, "could not tile a fused block");
+            if (st != QSA_OK) {
                 delete b;
-                return fail(QSA_E_ARG, "could not tile a fused block");
+                return st;
             }
-            b->blocks.push_back(bb);
+            for (int j = 0; j < g.k; ++j) g.pos[j] = tg[j];
+            src.push_back(g);
+            cost[t] += 2u << g.k;
         }
-        b->bstart.push_back(static_cast<uint32_t>(b->blocks.size()));
+        for (size_t i = 0; i < src.size(); ++i) src[i].mat = mats.data() + off[i];
+        std::vector<unsigned char> progs;
+        for (const GroupPass& p : group_build(n_qubits, src, &progs)) b->passes.push_back(p);
+        b->pstart.push_back(static_cast<uint32_t>(b->passes.size()));
+        b->prog_base.push_back(b->progs.size());
+        b->progs.insert(b->progs.end(), progs.begin(), progs.end());
     }
     // longest trajectories first, so the tail of the queue holds short work
     b->order.resize(n_traj);
     for (int t = 0; t < n_traj; ++t) b->order[t] = t;
-    std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) {
-        return b->bstart[x + 1] - b->bstart[x] > b->bstart[y + 1] - b->bstart[y];
-    });
+    std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
     cudaError_t e = cudaSuccess;
     auto up = [&](void** dst, const void* src, size_t bytes) {
         if (e != cudaSuccess) return;
         e = dev_malloc(dst, std::max<size_t>(bytes, 16));
         if (e == cudaSuccess && bytes) e = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
     };
-    up(reinterpret_cast<void**>(&b->d_blocks), b->blocks.data(), b->blocks.size() * sizeof(qsa::BatchBlock));
-    up(reinterpret_cast<void**>(&b->d_bstart), b->bstart.data(), b->bstart.size() * sizeof(uint32_t));
+    up(reinterpret_cast<void**>(&b->d_passes), b->passes.data(), b->passes.size() * sizeof(qsa::GroupPass));
+    up(reinterpret_cast<void**>(&b->d_pstart), b->pstart.data(), b->pstart.size() * sizeof(uint32_t));
     up(reinterpret_cast<void**>(&b->d_order), b->order.data(), b->order.size() * sizeof(int32_t));
-    up(reinterpret_cast<void**>(&b->d_mats), b->mats.data(), b->mats.size() * sizeof(float));
+    up(reinterpret_cast<void**>(&b->d_progs), b->progs.data(), b->progs.size());
+    up(reinterpret_cast<void**>(&b->d_prog_base), b->prog_base.data(), b->prog_base.size() * sizeof(uint64_t));
     if (e == cudaSuccess) e = dev_malloc(&b->d_queue, 2 * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
@@ -1198,7 +1317,7 @@ qsa_status qsa_batch_create(int n_qubits, int n_traj, const qsa_op* ops, const s
 
 qsa_status qsa_batch_info(qsa_batch b, size_t* total_blocks, size_t* total_ops, uint64_t* launches) {
     if (!b) return fail(QSA_E_ARG, "batch is NULL");
-    if (total_blocks) *total_blocks = b->blocks.size();
+    if (total_blocks) *total_blocks = b->total_blocks;
     if (total_ops) *total_ops = b->total_ops;
     if (launches) *launches = b->launches;
     return QSA_OK;
@@ -1290,9 +1409,9 @@ qsa_status qsa_batch_run(qsa_batch b, void* dev_states, size_t bytes, uint64_t s
         *stats = qsa_run_stats{};
         stats->seconds = ms * 1e-3;
         stats->apply_seconds = ms * 1e-3;
-        stats->blocks = b->blocks.size();
-        stats->passes = b->blocks.size();
-        stats->hbm_bytes = 16.0 * static_cast<double>(1ull << b->n) * static_cast<double>(b->blocks.size());
+        stats->blocks = b->total_blocks;
+        stats->passes = b->passes.size();
+        stats->hbm_bytes = 16.0 * static_cast<double>(1ull << b->n) * static_cast<double>(b->passes.size());
         stats->launches = use_graph ? 2 : 2;
     }
     if (err_word != 0)

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 #include "qsa.h"
 
@@ -45,6 +46,7 @@ void dev_free(void* p);
 uint64_t bounds_word_apply();
 uint64_t bounds_word_layer();
 uint64_t bounds_word_tc();
+uint64_t bounds_word_group();
 
 // Number of SMs of the current device (cached per device).
 int num_sms();
@@ -53,28 +55,74 @@ int num_sms();
 // attribute belongs to the device's context; cached per device and kernel).
 cudaError_t set_smem_attr(const void* kernel, int bytes);
 
-// One fused block of a trajectory in the batched kernel (k <= 4, tile bits 11).
-struct BatchBlock {
-    int32_t k, T, m, nx;
-    int32_t xpos[6], tl[6], tls[6];
-    uint32_t mat_off;   // float offset of G in the matrix table
-    int32_t form;       // 0 plain stage, 1 swizzled gathers, 2 swizzled with in-place write-back
-    uint8_t fv[16];     // slot vectors of the swizzled stage
+// ---- group passes (group.cuh, group_host.cpp) ------------------------------
+// A run of dense (k <= 4) and diagonal (k <= kGroupDiagMax) blocks applied in
+// one pass over tiles of 2^T amplitudes, T = min(kGroupTileBits, n).
+constexpr int kGroupTileBits = 12;
+constexpr int kGroupLowBits = 3;          // a tile's lowest positions: runs of at least 64 bytes
+constexpr int kGroupDiagMax = 8;
+constexpr int kGroupDiag = 0;             // GroupOp::code of a diagonal block
+constexpr uint32_t kGroupProgBytes = 38 * 1024;   // a pass's program: two CTAs' stages and programs fit an SM
+
+// An operator on physical positions: dense, 2 * 4^k floats row-major; or
+// diagonal, 2 * 2^k floats (entry c: bit j of c = position pos[j]).
+struct GroupSrc {
+    int k;
+    bool diag;
+    int pos[kGroupDiagMax];
+    const float* mat;
 };
+
+// One block of a round.  Dense: code = its register bits (1..15), the matrix at
+// off with its index bits in ascending register-bit order.  Diagonal: entry
+// index bit j = bit c[j] of (tile number, tile-local index); the parts of the
+// four register bits in ro[], om their mask.
+struct GroupOp {
+    uint8_t code, k, om, pad;
+    uint32_t off;                 // byte offset from par_off, 16-byte aligned
+    uint16_t ro[4];
+    uint8_t c[kGroupDiagMax];
+};
+// Four tile bits in registers (s: their slots), the other tile bits in thread
+// order (tb), and the blocks [op0, op1) applied meanwhile.
+struct GroupRound {
+    uint16_t s[4];
+    uint8_t tb[8];
+    uint16_t op0, op1;
+};
+struct GroupPass {
+    uint64_t ntiles;
+    int32_t T, m, nx;
+    int32_t xpos[kGroupTileBits];
+    int32_t nrounds;
+    uint32_t ops_off, par_off;    // byte offsets within the program
+    uint32_t prog;                // byte offset of the program in its buffer
+    uint32_t bytes;               // its length, a multiple of 16
+    int32_t only;                 // the operator of a pass that applies one, else -1
+};
+// Whether an operator can be part of a group pass.
+bool group_takes(int k, bool diag);
+// The passes that apply src[0..] in order (moved only across operators that act
+// on other positions, or across diagonal ones where both are); programs
+// appended to *progs, whose length stays a multiple of 16.
+std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std::vector<unsigned char>* progs);
+// zero: the state is taken as |0...0> and not read.
+cudaError_t launch_group(float2* psi, int n, const GroupPass& p, const unsigned char* d_progs, bool zero,
+                         cudaStream_t st, uint64_t* launches);
 
 struct BatchArgs {
     float2* states;            // n_traj consecutive states of 2^n amplitudes
     int n, n_traj;
-    const BatchBlock* blocks;
-    const uint32_t* bstart;    // n_traj + 1 block offsets
+    const GroupPass* passes;
+    const uint32_t* pstart;    // n_traj + 1 pass offsets
     const int32_t* order;      // trajectories in queue order (longest first)
-    const float* mats;
+    const unsigned char* progs;
+    const uint64_t* prog_base; // per trajectory: byte offset of its programs in progs
     unsigned int* queue;       // work counter, zero before the launch
     int* err;                  // set to 7 when the cycle budget runs out
-    unsigned long long budget; // clock64 cycles per CTA, 0 = unlimited
+    unsigned long long budget; // clock64 cycles per cluster, 0 = unlimited
 };
 
-bool make_batch_block(int n, const int* phys, int k, uint32_t mat_off, BatchBlock* b);
 cudaError_t launch_batch_evolve(const BatchArgs& a, cudaStream_t st, uint64_t* launches);
 
 // One CTA per trajectory: sample `shots` outcomes of every state (identity

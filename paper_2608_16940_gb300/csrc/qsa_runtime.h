@@ -85,6 +85,12 @@ struct PlanLayer {
     std::vector<LayerLaunch> launches;   // for the plan's layout (empty when N < 12)
 };
 
+// Consecutive blocks [b0, b1) that run as the group passes [p0, p1).
+struct PlanGroup {
+    size_t b0, b1, p0, p1;
+    uint64_t blocks = 0, diags = 0, prods = 0;   // of the passes with several blocks
+};
+
 struct qsa_plan_s {
     int n = 0;
     qsa_plan_opts opts{};
@@ -100,6 +106,11 @@ struct qsa_plan_s {
     std::vector<PlanLayer> layers;
     std::vector<unsigned char> host_layer;   // layer payloads (16-byte aligned)
     unsigned char* d_layer = nullptr;
+    // group passes for the layout L0 (GroupPass::only: a block index)
+    std::vector<PlanGroup> groups;
+    std::vector<qsa::GroupPass> gpasses;
+    std::vector<unsigned char> host_group;   // their programs
+    unsigned char* d_group = nullptr;
 };
 
 namespace qsa {
@@ -107,6 +118,13 @@ namespace qsa {
 // In-block bits: the low positions a tile of the FP32 kernels covers as one
 // contiguous run (2^11 amplitudes = 16 KiB).
 constexpr int kInBlockBits = 11;
+
+// Largest state whose plans run consecutive blocks as group passes.  Grouping
+// pays at every size (N = 25, 270 blocks of a QFT and random layers: see
+// group.cu), but it changes what a plan costs from its blocks to its passes,
+// and the learned planner scores blocks: on larger states, where it is what
+// chooses the plan, the blocks stay one pass each so that its scores hold.
+constexpr int kGroupMaxQubits = 25;
 
 qsa_status fail(qsa_status st, const std::string& msg);
 qsa_status cuda_fail(qsa_state s, cudaError_t e, const char* where);

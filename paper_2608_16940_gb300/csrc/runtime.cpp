@@ -331,7 +331,7 @@ uint64_t qsa_debug_live_allocations(void) {
 }
 
 uint64_t qsa_debug_bounds_status(void) {
-    for (uint64_t w : {bounds_word_apply(), bounds_word_layer(), bounds_word_tc()})
+    for (uint64_t w : {bounds_word_apply(), bounds_word_layer(), bounds_word_tc(), bounds_word_group()})
         if (w) return w;
     return 0;
 }
