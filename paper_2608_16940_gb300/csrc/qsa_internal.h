@@ -220,9 +220,11 @@ cudaError_t launch_reduce_z_multi(const float2* psi, int n, const uint64_t* phys
 cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double* d_partials, double* d_out,
                             cudaStream_t st, uint64_t* launches);
 
-// out[x] = |psi_{encode(x)}|^2 for logical x; d_layout = int32 L[0..n-1] on device.
-cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* d_layout, double* out,
-                                 cudaStream_t st, uint64_t* launches);
+// out[x] = |psi_{encode(x)}|^2 for logical x; layout_host = L[0..n-1].  With
+// d_norm, also the norm (FP64 sum) into *d_norm (device) via d_partials
+// (reduce_partials() doubles).
+cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout_host, double* out, double* d_partials,
+                                 double* d_norm, cudaStream_t st, uint64_t* launches);
 
 // Sampler scratch sizes and launch (see qsa_sample_counts).
 uint64_t next_pow2_u64(uint64_t v);

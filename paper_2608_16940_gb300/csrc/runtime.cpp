@@ -642,12 +642,26 @@ qsa_status qsa_state_sync(qsa_state s) {
 qsa_status qsa_probabilities_device(qsa_state s, double* out_dev, double* norm_out) {
     qsa_status st = check_state(s);
     if (st != QSA_OK) return st;
-    if (out_dev) {
-        cudaError_t e = launch_probs_logical(s->psi, s->n, s->L, out_dev, s->stream, &s->launches);
-        if (e != cudaSuccess) return cuda_fail(s, e, "probability kernel");
+    if (!out_dev) {
+        if (norm_out) return qsa_expectation_z(s, 0, norm_out);
+        cudaError_t e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "probabilities");
+        return QSA_OK;
     }
-    if (norm_out) return qsa_expectation_z(s, 0, norm_out);
-    cudaError_t e = cudaStreamSynchronize(s->stream);
+    double* d_norm = nullptr;
+    if (norm_out) {
+        st = ensure_dev(s, reinterpret_cast<void**>(&s->d_red), &s->red_cap, sizeof(double) * (reduce_partials() + 8));
+        if (st != QSA_OK) return st;
+        d_norm = s->d_red + reduce_partials();
+    }
+    cudaError_t e = launch_probs_logical(s->psi, s->n, s->L, out_dev, s->d_red, d_norm, s->stream, &s->launches);
+    if (e != cudaSuccess) return cuda_fail(s, e, "probability kernel");
+    if (norm_out) {
+        e = cudaMemcpyAsync(norm_out, d_norm, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "probability norm");
+        return sync_and_check(s, "probabilities");
+    }
+    e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "probabilities");
     return QSA_OK;
 }
@@ -655,26 +669,31 @@ qsa_status qsa_probabilities_device(qsa_state s, double* out_dev, double* norm_o
 qsa_status qsa_probabilities(qsa_state s, double* out_host, double* norm_out) {
     qsa_status st = check_state(s);
     if (st != QSA_OK) return st;
-    if (out_host) {
-        const size_t bytes = sizeof(double) << s->n;
-        double* tmp = nullptr;
-        cudaError_t e = dev_malloc(&tmp, bytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(QSA_E_NOMEM, "cudaMalloc of the probability buffer failed");
-        }
-        e = launch_probs_logical(s->psi, s->n, s->L, tmp, s->stream, &s->launches);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, tmp, bytes, cudaMemcpyDeviceToHost, s->stream);
-        if (e != cudaSuccess) {
-            dev_free(tmp);
-            return cuda_fail(s, e, "probabilities");
-        }
-        st = sync_and_check(s, "probabilities");
-        dev_free(tmp);
+    if (!out_host) return norm_out ? qsa_expectation_z(s, 0, norm_out) : QSA_OK;
+    double* d_norm = nullptr;
+    if (norm_out) {
+        st = ensure_dev(s, reinterpret_cast<void**>(&s->d_red), &s->red_cap, sizeof(double) * (reduce_partials() + 8));
         if (st != QSA_OK) return st;
+        d_norm = s->d_red + reduce_partials();
     }
-    if (norm_out) return qsa_expectation_z(s, 0, norm_out);
-    return QSA_OK;
+    const size_t bytes = sizeof(double) << s->n;
+    double* tmp = nullptr;
+    cudaError_t e = dev_malloc(&tmp, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(QSA_E_NOMEM, "cudaMalloc of the probability buffer failed");
+    }
+    e = launch_probs_logical(s->psi, s->n, s->L, tmp, s->d_red, d_norm, s->stream, &s->launches);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, tmp, bytes, cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess && norm_out)
+        e = cudaMemcpyAsync(norm_out, d_norm, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
+    if (e != cudaSuccess) {
+        dev_free(tmp);
+        return cuda_fail(s, e, "probabilities");
+    }
+    st = sync_and_check(s, "probabilities");
+    dev_free(tmp);
+    return st;
 }
 
 qsa_status qsa_sample_counts(qsa_state s, uint64_t shots, uint64_t seed, uint64_t* outcomes, uint64_t* counts,
