@@ -315,6 +315,7 @@ template <> struct ApplyCfg<3> { static constexpr int T = 11, R = 8, S = 2; stat
 // (2^11 left half of the CTA idle in the compute phase), two stages so that
 // three CTAs fit an SM (faster than three stages at two CTAs)
 template <> struct ApplyCfg<4> { static constexpr int T = 12, R = 16, S = 2; static constexpr bool SWZ = true; };
+// k = 5, 6: states below one tile of 2^12 amplitudes only (launch_apply_fp32)
 template <> struct ApplyCfg<5> { static constexpr int T = 12, R = 8, S = 2; static constexpr bool SWZ = false; };
 template <> struct ApplyCfg<6> { static constexpr int T = 12, R = 8, S = 2; static constexpr bool SWZ = false; };
 
@@ -432,6 +433,231 @@ cudaError_t launch_apply_k(float2* psi, int n, const int* phys, const float* d_m
     uint64_t grid = static_cast<uint64_t>(num_sms()) * occ;
     if (grid > g.ntiles) grid = g.ntiles;
     kern<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(a);
+    ++*launches;
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Apply, k = 5 and 6
+// ---------------------------------------------------------------------------
+// A 2^k x 2^k complex matrix on the tile's 2^(12-k) groups: bound by the FP32
+// pipe (128 / 256 real FMAs per amplitude against 16 bytes), so what matters is
+// how many FMAs each shared-memory load feeds.  A team of 128 threads takes a
+// tile; a thread accumulates 8 rows x 4 groups, so that one column step is 128
+// FMAs on 4 state loads (one amplitude of each group) and 4 matrix loads of 16
+// bytes (two rows' entries).  Scalar FMAs: a packed pair reads six registers and
+// issues every third cycle (84 FMAs per clock and SM with operands that change,
+// 95 with one held, measured), scalar ones reach 104.  The two half-warps of a
+// k = 6 team take neighbouring row pairs and read neighbouring 16-byte units.
+// Three teams per CTA, one CTA per SM, share the matrix; two stages per team
+// keep the next tile's copies under the arithmetic (with two teams 5 % slower,
+// four leave 128 registers a thread and spill).  The matrix's index bits are put
+// in ascending position order, so a target on position 0 (P0) is column bit 0
+// and both columns of a pair come in one 16-byte load.  Outputs go back to the
+// stage in place and leave in address order.
+// N = 26, random targets, k = 5 / 6: 0.48 / 0.985 ms with one row of the matrix
+// read per group (the kernel above, 8 rows per thread), 0.360 / 0.647 ms here,
+// 0.59 / 0.66 of 128 FMAs per clock and SM.
+constexpr int kWideT = 12, kWideTeam = 128, kWideTeams = 3, kWideR = 8, kWideG = 4;
+constexpr int kWideChunks = (1 << (kWideT - 1)) / kWideTeam;   // 16-byte units per thread
+
+struct WideArgs {
+    float2* psi;
+    uint64_t ntiles;
+    int m, nx;
+    int xpos[6];
+    const float* mat;
+    int src[6];                    // sorted index bit i is the operator's index bit src[i]
+    uint64_t poff[kWideT];         // global offset and slot of tile bit b
+    uint16_t pslot[kWideT];
+    uint64_t goff[kWideChunks];    // global offset and slot of tile-local 256 k
+    uint16_t gslot[kWideChunks];
+    uint16_t sloff[64];            // slot of column c (sorted index)
+    uint16_t fslot[8];             // slot of each non-target tile bit, ascending
+};
+
+template <int K>
+__host__ __device__ constexpr size_t wide_smem() {
+    return sizeof(float2) * 2 * kWideTeams * (1 << kWideT) + (8u << (2 * K));
+}
+
+template <int K, bool P0>
+__global__ void __launch_bounds__(kWideTeam * kWideTeams, 1) k_apply_wide(const __grid_constant__ WideArgs a) {
+    constexpr int D = 1 << K, NRB = D / kWideR, NF = kWideT - K;
+    static_assert((D / kWideR) * (1 << NF) / kWideG == kWideTeam, "a team covers the tile");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int team = threadIdx.x / kWideTeam, tid = threadIdx.x % kWideTeam;
+    float2* stage = reinterpret_cast<float2*>(smem_raw) + team * 2 * (1 << kWideT);
+    float2* Mt = reinterpret_cast<float2*>(smem_raw + sizeof(float2) * 2 * kWideTeams * (1 << kWideT));   // [column][row]
+
+    const float2* gm = reinterpret_cast<const float2*>(a.mat);
+    for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
+        const int r = i & (D - 1), c = i >> K;
+        int ro = 0, co = 0;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            ro |= ((r >> j) & 1) << a.src[j];
+            co |= ((c >> j) & 1) << a.src[j];
+        }
+        Mt[i] = gm[ro * D + co];
+    }
+    // this thread's copies: tile-local 2 tid + 256 k
+    uint64_t gld = 0;
+    int sld = 0;
+#pragma unroll
+    for (int b = 0; b < 7; ++b)
+        if ((tid >> b) & 1) {
+            gld |= a.poff[b + 1];
+            sld ^= a.pslot[b + 1];
+        }
+    // row block and groups of this thread: the lowest lane bits are groups
+    constexpr int LB = NF - 2;                       // thread bits that choose groups (two more: its four groups)
+    const int rb = tid >> LB;
+    const int rslot = a.sloff[2 * rb];               // of its first row
+    int gs[kWideG];
+    gs[0] = 0;
+#pragma unroll
+    for (int i = 0; i < LB; ++i)
+        if ((tid >> i) & 1) gs[0] ^= a.fslot[i];
+    gs[1] = gs[0] ^ a.fslot[LB];
+    gs[2] = gs[0] ^ a.fslot[LB + 1];
+    gs[3] = gs[1] ^ a.fslot[LB + 1];
+    __syncthreads();
+
+    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kWideTeams;
+    const uint64_t limit = a.ntiles << kWideT;
+    auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kWideTeam) : "memory"); };
+    auto tile_at = [&](uint64_t t) {
+        uint64_t base = t << a.m;
+#pragma unroll
+        for (int e = 0; e < 6; ++e)
+            if (e < a.nx) base = insert_zero(base, a.xpos[e]);
+        return base | gld;
+    };
+    auto load = [&](uint64_t base, float2* to) {
+#pragma unroll
+        for (int k = 0; k < kWideChunks; ++k)
+            if (dbg::in_bounds(base | a.goff[k], 2, limit, 7)) cp_async16(to + (sld ^ a.gslot[k]), a.psi + (base | a.goff[k]));
+    };
+    const uint64_t t0 = blockIdx.x + static_cast<uint64_t>(gridDim.x) * team;
+    uint64_t next = tile_at(t0);
+    if (t0 < a.ntiles) load(next, stage);
+    cp_async_commit();
+    int cur = 0;
+    for (uint64_t t = t0; t < a.ntiles; t += stride) {
+        const uint64_t base = next;
+        float2* st = stage + cur * (1 << kWideT);
+        cur ^= 1;
+        cp_async_wait<0>();
+        team_sync();   // the tile has landed, and the team has written the other stage's tile out
+        next = tile_at(t + stride);
+        if (t + stride < a.ntiles) load(next, stage + cur * (1 << kWideT));
+        cp_async_commit();
+        float2 acc[kWideR][kWideG];
+#pragma unroll
+        for (int r = 0; r < kWideR; ++r)
+#pragma unroll
+            for (int g = 0; g < kWideG; ++g) acc[r][g] = make_float2(0.f, 0.f);
+        auto column = [&](const float4* m, const float2 (&v)[kWideG]) {
+#pragma unroll
+            for (int r = 0; r < kWideR; r += 2) {
+                const float4 e = m[NRB * (r >> 1)];   // rows 2 (rb + NRB r / 2) and the next
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r][g].x = fmaf(e.x, v[g].x, acc[r][g].x);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r][g].y = fmaf(e.x, v[g].y, acc[r][g].y);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r][g].x = fmaf(-e.y, v[g].y, acc[r][g].x);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r][g].y = fmaf(e.y, v[g].x, acc[r][g].y);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].x = fmaf(e.z, v[g].x, acc[r + 1][g].x);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].y = fmaf(e.z, v[g].y, acc[r + 1][g].y);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].x = fmaf(-e.w, v[g].y, acc[r + 1][g].x);
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].y = fmaf(e.w, v[g].x, acc[r + 1][g].y);
+            }
+        };
+        // eight columns at a time: their low bits' slots enter from the parameter bank
+        constexpr int kWC = 8;
+#pragma unroll 1
+        for (int o = 0; o < D; o += kWC) {
+            const int hi = a.sloff[o];
+            const float4* m = reinterpret_cast<const float4*>(Mt + o * D) + rb;
+#pragma unroll
+            for (int c = 0; c < kWC; c += 2) {
+                float2 v0[kWideG], v1[kWideG];
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) {
+                    if constexpr (P0) {
+                        const float4 f = *reinterpret_cast<const float4*>(st + (gs[g] ^ hi ^ a.sloff[c]));
+                        v0[g] = make_float2(f.x, f.y);
+                        v1[g] = make_float2(f.z, f.w);
+                    } else {
+                        v0[g] = st[gs[g] ^ hi ^ a.sloff[c]];
+                        v1[g] = st[gs[g] ^ hi ^ a.sloff[c + 1]];
+                    }
+                }
+                column(m + c * (D / 2), v0);
+                column(m + (c + 1) * (D / 2), v1);
+            }
+        }
+        team_sync();   // every input of the tile has been read
+#pragma unroll
+        for (int r = 0; r < kWideR; ++r) {
+            const int so = rslot ^ a.sloff[2 * NRB * (r >> 1) + (r & 1)];
+#pragma unroll
+            for (int g = 0; g < kWideG; ++g) st[gs[g] ^ so] = acc[r][g];
+        }
+        team_sync();
+#pragma unroll
+        for (int k = 0; k < kWideChunks; ++k)
+            if (dbg::in_bounds(base | a.goff[k], 2, limit, 8))
+                __stcs(reinterpret_cast<float4*>(a.psi + (base | a.goff[k])),
+                       *reinterpret_cast<const float4*>(st + (sld ^ a.gslot[k])));
+    }
+    cp_async_wait<0>();
+}
+
+template <int K>
+cudaError_t launch_apply_wide(float2* psi, int n, const int* phys, const float* d_mat, cudaStream_t st,
+                              uint64_t* launches) {
+    TileGeom g;
+    if (!make_geom(n, phys, K, kWideT, &g) || g.T != kWideT) return cudaErrorInvalidValue;
+    WideArgs a{};
+    a.psi = psi;
+    a.ntiles = g.ntiles;
+    a.m = g.m;
+    a.nx = g.nx;
+    for (int e = 0; e < 6; ++e) a.xpos[e] = g.xpos[e];
+    a.mat = d_mat;
+    int tl[6], tls[6];
+    uint8_t fv[16];
+    local_targets(g, phys, K, tl, tls);
+    for (int i = 0; i < K; ++i) a.src[i] = static_cast<int>(std::find(tl, tl + K, tls[i]) - tl);
+    stage_slots(g.T, tls, K, fv);
+    int nf = 0;
+    for (int b = 0; b < kWideT; ++b) {
+        a.poff[b] = 1ull << (b < g.m ? b : g.xpos[b - g.m]);
+        a.pslot[b] = static_cast<uint16_t>((1 << b) ^ (b >= 4 ? fv[b] << 1 : 0));
+        if (std::find(tls, tls + K, b) == tls + K) a.fslot[nf++] = a.pslot[b];
+    }
+    for (int k = 0; k < kWideChunks; ++k)
+        for (int b = 0; b < 4; ++b)
+            if ((k >> b) & 1) {
+                a.goff[k] |= a.poff[8 + b];
+                a.gslot[k] = static_cast<uint16_t>(a.gslot[k] ^ a.pslot[8 + b]);
+            }
+    for (int c = 0; c < (1 << K); ++c)
+        for (int j = 0; j < K; ++j)
+            if ((c >> j) & 1) a.sloff[c] = static_cast<uint16_t>(a.sloff[c] ^ a.pslot[tls[j]]);
+    auto kern = tls[0] == 0 ? k_apply_wide<K, true> : k_apply_wide<K, false>;
+    cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(wide_smem<K>()));
+    if (e != cudaSuccess) return e;
+    const uint64_t grid = std::min<uint64_t>(g.ntiles, static_cast<uint64_t>(num_sms()));
+    kern<<<static_cast<unsigned>(grid), kWideTeam * kWideTeams, wide_smem<K>(), st>>>(a);
     ++*launches;
     return cudaGetLastError();
 }
@@ -760,8 +986,13 @@ cudaError_t launch_apply_fp32(float2* psi, int n, const int* phys, int k, const 
         case 2: return launch_apply_k<2>(psi, n, phys, d_mat, st, launches);
         case 3: return launch_apply_k<3>(psi, n, phys, d_mat, st, launches);
         case 4: return launch_apply_k<4>(psi, n, phys, d_mat, st, launches);
-        case 5: return launch_apply_k<5>(psi, n, phys, d_mat, st, launches);
-        case 6: return launch_apply_k<6>(psi, n, phys, d_mat, st, launches);
+        // states below one tile keep the kernel that takes any tile size
+        case 5:
+            return n >= kWideT ? launch_apply_wide<5>(psi, n, phys, d_mat, st, launches)
+                               : launch_apply_k<5>(psi, n, phys, d_mat, st, launches);
+        case 6:
+            return n >= kWideT ? launch_apply_wide<6>(psi, n, phys, d_mat, st, launches)
+                               : launch_apply_k<6>(psi, n, phys, d_mat, st, launches);
         default: return cudaErrorInvalidValue;
     }
 }
