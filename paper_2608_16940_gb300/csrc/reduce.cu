@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <utility>
 
 #include "qsa_device.cuh"
 #include "qsa_internal.h"
@@ -117,9 +118,12 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_z_multi(const float4* __
     }
 }
 
-// Fixed-order sum of the partials (deterministic for a given grid).
+// Fixed-order sum of the partials (deterministic for a given grid); CTA m sums
+// partials[m n ..) into out[m].
 __global__ void k_finalize_sum(const double* __restrict__ partials, int n, double* __restrict__ out) {
     __shared__ double sh[1024];
+    partials += static_cast<size_t>(blockIdx.x) * n;
+    out += blockIdx.x;
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
     sh[threadIdx.x] = v;
@@ -516,6 +520,19 @@ __global__ void k_scan_add(uint64_t* __restrict__ cum, uint64_t n, const uint64_
         cum[i] += parts[i / kScanSeg - 1];
 }
 
+// Shot s's draw u = floor(r * total / 2^64) and its block: the first with cum > u.
+__device__ __forceinline__ uint64_t draw_u(uint64_t s, uint64_t stream_id, uint64_t seed, uint64_t total) {
+    return __umul64hi(philox4x64_10_w0(s, stream_id, 0, 0, seed, 0), total);
+}
+__device__ __forceinline__ uint64_t find_block(const uint64_t* __restrict__ cum, uint64_t nblocks, uint64_t u) {
+    uint64_t lo = 0, hi = nblocks - 1;
+    while (lo < hi) {
+        const uint64_t mid = lo + ((hi - lo) >> 1);
+        if (cum[mid] > u) hi = mid; else lo = mid + 1;
+    }
+    return lo;
+}
+
 // One warp per shot: draw u, find the block (first cum > u), then the amplitude.
 __global__ void k_draw(const float2* __restrict__ psi, const uint64_t* __restrict__ cum, uint64_t nblocks, int bsz,
                        Layout lay, uint64_t shots, uint64_t seed, uint64_t stream_id, uint64_t* __restrict__ keys) {
@@ -527,15 +544,8 @@ __global__ void k_draw(const float2* __restrict__ psi, const uint64_t* __restric
         if (lane == 0) keys[s] = 0;
         return;
     }
-    const uint64_t r = philox4x64_10_w0(s, stream_id, 0, 0, seed, 0);
-    const uint64_t u = __umul64hi(r, total);  // floor(r * total / 2^64)
-    // first block b with cum[b] > u
-    uint64_t lo = 0, hi = nblocks - 1;
-    while (lo < hi) {
-        uint64_t mid = lo + ((hi - lo) >> 1);
-        if (cum[mid] > u) hi = mid; else lo = mid + 1;
-    }
-    const uint64_t b = lo;
+    const uint64_t u = draw_u(s, stream_id, seed, total);
+    const uint64_t b = find_block(cum, nblocks, u);
     const uint64_t ub = u - (b ? cum[b - 1] : 0);
     // lane l covers amplitudes [l*per, (l+1)*per) of the block
     const int per = (bsz + 31) >> 5;
@@ -561,6 +571,250 @@ __global__ void k_draw(const float2* __restrict__ psi, const uint64_t* __restric
         const uint64_t y = b * static_cast<uint64_t>(bsz) + static_cast<uint64_t>(lane * per + j);
         keys[s] = decode_physical(y, lay);
     }
+}
+
+// Many shots on blocks of 1024 amplitudes: the shots are sorted by block first
+// (key: block << kShotBits | shot), so that a block's 8 KiB are read once for
+// all of its shots instead of once per shot.
+constexpr int kShotBits = 26;   // shots are at most 2^26, blocks at most 2^24
+
+__global__ void __launch_bounds__(256) k_draw_blocks(const uint64_t* __restrict__ cum, uint64_t nblocks, uint64_t shots,
+                                                     uint64_t seed, uint64_t stream_id, uint64_t* __restrict__ out) {
+    const uint64_t s = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (s >= shots) return;
+    const uint64_t total = cum[nblocks - 1];
+    const uint64_t b = total ? find_block(cum, nblocks, draw_u(s, stream_id, seed, total)) : 0;
+    out[s] = (b << kShotBits) | s;
+}
+
+// A warp takes `per` consecutive shots of the sorted list; for each block among
+// them it forms the prefix of the block's 1024 weights in shared memory (lanes
+// over 16-byte pairs, 64 amplitudes a step) and every lane whose shot lies in
+// the block searches it.
+constexpr int kResolveWarps = 4;
+
+__global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float4* __restrict__ psi2,
+                                                                      const uint64_t* __restrict__ cum,
+                                                                      uint64_t nblocks, const __grid_constant__ Layout lay,
+                                                                      const uint64_t* __restrict__ draws, uint64_t shots,
+                                                                      uint64_t seed, uint64_t stream_id, int per,
+                                                                      uint64_t* __restrict__ keys) {
+    __shared__ __align__(16) uint64_t pre[kResolveWarps][1024];   // inclusive prefixes
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint64_t i = (static_cast<uint64_t>(blockIdx.x) * kResolveWarps + w) * per + lane;
+    const bool valid = lane < per && i < shots;
+    const uint64_t total = cum[nblocks - 1];
+    const uint64_t d = valid ? draws[i] : 0;
+    const uint64_t b = d >> kShotBits;
+    uint64_t ub = 0;
+    if (valid && total) ub = draw_u(d & ((1ull << kShotBits) - 1), stream_id, seed, total) - (b ? cum[b - 1] : 0);
+    bool open = valid && total;
+    uint64_t key = 0;
+    for (;;) {
+        const unsigned left = __ballot_sync(0xffffffffu, open);
+        if (!left) break;
+        const uint64_t bb = __shfl_sync(0xffffffffu, b, __ffs(left) - 1);
+        const float4* p = psi2 + bb * 512 + lane;
+        float4 a[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) a[k] = __ldg(p + 32 * k);
+        uint64_t run = 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const uint64_t w0 = sq_fixed60(a[k].x) + sq_fixed60(a[k].y), w1 = sq_fixed60(a[k].z) + sq_fixed60(a[k].w);
+            const uint64_t incl = warp_incl_scan_u64(w0 + w1) + run;
+            *reinterpret_cast<ulonglong2*>(&pre[w][2 * (lane + 32 * k)]) = make_ulonglong2(incl - w1, incl);
+            run = __shfl_sync(0xffffffffu, incl, 31);
+        }
+        __syncwarp();
+        if (open && b == bb) {
+            int lo = 0, hi = 1023;   // the first prefix above ub (the last one is: ub < cum[b] - cum[b - 1])
+#pragma unroll
+            for (int k = 0; k < 10; ++k) {
+                const int mid = (lo + hi) >> 1;
+                if (pre[w][mid] > ub) hi = mid; else lo = mid + 1;
+            }
+            key = decode_physical(bb * 1024 + static_cast<uint64_t>(lo), lay);
+            open = false;
+        }
+        __syncwarp();
+    }
+    if (valid) keys[i] = key;
+}
+
+// Stable radix sort of 64-bit keys by one 8-bit digit (least significant digit
+// first): per-tile digit counts (hist[digit][tile]), their prefixes per digit,
+// and the scatter, where a warp ranks its keys by matching digits 32 at a time.
+// Three launches a digit against (log2 P)^2 / 2 for a whole bitonic network:
+// 200 000 26-bit outcomes 542 us in 171 global bitonic steps, 65 us in the 12
+// launches here; their run-length encoding 294 us in one CTA, 17 us in tiles.
+constexpr int kRadixThreads = 256, kRadixPer = 8, kRadixTile = kRadixThreads * kRadixPer;
+
+__global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint64_t* __restrict__ keys, uint64_t n, int shift,
+                                                               uint32_t ntiles, uint32_t* __restrict__ hist) {
+    __shared__ uint32_t h[256];
+    h[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j) {
+        const uint64_t i = static_cast<uint64_t>(blockIdx.x) * kRadixTile + j * kRadixThreads + threadIdx.x;
+        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
+    }
+    __syncthreads();
+    hist[static_cast<uint64_t>(threadIdx.x) * ntiles + blockIdx.x] = h[threadIdx.x];
+}
+
+// CTA d: exclusive prefixes of digit d's tile counts in place, their sum to totals[d].
+__global__ void __launch_bounds__(kRadixThreads) k_radix_scan(uint32_t* __restrict__ hist, uint32_t ntiles,
+                                                               uint32_t* __restrict__ totals) {
+    __shared__ uint32_t ws[8];
+    uint32_t* h = hist + static_cast<uint64_t>(blockIdx.x) * ntiles;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t run = 0;
+    for (uint32_t t0 = 0; t0 < ntiles; t0 += kRadixThreads) {
+        const uint32_t t = t0 + threadIdx.x;
+        const uint32_t v = t < ntiles ? h[t] : 0;
+        uint32_t inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += x;
+        }
+        if (lane == 31) ws[w] = inc;
+        __syncthreads();
+        uint32_t before = run, all = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k < w) before += ws[k];
+            all += ws[k];
+        }
+        if (t < ntiles) h[t] = before + inc - v;
+        run += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = run;
+}
+
+__global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(const uint64_t* __restrict__ in, uint64_t n, int shift,
+                                                                  uint32_t ntiles, const uint32_t* __restrict__ hist,
+                                                                  const uint32_t* __restrict__ totals,
+                                                                  uint64_t* __restrict__ out) {
+    __shared__ uint32_t cnt[kRadixThreads / 32][256];
+    __shared__ uint32_t ws[8];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    for (int i = tid; i < 8 * 256; i += kRadixThreads) cnt[i >> 8][i & 255] = 0;
+    // digit tid's first place: every smaller digit, then this digit's tiles before
+    const uint32_t tot = totals[tid];
+    uint32_t inc = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane == 31) ws[w] = inc;
+    __syncthreads();
+    uint32_t place = inc - tot + hist[static_cast<uint64_t>(tid) * ntiles + blockIdx.x];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (k < w) place += ws[k];
+    // warp w ranks its 256 keys in order, 32 at a time
+    const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * kRadixTile + w * 32 * kRadixPer + lane;
+    uint64_t key[kRadixPer];
+    uint32_t rank[kRadixPer];
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j) key[j] = i0 + 32 * j < n ? in[i0 + 32 * j] : 0;
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j) {
+        const bool valid = i0 + 32 * j < n;
+        const unsigned vm = __ballot_sync(0xffffffffu, valid);
+        const uint32_t dg = static_cast<uint32_t>(key[j] >> shift) & 255u;
+        unsigned peers = 0;
+        if (valid) {
+            peers = __match_any_sync(vm, dg);
+            rank[j] = cnt[w][dg] + __popc(peers & ((1u << lane) - 1u));
+        }
+        __syncwarp();
+        if (valid && lane == __ffs(peers) - 1) cnt[w][dg] += __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint32_t c = cnt[k][tid];
+        cnt[k][tid] = place;
+        place += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j)
+        if (i0 + 32 * j < n) out[cnt[w][static_cast<uint32_t>(key[j] >> shift) & 255u] + rank[j]] = key[j];
+}
+
+// Run-length encoding of sorted keys in tiles: heads per tile, (their prefix by
+// k_scan_inclusive,) the distinct keys and where their runs start, the lengths.
+__device__ __forceinline__ uint32_t tile_heads(const uint64_t* __restrict__ keys, uint64_t n, uint64_t i0, uint32_t* flags) {
+    uint32_t c = 0, f = 0;
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j) {   // this thread's kRadixPer consecutive keys
+        const uint64_t i = i0 + j;
+        const uint32_t head = i < n && (i == 0 || keys[i] != keys[i - 1]) ? 1u : 0u;
+        f |= head << j;
+        c += head;
+    }
+    *flags = f;
+    return c;
+}
+
+__global__ void __launch_bounds__(kRadixThreads) k_rle_heads(const uint64_t* __restrict__ keys, uint64_t n,
+                                                              uint64_t* __restrict__ tile_count) {
+    __shared__ uint32_t ws[8];
+    uint32_t f;
+    uint32_t c = tile_heads(keys, n, static_cast<uint64_t>(blockIdx.x) * kRadixTile + threadIdx.x * kRadixPer, &f);
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0;
+        for (int k = 0; k < 8; ++k) t += ws[k];
+        tile_count[blockIdx.x] = t;
+    }
+}
+
+__global__ void __launch_bounds__(kRadixThreads) k_rle_write(const uint64_t* __restrict__ keys, uint64_t n,
+                                                              const uint64_t* __restrict__ tile_incl,
+                                                              uint64_t* __restrict__ out_keys, uint64_t* __restrict__ starts,
+                                                              uint64_t* __restrict__ n_distinct) {
+    __shared__ uint32_t ws[8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * kRadixTile + threadIdx.x * kRadixPer;
+    uint32_t f;
+    const uint32_t c = tile_heads(keys, n, i0, &f);
+    uint32_t inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane == 31) ws[w] = inc;
+    __syncthreads();
+    uint64_t pos = (blockIdx.x ? tile_incl[blockIdx.x - 1] : 0) + inc - c;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (k < w) pos += ws[k];
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j)
+        if ((f >> j) & 1u) {
+            out_keys[pos] = keys[i0 + j];
+            starts[pos++] = i0 + j;
+        }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_distinct = tile_incl[blockIdx.x];
+}
+
+__global__ void k_rle_counts(const uint64_t* __restrict__ starts, uint64_t n, const uint64_t* __restrict__ n_distinct,
+                             uint64_t* __restrict__ counts) {
+    const uint64_t nd = *n_distinct;
+    const uint64_t d = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (d < nd) counts[d] = (d + 1 < nd ? starts[d + 1] : n) - starts[d];
 }
 
 __global__ void k_fill_u64(uint64_t* a, uint64_t from, uint64_t to, uint64_t v) {
@@ -590,20 +844,6 @@ __global__ void __launch_bounds__(1024) k_bitonic_smem(uint64_t* keys, int P) {
         }
     }
     for (int i = threadIdx.x; i < P; i += blockDim.x) keys[i] = sk[i];
-}
-
-__global__ void k_bitonic_step(uint64_t* keys, uint64_t P, uint64_t j, uint64_t k) {
-    uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= P) return;
-    uint64_t l = i ^ j;
-    if (l > i) {
-        bool up = (i & k) == 0;
-        uint64_t a = keys[i], c = keys[l];
-        if ((a > c) == up) {
-            keys[i] = c;
-            keys[l] = a;
-        }
-    }
 }
 
 // Run-length encode the sorted keys[0..n-1] with one CTA: distinct keys and
@@ -644,6 +884,10 @@ inline uint64_t next_pow2(uint64_t v) {
     while (p < v) p <<= 1;
     return p;
 }
+
+// Sorts of up to this many keys run in one CTA's shared memory (a launch or
+// three cheaper than the radix sort's nine to fifteen).
+constexpr uint64_t kSortSmemMax = 4096;
 
 // Batched sampler: CTA t samples state t (identity layout) with Philox stream
 // id t.  Shared memory: cum[nblocks] (uint64) then keys[P] (uint32).
@@ -853,8 +1097,8 @@ cudaError_t launch_reduce_z_multi(const float2* psi, int n, const uint64_t* phys
     zm.n = nmasks;
     for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
     k_reduce_z_multi<<<nb, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), npairs, zm, d_partials);
-    for (int m = 0; m < nmasks; ++m) k_finalize_sum<<<1, 1024, 0, st>>>(d_partials + m * nb, nb, d_out + m);
-    *launches += 1 + nmasks;
+    k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_partials, nb, d_out);
+    *launches += 2;
     return cudaGetLastError();
 }
 
@@ -984,17 +1228,18 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
         if (nb > cap) nb = cap;
         kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, cum,
                                                                  zm, d_zpartials);
-        for (int m = 0; m < nmasks; ++m)
-            k_finalize_sum<<<1, 1024, 0, st>>>(d_zpartials + m * nb, static_cast<int>(nb), d_zout + m);
-        *launches += nmasks;
+        if (nmasks > 0) {
+            k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_zpartials, static_cast<int>(nb), d_zout);
+            ++*launches;
+        }
     } else if (nmasks > 0) {
         ZMasks zm{};
         zm.n = nmasks;
         for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
         const int nb = reduce_partials();
         k_block_weights_z<<<nb, kRedThreads, 0, st>>>(psi, nblocks, bsz, cum, zm, d_zpartials);
-        for (int m = 0; m < nmasks; ++m) k_finalize_sum<<<1, 1024, 0, st>>>(d_zpartials + m * nb, nb, d_zout + m);
-        *launches += nmasks;
+        k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_zpartials, nb, d_zout);
+        ++*launches;
     } else {
         k_block_weights<<<static_cast<unsigned>((nblocks + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, nblocks, bsz,
                                                                                                 cum);
@@ -1012,26 +1257,63 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
     } else {
         k_scan_inclusive<<<1, 1024, 0, st>>>(cum, nblocks);
     }
-    k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
-                                                                                 seed, stream_id, keys);
-    *launches += 3;
-    if (P > shots) {
-        k_fill_u64<<<static_cast<unsigned>((P - shots + 255) / 256), 256, 0, st>>>(keys, shots, P, ~0ull);
-        ++*launches;
-    }
-    if (P <= 4096) {
+    if (P <= kSortSmemMax) {
+        k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
+                                                                                     seed, stream_id, keys);
+        if (P > shots) {
+            k_fill_u64<<<static_cast<unsigned>((P - shots + 255) / 256), 256, 0, st>>>(keys, shots, P, ~0ull);
+            ++*launches;
+        }
         k_bitonic_smem<<<1, 1024, sizeof(uint64_t) * P, st>>>(keys, static_cast<int>(P));
-        ++*launches;
-    } else {
-        const unsigned nb = static_cast<unsigned>((P + 255) / 256);
-        for (uint64_t k = 2; k <= P; k <<= 1)
-            for (uint64_t j = k >> 1; j > 0; j >>= 1) {
-                k_bitonic_step<<<nb, 256, 0, st>>>(keys, P, j, k);
-                ++*launches;
-            }
+        k_rle<<<1, 1024, 0, st>>>(keys, shots, d_out_keys, starts, d_out_counts, d_n_distinct);
+        *launches += 5;
+        return cudaGetLastError();
     }
-    k_rle<<<1, 1024, 0, st>>>(keys, shots, d_out_keys, starts, d_out_counts, d_n_distinct);
-    ++*launches;
+    // Many shots: radix sorts between the arrays at hand (the digit counts go
+    // where the outcome counts end up).  The outcomes must end in `keys`.
+    const uint32_t ntiles = static_cast<uint32_t>((shots + kRadixTile - 1) / kRadixTile);
+    uint32_t* hist = reinterpret_cast<uint32_t*>(d_out_counts);
+    uint32_t* totals = hist + 256ull * ntiles;
+    auto sort = [&](uint64_t* from, uint64_t* other, int lo, int bits) {   // returns where the keys end
+        for (int sh = 0; sh < bits; sh += 8) {
+            k_radix_hist<<<ntiles, kRadixThreads, 0, st>>>(from, shots, lo + sh, ntiles, hist);
+            k_radix_scan<<<256, kRadixThreads, 0, st>>>(hist, ntiles, totals);
+            k_radix_scatter<<<ntiles, kRadixThreads, 0, st>>>(from, shots, lo + sh, ntiles, hist, totals, other);
+            std::swap(from, other);
+            *launches += 3;
+        }
+        return from;
+    };
+    const bool odd = ((n + 7) / 8) & 1;
+    uint64_t* first = odd ? d_out_keys : keys;    // the unsorted outcomes
+    uint64_t* second = odd ? keys : d_out_keys;
+    // Grouping by block costs a sort of the shots (about 40 us of launches) and saves about 4 ns a shot
+    // while blocks share shots: N = 26, 10 000 / 30 000 / 200 000 shots 350 / 440 / 790 us grouped,
+    // 324 / 441 / 1327 us shot by shot (whole calls); N = 28, 30 000 / 100 000: 697 / 930 and 671 / 1036.
+    if (bsz == 1024 && shots >= std::max<uint64_t>(16384, nblocks / 4)) {
+        uint64_t* d = starts;
+        k_draw_blocks<<<static_cast<unsigned>((shots + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, seed, stream_id, d);
+        d = sort(d, second, kShotBits, n - 10);
+        // shots per warp: few when most lie in blocks of their own, which a warp reads one after another
+        // (N = 24, 30 000 shots: 325 us with 8, 360 with 32), many when they share blocks (N = 12,
+        // 200 000: 255 and 207)
+        const int per = shots >= 8 * nblocks ? 32 : shots >= 3 * nblocks ? 16 : 8;
+        const uint64_t cta = static_cast<uint64_t>(per) * kResolveWarps;
+        k_draw_resolve<<<static_cast<unsigned>((shots + cta - 1) / cta), 32 * kResolveWarps, 0, st>>>(
+            reinterpret_cast<const float4*>(psi), cum, nblocks, lay, d, shots, seed, stream_id, per, first);
+        *launches += 2;
+    } else {
+        k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
+                                                                                     seed, stream_id, first);
+        ++*launches;
+    }
+    sort(first, second, 0, n);
+    uint64_t* tiles = d_out_counts;
+    k_rle_heads<<<ntiles, kRadixThreads, 0, st>>>(keys, shots, tiles);
+    k_scan_inclusive<<<1, 1024, 0, st>>>(tiles, ntiles);
+    k_rle_write<<<ntiles, kRadixThreads, 0, st>>>(keys, shots, tiles, d_out_keys, starts, d_n_distinct);
+    k_rle_counts<<<static_cast<unsigned>((shots + 255) / 256), 256, 0, st>>>(starts, shots, d_n_distinct, d_out_counts);
+    *launches += 6;
     return cudaGetLastError();
 }
 
