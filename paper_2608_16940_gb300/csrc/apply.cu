@@ -11,8 +11,8 @@
 //           amplitudes that differ only in the target bits,
 //           psi'[x|spread(r)] = sum_c G[r][c] psi[x|spread(c)];
 //   permute (§IV-D, Lemma "distributed promotion swap" with the rank bits read
-//           as out-of-block bits): psi'[tau(y)] = psi[y] for a product tau of
-//           disjoint bit transpositions.
+//           as out-of-block bits): psi'[tau(y)] = psi[y] for a permutation tau
+//           of the bit positions, in as few passes as its cycles allow.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,6 +20,7 @@
 #include <map>
 #include <mutex>
 #include <utility>
+#include <vector>
 
 #include "qsa_bounds.cuh"
 #include "qsa_device.cuh"
@@ -835,59 +836,74 @@ __global__ void __launch_bounds__(kThreads) k_apply_prod(ProdArgs a) {
 // ---------------------------------------------------------------------------
 // Permute
 // ---------------------------------------------------------------------------
+// A permutation of the tile's bits, in place: the tile (2^T amplitudes, 16-byte
+// copies) is in shared memory before any of it is written.  Bound by HBM; what
+// counts is the number of passes a permutation of the state's positions takes,
+// so tiles are wide (2^13 amplitudes, runs of at least 64 bytes): ten positions
+// above the lowest three can move in one pass (plan_permutation).  One stage
+// per CTA, three CTAs of 512 threads per SM hide each other's latency.
+// N = 28, two random layouts and five bit swaps: 22 passes of 0.71 ms in
+// 2^11-amplitude tiles with up to six swaps each (14.5 ms), 7 of 0.69 ms here.
+constexpr int kPermT = 13, kPermThreads = 512, kPermLow = 3;
+
 struct PermArgs {
-    TileArgs t;
-    int npairs;
-    int la[6], lb[6];   // tile-local positions of each pair
+    float2* psi;
+    uint64_t ntiles;
+    int T, m, nx;
+    int xpos[kPermT];
+    uint64_t poff[kPermT];    // global offset and slot of tile bit b
+    uint16_t pslot[kPermT];
+    uint16_t sslot[kPermT];   // slot of the tile bit whose content tile bit b receives
 };
 
-template <int S>
-__global__ void __launch_bounds__(kThreads) k_permute(PermArgs a) {
+__global__ void __launch_bounds__(kPermThreads, 3) k_permute(const __grid_constant__ PermArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tileAmps = 1 << a.t.T;
-    float2* stage = reinterpret_cast<float2*>(smem_raw);
-    uint64_t* runoff = reinterpret_cast<uint64_t*>(stage + S * tileAmps);
-    build_runoff(a.t, runoff);
-    __syncthreads();
-    const uint64_t stride = gridDim.x;
+    float2* st = reinterpret_cast<float2*>(smem_raw);
+    constexpr int LT = 9;   // thread bits
+    static_assert(1 << LT == kPermThreads, "thread bits");
+    const int tid = threadIdx.x;
+    uint64_t g0 = 0;
+    uint32_t sl = 0, ss = 0;
 #pragma unroll
-    for (int s = 0; s < S - 1; ++s) {
-        uint64_t t = blockIdx.x + s * stride;
-        if (t < a.t.ntiles) load_tile(a.t, runoff, t, stage + s * tileAmps);
+    for (int b = 0; b < LT; ++b)
+        if ((tid >> b) & 1) {
+            g0 |= a.poff[b + 1];
+            sl ^= a.pslot[b + 1];
+            ss ^= a.sslot[b + 1];
+        }
+    const uint32_t chunks = 1u << (a.T - 1);
+    const int nk = chunks > kPermThreads ? static_cast<int>(chunks / kPermThreads) : 1;
+    const bool copies = static_cast<uint32_t>(tid) < chunks;
+    const uint64_t limit = a.ntiles << a.T;
+    const uint32_t s0 = a.sslot[0];
+    for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
+        uint64_t base = t << a.m;
+#pragma unroll
+        for (int e = 0; e < kPermT - kPermLow; ++e)
+            if (e < a.nx) base = insert_zero(base, a.xpos[e]);
+        base |= g0;
+        uint64_t g[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            g[k] = base | (k & 1 ? a.poff[LT + 1] : 0ull) | (k & 2 ? a.poff[LT + 2] : 0ull) | (k & 4 ? a.poff[LT + 3] : 0ull);
+            const uint32_t s = sl ^ (k & 1 ? a.pslot[LT + 1] : 0u) ^ (k & 2 ? a.pslot[LT + 2] : 0u) ^
+                               (k & 4 ? a.pslot[LT + 3] : 0u);
+            if (k < nk && copies && dbg::in_bounds(g[k], 2, limit, 6)) cp_async16(st + s, a.psi + g[k]);
+        }
         cp_async_commit();
-    }
-    int it_stage = 0;
-    const uint32_t chunks = static_cast<uint32_t>(tileAmps) >> 1;
-    for (uint64_t t = blockIdx.x; t < a.t.ntiles; t += stride) {
-        uint64_t tn = t + (S - 1) * stride;
-        int ld_stage = it_stage + (S - 1);
-        if (ld_stage >= S) ld_stage -= S;
-        if (tn < a.t.ntiles) load_tile(a.t, runoff, tn, stage + ld_stage * tileAmps);
-        cp_async_commit();
-        cp_async_wait<S - 1>();
+        cp_async_wait<0>();
         __syncthreads();
-        const float2* st = stage + it_stage * tileAmps;
-        const uint64_t base = tile_base(a.t, t);
-        for (uint32_t q = threadIdx.x; q < chunks; q += blockDim.x) {
-            uint32_t d0 = q << 1, d1 = d0 | 1u;
-            uint32_t s0 = d0, s1 = d1;
 #pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                if (i >= a.npairs) break;
-                uint32_t x0 = ((s0 >> a.la[i]) ^ (s0 >> a.lb[i])) & 1u;
-                s0 ^= (x0 << a.la[i]) | (x0 << a.lb[i]);
-                uint32_t x1 = ((s1 >> a.la[i]) ^ (s1 >> a.lb[i])) & 1u;
-                s1 ^= (x1 << a.la[i]) | (x1 << a.lb[i]);
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t s = ss ^ (k & 1 ? a.sslot[LT + 1] : 0u) ^ (k & 2 ? a.sslot[LT + 2] : 0u) ^
+                               (k & 4 ? a.sslot[LT + 3] : 0u);
+            if (k < nk && copies && dbg::in_bounds(g[k], 2, limit, 6)) {
+                const float2 v0 = st[s], v1 = st[s ^ s0];
+                __stcs(reinterpret_cast<float4*>(a.psi + g[k]), make_float4(v0.x, v0.y, v1.x, v1.y));
             }
-            float2 v0 = st[s0], v1 = st[s1];
-            const uint64_t gd = tile_global(a.t, runoff, base, d0);
-            if (dbg::in_bounds(gd, 2, a.t.ntiles << a.t.T, 6))
-                __stcs(reinterpret_cast<float4*>(a.t.psi + gd), make_float4(v0.x, v0.y, v1.x, v1.y));
         }
         __syncthreads();
-        if (++it_stage == S) it_stage = 0;
     }
-    cp_async_wait<0>();
 }
 
 __global__ void k_set_one(float2* psi) { psi[0] = make_float2(1.f, 0.f); }
@@ -1051,71 +1067,117 @@ cudaError_t launch_apply_prod(float2* psi, int n, const int* phys, int k, const 
     return cudaSuccess;
 }
 
-cudaError_t launch_permute(float2* psi, int n, const int* pa, const int* pb, int npairs, cudaStream_t st,
-                           uint64_t* launches) {
-    constexpr int S = 3, T = 11;
-    int i0 = 0;
-    while (i0 < npairs) {
-        // grow the pass while its extra tile bits fit
-        int i1 = i0 + 1;
-        TileGeom g;
-        int spec[12];
-        for (;;) {
-            int ns = 0;
-            for (int i = i0; i < i1; ++i) {
-                spec[ns++] = pa[i];
-                spec[ns++] = pb[i];
+std::vector<std::vector<int>> plan_permutation(int n, const int* dest, int T) {
+    const int cap = T - kPermLow;   // positions at kPermLow or above in one pass
+    std::vector<int> to(dest, dest + n);
+    std::vector<std::vector<int>> passes;
+    auto high = [](int p) { return p >= kPermLow ? 1 : 0; };
+    for (;;) {
+        // the cycles left, longest (in high positions) first
+        std::vector<std::vector<int>> cyc;
+        std::vector<char> seen(n, 0);
+        for (int p = 0; p < n; ++p) {
+            if (seen[p] || to[p] == p) continue;
+            std::vector<int> c;
+            for (int x = p; !seen[x]; x = to[x]) {
+                seen[x] = 1;
+                c.push_back(x);
             }
-            if (!make_geom(n, spec, ns, T, &g)) {
-                if (i1 == i0 + 1) return cudaErrorInvalidValue;
-                --i1;
-                ns = 0;
-                for (int i = i0; i < i1; ++i) {
-                    spec[ns++] = pa[i];
-                    spec[ns++] = pb[i];
-                }
-                make_geom(n, spec, ns, T, &g);
-                break;
-            }
-            if (i1 == npairs || i1 - i0 == 6) break;
-            ++i1;
+            cyc.push_back(c);
         }
-        PermArgs a{};
-        a.t.psi = psi;
-        a.t.ntiles = g.ntiles;
-        a.t.T = g.T;
-        a.t.m = g.m;
-        a.t.nx = g.nx;
-        for (int e = 0; e < 6; ++e) a.t.xpos[e] = g.xpos[e];
-        a.npairs = i1 - i0;
-        auto local = [&](int p) {
-            if (p < g.m) return p;
-            int e = 0;
-            while (g.xpos[e] != p) ++e;
-            return g.m + e;
+        if (cyc.empty()) return passes;
+        auto highs = [&](const std::vector<int>& c) {
+            int h = 0;
+            for (int p : c) h += high(p);
+            return h;
         };
-        for (int i = i0; i < i1; ++i) {
-            a.la[i - i0] = local(pa[i]);
-            a.lb[i - i0] = local(pb[i]);
+        std::stable_sort(cyc.begin(), cyc.end(),
+                         [&](const std::vector<int>& x, const std::vector<int>& y) { return highs(x) > highs(y); });
+        std::vector<int> pass(n);
+        for (int p = 0; p < n; ++p) pass[p] = p;
+        // contents of c[0..k) move one place along; the last one's goes back to c[0], from where it still has
+        // to reach its destination
+        int room = cap;
+        auto move = [&](const std::vector<int>& c, size_t k) {
+            for (size_t i = 0; i < k; ++i) {
+                pass[c[i]] = c[(i + 1) % k];
+                room -= high(c[i]);
+            }
+            const int last = to[c[k - 1]];
+            for (size_t i = 0; i + 1 < k; ++i) to[c[i + 1]] = c[i + 1];
+            to[c[0]] = k == c.size() ? c[0] : last;
+        };
+        std::vector<char> done(cyc.size(), 0);
+        for (size_t i = 0; i < cyc.size(); ++i)   // whole cycles that fit
+            if (highs(cyc[i]) <= room) {
+                move(cyc[i], cyc[i].size());
+                done[i] = 1;
+            }
+        for (size_t i = 0; i < cyc.size(); ++i) {   // then the first positions of others, from a low one if there is one
+            if (done[i]) continue;
+            std::vector<int> c = cyc[i];
+            for (size_t r = 0; r < c.size(); ++r)
+                if (!high(c[r])) {
+                    std::rotate(c.begin(), c.begin() + static_cast<long>(r), c.end());
+                    break;
+                }
+            size_t k = 0;
+            for (int h = 0; k < c.size() && h + high(c[k]) <= room; ++k) h += high(c[k]);
+            if (k >= 2) move(c, k);
         }
-        const size_t smem = sizeof(float2) * (static_cast<size_t>(S) << g.T) + sizeof(uint64_t) * 64;
-        auto kern = k_permute<S>;
-        {
-            const size_t full = sizeof(float2) * (static_cast<size_t>(S) << T) + sizeof(uint64_t) * 64;
-            cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(full));
-            if (e != cudaSuccess) return e;
+        passes.push_back(pass);
+    }
+}
+
+cudaError_t launch_permute(float2* psi, int n, const int* dest, cudaStream_t st, uint64_t* launches) {
+    const int T = std::min(kPermT, n);
+    for (const std::vector<int>& pass : plan_permutation(n, dest, kPermT)) {
+        PermArgs a{};
+        a.psi = psi;
+        a.T = T;
+        a.ntiles = 1ull << (n - T);
+        uint64_t moved = 0;
+        for (int p = 0; p < n; ++p)
+            if (pass[p] != p) moved |= 1ull << p;
+        int m = T;
+        while (m + __builtin_popcountll(moved >> m) > T) --m;
+        if (m < 1) return cudaErrorInvalidValue;
+        a.m = m;
+        for (int p = m; p < n; ++p)
+            if ((moved >> p) & 1) a.xpos[a.nx++] = p;
+        auto position = [&](int b) { return b < m ? b : a.xpos[b - m]; };
+        int bit_of[QSA_MAX_QUBITS] = {}, from[kPermT] = {};
+        for (int b = 0; b < T; ++b) bit_of[position(b)] = b;
+        for (int b = 0; b < T; ++b) from[bit_of[pass[position(b)]]] = b;
+        // The reading lanes vary the destination's bits 1..4: their source bits at 4 or above take slot
+        // bits 1..3 that no other of them has.
+        uint32_t used = 0, vec[kPermT] = {};
+        for (int b = 1; b <= 4 && b < T; ++b)
+            if (from[b] >= 1 && from[b] <= 3) used |= 1u << from[b];
+        for (int b = 1; b <= 4 && b < T; ++b)
+            if (from[b] >= 4)
+                for (int j = 1; j <= 3; ++j)
+                    if (!((used >> j) & 1)) {
+                        used |= 1u << j;
+                        vec[from[b]] = 1u << j;
+                        break;
+                    }
+        for (int b = 0; b < T; ++b) {
+            a.poff[b] = 1ull << position(b);
+            a.pslot[b] = static_cast<uint16_t>((1u << b) ^ vec[b]);
         }
-        int occ = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem);
+        for (int b = 0; b < T; ++b) a.sslot[b] = a.pslot[from[b]];
+        const size_t smem = sizeof(float2) << T;
+        cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(k_permute), static_cast<int>(sizeof(float2) << kPermT));
         if (e != cudaSuccess) return e;
-        if (occ < 1) occ = 1;
-        uint64_t grid = static_cast<uint64_t>(num_sms()) * occ;
-        if (grid > g.ntiles) grid = g.ntiles;
-        kern<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(a);
+        int occ = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_permute, kPermThreads, smem);
+        if (e != cudaSuccess) return e;
+        const uint64_t grid = std::min<uint64_t>(a.ntiles, static_cast<uint64_t>(num_sms()) * std::max(occ, 1));
+        k_permute<<<static_cast<unsigned>(grid), kPermThreads, smem, st>>>(a);
         ++*launches;
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        i0 = i1;
     }
     return cudaSuccess;
 }

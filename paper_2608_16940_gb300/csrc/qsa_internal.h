@@ -201,9 +201,13 @@ cudaError_t launch_layer_records(float2* psi, int n, const LayerGeom& g, const u
 cudaError_t launch_apply_layer(float2* psi, int n, const LayerGeom& g, const unsigned char* d_payload,
                                const LayerPayload& p, void* d_rec, cudaStream_t st, uint64_t* launches);
 
-// In-place swap of physical bit pairs (pa[i] <-> pb[i]), all positions distinct.
-cudaError_t launch_permute(float2* psi, int n, const int* pa, const int* pb, int npairs, cudaStream_t st,
-                           uint64_t* launches);
+// In-place permutation of physical positions: the content of position p moves
+// to dest[p] (a bijection), in as few passes as plan_permutation finds.
+cudaError_t launch_permute(float2* psi, int n, const int* dest, cudaStream_t st, uint64_t* launches);
+// The passes of such a permutation through tiles of 2^T amplitudes (T - 3
+// positions at 3 or above each): per pass, where each position's content goes;
+// their product is dest.
+std::vector<std::vector<int>> plan_permutation(int n, const int* dest, int T);
 
 // FP64 sum of (-1)^{popcount(y & physmask)} |psi_y|^2 into *d_out (device).
 // d_partials must hold reduce_partials() doubles.

@@ -129,8 +129,11 @@ qsa_status validate_targets(int n, const int32_t* targets, int k, int kmax) {
 // Swap physical positions pairs (pa[i], pb[i]) in data and layout.
 qsa_status permute_positions(qsa_state s, const int* pa, const int* pb, int np, qsa_run_stats* rs) {
     if (np == 0) return QSA_OK;
+    int dest[QSA_MAX_QUBITS];
+    for (int p = 0; p < s->n; ++p) dest[p] = p;
+    for (int i = 0; i < np; ++i) std::swap(dest[pa[i]], dest[pb[i]]);
     Timer tm(s, rs ? &rs->permute_seconds : nullptr);
-    cudaError_t e = launch_permute(s->psi, s->n, pa, pb, np, s->stream, &s->launches);
+    cudaError_t e = launch_permute(s->psi, s->n, dest, s->stream, &s->launches);
     tm.stop();
     if (e != cudaSuccess) return cuda_fail(s, e, "permute kernel");
     int inv[64];
@@ -487,27 +490,12 @@ qsa_status qsa_set_layout(qsa_state s, const int32_t* phys_of_logical, int mater
         for (int q = 0; q < s->n; ++q) s->L[q] = phys_of_logical[q];
         return QSA_OK;
     }
-    // Passes of disjoint transpositions; each swap puts one logical qubit in
-    // its final position.
-    for (int guard = 0; guard < 2 * QSA_MAX_QUBITS; ++guard) {
-        int pa[QSA_MAX_QUBITS], pb[QSA_MAX_QUBITS], np = 0;
-        uint64_t used = 0;
-        for (int q = 0; q < s->n; ++q) {
-            int a = s->L[q], b = phys_of_logical[q];
-            if (a == b || ((used >> a) & 1) || ((used >> b) & 1)) continue;
-            used |= (1ull << a) | (1ull << b);
-            pa[np] = a;
-            pb[np] = b;
-            ++np;
-        }
-        if (np == 0) break;
-        for (int i = 0; i < np; i += 6) {
-            st = permute_positions(s, pa + i, pb + i, std::min(6, np - i), nullptr);
-            if (st != QSA_OK) return st;
-        }
-    }
-    for (int q = 0; q < s->n; ++q)
-        if (s->L[q] != phys_of_logical[q]) return fail(QSA_E_STATE, "layout materialisation did not converge");
+    // qubit q's position moves from L[q] to its new one
+    int dest[QSA_MAX_QUBITS];
+    for (int q = 0; q < s->n; ++q) dest[s->L[q]] = phys_of_logical[q];
+    cudaError_t e = launch_permute(s->psi, s->n, dest, s->stream, &s->launches);
+    if (e != cudaSuccess) return cuda_fail(s, e, "permute kernel");
+    for (int q = 0; q < s->n; ++q) s->L[q] = phys_of_logical[q];
     return QSA_OK;
 }
 
@@ -525,11 +513,7 @@ qsa_status qsa_permute_bits(qsa_state s, const int32_t* phys_a, const int32_t* p
         a[i] = x;
         b[i] = y;
     }
-    for (int i = 0; i < n_pairs; i += 6) {
-        st = permute_positions(s, a.data() + i, b.data() + i, std::min(6, n_pairs - i), nullptr);
-        if (st != QSA_OK) return st;
-    }
-    return QSA_OK;
+    return permute_positions(s, a.data(), b.data(), n_pairs, nullptr);
 }
 
 qsa_status qsa_apply_fused_ex(qsa_state s, const int32_t* targets, int k, const double* matrix, int lowering,
