@@ -10,15 +10,17 @@
 // there, so blocks on the same four bits cost no shared-memory traffic between
 // them.
 //
-// What bounds a pass: the FP32 pipe.  A one-qubit block is 8 FMAs per amplitude
-// (256 SM cycles per tile), while its own pass over HBM is about 2800 SM
-// cycles per tile at the copy rate; with the blocks of a pass sharing one read
-// and one write, a run of k = 1, 2 blocks costs its FMAs instead of its passes.
-// Measured against one pass per block: QFT + 3 random layers at N = 25, DP plan
-// of k <= 4 blocks, 24.6 -> 4.58 ms; the 12-qubit brick circuit of 20 layers
-// from |0...0> (one tile: two launches instead of about 250) with its
-// probabilities and norm, 1.77 -> 0.162 ms; 128 trajectories at N = 20 of
-// 10..40 layers with their samples, 295 -> 45.9 ms.
+// What bounds a pass: instruction issue and the FP32 pipe, no longer HBM (a
+// pass of its own over HBM is about 2800 SM cycles per tile at the copy rate).
+// So unitary one-qubit blocks run as one FMA per amplitude (a scaled real
+// rotation, 64 SM cycles per tile where the complex 2 x 2 took 256), and
+// their phases share tables with the diagonal blocks around them (group_host.cpp).
+// Measured, one pass per block / group passes with complex 2 x 2 blocks / with
+// rotations: QFT + 3 random layers at N = 25, DP plan of k <= 4 blocks, 24.6 /
+// 4.58 / 3.72 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
+// tile: two launches instead of about 250) with its probabilities and norm, 1.77
+// / 0.159 / 0.125 ms; 128 trajectories at N = 20 of 10..40 layers with their
+// samples, 295 / 45.9 / 35.2 ms.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -182,31 +184,92 @@ __device__ __forceinline__ void dense4(uint64_t (&v)[16], const ulonglong2* __re
     }
 }
 
-__device__ __forceinline__ uint64_t cmul_pk(uint64_t v, float2 d) {
-    return fma2(pack2(d.y, d.y), rot90(v), mul2(pack2(d.x, d.x), v));
+// Scaled real rotation on register bit B, one packed FMA per amplitude (both
+// components share the real coefficient).  Tangent form:
+// (x0, x1) <- (x0 - t x1, x1 + t x0); cotangent form, row 0 negated:
+// (x0, x1) <- (x1 - t x0, x0 + t x1).
+template <int B, bool COT>
+__device__ __forceinline__ void rotate(uint64_t (&v)[16], float t) {
+    const uint64_t t2 = pack2(t, t), nt2 = pack2(-t, -t);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        if ((i >> B) & 1) continue;
+        const uint64_t x0 = v[i], x1 = v[i | (1 << B)];
+        v[i] = COT ? fma2(nt2, x0, x1) : fma2(nt2, x1, x0);
+        v[i | (1 << B)] = COT ? fma2(t2, x1, x0) : fma2(t2, x0, x1);
+    }
 }
 
-// A diagonal block: c = the thread's index (tile number above the tile bits,
-// register bits zero), the register bits' parts of the entry index in ro[].
-__device__ __forceinline__ void diagonal(uint64_t (&v)[16], const GroupOp& op, const float2* __restrict__ d, uint32_t c) {
-    uint32_t x = 0;
-    for (int j = 0; j < op.k; ++j) x |= ((c >> op.c[j]) & 1u) << j;
-    if (op.om == 0) {
-        const float2 f = d[x];
+template <int B>
+__device__ __forceinline__ void rotate_if(uint64_t (&v)[16], const GroupOp& op) {
+    if (!((op.k >> B) & 1)) return;
+    if ((op.om >> B) & 1)
+        rotate<B, true>(v, op.t[B]);
+    else
+        rotate<B, false>(v, op.t[B]);
+}
+
+__device__ __forceinline__ uint64_t cmul(uint64_t v, float2 d) {
+    const float2 x = unpack2(v);
+    return pack2(fmaf(-x.y, d.y, x.x * d.x), fmaf(x.x, d.y, x.y * d.x));
+}
+
+// A diagonal block whose entry index takes the register bits of OM: base = the
+// thread's entry, o[] the register bits' byte offsets.
+template <int OM>
+__device__ __forceinline__ void diagonal_om(uint64_t (&v)[16], const unsigned char* base, const uint16_t* ro) {
+    uint32_t o[4];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = cmul_pk(v[i], f);
-        return;
+    for (int b = 0; b < 4; ++b) o[b] = (OM >> b) & 1 ? ro[b] : 0u;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        if (e & ~OM) continue;
+        const float2 f = *reinterpret_cast<const float2*>(base + (e & 1 ? o[0] : 0u) + (e & 2 ? o[1] : 0u) +
+                                                          (e & 4 ? o[2] : 0u) + (e & 8 ? o[3] : 0u));
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if ((i & OM) == e) v[i] = cmul(v[i], f);
     }
-    const uint32_t o0 = op.ro[0], o1 = op.ro[1], o2 = op.ro[2], o3 = op.ro[3];
+}
+
+// c: the thread's index (tile number above the tile bits, register bits zero).
+__device__ __forceinline__ void diagonal(uint64_t (&v)[16], const GroupOp& op, const unsigned char* d, uint32_t c) {
+    const uint32_t c0 = *reinterpret_cast<const uint32_t*>(op.c), c1 = *reinterpret_cast<const uint32_t*>(op.c + 4);
+    uint32_t x = 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-        v[i] = cmul_pk(v[i], d[x | (i & 1 ? o0 : 0u) | (i & 2 ? o1 : 0u) | (i & 4 ? o2 : 0u) | (i & 8 ? o3 : 0u)]);
+    for (int j = 0; j < 8; ++j) x |= ((c >> (((j < 4 ? c0 : c1) >> (8 * (j & 3))) & 31u)) & 1u) << (j + 3);
+    d += x;
+    switch (op.om) {
+        case 0: diagonal_om<0>(v, d, op.ro); break;
+        case 1: diagonal_om<1>(v, d, op.ro); break;
+        case 2: diagonal_om<2>(v, d, op.ro); break;
+        case 3: diagonal_om<3>(v, d, op.ro); break;
+        case 4: diagonal_om<4>(v, d, op.ro); break;
+        case 5: diagonal_om<5>(v, d, op.ro); break;
+        case 6: diagonal_om<6>(v, d, op.ro); break;
+        case 7: diagonal_om<7>(v, d, op.ro); break;
+        case 8: diagonal_om<8>(v, d, op.ro); break;
+        case 9: diagonal_om<9>(v, d, op.ro); break;
+        case 10: diagonal_om<10>(v, d, op.ro); break;
+        case 11: diagonal_om<11>(v, d, op.ro); break;
+        case 12: diagonal_om<12>(v, d, op.ro); break;
+        case 13: diagonal_om<13>(v, d, op.ro); break;
+        case 14: diagonal_om<14>(v, d, op.ro); break;
+        default: diagonal_om<15>(v, d, op.ro); break;
+    }
 }
 
 __device__ __forceinline__ void run_op(uint64_t (&v)[16], const GroupOp& op, const unsigned char* par, uint32_t c) {
+    if (op.code == kGroupRot) {
+        rotate_if<0>(v, op);
+        rotate_if<1>(v, op);
+        rotate_if<2>(v, op);
+        rotate_if<3>(v, op);
+        return;
+    }
     const ulonglong2* g = reinterpret_cast<const ulonglong2*>(par + op.off);
     switch (op.code) {
-        case kGroupDiag: diagonal(v, op, reinterpret_cast<const float2*>(g), c); break;
+        case kGroupDiag: diagonal(v, op, par + op.off, c); break;
         case 1: dense1<0>(v, g); break;
         case 2: dense1<1>(v, g); break;
         case 4: dense1<2>(v, g); break;

@@ -16,6 +16,35 @@
 
 namespace qsa {
 
+// F = diag(p) [[c, -s], [s, c]] diag(q) with q[0] = 1, c = |F00|, s = |F01|;
+// false unless the product reproduces F to 1e-10 (a unitary F does).
+bool split_rotation(const std::array<std::complex<double>, 4>& F, double* c, double* s, std::complex<double>* p,
+                    std::complex<double>* q) {
+    const std::complex<double> a = F[0], b = F[1], cc = F[2], d = F[3];
+    const double ca = std::abs(a), sb = std::abs(b);
+    if (ca == 0.0 && sb == 0.0) return false;
+    *c = ca;
+    *s = sb;
+    q[0] = 1.0;
+    if (ca > 0.0 && sb > 0.0) {
+        p[0] = a / ca;
+        q[1] = -b / (p[0] * sb);
+        p[1] = cc / sb;
+    } else if (sb == 0.0) {
+        p[0] = a / ca;
+        q[1] = 1.0;
+        p[1] = d / ca;
+    } else {
+        q[1] = 1.0;
+        p[0] = -b / sb;
+        p[1] = cc / sb;
+    }
+    const std::complex<double> rec[4] = {p[0] * ca * q[0], -p[0] * sb * q[1], p[1] * sb * q[0], p[1] * ca * q[1]};
+    for (int i = 0; i < 4; ++i)
+        if (std::abs(rec[i] - F[i]) > 1e-10) return false;
+    return true;
+}
+
 namespace {
 
 constexpr int kTile = QSA_LAYER_TILE_BITS;
@@ -64,35 +93,6 @@ float2 f2(std::complex<double> z) { return make_float2(static_cast<float>(z.real
 
 float2 f2m(std::complex<double> z, double weight, ModulusCarry* carry) {
     return f2_modulus(z, std::norm(z), weight, carry);
-}
-
-// F = diag(p) [[c, -s], [s, c]] diag(q) with q[0] = 1, c = |F00|, s = |F01|;
-// false unless the product reproduces F to 1e-10 (a unitary F does).
-bool split_rotation(const std::array<std::complex<double>, 4>& F, double* c, double* s, std::complex<double>* p,
-                    std::complex<double>* q) {
-    const std::complex<double> a = F[0], b = F[1], cc = F[2], d = F[3];
-    const double ca = std::abs(a), sb = std::abs(b);
-    if (ca == 0.0 && sb == 0.0) return false;
-    *c = ca;
-    *s = sb;
-    q[0] = 1.0;
-    if (ca > 0.0 && sb > 0.0) {
-        p[0] = a / ca;
-        q[1] = -b / (p[0] * sb);
-        p[1] = cc / sb;
-    } else if (sb == 0.0) {
-        p[0] = a / ca;
-        q[1] = 1.0;
-        p[1] = d / ca;
-    } else {
-        q[1] = 1.0;
-        p[0] = -b / sb;
-        p[1] = cc / sb;
-    }
-    const std::complex<double> rec[4] = {p[0] * ca * q[0], -p[0] * sb * q[1], p[1] * sb * q[0], p[1] * ca * q[1]};
-    for (int i = 0; i < 4; ++i)
-        if (std::abs(rec[i] - F[i]) > 1e-10) return false;
-    return true;
 }
 
 // The rotation [[c, -s], [s, c]] runs in the cotangent form when s > c.

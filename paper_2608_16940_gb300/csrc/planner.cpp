@@ -244,7 +244,8 @@ void build_next_use(qsa_plan_s* p) {
 // Runs of consecutive dense (k <= 4), diagonal and product blocks become group
 // passes (several blocks per pass over the state) for the plan's layout.
 // Per-gate plans keep one pass per op, and permuting plans one layout per block.
-void build_groups(qsa_plan_s* p) {
+// mat64: the blocks' matrices before rounding, at their offsets in host_mat.
+void build_groups(qsa_plan_s* p, const std::vector<double>& mat64) {
     if (p->n > kGroupMaxQubits || p->opts.planner == QSA_PLAN_PER_GATE || p->opts.lowering == QSA_LOWER_PERMUTE) return;
     auto takes = [](const PlanBlock& b) { return b.layer < 0 && (b.prod || group_takes(b.k, b.diag)); };
     const size_t nb = p->blocks.size();
@@ -256,7 +257,7 @@ void build_groups(qsa_plan_s* p) {
             std::vector<int> whole;   // the block an operator is all of, or -1 (a product's factor)
             for (size_t x = i; x < e; ++x) {
                 const PlanBlock& b = p->blocks[x];
-                const float* mat = p->host_mat.data() + b.off;
+                const double* mat = mat64.data() + b.off;
                 if (b.prod) {
                     for (int j = 0; j < b.k; ++j) {
                         src.push_back({1, false, {p->L0[b.t[j]]}, mat + 8 * j});
@@ -653,6 +654,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
     p->blocks.resize(blocks.size());
     std::vector<double> M;
     ModulusCarry carry;   // modulus errors of the plan's FP32 constants (error feedback)
+    std::vector<double> mat64;   // host_mat before rounding
     for (size_t i = 0; i < blocks.size(); ++i) {
         const Unit& u = blocks[i];
         PlanBlock& b = p->blocks[i];
@@ -762,7 +764,10 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
                 F[4 * j + 3] = h[2] * f[1] + h[3] * f[3];
             }
             p->host_mat.resize(b.off + 8 * t);
+            mat64.resize(b.off + 8 * t);
             for (int c = 0; c < 4 * t; ++c) {
+                mat64[b.off + 2 * c] = F[c].real();
+                mat64[b.off + 2 * c + 1] = F[c].imag();
                 p->host_mat[b.off + 2 * c] = static_cast<float>(F[c].real());
                 p->host_mat[b.off + 2 * c + 1] = static_cast<float>(F[c].imag());
             }
@@ -776,6 +781,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
             p->host_mat.resize(b.off + M.size());
             to_float_moduli(M.data(), M.size() / 2, p->host_mat.data() + b.off, 1.0 / static_cast<double>(M.size() / 2),
                             &carry);
+            mat64.insert(mat64.end(), M.begin(), M.end());
         } else if (u.e - u.s == 1) {
             const qsa_op& op = ops[u.s];
             b.k = op.k;
@@ -783,6 +789,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
             const size_t cnt = 2ull << (2 * op.k);
             p->host_mat.resize(b.off + cnt);
             to_float_matrix(op.matrix, op.k, p->host_mat.data() + b.off);
+            mat64.insert(mat64.end(), op.matrix, op.matrix + cnt);
         } else {
             st = fuse_range(ops, u.s, u.e, b.t, &b.k, &M);
             if (st != QSA_OK) {
@@ -791,9 +798,11 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
             }
             p->host_mat.resize(b.off + M.size());
             for (size_t j = 0; j < M.size(); ++j) p->host_mat[b.off + j] = static_cast<float>(M[j]);
+            mat64.insert(mat64.end(), M.begin(), M.end());
         }
         p->max_width = std::max(p->max_width, b.k);
         while (p->host_mat.size() % 4) p->host_mat.push_back(0.f);  // 16-byte aligned matrices
+        mat64.resize(p->host_mat.size());
     }
     // the zero-state block takes over the layer block after it: the generated
     // product state passes through that block's diagonal part and factors in
@@ -820,7 +829,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
     for (PlanLayer& pl : p->layers)
         pl.launches = prepare_layer(n_qubits, p->L0.data(), pl.spec, &p->host_layer, &carry);
     build_next_use(p);
-    build_groups(p);
+    build_groups(p, mat64);
     *out = p;
     return QSA_OK;
 }
@@ -1254,7 +1263,7 @@ qsa_status qsa_batch_create(int n_qubits, int n_traj, const qsa_op* ops, const s
         std::vector<size_t> order;   // the identity: batches take no layer units
         auto units = plan(tops, cnt, n_qubits, o, nullptr, &order, costmodel_global());
         b->total_blocks += units.size();
-        std::vector<float> mats;     // addressed by offset until all are in place
+        std::vector<double> mats;    // addressed by offset until all are in place
         std::vector<size_t> off;
         std::vector<GroupSrc> src;
         for (const Unit& u : units) {
@@ -1271,7 +1280,7 @@ qsa_status qsa_batch_create(int n_qubits, int n_traj, const qsa_op* ops, const s
             } else {
                 st = fuse_range(tops, u.s, u.e, tg, &g.k, &M);
             }
-            for (double x : M) mats.push_back(static_cast<float>(x));
+            mats.insert(mats.end(), M.begin(), M.end());
             if (st == QSA_OK && !group_takes(g.k, g.diag)) st = fail(QSA_E_ARG, "could not tile a fused block");
             if (st != QSA_OK) {
                 delete b;

@@ -62,26 +62,34 @@ constexpr int kGroupTileBits = 12;
 constexpr int kGroupLowBits = 3;          // a tile's lowest positions: runs of at least 64 bytes
 constexpr int kGroupDiagMax = 8;
 constexpr int kGroupDiag = 0;             // GroupOp::code of a diagonal block
+constexpr int kGroupRot = 16;             // ... of rotations
 constexpr uint32_t kGroupProgBytes = 38 * 1024;   // a pass's program: two CTAs' stages and programs fit an SM
 
-// An operator on physical positions: dense, 2 * 4^k floats row-major; or
-// diagonal, 2 * 2^k floats (entry c: bit j of c = position pos[j]).
+// An operator on physical positions: dense, 2 * 4^k doubles row-major; or
+// diagonal, 2 * 2^k doubles (entry c: bit j of c = position pos[j]).
 struct GroupSrc {
     int k;
     bool diag;
     int pos[kGroupDiagMax];
-    const float* mat;
+    const double* mat;
 };
 
-// One block of a round.  Dense: code = its register bits (1..15), the matrix at
-// off with its index bits in ascending register-bit order.  Diagonal: entry
-// index bit j = bit c[j] of (tile number, tile-local index); the parts of the
-// four register bits in ro[], om their mask.
+// One operator of a round.  Dense: code = its register bits (1..15), the matrix
+// at off with its index bits in ascending register-bit order.  Diagonal: entry
+// index bit j = bit c[j] of (tile number, tile-local index), unused ones bit 31
+// (always 0); byte offsets of the four register bits' parts in ro[], om their
+// mask.  Rotations: scaled real rotations on the register bits of k, in the
+// cotangent form on those of om, coefficients t[].
 struct GroupOp {
     uint8_t code, k, om, pad;
     uint32_t off;                 // byte offset from par_off, 16-byte aligned
-    uint16_t ro[4];
-    uint8_t c[kGroupDiagMax];
+    union {
+        struct {
+            uint16_t ro[4];
+            uint8_t c[kGroupDiagMax];
+        };
+        float t[4];
+    };
 };
 // Four tile bits in registers (s: their slots), the other tile bits in thread
 // order (tb), and the blocks [op0, op1) applied meanwhile.

@@ -145,6 +145,10 @@ float2 f2_modulus(std::complex<double> z, double m2, double weight = 1.0, Modulu
 // A table of `count` interleaved complex numbers rounded that way, each with
 // its own modulus as the target and the given weight.
 void to_float_moduli(const double* z, size_t count, float* out, double weight, ModulusCarry* carry);
+// F = diag(p) [[c, -s], [s, c]] diag(q) with c, s >= 0 and q[0] = 1; false unless
+// the product reproduces F to 1e-10 (a unitary F does).
+bool split_rotation(const std::array<std::complex<double>, 4>& F, double* c, double* s, std::complex<double>* p,
+                    std::complex<double>* q);
 qsa_status validate_targets(int n, const int32_t* targets, int k, int kmax = QSA_MAX_K);
 qsa_status apply_logical(qsa_state s, const int32_t* targets, int k, const float* d_mat, int lowering,
                          int precision, qsa_run_stats* rs);
