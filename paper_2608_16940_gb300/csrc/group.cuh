@@ -12,15 +12,17 @@
 //
 // What bounds a pass: instruction issue and the FP32 pipe, no longer HBM (a
 // pass of its own over HBM is about 2800 SM cycles per tile at the copy rate).
-// So unitary one-qubit blocks run as one FMA per amplitude (a scaled real
-// rotation, 64 SM cycles per tile where the complex 2 x 2 took 256), and
-// their phases share tables with the diagonal blocks around them (group_host.cpp).
+// So unitary one-qubit blocks run as real rotations in two in-place shears, one
+// FMA per amplitude (64 SM cycles per tile where the complex 2 x 2 took 256), and
+// their phases share tables with the diagonal blocks around them
+// (group_host.cpp); what a thread needs to find its places and entries comes
+// from small tables in the program instead of bit arithmetic.
 // Measured, one pass per block / group passes with complex 2 x 2 blocks / with
-// rotations: QFT + 3 random layers at N = 25, DP plan of k <= 4 blocks, 24.6 /
-// 4.58 / 3.72 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
-// tile: two launches instead of about 250) with its probabilities and norm, 1.77
-// / 0.159 / 0.125 ms; 128 trajectories at N = 20 of 10..40 layers with their
-// samples, 295 / 45.9 / 35.2 ms.
+// rotations: QFT + 3 random layers at N = 25, DP plan of k <= 4 blocks, 24.5 /
+// 4.58 / 3.30 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
+// tile: one launch instead of about 250) with its probabilities and norm, 1.77
+// / 0.159 / 0.107 ms; 128 trajectories at N = 20 of 10..40 layers with their
+// samples, 295 / 45.9 / 28.4 ms.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -61,7 +63,6 @@ __host__ __device__ constexpr int slot_of(int j) {
 struct Tables {
     uint64_t goff[8];        // global offsets of the copy loop's strides (tile-local 512 k)
     uint64_t runoff[512];    // global offset of the tile's bits m..T-1
-    uint8_t h[256];          // slot vector of the tile-local bits 4..11
 };
 
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
@@ -184,29 +185,31 @@ __device__ __forceinline__ void dense4(uint64_t (&v)[16], const ulonglong2* __re
     }
 }
 
-// Scaled real rotation on register bit B, one packed FMA per amplitude (both
-// components share the real coefficient).  Tangent form:
-// (x0, x1) <- (x0 - t x1, x1 + t x0); cotangent form, row 0 negated:
-// (x0, x1) <- (x1 - t x0, x0 + t x1).
-template <int B, bool COT>
-__device__ __forceinline__ void rotate(uint64_t (&v)[16], float t) {
-    const uint64_t t2 = pack2(t, t), nt2 = pack2(-t, -t);
+// Real rotation by atan t on register bit B up to a factor per row, as two
+// shears in place (no temporaries), one packed FMA per amplitude (both
+// components share the real coefficient); a = t / (1 + t^2), kappa = 1 / sqrt(1 + t^2):
+// first order x0 -= t x1, x1 += a x0 gives diag(1 / kappa, kappa) R, second order
+// x1 += t x0, x0 -= a x1 gives diag(kappa, 1 / kappa) R.
+template <int B, bool SECOND>
+__device__ __forceinline__ void rotate(uint64_t (&v)[16], float t, float a) {
+    const uint64_t t2 = SECOND ? pack2(t, t) : pack2(-t, -t), a2 = SECOND ? pack2(-a, -a) : pack2(a, a);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         if ((i >> B) & 1) continue;
-        const uint64_t x0 = v[i], x1 = v[i | (1 << B)];
-        v[i] = COT ? fma2(nt2, x0, x1) : fma2(nt2, x1, x0);
-        v[i | (1 << B)] = COT ? fma2(t2, x1, x0) : fma2(t2, x0, x1);
+        uint64_t& x = v[SECOND ? i | (1 << B) : i];
+        uint64_t& y = v[SECOND ? i : i | (1 << B)];
+        x = fma2(t2, y, x);
+        y = fma2(a2, x, y);
     }
 }
 
 template <int B>
-__device__ __forceinline__ void rotate_if(uint64_t (&v)[16], const GroupOp& op) {
-    if (!((op.k >> B) & 1)) return;
-    if ((op.om >> B) & 1)
-        rotate<B, true>(v, op.t[B]);
+__device__ __forceinline__ void rotate_if(uint64_t (&v)[16], uint32_t head, float t, float a) {
+    if (!((head >> (8 + B)) & 1)) return;
+    if ((head >> (16 + B)) & 1)
+        rotate<B, true>(v, t, a);
     else
-        rotate<B, false>(v, op.t[B]);
+        rotate<B, false>(v, t, a);
 }
 
 __device__ __forceinline__ uint64_t cmul(uint64_t v, float2 d) {
@@ -217,10 +220,8 @@ __device__ __forceinline__ uint64_t cmul(uint64_t v, float2 d) {
 // A diagonal block whose entry index takes the register bits of OM: base = the
 // thread's entry, o[] the register bits' byte offsets.
 template <int OM>
-__device__ __forceinline__ void diagonal_om(uint64_t (&v)[16], const unsigned char* base, const uint16_t* ro) {
-    uint32_t o[4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) o[b] = (OM >> b) & 1 ? ro[b] : 0u;
+__device__ __forceinline__ void diagonal_om(uint64_t (&v)[16], const unsigned char* base, uint32_t ro01, uint32_t ro23) {
+    const uint32_t o[4] = {ro01 & 0xffffu, ro01 >> 16, ro23 & 0xffffu, ro23 >> 16};
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
         if (e & ~OM) continue;
@@ -232,44 +233,48 @@ __device__ __forceinline__ void diagonal_om(uint64_t (&v)[16], const unsigned ch
     }
 }
 
-// c: the thread's index (tile number above the tile bits, register bits zero).
-__device__ __forceinline__ void diagonal(uint64_t (&v)[16], const GroupOp& op, const unsigned char* d, uint32_t c) {
-    const uint32_t c0 = *reinterpret_cast<const uint32_t*>(op.c), c1 = *reinterpret_cast<const uint32_t*>(op.c + 4);
-    uint32_t x = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) x |= ((c >> (((j < 4 ? c0 : c1) >> (8 * (j & 3))) & 31u)) & 1u) << (j + 3);
-    d += x;
-    switch (op.om) {
-        case 0: diagonal_om<0>(v, d, op.ro); break;
-        case 1: diagonal_om<1>(v, d, op.ro); break;
-        case 2: diagonal_om<2>(v, d, op.ro); break;
-        case 3: diagonal_om<3>(v, d, op.ro); break;
-        case 4: diagonal_om<4>(v, d, op.ro); break;
-        case 5: diagonal_om<5>(v, d, op.ro); break;
-        case 6: diagonal_om<6>(v, d, op.ro); break;
-        case 7: diagonal_om<7>(v, d, op.ro); break;
-        case 8: diagonal_om<8>(v, d, op.ro); break;
-        case 9: diagonal_om<9>(v, d, op.ro); break;
-        case 10: diagonal_om<10>(v, d, op.ro); break;
-        case 11: diagonal_om<11>(v, d, op.ro); break;
-        case 12: diagonal_om<12>(v, d, op.ro); break;
-        case 13: diagonal_om<13>(v, d, op.ro); break;
-        case 14: diagonal_om<14>(v, d, op.ro); break;
-        default: diagonal_om<15>(v, d, op.ro); break;
+// w: the operator's first 16 bytes; d: the thread's entry.
+__device__ __forceinline__ void diagonal(uint64_t (&v)[16], uint4 w, const unsigned char* d) {
+    switch ((w.x >> 16) & 15u) {
+        case 0: diagonal_om<0>(v, d, w.z, w.w); break;
+        case 1: diagonal_om<1>(v, d, w.z, w.w); break;
+        case 2: diagonal_om<2>(v, d, w.z, w.w); break;
+        case 3: diagonal_om<3>(v, d, w.z, w.w); break;
+        case 4: diagonal_om<4>(v, d, w.z, w.w); break;
+        case 5: diagonal_om<5>(v, d, w.z, w.w); break;
+        case 6: diagonal_om<6>(v, d, w.z, w.w); break;
+        case 7: diagonal_om<7>(v, d, w.z, w.w); break;
+        case 8: diagonal_om<8>(v, d, w.z, w.w); break;
+        case 9: diagonal_om<9>(v, d, w.z, w.w); break;
+        case 10: diagonal_om<10>(v, d, w.z, w.w); break;
+        case 11: diagonal_om<11>(v, d, w.z, w.w); break;
+        case 12: diagonal_om<12>(v, d, w.z, w.w); break;
+        case 13: diagonal_om<13>(v, d, w.z, w.w); break;
+        case 14: diagonal_om<14>(v, d, w.z, w.w); break;
+        default: diagonal_om<15>(v, d, w.z, w.w); break;
     }
 }
 
-__device__ __forceinline__ void run_op(uint64_t (&v)[16], const GroupOp& op, const unsigned char* par, uint32_t c) {
-    if (op.code == kGroupRot) {
-        rotate_if<0>(v, op);
-        rotate_if<1>(v, op);
-        rotate_if<2>(v, op);
-        rotate_if<3>(v, op);
+// w: the operator's first 16 bytes; t: the tile's number.
+__device__ __forceinline__ void run_op(uint64_t (&v)[16], const GroupOp& op, uint4 w, const unsigned char* par, uint32_t t) {
+    const float4 rt = *reinterpret_cast<const float4*>(op.t), ra = *reinterpret_cast<const float4*>(op.a);
+    uint32_t x = op.lo[threadIdx.x & 15] + op.hi[threadIdx.x >> 4];
+    const uint32_t code = w.x & 255u;
+    if (code == kGroupRot) {
+        rotate_if<0>(v, w.x, rt.x, ra.x);
+        rotate_if<1>(v, w.x, rt.y, ra.y);
+        rotate_if<2>(v, w.x, rt.z, ra.z);
+        rotate_if<3>(v, w.x, rt.w, ra.w);
         return;
     }
-    const ulonglong2* g = reinterpret_cast<const ulonglong2*>(par + op.off);
-    switch (op.code) {
-        case kGroupDiag: diagonal(v, op, par + op.off, c); break;
+    const ulonglong2* g = reinterpret_cast<const ulonglong2*>(par + w.y);
+    switch (code) {
+        case kGroupDiag: {
+            const int k = (w.x >> 8) & 255u;
+            for (int j = 0; j < k; ++j) x += ((t >> op.out[j]) & 1u) << op.obit[j];
+            diagonal(v, w, par + w.y + x);
+            break;
+        }
         case 1: dense1<0>(v, g); break;
         case 2: dense1<1>(v, g); break;
         case 4: dense1<2>(v, g); break;
@@ -301,7 +306,6 @@ __device__ __forceinline__ void run_pass(const GroupPass& p, float2* psi, float2
             if ((r >> e) & 1) off |= 1ull << p.xpos[e];
         tb.runoff[r] = off;
     }
-    tb.h[tid & 255] = static_cast<uint8_t>((slot_of((tid & 255) << 4) >> 1) & 7);
     __syncthreads();
     auto offset = [&](int j) { return static_cast<uint64_t>(j & ((1 << m) - 1)) | tb.runoff[j >> m]; };
     const uint32_t chunks = T == 0 ? 0u : 1u << (T - 1);      // 16-byte units of the tile
@@ -310,6 +314,9 @@ __device__ __forceinline__ void run_pass(const GroupPass& p, float2* psi, float2
     if (tid < 8) tb.goff[tid] = tid < nk ? offset(512 * tid) : 0;
     const uint64_t gld = copies ? offset(2 * tid) : 0;
     const int sld = slot_of(2 * tid);
+    // the pass leaves some bits inverted: amplitude j stands in place j ^ flip
+    const int sst = sld ^ slot_of(static_cast<int>(p.flip & ~1u));
+    const bool swap = p.flip & 1u;
     if (T < 4)   // the registers' bits above the state's: amplitudes that stay zero
         for (int j = tid; j < 16; j += kThreads) stage[j] = stage[kAmps + j] = make_float2(0.f, 0.f);
     __syncthreads();
@@ -350,11 +357,7 @@ __device__ __forceinline__ void run_pass(const GroupPass& p, float2* psi, float2
         for (int r = 0; r < p.nrounds; ++r) {
             const GroupRound& rd = rounds[r];
             if (active) {
-                int jb = 0;
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (i < tbits) jb |= ((tid >> i) & 1) << rd.tb[i];
-                const int sb = jb ^ (static_cast<int>(tb.h[jb >> 4]) << 1);
+                const int sb = rd.lo[tid & 15] ^ rd.hi[tid >> 4];
                 const int s0 = rd.s[0], s1 = rd.s[1], s2 = rd.s[2], s3 = rd.s[3];
                 uint64_t v[16];
                 if (s0 == 1) {   // tile bit 0 is the first register bit: pairs in one 16-byte access
@@ -371,8 +374,9 @@ __device__ __forceinline__ void run_pass(const GroupPass& p, float2* psi, float2
                         v[i] = *reinterpret_cast<const uint64_t*>(
                             st + (sb ^ (i & 1 ? s0 : 0) ^ (i & 2 ? s1 : 0) ^ (i & 4 ? s2 : 0) ^ (i & 8 ? s3 : 0)));
                 }
-                const uint32_t c = static_cast<uint32_t>(t << T) | static_cast<uint32_t>(jb);
-                for (int o = rd.op0; o < rd.op1; ++o) run_op(v, ops[o], par, c);
+                const int o1 = rd.op1;
+                for (int o = rd.op0; o < o1; ++o)
+                    run_op(v, ops[o], *reinterpret_cast<const uint4*>(ops + o), par, static_cast<uint32_t>(t));
                 if (s0 == 1) {
 #pragma unroll
                     for (int i = 0; i < 16; i += 2)
@@ -394,9 +398,9 @@ __device__ __forceinline__ void run_pass(const GroupPass& p, float2* psi, float2
             for (int k = 0; k < 8; ++k) {
                 if (k >= nk) break;
                 const uint64_t gi = base | tb.goff[k];
-                if (dbg::in_bounds(gi, 2, limit, 15))
-                    *reinterpret_cast<float4*>(psi + gi) =
-                        *reinterpret_cast<const float4*>(st + (sld ^ slot_of(512 * k)));
+                float4 x = *reinterpret_cast<const float4*>(st + (sst ^ slot_of(512 * k)));
+                if (swap) x = make_float4(x.z, x.w, x.x, x.y);
+                if (dbg::in_bounds(gi, 2, limit, 15)) *reinterpret_cast<float4*>(psi + gi) = x;
             }
         }
         cur ^= 1;

@@ -28,12 +28,13 @@ constexpr int kSlotVec[kGroupTileBits] = {0, 1, 2, 4, 3, 5, 6, 7, 1, 2, 4, 7};
 // Operators looked at past the first one left behind, so that building stays
 // linear in the length of a long run.
 constexpr size_t kLookahead = 512;
-constexpr size_t kMaxOps = 512;
+constexpr size_t kMaxOps = 2048;
 
 int slot_of_bit(int b) { return b < 4 ? 1 << b : (1 << b) ^ (kSlotVec[b] << 1); }
 
 uint32_t dense_bytes(int k) { return k == 4 ? 2048u : 16u << (2 * k); }
 uint32_t diag_bytes(int k) { return std::max(16u, 8u << k); }
+static_assert(sizeof(GroupOp) == 112 && sizeof(GroupRound) % 16 == 0, "16-byte aligned program");
 
 using Cx = std::complex<double>;
 
@@ -42,18 +43,21 @@ using Cx = std::complex<double>;
 // before R, and diag(p) waits for the next operator on its qubit that is not
 // diagonal and joins its matrix, so the phases between two operators of a qubit
 // are one diagonal, which shares a table with other diagonal operators, and the
-// rotation is one FMA per amplitude: R = kappa M with one coefficient of each
-// row of M equal to 1 (tangent form when c >= s, else cotangent, whose first row
-// is negated into p), kappa in the diagonal.
+// rotation is one FMA per amplitude.  It runs as two shears (group.cuh), which
+// leave the rows scaled by 1 / kappa and kappa: their inverses join p.  An angle
+// above 45 degrees is one below times X Z: Z joins q, and the pass keeps the
+// qubit's bit inverted (X) from there on, in the operators that follow and in
+// the places where it stores.
 struct Fine {
     enum Kind { kRot, kDense, kDiag } kind;
     uint64_t mask;           // positions
     int k;
     int pos[kGroupDiagMax];
-    float t = 0.f;           // rotation
-    bool cot = false;
+    float t = 0.f;           // rotation: tangent, and whether the bit is inverted after it
+    bool flip = false;
     std::vector<Cx> m;       // dense: row-major; diagonal: entries
     int src = -1;            // the source operator it is all of, unchanged
+    uint32_t inv = 0;        // index bits on positions that are inverted when it runs
 };
 
 std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
@@ -76,7 +80,39 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
         const size_t D = size_t(1) << s.k, cnt = s.diag ? D : D * D;
         f.m.resize(cnt);
         for (size_t e = 0; e < cnt; ++e) f.m[e] = Cx(s.mat[2 * e], s.mat[2 * e + 1]);
-        if (!s.diag) {
+        if (!s.diag && s.k == 1) {
+            const int at = s.pos[0];
+            // the phases that wait join the operator, their moduli (the factors of a rotation's rows) stay
+            // with the diagonal before it, so that it is still unitary
+            const double m0 = std::abs(wait[at][0]), m1 = std::abs(wait[at][1]);
+            const Cx w0 = wait[at][0] / m0, w1 = wait[at][1] / m1;
+            double scale = 0.0;
+            for (const Cx& z : f.m) scale = std::max(scale, std::abs(z));
+            double c = 0.0, sn = 0.0;
+            Cx p[2], q[2];
+            if (m0 > 0.0 && m1 > 0.0 && scale > 0.0 && scale < 1e30 &&
+                split_rotation({f.m[0] * w0 / scale, f.m[1] * w1 / scale, f.m[2] * w0 / scale, f.m[3] * w1 / scale}, &c,
+                               &sn, p, q)) {
+                if (sn == 0.0) {   // diagonal after all
+                    wait[at] = {scale * c * p[0] * m0, scale * c * p[1] * m1};
+                    continue;
+                }
+                const bool flip = sn > c;
+                f.t = static_cast<float>(flip ? c / sn : sn / c);
+                // exact for the rounded tangent: what is left over is a common factor
+                const double t = f.t, kappa = 1.0 / std::sqrt(1.0 + t * t), norm = scale * std::sqrt(c * c + sn * sn);
+                wait[at] = {p[0] * norm * (flip ? 1.0 / kappa : kappa), p[1] * norm * (flip ? kappa : 1.0 / kappa)};
+                const Cx q0 = m0, q1 = (flip ? -q[1] : q[1]) * m1;
+                if (std::abs(q0 - 1.0) > 1e-14 || std::abs(q1 - 1.0) > 1e-14) diag1(at, q0, q1);
+                f.kind = Fine::kRot;
+                f.flip = flip;
+                f.src = -1;
+                f.m.clear();
+                out.push_back(std::move(f));
+                continue;
+            }
+        }
+        if (!s.diag)
             for (int j = 0; j < s.k; ++j) {
                 if (!waiting(s.pos[j])) continue;
                 for (size_t r = 0; r < D; ++r)
@@ -84,37 +120,6 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
                 wait[s.pos[j]] = {1.0, 1.0};
                 f.src = -1;
             }
-            double scale = 0.0;
-            for (const Cx& z : f.m) scale = std::max(scale, std::abs(z));
-            double c = 0.0, sn = 0.0;
-            Cx p[2], q[2];
-            if (s.k == 1 && scale > 0.0 && scale < 1e30 &&
-                split_rotation({f.m[0] / scale, f.m[1] / scale, f.m[2] / scale, f.m[3] / scale}, &c, &sn, p, q)) {
-                const int at = s.pos[0];
-                if (sn == 0.0) {   // diagonal after all
-                    wait[at] = {scale * c * p[0], scale * c * p[1]};
-                    continue;
-                }
-                const bool cot = sn > c;
-                const double t = cot ? c / sn : sn / c;
-                const float tf = static_cast<float>(t);
-                // kappa for the rounded coefficient: the pass applies an exact multiple of a rotation
-                const double kappa =
-                    scale * std::sqrt((c * c + sn * sn) / (1.0 + static_cast<double>(tf) * static_cast<double>(tf)));
-                wait[at] = {cot ? -p[0] : p[0], p[1]};
-                if (std::abs(q[1] - 1.0) > 1e-14) {
-                    diag1(at, kappa, kappa * q[1]);
-                } else {
-                    wait[at][0] *= kappa;
-                    wait[at][1] *= kappa;
-                }
-                f.kind = Fine::kRot;
-                f.t = tf;
-                f.cot = cot;
-                f.src = -1;
-                f.m.clear();
-            }
-        }
         out.push_back(std::move(f));
     }
     for (int q = 0; q < n; ++q)
@@ -254,20 +259,23 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
     std::vector<const Fine*> left(fine.size());
     for (size_t i = 0; i < fine.size(); ++i) left[i] = &fine[i];
     ModulusCarry carry;
+    // What a pass may take, by the sizes before diagonal operators share tables and rotations share
+    // entries; less of it where the program comes out too long after all.
+    double room = 2.0 * kGroupProgBytes;
     while (!left.empty()) {
         // the operators of this pass
         std::vector<Fine> take;
         std::vector<const Fine*> later;
         uint64_t tile = 0, held_dense = 0, held_diag = 0;
-        uint32_t bytes = 0;
+        double bytes = 0.0;
         size_t i = 0;
         for (; i < left.size(); ++i) {
             const Fine& f = *left[i];
             if (later.size() >= kLookahead) break;
             const bool dg = f.kind == Fine::kDiag;
-            const uint32_t b = op_bytes(f) + sizeof(GroupOp) + sizeof(GroupRound);
+            const double b = op_bytes(f) + (dg && f.k < 3 ? 16.0 : 64.0);
             bool ok = !(f.mask & held_dense) && (dg || !(f.mask & held_diag));
-            ok = ok && take.size() < kMaxOps && bytes + b + 64 <= kGroupProgBytes;
+            ok = ok && take.size() < kMaxOps && bytes + b <= room;
             if (ok && !dg && n > kGroupTileBits) ok = popc((tile | f.mask) >> kGroupLowBits) <= max_high;
             if (ok) {
                 take.push_back(f);
@@ -279,7 +287,6 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
             }
         }
         later.insert(later.end(), left.begin() + static_cast<long>(i), left.end());
-        left.swap(later);
 
         GroupPass p{};
         p.only = take.size() == 1 ? take[0].src : -1;
@@ -304,15 +311,17 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
             return T + popc(~tmask & ((1ull << q) - 1));
         };
 
-        // diagonal operators share tables of 2^6 entries (lanes read 512 bytes); smaller ones where the
-        // program would not fit
-        std::vector<Fine> ops;
-        for (int cap : {6, 4, 0}) {
-            ops = cap ? merge_diagonals(take, cap) : take;
-            uint32_t total = 64;
-            for (const Fine& f : ops) total += op_bytes(f) + sizeof(GroupOp) + sizeof(GroupRound);
-            if (total <= kGroupProgBytes) break;
+        // diagonal operators share tables of up to 2^6 entries (lanes read 512 bytes)
+        std::vector<Fine> ops = merge_diagonals(take, 6);
+
+        // inverted bits, as the operators in order leave them
+        uint64_t flipped = 0;
+        for (Fine& f : ops) {
+            for (int j = 0; j < f.k; ++j) f.inv |= static_cast<uint32_t>((flipped >> f.pos[j]) & 1) << j;
+            if (f.flip) flipped ^= f.mask;
         }
+        for (int q = 0; q < n; ++q)
+            if ((flipped >> q) & 1) p.flip |= 1u << cbit(q);
 
         // rounds
         std::vector<GroupRound> rounds;
@@ -350,9 +359,16 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                 }
             GroupRound rd{};
             for (int b = 0; b < 4; ++b) rd.s[b] = static_cast<uint16_t>(slot_of_bit(rb[b]));
-            order_threads(reg, rd.tb);
+            uint8_t tb[8];
+            order_threads(reg, tb);
             // a tile of fewer bits: its thread bits come first, the others are never set
-            std::stable_partition(rd.tb, rd.tb + 8, [&](uint8_t b) { return b < std::max(T, 4); });
+            std::stable_partition(tb, tb + 8, [&](uint8_t b) { return b < std::max(T, 4); });
+            for (int x = 0; x < 16; ++x)
+                for (int b = 0; b < 4; ++b)
+                    if ((x >> b) & 1) {
+                        rd.lo[x] = static_cast<uint16_t>(rd.lo[x] ^ slot_of_bit(tb[b]));
+                        rd.hi[x] = static_cast<uint16_t>(rd.hi[x] ^ slot_of_bit(tb[4 + b]));
+                    }
             rd.op0 = static_cast<uint16_t>(code.size());
             std::vector<uint64_t> masks;   // positions of this round's codes
             for (const Fine* f : now) {
@@ -374,15 +390,17 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                     }
                     GroupOp& g = code[rd.op0 + x];
                     g.k |= static_cast<uint8_t>(1u << r);
-                    if (f->cot) g.om |= static_cast<uint8_t>(1u << r);
-                    g.t[r] = f->t;
+                    // on an inverted bit: the other way round, the rows' factors exchanged
+                    const bool inv = f->inv != 0;
+                    if (inv) g.om |= static_cast<uint8_t>(1u << r);
+                    const double t = inv ? -f->t : f->t;
+                    g.t[r] = static_cast<float>(t);
+                    g.a[r] = static_cast<float>(t / (1.0 + t * t));
                     masks[x] |= f->mask;
                     continue;
                 }
-                op.k = static_cast<uint8_t>(f->k);
                 op.off = static_cast<uint32_t>(par.size());
                 par.resize(op.off + op_bytes(*f));
-                float* g = reinterpret_cast<float*>(par.data() + op.off);
                 if (f->kind == Fine::kDiag) {
                     // index bits: the thread bits in lane order (neighbouring lanes read neighbouring
                     // entries), then the register bits, then the bits outside the tile
@@ -392,33 +410,42 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                         const int c = cbit(f->pos[j]);
                         ord[j] = j;
                         key[j] = c >= kGroupTileBits ? 64 + c : (reg >> c) & 1 ? 32 + c
-                                 : static_cast<int>(std::find(rd.tb, rd.tb + 8, c) - rd.tb);
+                                 : static_cast<int>(std::find(tb, tb + 8, c) - tb);
                     }
                     std::sort(ord, ord + f->k, [&](int x, int y) { return key[x] < key[y]; });
-                    for (int j = 0; j < kGroupDiagMax; ++j) op.c[j] = 31;   // no bit
                     for (int j = 0; j < f->k; ++j) {
-                        const int c = cbit(f->pos[ord[j]]);
-                        op.c[j] = static_cast<uint8_t>(c);
-                        if (c < kGroupTileBits && ((reg >> c) & 1)) {
-                            op.ro[reg_of[c]] = static_cast<uint16_t>(8u << j);
-                            op.om |= static_cast<uint8_t>(1u << reg_of[c]);
+                        const int key_j = key[ord[j]];
+                        if (key_j >= 64) {
+                            op.out[op.k] = static_cast<uint8_t>(key_j - 64 - T);
+                            op.obit[op.k++] = static_cast<uint8_t>(j + 3);
+                        } else if (key_j >= 32) {
+                            op.ro[reg_of[key_j - 32]] = static_cast<uint16_t>(8u << j);
+                            op.om |= static_cast<uint8_t>(1u << reg_of[key_j - 32]);
+                        } else {
+                            for (int x = 0; x < 16; ++x)
+                                if ((x >> (key_j & 3)) & 1) {
+                                    uint16_t& o = key_j < 4 ? op.lo[x] : op.hi[x];
+                                    o = static_cast<uint16_t>(o + (8u << j));
+                                }
                         }
                     }
+                    float* g = reinterpret_cast<float*>(par.data() + op.off);
                     const double share = 1.0 / static_cast<double>(f->m.size());
                     for (size_t x = 0; x < f->m.size(); ++x) {
                         size_t y = 0;
                         for (int j = 0; j < f->k; ++j) y |= ((x >> j) & 1) << ord[j];
-                        const double m2 = std::norm(f->m[y]);
+                        const Cx z = f->m[y ^ f->inv];
+                        const double m2 = std::norm(z);
                         // rounded with error feedback on the modulus, relative to the entry's own
                         const float2 e = m2 > 1e-30 && m2 < 1e30
-                                             ? f2_modulus(f->m[y], m2, share / m2, &carry)
-                                             : make_float2(static_cast<float>(f->m[y].real()),
-                                                           static_cast<float>(f->m[y].imag()));
+                                             ? f2_modulus(z, m2, share / m2, &carry)
+                                             : make_float2(static_cast<float>(z.real()), static_cast<float>(z.imag()));
                         g[2 * x] = e.x;
                         g[2 * x + 1] = e.y;
                     }
                 } else {
                     // index bits in ascending register-bit order
+                    float* g = reinterpret_cast<float*>(par.data() + op.off);
                     int rbit[4], ord[4];
                     for (int j = 0; j < f->k; ++j) {
                         rbit[j] = reg_of[cbit(f->pos[j])];
@@ -431,7 +458,7 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                         int y = 0;
                         for (int j = 0; j < f->k; ++j)
                             if ((x >> j) & 1) y |= 1 << ord[j];
-                        return y;
+                        return y ^ static_cast<int>(f->inv);
                     };
                     for (int r = 0; r < D; ++r)
                         for (int c = 0; c < D; ++c) {
@@ -455,6 +482,12 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
         p.ops_off = up16(rounds.size() * sizeof(GroupRound));
         p.par_off = up16(p.ops_off + code.size() * sizeof(GroupOp));
         p.bytes = up16(p.par_off + par.size());
+        if (p.bytes > kGroupProgBytes) {
+            room *= 0.7;   // the same operators again, fewer of them
+            continue;
+        }
+        room = 2.0 * kGroupProgBytes;
+        left.swap(later);
         p.prog = static_cast<uint32_t>(progs->size());
         progs->resize(p.prog + p.bytes);
         unsigned char* d = progs->data() + p.prog;

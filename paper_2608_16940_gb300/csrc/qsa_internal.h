@@ -74,35 +74,43 @@ struct GroupSrc {
     const double* mat;
 };
 
-// One operator of a round.  Dense: code = its register bits (1..15), the matrix
-// at off with its index bits in ascending register-bit order.  Diagonal: entry
-// index bit j = bit c[j] of (tile number, tile-local index), unused ones bit 31
-// (always 0); byte offsets of the four register bits' parts in ro[], om their
-// mask.  Rotations: scaled real rotations on the register bits of k, in the
-// cotangent form on those of om, coefficients t[].
+// One operator of a round.  Dense: code = its register bits (1..15); the matrix
+// at off with its index bits in ascending register-bit order.  Rotations: on the
+// register bits of k, in the second order on those of om.  Diagonal: entries at
+// off; byte offsets of an entry's index parts: ro of the four register bits (om
+// their mask), lo and hi of thread bits 0..3 and 4..7, and k bits of the tile
+// number.  Everything that a thread needs before the entries or the matrix sits
+// at a fixed place, so its loads do not wait for one another.
 struct GroupOp {
     uint8_t code, k, om, pad;
-    uint32_t off;                 // byte offset from par_off, 16-byte aligned
+    uint32_t off;                         // byte offset from par_off, 16-byte aligned
+    uint16_t ro[4];
     union {
         struct {
-            uint16_t ro[4];
-            uint8_t c[kGroupDiagMax];
+            float t[4], a[4];             // rotations
         };
-        float t[4];
+        struct {
+            uint8_t out[kGroupDiagMax];   // diagonal: bits of the tile number ...
+            uint8_t obit[kGroupDiagMax];  // ... and the shifts to their byte offsets
+        };
     };
+    uint16_t lo[16], hi[16];
 };
-// Four tile bits in registers (s: their slots), the other tile bits in thread
-// order (tb), and the blocks [op0, op1) applied meanwhile.
+// Four tile bits in registers (s: their slots), the other tile bits in threads
+// (slots of thread bits 0..3 and 4..7), and the operators [op0, op1) applied
+// meanwhile.
 struct GroupRound {
     uint16_t s[4];
-    uint8_t tb[8];
     uint16_t op0, op1;
+    uint16_t pad[2];
+    uint16_t lo[16], hi[16];
 };
 struct GroupPass {
     uint64_t ntiles;
     int32_t T, m, nx;
     int32_t xpos[kGroupTileBits];
     int32_t nrounds;
+    uint32_t flip;                // tile bits that the pass leaves inverted until it stores
     uint32_t ops_off, par_off;    // byte offsets within the program
     uint32_t prog;                // byte offset of the program in its buffer
     uint32_t bytes;               // its length, a multiple of 16
