@@ -113,7 +113,10 @@ cudaError_t launch_batch_evolve(const BatchArgs& a, cudaStream_t st, uint64_t* l
     if (e != cudaSuccess) return e;
     // a trajectory's passes run one after another, so the batch ends when its
     // deepest trajectory does: up to four CTAs share one, as many as it has tiles
-    const unsigned csize = a.n >= kGroupTileBits + 2 ? 4 : a.n == kGroupTileBits + 1 ? 2 : 1;
+    unsigned csize = a.n >= kGroupTileBits + 2 ? 4 : a.n == kGroupTileBits + 1 ? 2 : 1;
+    // eight when the trajectories would leave half of the CTA slots empty with four (with more of them
+    // than slots, larger clusters only add waiting: 128 at N = 20, 29.5 / 30.0 / 35.2 ms with 4 / 8 / 16)
+    if (a.n >= kGroupTileBits + 4 && a.n_traj * 8 <= 2 * num_sms()) csize = 8;
     // one cluster per trajectory in flight (clusters that find the queue empty leave at once)
     unsigned clusters = std::max(1u, static_cast<unsigned>(2 * num_sms()) / csize);
     clusters = std::min(clusters, static_cast<unsigned>(a.n_traj));

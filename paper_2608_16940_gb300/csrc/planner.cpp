@@ -1182,13 +1182,14 @@ struct qsa_batch_s {
     unsigned* d_queue = nullptr;   // [0] work counter, [1] error word
     uint32_t* d_out = nullptr;     // keys, counts (n_traj * shots each), n_distinct (n_traj)
     size_t out_cap = 0;
+    bool no_scratch = false;       // the sampler's scratch did not fit once
     uint64_t shots = 0;
     cudaStream_t cap_stream = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     void* g_states = nullptr;
     uint64_t g_shots = 0, g_seed = 0, g_budget = 0;
-    uint64_t launches = 0;
+    uint64_t launches = 0, per_run = 0;   // kernels launched, and by one run
 };
 
 namespace {
@@ -1203,12 +1204,22 @@ void batch_free_device(qsa_batch b) {
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
 }
 
+// Bytes of a run's outputs (keys, counts, n_distinct); the sampler's scratch follows.
+size_t batch_output_bytes(qsa_batch b, uint64_t shots) {
+    return (sizeof(uint32_t) * (2 * static_cast<size_t>(b->n_traj) * shots + b->n_traj) + 15) & ~static_cast<size_t>(15);
+}
+
 cudaError_t batch_enqueue(qsa_batch b, float2* states, uint64_t shots, uint64_t seed, uint64_t budget, cudaStream_t st) {
     uint32_t* keys = b->d_out;
     uint32_t* cnts = keys + static_cast<size_t>(b->n_traj) * shots;
     uint32_t* nd = cnts + static_cast<size_t>(b->n_traj) * shots;
+    const size_t outs = batch_output_bytes(b, shots);
+    void* scratch = outs + qsa::batch_sample_scratch_bytes(b->n, b->n_traj, static_cast<uint32_t>(shots)) <= b->out_cap
+                        ? reinterpret_cast<char*>(b->d_out) + outs
+                        : nullptr;
     cudaError_t e = cudaMemsetAsync(b->d_queue, 0, 2 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
+    const uint64_t l0 = b->launches;
     qsa::BatchArgs a{};
     a.states = states;
     a.n = b->n;
@@ -1223,8 +1234,10 @@ cudaError_t batch_enqueue(qsa_batch b, float2* states, uint64_t shots, uint64_t 
     a.budget = budget;
     e = qsa::launch_batch_evolve(a, st, &b->launches);
     if (e != cudaSuccess) return e;
-    return qsa::launch_batch_sample(states, b->n, b->n_traj, static_cast<uint32_t>(shots), seed, keys, cnts, nd, st,
-                                    &b->launches);
+    e = qsa::launch_batch_sample(states, b->n, b->n_traj, static_cast<uint32_t>(shots), seed, keys, cnts, nd,
+                                 scratch, st, &b->launches);
+    b->per_run = b->launches - l0;
+    return e;
 }
 
 }  // namespace
@@ -1340,8 +1353,9 @@ qsa_status qsa_batch_run(qsa_batch b, void* dev_states, size_t bytes, uint64_t s
     if (reinterpret_cast<uintptr_t>(dev_states) % 16) return fail(QSA_E_ARG, "states must be 16-byte aligned");
     if (shots < 1 || shots > 16384) return fail(QSA_E_ARG, "batched sampling takes 1..16384 shots per trajectory");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    const size_t need = sizeof(uint32_t) * (2 * static_cast<size_t>(b->n_traj) * shots + b->n_traj);
-    if (need > b->out_cap) {
+    const size_t outs = batch_output_bytes(b, shots);
+    size_t need = outs + qsa::batch_sample_scratch_bytes(b->n, b->n_traj, static_cast<uint32_t>(shots));
+    if (need > b->out_cap && (outs > b->out_cap || !b->no_scratch)) {
         if (b->d_out) {
             cudaDeviceSynchronize();
             dev_free(b->d_out);
@@ -1355,6 +1369,12 @@ qsa_status qsa_batch_run(qsa_batch b, void* dev_states, size_t bytes, uint64_t s
             b->graph = nullptr;
         }
         cudaError_t e = dev_malloc(&b->d_out, need);
+        if (e != cudaSuccess && need > outs) {   // no room for the scratch: one CTA per trajectory samples
+            cudaGetLastError();
+            need = outs;
+            b->no_scratch = true;
+            e = dev_malloc(&b->d_out, need);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(QSA_E_NOMEM, "cudaMalloc of batch outputs failed");
@@ -1400,7 +1420,7 @@ qsa_status qsa_batch_run(qsa_batch b, void* dev_states, size_t bytes, uint64_t s
         cudaEventRecord(e0, st);
         e = cudaGraphLaunch(b->gexec, st);
         cudaEventRecord(e1, st);
-        if (e == cudaSuccess) b->launches += 2;
+        if (e == cudaSuccess) b->launches += b->per_run;
     } else {
         cudaEventRecord(e0, st);
         e = batch_enqueue(b, states, shots, seed, budget_cycles, st);
@@ -1421,7 +1441,7 @@ qsa_status qsa_batch_run(qsa_batch b, void* dev_states, size_t bytes, uint64_t s
         stats->blocks = b->total_blocks;
         stats->passes = b->passes.size();
         stats->hbm_bytes = 16.0 * static_cast<double>(1ull << b->n) * static_cast<double>(b->passes.size());
-        stats->launches = use_graph ? 2 : 2;
+        stats->launches = b->per_run;
     }
     if (err_word != 0)
         return fail(QSA_E_TIMEOUT, "batched trajectories: the cycle budget ran out (error word " +

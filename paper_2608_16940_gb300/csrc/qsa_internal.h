@@ -141,12 +141,15 @@ struct BatchArgs {
 
 cudaError_t launch_batch_evolve(const BatchArgs& a, cudaStream_t st, uint64_t* launches);
 
-// One CTA per trajectory: sample `shots` outcomes of every state (identity
-// layout) with Philox stream id = trajectory index, sort, run-length encode.
-// Outputs per trajectory t at t * shots: outcomes, counts; n_distinct[t].
+// Sample `shots` outcomes of every state (identity layout) with Philox stream
+// id = trajectory index, sort, run-length encode.  Outputs per trajectory t at
+// t * shots: outcomes, counts; n_distinct[t].  With d_scratch (8-byte aligned,
+// batch_sample_scratch_bytes, which is 0 where it is not used) the shots of all
+// trajectories are drawn and sorted together, else one CTA takes a trajectory.
+size_t batch_sample_scratch_bytes(int n, int n_traj, uint32_t shots);
 cudaError_t launch_batch_sample(const float2* states, int n, int n_traj, uint32_t shots, uint64_t seed,
-                                uint32_t* out_keys, uint32_t* out_counts, uint32_t* n_distinct, cudaStream_t st,
-                                uint64_t* launches);
+                                uint32_t* out_keys, uint32_t* out_counts, uint32_t* n_distinct, void* d_scratch,
+                                cudaStream_t st, uint64_t* launches);
 
 // ---- launchers (return the first CUDA error; *launches incremented) --------
 cudaError_t launch_init_zero(float2* psi, int n, cudaStream_t st, uint64_t* launches);

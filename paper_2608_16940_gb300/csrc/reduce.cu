@@ -578,13 +578,18 @@ __global__ void k_draw(const float2* __restrict__ psi, const uint64_t* __restric
 // all of its shots instead of once per shot.
 constexpr int kShotBits = 26;   // shots are at most 2^26, blocks at most 2^24
 
+// `count` shots in all, `shots` of each state: state t (its nblocks blocks from
+// block t nblocks on) has shots t * shots ... with stream stream_id + t.
 __global__ void __launch_bounds__(256) k_draw_blocks(const uint64_t* __restrict__ cum, uint64_t nblocks, uint64_t shots,
-                                                     uint64_t seed, uint64_t stream_id, uint64_t* __restrict__ out) {
+                                                     uint64_t count, uint64_t seed, uint64_t stream_id,
+                                                     uint64_t* __restrict__ out) {
     const uint64_t s = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s >= shots) return;
+    if (s >= count) return;
+    const uint64_t t = s / shots;
+    cum += t * nblocks;
     const uint64_t total = cum[nblocks - 1];
-    const uint64_t b = total ? find_block(cum, nblocks, draw_u(s, stream_id, seed, total)) : 0;
-    out[s] = (b << kShotBits) | s;
+    const uint64_t b = total ? find_block(cum, nblocks, draw_u(s - t * shots, stream_id + t, seed, total)) : 0;
+    out[s] = ((t * nblocks + b) << kShotBits) | s;
 }
 
 // A warp takes `per` consecutive shots of the sorted list; for each block among
@@ -597,19 +602,19 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float
                                                                       const uint64_t* __restrict__ cum,
                                                                       uint64_t nblocks, const __grid_constant__ Layout lay,
                                                                       const uint64_t* __restrict__ draws, uint64_t shots,
-                                                                      uint64_t seed, uint64_t stream_id, int per,
-                                                                      uint64_t* __restrict__ keys) {
+                                                                      uint64_t count, uint64_t seed, uint64_t stream_id,
+                                                                      int per, uint64_t* __restrict__ keys) {
     __shared__ __align__(16) uint64_t pre[kResolveWarps][1024];   // inclusive prefixes
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint64_t i = (static_cast<uint64_t>(blockIdx.x) * kResolveWarps + w) * per + lane;
-    const bool valid = lane < per && i < shots;
-    const uint64_t total = cum[nblocks - 1];
+    const bool valid = lane < per && i < count;
     const uint64_t d = valid ? draws[i] : 0;
-    const uint64_t b = d >> kShotBits;
+    const uint64_t b = d >> kShotBits, sh = d & ((1ull << kShotBits) - 1), t = sh / shots, b0 = t * nblocks;
+    const uint64_t total = cum[b0 + nblocks - 1];
     uint64_t ub = 0;
-    if (valid && total) ub = draw_u(d & ((1ull << kShotBits) - 1), stream_id, seed, total) - (b ? cum[b - 1] : 0);
+    if (valid && total) ub = draw_u(sh - t * shots, stream_id + t, seed, total) - (b > b0 ? cum[b - 1] : 0);
     bool open = valid && total;
-    uint64_t key = 0;
+    uint64_t key = lay.n ? 0 : b0 * 1024;   // a state of zero weight: its first index
     for (;;) {
         const unsigned left = __ballot_sync(0xffffffffu, open);
         if (!left) break;
@@ -634,7 +639,8 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float
                 const int mid = (lo + hi) >> 1;
                 if (pre[w][mid] > ub) hi = mid; else lo = mid + 1;
             }
-            key = decode_physical(bb * 1024 + static_cast<uint64_t>(lo), lay);
+            key = bb * 1024 + static_cast<uint64_t>(lo);
+            if (lay.n) key = decode_physical(key, lay);   // else the index through all states
             open = false;
         }
         __syncwarp();
@@ -889,6 +895,58 @@ inline uint64_t next_pow2(uint64_t v) {
 // three cheaper than the radix sort's nine to fifteen).
 constexpr uint64_t kSortSmemMax = 4096;
 
+// Run-length encoding of one CTA's sorted keys (any indexable), wsum and carry
+// in shared memory.
+template <typename Keys>
+__device__ __forceinline__ void rle_cta(const Keys& keys, uint32_t shots, uint32_t* wsum, uint32_t& carry, uint32_t* okeys,
+                                        uint32_t* ocnt, uint32_t* n_distinct) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    // run-length encode: heads get their output slot; out_counts holds the
+    // run starts until they are turned into counts
+    if (threadIdx.x == 0) carry = 0;
+    __syncthreads();
+    for (uint32_t base = 0; base < shots; base += blockDim.x) {
+        const uint32_t i = base + threadIdx.x;
+        const uint32_t head = (i < shots && (i == 0 || keys[i] != keys[i - 1])) ? 1u : 0u;
+        uint32_t inc = head;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t v = lane < nw ? wsum[lane] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += t;
+            }
+            wsum[lane] = v;
+        }
+        __syncthreads();
+        const uint32_t pos = carry + (warp ? wsum[warp - 1] : 0) + inc - head;
+        if (head) {
+            okeys[pos] = keys[i];
+            ocnt[pos] = i;
+        }
+        __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) carry = pos + head;
+        __syncthreads();
+    }
+    const uint32_t nd = carry;
+    for (uint32_t base = 0; base < nd; base += blockDim.x) {
+        const uint32_t d = base + threadIdx.x;
+        uint32_t c = 0;
+        if (d < nd) c = (d + 1 < nd ? ocnt[d + 1] : shots) - ocnt[d];
+        __syncthreads();
+        if (d < nd) ocnt[d] = c;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *n_distinct = nd;
+}
+
 // Batched sampler: CTA t samples state t (identity layout) with Philox stream
 // id t.  Shared memory: cum[nblocks] (uint64) then keys[P] (uint32).
 constexpr int kBatchSampleThreads = 512;
@@ -977,61 +1035,129 @@ __global__ void __launch_bounds__(kBatchSampleThreads)
             }
             __syncthreads();
         }
-    // run-length encode: heads get their output slot; out_counts holds the
-    // run starts until they are turned into counts
-    uint32_t* okeys = out_keys + static_cast<uint64_t>(traj) * shots;
-    uint32_t* ocnt = out_counts + static_cast<uint64_t>(traj) * shots;
-    if (threadIdx.x == 0) carry = 0;
+    rle_cta(keys, shots, wsum, carry, out_keys + static_cast<uint64_t>(traj) * shots,
+            out_counts + static_cast<uint64_t>(traj) * shots, n_distinct + traj);
+}
+
+// Samples of all trajectories sorted by (trajectory, outcome): CTA t encodes
+// trajectory t's.
+__global__ void __launch_bounds__(kBatchSampleThreads)
+    k_batch_rle(const uint64_t* __restrict__ keys, int n, uint32_t shots, uint32_t* __restrict__ out_keys,
+                uint32_t* __restrict__ out_counts, uint32_t* __restrict__ n_distinct) {
+    __shared__ uint32_t wsum[32];
+    __shared__ uint32_t carry;
+    const uint64_t at = static_cast<uint64_t>(blockIdx.x) * shots;
+    const uint64_t mask = (1ull << n) - 1;
+    struct Outcomes {
+        const uint64_t* k;
+        uint64_t mask;
+        __device__ uint32_t operator[](uint32_t i) const { return static_cast<uint32_t>(k[i] & mask); }
+    };
+    rle_cta(Outcomes{keys + at, mask}, shots, wsum, carry, out_keys + at, out_counts + at, n_distinct + blockIdx.x);
+}
+
+// Inclusive prefixes of the block weights of each state, a CTA per state of up
+// to 4096 blocks.
+__global__ void __launch_bounds__(1024) k_batch_scan(uint64_t* __restrict__ cum, int nblocks) {
+    __shared__ uint64_t wsum[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t* c = cum + static_cast<uint64_t>(blockIdx.x) * nblocks;
+    const int i0 = 4 * threadIdx.x;
+    uint64_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = i0 + k < nblocks ? c[i0 + k] : 0;
+    v[1] += v[0];
+    v[2] += v[1];
+    v[3] += v[2];
+    const uint64_t inc = warp_incl_scan_u64(v[3]);
+    if (lane == 31) wsum[wid] = inc;
     __syncthreads();
-    for (uint32_t base = 0; base < shots; base += blockDim.x) {
-        const uint32_t i = base + threadIdx.x;
-        const uint32_t head = (i < shots && (i == 0 || keys[i] != keys[i - 1])) ? 1u : 0u;
-        uint32_t inc = head;
+    if (wid == 0) wsum[lane] = warp_incl_scan_u64(wsum[lane]);
+    __syncthreads();
+    const uint64_t off = inc - v[3] + (wid ? wsum[wid - 1] : 0);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += t;
-        }
-        if (lane == 31) wsum[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t v = lane < nw ? wsum[lane] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += t;
-            }
-            wsum[lane] = v;
-        }
-        __syncthreads();
-        const uint32_t pos = carry + (warp ? wsum[warp - 1] : 0) + inc - head;
-        if (head) {
-            okeys[pos] = keys[i];
-            ocnt[pos] = i;
-        }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = pos + head;
-        __syncthreads();
-    }
-    const uint32_t nd = carry;
-    for (uint32_t base = 0; base < nd; base += blockDim.x) {
-        const uint32_t d = base + threadIdx.x;
-        uint32_t c = 0;
-        if (d < nd) c = (d + 1 < nd ? ocnt[d + 1] : shots) - ocnt[d];
-        __syncthreads();
-        if (d < nd) ocnt[d] = c;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) n_distinct[traj] = nd;
+    for (int k = 0; k < 4; ++k)
+        if (i0 + k < nblocks) c[i0 + k] = v[k] + off;
 }
 
 }  // namespace
 
 uint64_t next_pow2_u64(uint64_t v) { return next_pow2(v); }
 
+namespace {
+
+// Sorts n keys by their bits [lo, lo + bits), a digit of eight at a time, between
+// the two arrays; returns the one they end in.  hist: 256 (tiles + 1) words.
+uint64_t* radix_sort(uint64_t* from, uint64_t* other, uint64_t n, int lo, int bits, uint32_t* hist, cudaStream_t st,
+                     uint64_t* launches) {
+    const uint32_t ntiles = static_cast<uint32_t>((n + kRadixTile - 1) / kRadixTile);
+    uint32_t* totals = hist + 256ull * ntiles;
+    for (int sh = 0; sh < bits; sh += 8) {
+        k_radix_hist<<<ntiles, kRadixThreads, 0, st>>>(from, n, lo + sh, ntiles, hist);
+        k_radix_scan<<<256, kRadixThreads, 0, st>>>(hist, ntiles, totals);
+        k_radix_scatter<<<ntiles, kRadixThreads, 0, st>>>(from, n, lo + sh, ntiles, hist, totals, other);
+        std::swap(from, other);
+        *launches += 3;
+    }
+    return from;
+}
+
+int bits_of(uint64_t count) {   // bits of 0 .. count - 1
+    int b = 0;
+    while ((1ull << b) < count) ++b;
+    return b;
+}
+
+// shots per resolving warp: few when most lie in blocks of their own, which a
+// warp reads one after another (N = 24, 30 000 shots: 325 us with 8, 360 with
+// 32), many when they share blocks (N = 12, 200 000: 255 and 207)
+int resolve_per(uint64_t shots, uint64_t nblocks) { return shots >= 8 * nblocks ? 32 : shots >= 3 * nblocks ? 16 : 8; }
+
+// The batch's samples of all trajectories at once, where the shots' numbers fit
+// their keys: a CTA per trajectory reads a block of 8 KiB for every shot and sorts
+// in one CTA, which is slower at every size measured (whole runs of shallow
+// trajectories, N = 10 / 14 / 20: one with 100 shots 113 / 131 / 850 us against
+// 57 / 85 / 468, 64 with 16 000 shots each 11.2 / 12.2 / 14.3 ms against 0.21 /
+// 0.27 / 1.64).  It remains for states below one block of 1024 amplitudes and
+// where the scratch could not be allocated.
+bool batch_samples_together(int n, int n_traj, uint32_t shots) {
+    const uint64_t total = static_cast<uint64_t>(n_traj) * shots;
+    return n >= 10 && total <= (1ull << kShotBits);
+}
+
+}  // namespace
+
+size_t batch_sample_scratch_bytes(int n, int n_traj, uint32_t shots) {
+    if (!batch_samples_together(n, n_traj, shots)) return 0;
+    const uint64_t total = static_cast<uint64_t>(n_traj) * shots, ntiles = (total + kRadixTile - 1) / kRadixTile;
+    return sizeof(uint64_t) * ((static_cast<uint64_t>(n_traj) << (n - 10)) + 2 * total) + sizeof(uint32_t) * 256 * (ntiles + 1);
+}
+
 cudaError_t launch_batch_sample(const float2* states, int n, int n_traj, uint32_t shots, uint64_t seed,
-                                uint32_t* out_keys, uint32_t* out_counts, uint32_t* n_distinct, cudaStream_t st,
-                                uint64_t* launches) {
+                                uint32_t* out_keys, uint32_t* out_counts, uint32_t* n_distinct, void* d_scratch,
+                                cudaStream_t st, uint64_t* launches) {
+    if (d_scratch && batch_samples_together(n, n_traj, shots)) {
+        const uint64_t nblocks = 1ull << (n - 10), all = nblocks * n_traj, total = static_cast<uint64_t>(n_traj) * shots;
+        uint64_t* cum = static_cast<uint64_t*>(d_scratch);
+        uint64_t* x = cum + all;
+        uint64_t* y = x + total;
+        uint32_t* hist = reinterpret_cast<uint32_t*>(y + total);
+        const uint64_t nb = std::min<uint64_t>((all + 7) / 8, 2ull * num_sms());   // two CTAs of 8 warps fit an SM
+        k_weights_z1024<0><<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(states), all,
+                                                                            cum, ZMasks{}, nullptr);
+        k_batch_scan<<<n_traj, 1024, 0, st>>>(cum, static_cast<int>(nblocks));
+        k_draw_blocks<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, total, seed, 0, x);
+        uint64_t* d = radix_sort(x, y, total, kShotBits, bits_of(all), hist, st, launches);
+        uint64_t* keys = d == x ? y : x;
+        const int per = resolve_per(shots, nblocks);
+        const uint64_t cta = static_cast<uint64_t>(per) * kResolveWarps;
+        k_draw_resolve<<<static_cast<unsigned>((total + cta - 1) / cta), 32 * kResolveWarps, 0, st>>>(
+            reinterpret_cast<const float4*>(states), cum, nblocks, Layout{}, d, shots, total, seed, 0, per, keys);
+        keys = radix_sort(keys, d, total, 0, n + bits_of(n_traj), hist, st, launches);
+        k_batch_rle<<<n_traj, kBatchSampleThreads, 0, st>>>(keys, n, shots, out_keys, out_counts, n_distinct);
+        *launches += 5;
+        return cudaGetLastError();
+    }
     const int bsz = n >= 10 ? 1024 : (1 << n);
     const uint64_t nb = (1ull << n) / bsz;
     const uint32_t P = static_cast<uint32_t>(next_pow2(shots));
@@ -1273,16 +1399,8 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
     // where the outcome counts end up).  The outcomes must end in `keys`.
     const uint32_t ntiles = static_cast<uint32_t>((shots + kRadixTile - 1) / kRadixTile);
     uint32_t* hist = reinterpret_cast<uint32_t*>(d_out_counts);
-    uint32_t* totals = hist + 256ull * ntiles;
-    auto sort = [&](uint64_t* from, uint64_t* other, int lo, int bits) {   // returns where the keys end
-        for (int sh = 0; sh < bits; sh += 8) {
-            k_radix_hist<<<ntiles, kRadixThreads, 0, st>>>(from, shots, lo + sh, ntiles, hist);
-            k_radix_scan<<<256, kRadixThreads, 0, st>>>(hist, ntiles, totals);
-            k_radix_scatter<<<ntiles, kRadixThreads, 0, st>>>(from, shots, lo + sh, ntiles, hist, totals, other);
-            std::swap(from, other);
-            *launches += 3;
-        }
-        return from;
+    auto sort = [&](uint64_t* from, uint64_t* other, int lo, int bits) {
+        return radix_sort(from, other, shots, lo, bits, hist, st, launches);
     };
     const bool odd = ((n + 7) / 8) & 1;
     uint64_t* first = odd ? d_out_keys : keys;    // the unsorted outcomes
@@ -1292,15 +1410,13 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
     // 324 / 441 / 1327 us shot by shot (whole calls); N = 28, 30 000 / 100 000: 697 / 930 and 671 / 1036.
     if (bsz == 1024 && shots >= std::max<uint64_t>(16384, nblocks / 4)) {
         uint64_t* d = starts;
-        k_draw_blocks<<<static_cast<unsigned>((shots + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, seed, stream_id, d);
+        k_draw_blocks<<<static_cast<unsigned>((shots + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, shots, seed, stream_id,
+                                                                                  d);
         d = sort(d, second, kShotBits, n - 10);
-        // shots per warp: few when most lie in blocks of their own, which a warp reads one after another
-        // (N = 24, 30 000 shots: 325 us with 8, 360 with 32), many when they share blocks (N = 12,
-        // 200 000: 255 and 207)
-        const int per = shots >= 8 * nblocks ? 32 : shots >= 3 * nblocks ? 16 : 8;
+        const int per = resolve_per(shots, nblocks);
         const uint64_t cta = static_cast<uint64_t>(per) * kResolveWarps;
         k_draw_resolve<<<static_cast<unsigned>((shots + cta - 1) / cta), 32 * kResolveWarps, 0, st>>>(
-            reinterpret_cast<const float4*>(psi), cum, nblocks, lay, d, shots, seed, stream_id, per, first);
+            reinterpret_cast<const float4*>(psi), cum, nblocks, lay, d, shots, shots, seed, stream_id, per, first);
         *launches += 2;
     } else {
         k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
