@@ -407,7 +407,7 @@ std::vector<LayerLaunch> prepare_layer(int n, const int32_t* L, const LayerSpec&
 }
 
 qsa_status run_layer_launches(qsa_state s, const std::vector<LayerLaunch>& ls, const unsigned char* d_base,
-                              qsa_run_stats* rs) {
+                              qsa_run_stats* rs, bool product) {
     for (const LayerLaunch& ll : ls) {
         if (ll.p.rotation && (ll.p.ncross > 0 || ll.p.nout > 0)) {
             qsa_status st = ensure_dev(s, &s->d_lrec, &s->lrec_cap, layer_record_bytes(s->n));
@@ -418,7 +418,7 @@ qsa_status run_layer_launches(qsa_state s, const std::vector<LayerLaunch>& ls, c
                                              &s->launches);
         if (e != cudaSuccess) return cuda_fail(s, e, "layer records kernel");
         {
-            Timer tm(s, rs ? &rs->layer_seconds : nullptr);
+            Timer tm(s, rs ? (product ? &rs->prod_seconds : &rs->layer_seconds) : nullptr);
             e = launch_apply_layer(s->psi, s->n, ll.g, d_base + ll.dev_off, ll.p, s->d_lrec, s->stream,
                                    &s->launches);
             tm.stop();
@@ -432,9 +432,26 @@ qsa_status run_layer_launches(qsa_state s, const std::vector<LayerLaunch>& ls, c
     }
     if (rs) {
         rs->blocks += 1;
-        rs->layer_blocks += 1;
+        (product ? rs->prod_blocks : rs->layer_blocks) += 1;
     }
     return QSA_OK;
+}
+
+bool product_as_layer(const int32_t* targets, int k, const double* factors, LayerSpec* spec) {
+    for (int j = 0; j < k; ++j) {
+        std::array<std::complex<double>, 4> F;
+        double big = 0.0;
+        for (int c = 0; c < 4; ++c) {
+            F[c] = std::complex<double>(factors[8 * j + 2 * c], factors[8 * j + 2 * c + 1]);
+            big = std::max(big, std::abs(F[c]));
+        }
+        double c, sn;
+        std::complex<double> p[2], q[2];
+        if (!(big > 0.5 && big < 1.5) || !split_rotation(F, &c, &sn, p, q)) return false;
+        spec->t.push_back(targets[j]);
+        spec->f.push_back(F);
+    }
+    return true;
 }
 
 qsa_status apply_layer_logical(qsa_state s, const LayerSpec& spec, qsa_run_stats* rs) {

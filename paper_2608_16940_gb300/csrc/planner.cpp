@@ -771,6 +771,11 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
                 p->host_mat[b.off + 2 * c] = static_cast<float>(F[c].real());
                 p->host_mat[b.off + 2 * c + 1] = static_cast<float>(F[c].imag());
             }
+            PlanLayer pl;
+            if (n_qubits >= kProdLayerQubits && product_as_layer(b.t, t, mat64.data() + b.off, &pl.spec)) {
+                b.prod_layer = static_cast<int>(p->layers.size());
+                p->layers.push_back(std::move(pl));
+            }
         } else if (u.diag) {
             b.diag = true;
             st = fuse_diag_range(ops, u.s, u.e, b.t, &b.k, &M);
@@ -1033,7 +1038,11 @@ qsa_status run_block(qsa_state s, qsa_plan p, size_t i, qsa_run_stats* rs) {
             return run_layer_launches(s, pl.launches, p->d_layer, rs);
         return apply_layer_logical(s, pl.spec, rs);   // another layout: prepare again
     }
-    if (b.prod) return apply_prod_logical(s, b.t, b.k, p->d_mat + b.off, rs);
+    if (b.prod) {
+        if (b.prod_layer >= 0 && std::equal(p->L0.begin(), p->L0.end(), s->L))
+            return run_layer_launches(s, p->layers[b.prod_layer].launches, p->d_layer, rs, true);
+        return apply_prod_logical(s, b.t, b.k, p->d_mat + b.off, rs);
+    }
     if (b.diag) return apply_diag_logical(s, b.t, b.k, p->d_mat + b.off, rs);
     if (p->opts.lowering == QSA_LOWER_PERMUTE) {
         // promote the targets into the in-block frames, victims per the plan's rule

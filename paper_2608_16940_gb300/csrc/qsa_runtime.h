@@ -74,6 +74,7 @@ struct PlanBlock {
     bool diag = false;         // diagonal mode: 2^k entries, streaming kernel
     bool prod = false;         // product of one-qubit factors: 8 floats per factor, product kernel
     int layer = -1;            // layer block: index into qsa_plan_s::layers
+    int prod_layer = -1;       // product block that runs as a layer: likewise
     bool init = false;         // zero-state preparation (a write-only layer block)
     int n_diag = 0;            // layer block: ops of its diagonal part
     size_t off = 0;            // float offset of its matrix / diagonal in host_mat / d_mat
@@ -179,7 +180,15 @@ bool layer_fits(int n, const int* pos, int k);
 std::vector<LayerLaunch> prepare_layer(int n, const int32_t* L, const LayerSpec& spec,
                                        std::vector<unsigned char>* bytes, ModulusCarry* carry = nullptr);
 qsa_status run_layer_launches(qsa_state s, const std::vector<LayerLaunch>& ls, const unsigned char* d_base,
-                              qsa_run_stats* rs);
+                              qsa_run_stats* rs, bool product = false);
+// Smallest state on which a product of unitary factors runs as a layer: the layer
+// kernel takes 0.36 ms for seven factors on random targets at N = 27 where the
+// product kernel's complex butterflies take 0.64, but forming its tables costs
+// the host about 10 us, which a smaller state's pass does not hide.
+constexpr int kProdLayerQubits = 24;
+// A product block as a layer without diagonal ops (8 doubles per factor), if
+// every factor is unitary.
+bool product_as_layer(const int32_t* targets, int k, const double* factors, LayerSpec* spec);
 // Prepare for the state's current layout, upload to scratch and run (N < 12:
 // the diagonal and product kernels, op by op).
 qsa_status apply_layer_logical(qsa_state s, const LayerSpec& spec, qsa_run_stats* rs);

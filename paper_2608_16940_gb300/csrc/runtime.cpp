@@ -546,6 +546,11 @@ qsa_status qsa_apply_product(qsa_state s, const int32_t* targets, int k, const d
     st = validate_targets(s->n, targets, k, QSA_MAX_PROD);
     if (st != QSA_OK) return st;
     if (!factors) return fail(QSA_E_ARG, "factors is NULL");
+    // Unitary factors of a large state run as a layer (real rotations, nine
+    // positions above the lowest three in one pass).
+    LayerSpec spec;
+    if (s->n >= kProdLayerQubits && product_as_layer(targets, k, factors, &spec))
+        return apply_layer_logical(s, spec, nullptr);
     const size_t cnt = 8ull * k;
     std::vector<float> hf(cnt);
     for (size_t i = 0; i < cnt; ++i) hf[i] = static_cast<float>(factors[i]);
