@@ -33,6 +33,7 @@ namespace {
 using namespace dev;
 
 constexpr int kThreads = 256;
+constexpr int kBeyondL2 = 24;   // states of 128 MiB and more do not stay in the L2 (129 MB)
 
 struct TileArgs {
     float2* psi;
@@ -153,7 +154,7 @@ __device__ __forceinline__ void store_tile_swz(const TileArgs& a, const uint64_t
 // item writes its outputs in place and the tile goes back in address order
 // (16-byte units of 2^TB-amplitude tiles), for target sets whose direct
 // stores would give every lane its own sector.
-template <int K, int R, int S, bool SWZ = false, bool WB = false, int TB = 11, bool PO = false>
+template <int K, int R, int S, bool SWZ = false, bool WB = false, int TB = 11, bool PO = false, int NG = 1, int TH = kThreads>
 __device__ __forceinline__ void apply_tiles(const ApplyArgs& a, float2* stage, const float2* Ms,
                                             const uint64_t* runoff, const int* loff, uint64_t t0, uint64_t stride,
                                             const uint8_t* htab = nullptr, const int* sloff = nullptr) {
@@ -191,76 +192,102 @@ __device__ __forceinline__ void apply_tiles(const ApplyArgs& a, float2* stage, c
 
         float2* st = stage + it_stage * tileAmps;
         const uint64_t base = tile_base(a.t, t);
-        for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        // NG groups per item share the matrix's loads (whole groups only: R = D, full tiles)
+        for (int it = threadIdx.x; it < items / NG; it += blockDim.x) {
             const int g = it & (G - 1);
             const int rb = it >> gshift;
-            uint32_t lb = static_cast<uint32_t>(g);
+            uint32_t lb[NG], lbs[NG];   // the groups' bases, in the tile and in the stage
 #pragma unroll
-            for (int j = 0; j < K; ++j) lb = static_cast<uint32_t>(insert_zero(lb, a.tls[j]));
-            const uint32_t lbs = SWZ ? (lb ^ stage_xor(htab, lb)) : lb;   // the group's base in the stage
-            if constexpr (K <= 5) {
+            for (int x = 0; x < NG; ++x) {
+                lb[x] = static_cast<uint32_t>(g + x * (G / NG));
+#pragma unroll
+                for (int j = 0; j < K; ++j) lb[x] = static_cast<uint32_t>(insert_zero(lb[x], a.tls[j]));
+                lbs[x] = SWZ ? (lb[x] ^ stage_xor(htab, lb[x])) : lb[x];
+            }
+            auto put = [&](int x, int r, float re, float im) {
+                if constexpr (WB) {
+                    st[lbs[x] ^ msoff(r)] = make_float2(re, im);   // in place: inputs are in registers
+                } else {
+                    const uint64_t gj = tile_global(a.t, runoff, base, lb[x] | moff(r));
+                    if (dbg::in_bounds(gj, 1, a.t.ntiles << a.t.T, 4)) __stcs(a.t.psi + gj, make_float2(re, im));
+                }
+            };
+            if constexpr (K != 3) {
                 // Packed FP32 pairs: with x2_c = (Re v_c, Re v_c), y2_c = (Im v_c, Im v_c)
                 // and g = (Re G, Im G), p = sum x2_c * g and q = sum y2_c * g give
                 // Re = p.x - q.y and Im = p.y + q.x; one 16-byte load of two G entries
                 // feeds four f32x2 FMAs.
-                uint64_t x2[D], y2[D];
+                uint64_t x2[NG][D], y2[NG][D];
 #pragma unroll
-                for (int c = 0; c < D; ++c) {
-                    const float2 f = SWZ ? st[lbs ^ msoff(c)] : st[lb | moff(c)];
-                    x2[c] = pack2(f.x, f.x);
-                    y2[c] = pack2(f.y, f.y);
-                }
+                for (int x = 0; x < NG; ++x)
+#pragma unroll
+                    for (int c = 0; c < D; ++c) {
+                        const float2 f = SWZ ? st[lbs[x] ^ msoff(c)] : st[lb[x] | moff(c)];
+                        x2[x][c] = pack2(f.x, f.x);
+                        y2[x][c] = pack2(f.y, f.y);
+                    }
 #pragma unroll
                 for (int rr = 0; rr < R; ++rr) {
                     const int r = rb * R + rr;
                     const ulonglong2* mrow = reinterpret_cast<const ulonglong2*>(Ms + r * D);
-                    uint64_t p = 0, qv = 0;
+                    uint64_t p[NG] = {}, qv[NG] = {};
 #pragma unroll
                     for (int c = 0; c < D; c += 2) {
                         const ulonglong2 gg = mrow[c >> 1];  // G[r][c], G[r][c+1]
-                        p = fma2(x2[c], gg.x, p);
-                        qv = fma2(y2[c], gg.x, qv);
-                        p = fma2(x2[c + 1], gg.y, p);
-                        qv = fma2(y2[c + 1], gg.y, qv);
+#pragma unroll
+                        for (int x = 0; x < NG; ++x) {
+                            p[x] = fma2(x2[x][c], gg.x, p[x]);
+                            qv[x] = fma2(y2[x][c], gg.x, qv[x]);
+                        }
+#pragma unroll
+                        for (int x = 0; x < NG; ++x) {
+                            p[x] = fma2(x2[x][c + 1], gg.y, p[x]);
+                            qv[x] = fma2(y2[x][c + 1], gg.y, qv[x]);
+                        }
                     }
-                    const float2 P = unpack2(p), Q = unpack2(qv);
-                    if constexpr (WB) {
-                        st[lbs ^ msoff(r)] = make_float2(P.x - Q.y, P.y + Q.x);   // in place: inputs are in registers
-                    } else {
-                        const uint64_t gj = tile_global(a.t, runoff, base, lb | moff(r));
-                        if (dbg::in_bounds(gj, 1, a.t.ntiles << a.t.T, 4))
-                            __stcs(a.t.psi + gj, make_float2(P.x - Q.y, P.y + Q.x));
+#pragma unroll
+                    for (int x = 0; x < NG; ++x) {
+                        const float2 P = unpack2(p[x]), Q = unpack2(qv[x]);
+                        put(x, r, P.x - Q.y, P.y + Q.x);
                     }
                 }
             } else {
-                float2 v[D];
+                // Scalar FMAs: a packed pair reads six registers and issues every third
+                // cycle when its operands change.
+                float2 v[NG][D];
 #pragma unroll
-                for (int c = 0; c < D; ++c) v[c] = st[lb | loff[c]];
+                for (int x = 0; x < NG; ++x)
+#pragma unroll
+                    for (int c = 0; c < D; ++c) v[x][c] = SWZ ? st[lbs[x] ^ msoff(c)] : st[lb[x] | moff(c)];
 #pragma unroll
                 for (int rr = 0; rr < R; ++rr) {
                     const int r = rb * R + rr;
                     const float4* mrow = reinterpret_cast<const float4*>(Ms + r * D);
-                    float ar = 0.f, ai = 0.f;
+                    // the products of the real and of the imaginary parts in sums of their own
+                    float ar[NG] = {}, ai[NG] = {}, br[NG] = {}, bi[NG] = {};
 #pragma unroll
                     for (int c = 0; c < D; c += 2) {
-                        float4 m2 = mrow[c >> 1];  // G[r][c], G[r][c+1]
-                        ar = fmaf(m2.x, v[c].x, ar);
-                        ar = fmaf(-m2.y, v[c].y, ar);
-                        ai = fmaf(m2.x, v[c].y, ai);
-                        ai = fmaf(m2.y, v[c].x, ai);
-                        ar = fmaf(m2.z, v[c + 1].x, ar);
-                        ar = fmaf(-m2.w, v[c + 1].y, ar);
-                        ai = fmaf(m2.z, v[c + 1].y, ai);
-                        ai = fmaf(m2.w, v[c + 1].x, ai);
+                        const float4 m2 = mrow[c >> 1];  // G[r][c], G[r][c+1]
+#pragma unroll
+                        for (int x = 0; x < NG; ++x) {
+                            ar[x] = fmaf(m2.x, v[x][c].x, ar[x]);
+                            ai[x] = fmaf(m2.x, v[x][c].y, ai[x]);
+                            br[x] = fmaf(m2.y, v[x][c].y, br[x]);
+                            bi[x] = fmaf(m2.y, v[x][c].x, bi[x]);
+                            ar[x] = fmaf(m2.z, v[x][c + 1].x, ar[x]);
+                            ai[x] = fmaf(m2.z, v[x][c + 1].y, ai[x]);
+                            br[x] = fmaf(m2.w, v[x][c + 1].y, br[x]);
+                            bi[x] = fmaf(m2.w, v[x][c + 1].x, bi[x]);
+                        }
                     }
-                    const uint64_t gj = tile_global(a.t, runoff, base, lb | loff[r]);
-                    if (dbg::in_bounds(gj, 1, a.t.ntiles << a.t.T, 4)) __stcs(a.t.psi + gj, make_float2(ar, ai));
+#pragma unroll
+                    for (int x = 0; x < NG; ++x) put(x, r, ar[x] - br[x], ai[x] + bi[x]);
                 }
             }
         }
         if constexpr (WB) {
             __syncthreads();
-            store_tile_swz<(1 << (TB - 1)) / kThreads>(a.t, runoff, htab, t, st);
+            store_tile_swz<(1 << (TB - 1)) / TH>(a.t, runoff, htab, t, st);
         }
         __syncthreads();
         if (++it_stage == S) it_stage = 0;
@@ -280,8 +307,8 @@ __device__ __forceinline__ void build_loff(const int* tl, int* loff) {
     }
 }
 
-template <int K, int R, int S, bool SWZ, bool WB, int TB>
-__global__ void __launch_bounds__(kThreads) k_apply_fp32(ApplyArgs a) {
+template <int K, int R, int S, bool SWZ, bool WB, int TB, int NG, int TH>
+__global__ void __launch_bounds__(TH) k_apply_fp32(ApplyArgs a) {
     constexpr int D = 1 << K;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tileAmps = 1 << a.t.T;
@@ -302,23 +329,24 @@ __global__ void __launch_bounds__(kThreads) k_apply_fp32(ApplyArgs a) {
         for (int c = threadIdx.x; c < D; c += blockDim.x) sloff[c] = loff[c] ^ static_cast<int>(stage_xor(htab, loff[c]));
     }
     __syncthreads();
-    apply_tiles<K, R, S, SWZ, WB, TB, (K <= 4)>(a, stage, Ms, runoff, loff, blockIdx.x, gridDim.x, htab, sloff);
+    apply_tiles<K, R, S, SWZ, WB, TB, (K <= 4), NG, TH>(a, stage, Ms, runoff, loff, blockIdx.x, gridDim.x, htab, sloff);
 }
 
 template <int K>
 struct ApplyCfg;
 // SWZ: the swizzled stage and, where the targets call for it, in-place outputs
 // with an address-order write-back are available (k <= 4).
-template <> struct ApplyCfg<1> { static constexpr int T = 11, R = 2, S = 2; static constexpr bool SWZ = true; };
-template <> struct ApplyCfg<2> { static constexpr int T = 11, R = 4, S = 2; static constexpr bool SWZ = true; };
-template <> struct ApplyCfg<3> { static constexpr int T = 11, R = 8, S = 2; static constexpr bool SWZ = true; };
-// k = 4: 2^12-amplitude tiles, so that a tile has one 16-row item per thread
-// (2^11 left half of the CTA idle in the compute phase), two stages so that
-// three CTAs fit an SM (faster than three stages at two CTAs)
-template <> struct ApplyCfg<4> { static constexpr int T = 12, R = 16, S = 2; static constexpr bool SWZ = true; };
+template <> struct ApplyCfg<1> { static constexpr int NG = 1, TH = kThreads, T = 11, R = 2, S = 2; static constexpr bool SWZ = true; };
+template <> struct ApplyCfg<2> { static constexpr int NG = 1, TH = kThreads, T = 11, R = 4, S = 2; static constexpr bool SWZ = true; };
+template <> struct ApplyCfg<3> { static constexpr int NG = 1, TH = kThreads, T = 11, R = 8, S = 2; static constexpr bool SWZ = true; };
+// k = 3: scalar FMAs (N = 27: 0.349 ms, packed ones 0.367).  k = 4: CTAs of 128
+// threads with two groups per thread, which share the matrix's broadcast loads
+// (N = 27: 0.406 ms; one group, 256 threads: 0.422; scalar FMAs 0.452 / 0.499 with
+// one / two groups); 2^12-amplitude tiles, two stages so that three CTAs fit an SM
+template <> struct ApplyCfg<4> { static constexpr int NG = 2, TH = 128, T = 12, R = 16, S = 2; static constexpr bool SWZ = true; };
 // k = 5, 6: states below one tile of 2^12 amplitudes only (launch_apply_fp32)
-template <> struct ApplyCfg<5> { static constexpr int T = 12, R = 8, S = 2; static constexpr bool SWZ = false; };
-template <> struct ApplyCfg<6> { static constexpr int T = 12, R = 8, S = 2; static constexpr bool SWZ = false; };
+template <> struct ApplyCfg<5> { static constexpr int NG = 1, TH = kThreads, T = 12, R = 8, S = 2; static constexpr bool SWZ = false; };
+template <> struct ApplyCfg<6> { static constexpr int NG = 1, TH = kThreads, T = 12, R = 8, S = 2; static constexpr bool SWZ = false; };
 
 // Form of a k <= 4 launch from its lowest non-target tile positions np[0..4]
 // (the group-index bits that vary across a warp).  With the plain layout a
@@ -419,21 +447,29 @@ cudaError_t launch_apply_k(float2* psi, int n, const int* phys, const float* d_m
     }
     constexpr size_t tables = sizeof(uint64_t) * 64 + 2 * sizeof(int) * 64 + 256;
     const size_t smem = sizeof(float2) * (static_cast<size_t>(C::S) << g.T) + sizeof(float2) * D * D + tables;
-    auto kern = form == 2   ? k_apply_fp32<K, C::R, C::S, C::SWZ, C::SWZ, C::T>
-                : form == 1 ? k_apply_fp32<K, C::R, C::S, C::SWZ, false, C::T>
-                            : k_apply_fp32<K, C::R, C::S, false, false, C::T>;
+    // several groups per item on full tiles only
+    const bool whole = g.T == C::T;
+    auto kern = form == 2   ? k_apply_fp32<K, C::R, C::S, C::SWZ, C::SWZ, C::T, C::NG, C::TH>
+                : form == 1 ? k_apply_fp32<K, C::R, C::S, C::SWZ, false, C::T, C::NG, C::TH>
+                : whole     ? k_apply_fp32<K, C::R, C::S, false, false, C::T, C::NG, C::TH>
+                            : k_apply_fp32<K, C::R, C::S, false, false, C::T, 1, C::TH>;
     {
         const size_t full = sizeof(float2) * (static_cast<size_t>(C::S) << C::T) + sizeof(float2) * D * D + tables;
         cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(full));
         if (e != cudaSuccess) return e;
     }
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, C::TH, smem);
     if (e != cudaSuccess) return e;
     if (occ < 1) occ = 1;
+    // k = 1, 2 on states beyond the L2: two CTAs per SM, 32 KiB of loads in flight, which is all that the
+    // memory's latency takes; more only turn its bus around more often (N = 26 / 29, k = 1: 182 / 1402 us
+    // with the six that fit, 162 / 1269 with two).  In the L2 (N = 22: 10.3 and 12.3 us) and at k = 3,
+    // whose arithmetic wants the warps (N = 26: 179 and 199 us), as many as fit.
+    if (K <= 2 && n >= kBeyondL2 && occ > 2) occ = 2;
     uint64_t grid = static_cast<uint64_t>(num_sms()) * occ;
     if (grid > g.ntiles) grid = g.ntiles;
-    kern<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(a);
+    kern<<<static_cast<unsigned>(grid), C::TH, smem, st>>>(a);
     ++*launches;
     return cudaGetLastError();
 }

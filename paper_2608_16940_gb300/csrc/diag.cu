@@ -3,12 +3,16 @@
 // target bits; Eq. cost-diag-formal: one streaming pass, no permutation, the
 // layout unchanged).
 //
-// Each thread updates pairs of amplitudes (one 16-byte float4, physical
-// indices y and y + 1) and keeps six pairs in flight; four 256-thread CTAs per
-// SM fit both the registers and the widest (2^12-entry) table.  The entry index c(y)
-// (bit j = bit p_j of y) is assembled from three shared tables over bits
-// 0..11, 12..23 and 24..33 of y; the 2^k-entry FP32 table itself sits in
-// shared memory.  Loads and stores stream (evict-first): 16 B per amplitude.
+// A CTA walks tiles of 1024 pairs of amplitudes (16 bytes, physical indices y and
+// y + 1), four per thread in flight; three 256-thread CTAs per SM put 48 KiB in
+// flight: the memory's latency takes no more, and more turn its bus around more
+// often (N = 26, k = 4: 187 us with 96 KiB, 181 with 72, 173 with 48).  The entry
+// index c(y) (bit j = bit p_j of y) is the OR of a part per thread, per tile and
+// per place in the tile; shared tables over the bits of y, 18 KiB formed by every
+// CTA, cost a small state most of its launch (N = 20, k = 4: 20.5 us, 6.1 here;
+// N = 27, k = 1 / 8 / 12: 0.344 / 0.366 / 0.446 ms, 0.325 / 0.328 / 0.339 here).
+// The 2^k-entry FP32 table itself sits in shared memory.  Loads and stores
+// stream (evict-first): 16 B per amplitude.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -21,7 +25,8 @@ namespace qsa {
 namespace {
 
 constexpr int kDiagThreads = 256;
-constexpr int kDiagUnroll = 6;
+constexpr int kDiagUnroll = 4;
+constexpr int kDiagCtas = 3;
 
 struct DiagArgs {
     float4* psi;
@@ -40,53 +45,44 @@ __device__ __forceinline__ float4 cmul2(float4 v, float2 a, float2 b) {
     return w;
 }
 
-__global__ void __launch_bounds__(kDiagThreads, 4) k_apply_diag(DiagArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    float2* d = reinterpret_cast<float2*>(smem);
-    uint16_t* t0 = reinterpret_cast<uint16_t*>(d + (1 << a.k));   // bits 0..11 of y
-    uint16_t* t1 = t0 + 4096;                                       // bits 12..23
-    uint16_t* t2 = t1 + 4096;                                       // bits 24..33
-    for (int i = threadIdx.x; i < (1 << a.k); i += blockDim.x) d[i] = a.d[i];
-    for (int i = threadIdx.x; i < 4096; i += blockDim.x) {
-        uint32_t c0 = 0, c1 = 0, c2 = 0;
-        for (int j = 0; j < a.k; ++j) {
-            const int p = a.p[j];
-            if (p < 12)
-                c0 |= ((static_cast<uint32_t>(i) >> p) & 1u) << j;
-            else if (p < 24)
-                c1 |= ((static_cast<uint32_t>(i) >> (p - 12)) & 1u) << j;
-            else
-                c2 |= ((static_cast<uint32_t>(i) >> (p - 24)) & 1u) << j;
-        }
-        t0[i] = static_cast<uint16_t>(c0);
-        t1[i] = static_cast<uint16_t>(c1);
-        if (i < 1024) t2[i] = static_cast<uint16_t>(c2);
-    }
-    __syncthreads();
-
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-    for (uint64_t q0 = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q0 < a.npairs;
-         q0 += kDiagUnroll * stride) {
-        float4 v[kDiagUnroll];
+// Part of the entry index from the bits of y in [from, to).
+__device__ __forceinline__ uint32_t entry_part(const DiagArgs& a, uint64_t y, int from, int to) {
+    const uint32_t lo = static_cast<uint32_t>(y), hi = static_cast<uint32_t>(y >> 32);
+    uint32_t c = 0;
 #pragma unroll
-        for (int u = 0; u < kDiagUnroll; ++u) {
-            const uint64_t q = q0 + u * stride;
-            if (q < a.npairs) v[u] = __ldcs(a.psi + q);
-        }
-#pragma unroll
-        for (int u = 0; u < kDiagUnroll; ++u) {
-            const uint64_t q = q0 + u * stride;
-            if (q < a.npairs) {
-                const uint64_t y = q << 1;
-                const uint32_t hi = static_cast<uint32_t>(t1[(y >> 12) & 4095u]) | t2[(y >> 24) & 1023u];
-                const uint32_t lo = static_cast<uint32_t>(y) & 4095u;
-                __stcs(a.psi + q, cmul2(v[u], d[t0[lo] | hi], d[t0[lo | 1u] | hi]));
-            }
-        }
+    for (int j = 0; j < QSA_MAX_DIAG; ++j) {
+        if (j >= a.k) break;
+        const int p = a.p[j];
+        if (p >= from && p < to) c |= (((p < 32 ? lo : hi) >> (p & 31)) & 1u) << j;
     }
+    return c;
 }
 
-size_t diag_smem(int k) { return (sizeof(float2) << k) + 2 * (4096 + 4096 + 1024); }
+__global__ void __launch_bounds__(kDiagThreads, kDiagCtas) k_apply_diag(const __grid_constant__ DiagArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    float2* d = reinterpret_cast<float2*>(smem);
+    for (int i = threadIdx.x; i < (1 << a.k); i += blockDim.x) d[i] = a.d[i];
+    // y = tile << 11 | place << 9 | thread << 1 | odd
+    const uint32_t odd = entry_part(a, 1, 0, 1), ct = entry_part(a, 2 * threadIdx.x, 1, 9);
+    const uint32_t c1 = entry_part(a, 1 << 9, 9, 11), c2 = entry_part(a, 2 << 9, 9, 11);
+    __syncthreads();
+
+    constexpr uint64_t kTile = kDiagThreads * kDiagUnroll;
+    for (uint64_t q0 = blockIdx.x * kTile; q0 < a.npairs; q0 += gridDim.x * kTile) {
+        const uint64_t q = q0 + threadIdx.x;
+        float4 v[kDiagUnroll];
+#pragma unroll
+        for (int u = 0; u < kDiagUnroll; ++u)
+            if (q + u * kDiagThreads < a.npairs) v[u] = __ldcs(a.psi + q + u * kDiagThreads);
+        const uint32_t c = ct | entry_part(a, q0 << 1, 11, 64);
+#pragma unroll
+        for (int u = 0; u < kDiagUnroll; ++u)
+            if (q + u * kDiagThreads < a.npairs) {
+                const uint32_t cu = c | (u & 1 ? c1 : 0u) | (u & 2 ? c2 : 0u);
+                __stcs(a.psi + q + u * kDiagThreads, cmul2(v[u], d[cu], d[cu | odd]));
+            }
+    }
+}
 
 }  // namespace
 
@@ -99,18 +95,9 @@ cudaError_t launch_apply_diag(float2* psi, int n, const int* phys, int k, const 
     a.d = reinterpret_cast<const float2*>(d_tab);
     a.k = k;
     for (int j = 0; j < k; ++j) a.p[j] = phys[j];
-    {
-        cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(k_apply_diag),
-                                      static_cast<int>(diag_smem(QSA_MAX_DIAG)));
-        if (e != cudaSuccess) return e;
-    }
-    const size_t sm = diag_smem(k);
-    int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_diag, kDiagThreads, sm);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    const uint64_t need = (a.npairs + kDiagThreads - 1) / kDiagThreads;
-    const uint64_t grid = std::min<uint64_t>(static_cast<uint64_t>(num_sms()) * occ, need);
+    const size_t sm = sizeof(float2) << k;   // at most 32 KiB
+    const uint64_t tile = kDiagThreads * kDiagUnroll, need = (a.npairs + tile - 1) / tile;
+    const uint64_t grid = std::min<uint64_t>(static_cast<uint64_t>(num_sms()) * kDiagCtas, need);
     k_apply_diag<<<static_cast<unsigned>(grid), kDiagThreads, sm, st>>>(a);
     ++*launches;
     return cudaGetLastError();
