@@ -175,8 +175,9 @@ __device__ __forceinline__ double square_exact(float v) {
 // the tile bits that the writing lanes vary (formed on the host).  With
 // partials the norm is taken in the same read (double-float per thread, as
 // k_reduce_z).  N = 27, random layout, probabilities and norm:
-// 2.01 ms by gather and a second pass, 0.474 ms here (0.317 ms at the copy rate).
-constexpr int kProbT = 12;
+// 2.01 ms by gather and a second pass, 0.458 ms here (0.317 ms at the copy rate;
+// 0.478 with four CTAs per SM and no loads in flight while a tile is written).
+constexpr int kProbT = 12, kProbCtas = 3;
 
 struct ProbArgs {
     const float2* psi;
@@ -191,7 +192,7 @@ struct ProbArgs {
     uint16_t lslot[kProbT];    // slot of the tile bit that holds the i-th logical qubit
 };
 
-__global__ void __launch_bounds__(kRedThreads, 4) k_probs_tile(const __grid_constant__ ProbArgs a) {
+__global__ void __launch_bounds__(kRedThreads, kProbCtas) k_probs_tile(const __grid_constant__ ProbArgs a) {
     __shared__ __align__(16) double st[1 << kProbT];
     const int tid = threadIdx.x, lane = tid & 31;
     uint64_t gl = 0, gs = 0;
@@ -206,21 +207,22 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_probs_tile(const __grid_cons
         }
     const int op = lane < a.nouter ? a.opos[lane] : 0, oq = lane < a.nouter ? a.oq[lane] : 0;
     float zs = 0.f, zc = 0.f;
-    for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-        // the tile's base in both orders: lane i places outer bit i
-        const uint64_t bit = lane < a.nouter ? (t >> lane) & 1ull : 0ull;
-        const uint64_t pb = bit << op, lb = bit << oq;
-        const uint64_t pbase = (static_cast<uint64_t>(__reduce_or_sync(0xffffffffu, static_cast<uint32_t>(pb >> 32))) << 32) |
-                               __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(pb));
-        const uint64_t lbase = (static_cast<uint64_t>(__reduce_or_sync(0xffffffffu, static_cast<uint32_t>(lb >> 32))) << 32) |
-                               __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(lb));
-        float4 v[8];
+    // the tile's base in both orders: lane i places outer bit i
+    auto place = [&](uint64_t t, int at) {
+        const uint64_t b = lane < a.nouter ? ((t >> lane) & 1ull) << at : 0ull;
+        return (static_cast<uint64_t>(__reduce_or_sync(0xffffffffu, static_cast<uint32_t>(b >> 32))) << 32) |
+               __reduce_or_sync(0xffffffffu, static_cast<uint32_t>(b));
+    };
+    float4 v[8];
+    auto load = [&](uint64_t t) {
+        const uint64_t base = place(t, op) | gl;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const uint64_t g = pbase | gl | (k & 1 ? a.poff[9] : 0ull) | (k & 2 ? a.poff[10] : 0ull) |
-                               (k & 4 ? a.poff[11] : 0ull);
-            v[k] = __ldcs(reinterpret_cast<const float4*>(a.psi + g));
-        }
+        for (int k = 0; k < 8; ++k)
+            v[k] = __ldcs(reinterpret_cast<const float4*>(a.psi + (base | (k & 1 ? a.poff[9] : 0ull) |
+                                                                   (k & 2 ? a.poff[10] : 0ull) | (k & 4 ? a.poff[11] : 0ull))));
+    };
+    if (blockIdx.x < a.ntiles) load(blockIdx.x);
+    for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
         __syncthreads();   // the tile before has been read
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -235,12 +237,14 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_probs_tile(const __grid_cons
                 acc_square(zs, zc, v[k].w, false);
             }
         }
+        if (t + gridDim.x < a.ntiles) load(t + gridDim.x);   // in flight while this tile is written
         __syncthreads();
+        const uint64_t lbase = place(t, oq) | gs;
         const uint32_t s0 = a.lslot[0];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const uint32_t s = ss ^ (k & 1 ? a.lslot[9] : 0u) ^ (k & 2 ? a.lslot[10] : 0u) ^ (k & 4 ? a.lslot[11] : 0u);
-            const uint64_t g = lbase | gs | (k & 1 ? a.loff[9] : 0ull) | (k & 2 ? a.loff[10] : 0ull) |
+            const uint64_t g = lbase | (k & 1 ? a.loff[9] : 0ull) | (k & 2 ? a.loff[10] : 0ull) |
                                (k & 4 ? a.loff[11] : 0ull);
             __stcs(reinterpret_cast<double2*>(a.out + g), make_double2(st[s], st[s ^ s0]));
         }
@@ -455,6 +459,75 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_weights_z1024(const float4* 
             }
             __syncthreads();
         }
+    }
+}
+
+// The sums alone, for states of at least one block of 1024 amplitudes: as
+// k_weights_z1024 (each mask's terms in the same order whatever the other masks,
+// so a mask's result does not depend on them), kZLoads 16-byte loads per lane in
+// flight (64 KiB per SM).  N = 27: one mask 0.283 ms with one load per thread and
+// the signs selected per component, 0.197 here (two / four masks 0.207 / 0.272;
+// 0.158 ms at the copy rate).
+constexpr int kZLoads = 4, kZCtas = 4;
+template <int NM>
+__global__ void __launch_bounds__(kRedThreads, NM <= 2 ? kZCtas : 1) k_zsums1024(const float4* __restrict__ psi2, uint64_t nblocks,
+                                                           const __grid_constant__ ZMasks masks,
+                                                           double* __restrict__ partials) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t warps = static_cast<uint64_t>(gridDim.x) * (blockDim.x >> 5);
+    float zs[NM] = {}, zc[NM] = {};
+    uint32_t kb[NM] = {}, lb[NM] = {}, fr[NM] = {};
+    float bf[NM] = {};
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+        for (int k = 0; k < 16; ++k) kb[m] |= static_cast<uint32_t>(__popcll((64ull * k) & masks.m[m]) & 1) << k;
+        lb[m] = __popcll((2ull * lane) & masks.m[m]) & 1;
+        bf[m] = (masks.m[m] & 1ull) ? -1.f : 1.f;
+    }
+    for (uint64_t w = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; w < nblocks; w += warps) {
+        const float4* p = psi2 + w * 512 + lane;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const uint32_t f = (__popcll((w << 10) & masks.m[m]) & 1) ^ lb[m];
+            if (f != fr[m]) {
+                zs[m] = -zs[m];
+                zc[m] = -zc[m];
+                fr[m] = f;
+            }
+        }
+#pragma unroll
+        for (int k0 = 0; k0 < 16; k0 += kZLoads) {
+            float4 a[kZLoads];
+#pragma unroll
+            for (int k = 0; k < kZLoads; ++k) a[k] = __ldcs(p + 32 * (k0 + k));
+#pragma unroll
+            for (int k = 0; k < kZLoads; ++k) {
+                float h0, l0, h1, l1;
+                square_pair(a[k].x, a[k].y, h0, l0);
+                square_pair(a[k].z, a[k].w, h1, l1);
+#pragma unroll
+                for (int m = 0; m < NM; ++m) {
+                    const float g0 = __uint_as_float(0x3f800000u | (((kb[m] >> (k0 + k)) & 1u) << 31));
+                    add_scaled(zs[m], zc[m], h0, l0, g0);
+                    add_scaled(zs[m], zc[m], h1, l1, g0 * bf[m]);
+                }
+            }
+        }
+    }
+    __shared__ double ws[kRedThreads / 32];
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+        const double sg = fr[m] ? -1.0 : 1.0;   // back from the thread's frame
+        double acc = sg * static_cast<double>(zs[m]) + sg * static_cast<double>(zc[m]);
+        acc = warp_sum_d(acc);
+        if (lane == 0) ws[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            double v = threadIdx.x < (kRedThreads / 32) ? ws[threadIdx.x] : 0.0;
+            v = warp_sum_d(v);
+            if (threadIdx.x == 0) partials[static_cast<uint64_t>(m) * gridDim.x + blockIdx.x] = v;
+        }
+        __syncthreads();
     }
 }
 
@@ -1200,6 +1273,25 @@ __global__ void __launch_bounds__(kRedThreads) k_dm_diag(const float2* __restric
 
 int reduce_partials() { return num_sms() * kRedBlocksPerSM; }
 
+namespace {
+
+cudaError_t launch_zsums(const float2* psi, int n, const uint64_t* physmasks, int nmasks, double* d_partials, double* d_out,
+                         cudaStream_t st, uint64_t* launches) {
+    const uint64_t nblocks = 1ull << (n - 10);
+    ZMasks zm{};
+    zm.n = nmasks;
+    for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
+    // the same grid for any number of masks: a mask's partial sums are the same in all of them
+    const uint64_t nb = std::min<uint64_t>((nblocks + 7) / 8, static_cast<uint64_t>(kZCtas) * num_sms());
+    auto kern = nmasks == 1 ? k_zsums1024<1> : nmasks == 2 ? k_zsums1024<2> : nmasks == 3 ? k_zsums1024<3> : k_zsums1024<4>;
+    kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, zm, d_partials);
+    k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_partials, static_cast<int>(nb), d_out);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double* d_partials, double* d_out,
                             cudaStream_t st, uint64_t* launches) {
     const uint64_t npairs = (1ull << n) >> 1;
@@ -1208,6 +1300,7 @@ cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double*
         // n = 1 is still >= one pair; n >= 1 always holds here
         return cudaErrorInvalidValue;
     }
+    if (n >= 10) return launch_zsums(psi, n, &physmask, 1, d_partials, d_out, st, launches);
     k_reduce_z<<<nb, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), npairs, physmask, d_partials);
     k_finalize_sum<<<1, 1024, 0, st>>>(d_partials, nb, d_out);
     *launches += 2;
@@ -1217,6 +1310,7 @@ cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double*
 cudaError_t launch_reduce_z_multi(const float2* psi, int n, const uint64_t* physmasks, int nmasks,
                                   double* d_partials, double* d_out, cudaStream_t st, uint64_t* launches) {
     if (nmasks < 1 || nmasks > kMaxZMasks || n < 1) return cudaErrorInvalidValue;
+    if (n >= 10) return launch_zsums(psi, n, physmasks, nmasks, d_partials, d_out, st, launches);
     const uint64_t npairs = (1ull << n) >> 1;
     const int nb = reduce_partials();
     ZMasks zm{};
@@ -1297,8 +1391,8 @@ cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout
                 }
     for (int b = 0; b < kProbT; ++b) a.pslot[b] = static_cast<uint16_t>((1u << b) ^ vec[b]);
     for (int i = 0; i < kProbT; ++i) a.lslot[i] = a.pslot[lt[i]];
-    // as many CTAs as stay resident (four to an SM); at most reduce_partials()
-    const uint64_t nb = std::min<uint64_t>(a.ntiles, 4ull * num_sms());
+    // as many CTAs as stay resident; at most reduce_partials()
+    const uint64_t nb = std::min<uint64_t>(a.ntiles, static_cast<uint64_t>(kProbCtas) * num_sms());
     k_probs_tile<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(a);
     ++*launches;
     if (d_norm) {
