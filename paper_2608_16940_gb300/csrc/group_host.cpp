@@ -11,6 +11,7 @@
 #include <cmath>
 #include <complex>
 #include <cstring>
+#include <deque>
 #include <utility>
 #include <vector>
 
@@ -37,6 +38,11 @@ uint32_t diag_bytes(int k) { return std::max(16u, 8u << k); }
 static_assert(sizeof(GroupOp) == 112 && sizeof(GroupRound) % 16 == 0, "16-byte aligned program");
 
 using Cx = std::complex<double>;
+
+// Plain products and moduli: the library's complex product tests for NaN and its
+// modulus guards against overflow, several times the cost of the arithmetic here.
+Cx mul(Cx a, Cx b) { return {a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real()}; }
+double modulus(Cx z) { return std::sqrt(std::norm(z)); }
 
 // What the passes are made of.  A unitary one-qubit operator is split as
 // diag(p) R diag(q) with a real rotation R: diag(q) becomes a diagonal operator
@@ -84,15 +90,15 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
             const int at = s.pos[0];
             // the phases that wait join the operator, their moduli (the factors of a rotation's rows) stay
             // with the diagonal before it, so that it is still unitary
-            const double m0 = std::abs(wait[at][0]), m1 = std::abs(wait[at][1]);
+            const double m0 = modulus(wait[at][0]), m1 = modulus(wait[at][1]);
             const Cx w0 = wait[at][0] / m0, w1 = wait[at][1] / m1;
             double scale = 0.0;
-            for (const Cx& z : f.m) scale = std::max(scale, std::abs(z));
+            for (const Cx& z : f.m) scale = std::max(scale, modulus(z));
             double c = 0.0, sn = 0.0;
             Cx p[2], q[2];
             if (m0 > 0.0 && m1 > 0.0 && scale > 0.0 && scale < 1e30 &&
-                split_rotation({f.m[0] * w0 / scale, f.m[1] * w1 / scale, f.m[2] * w0 / scale, f.m[3] * w1 / scale}, &c,
-                               &sn, p, q)) {
+                split_rotation({mul(f.m[0], w0) / scale, mul(f.m[1], w1) / scale, mul(f.m[2], w0) / scale,
+                                mul(f.m[3], w1) / scale}, &c, &sn, p, q)) {
                 if (sn == 0.0) {   // diagonal after all
                     wait[at] = {scale * c * p[0] * m0, scale * c * p[1] * m1};
                     continue;
@@ -103,7 +109,7 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
                 const double t = f.t, kappa = 1.0 / std::sqrt(1.0 + t * t), norm = scale * std::sqrt(c * c + sn * sn);
                 wait[at] = {p[0] * norm * (flip ? 1.0 / kappa : kappa), p[1] * norm * (flip ? kappa : 1.0 / kappa)};
                 const Cx q0 = m0, q1 = (flip ? -q[1] : q[1]) * m1;
-                if (std::abs(q0 - 1.0) > 1e-14 || std::abs(q1 - 1.0) > 1e-14) diag1(at, q0, q1);
+                if (std::norm(q0 - 1.0) > 1e-28 || std::norm(q1 - 1.0) > 1e-28) diag1(at, q0, q1);
                 f.kind = Fine::kRot;
                 f.flip = flip;
                 f.src = -1;
@@ -132,18 +138,22 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
 // one of its positions without being diagonal; until then it is open.  It still
 // takes an operator afterwards, on positions that nothing but diagonal operators
 // has touched since where it stands.
-std::vector<Fine> merge_diagonals(const std::vector<Fine>& ops, int cap) {
+// New blocks are kept in *made.
+std::vector<Fine*> merge_diagonals(const std::vector<Fine*>& ops, int cap, std::deque<Fine>* made) {
     struct Block {
         uint64_t mask = 0, closed = 0;
         int64_t place = -1;          // index in seq, -1: not placed yet
-        std::vector<const Fine*> of;
+        std::vector<Fine*> of;
     };
     std::vector<Block> blocks;
-    std::vector<std::pair<const Fine*, int>> seq;   // an operator, or a block's index
+    std::vector<std::pair<Fine*, int>> seq;         // an operator, or a block's index
     std::vector<int64_t> last(64, -1);              // per position: the last operator that is not diagonal
-    for (const Fine& f : ops) {
+    size_t open = 0;   // blocks before this one are closed on every position
+    for (Fine* fp : ops) {
+        Fine& f = *fp;
         if (f.kind != Fine::kDiag) {
-            for (size_t b = 0; b < blocks.size(); ++b) {
+            while (open < blocks.size() && blocks[open].closed == blocks[open].mask) ++open;
+            for (size_t b = open; b < blocks.size(); ++b) {
                 if (!(blocks[b].mask & f.mask)) continue;
                 if (blocks[b].place < 0) {
                     blocks[b].place = static_cast<int64_t>(seq.size());
@@ -152,11 +162,11 @@ std::vector<Fine> merge_diagonals(const std::vector<Fine>& ops, int cap) {
                 blocks[b].closed |= blocks[b].mask & f.mask;
             }
             for (int j = 0; j < f.k; ++j) last[f.pos[j]] = static_cast<int64_t>(seq.size());
-            seq.push_back({&f, -1});
+            seq.push_back({fp, -1});
             continue;
         }
         int best = -1, gain = -1;
-        for (size_t b = 0; b < blocks.size(); ++b) {
+        for (size_t b = blocks.size() > 24 ? blocks.size() - 24 : 0; b < blocks.size(); ++b) {
             Block& B = blocks[b];
             if ((B.closed & f.mask) || popc(B.mask | f.mask) > cap) continue;
             bool ok = true;
@@ -171,35 +181,52 @@ std::vector<Fine> merge_diagonals(const std::vector<Fine>& ops, int cap) {
             blocks.emplace_back();
         }
         blocks[best].mask |= f.mask;
-        blocks[best].of.push_back(&f);
+        blocks[best].of.push_back(fp);
     }
     for (size_t b = 0; b < blocks.size(); ++b)
         if (blocks[b].place < 0) seq.push_back({nullptr, static_cast<int>(b)});
-    std::vector<Fine> out;
+    std::vector<Fine*> out;
     for (const auto& it : seq) {
         if (it.first) {
-            out.push_back(*it.first);
+            out.push_back(it.first);
             continue;
         }
         const Block& B = blocks[it.second];
         if (B.of.size() == 1) {
-            out.push_back(*B.of[0]);
+            out.push_back(B.of[0]);
             continue;
         }
-        Fine f{Fine::kDiag, B.mask, 0, {}};
+        made->push_back(Fine{Fine::kDiag, B.mask, 0, {}});
+        Fine& f = made->back();
+        int bit_of[64];
         for (int q = 0; q < 64; ++q)
-            if ((B.mask >> q) & 1) f.pos[f.k++] = q;
-        f.m.assign(size_t(1) << f.k, 1.0);
+            if ((B.mask >> q) & 1) {
+                bit_of[q] = f.k;
+                f.pos[f.k++] = q;
+            }
+        // one-qubit members as an outer product, then the others
+        std::array<std::array<Cx, 2>, kGroupDiagMax> one;
+        one.fill({1.0, 1.0});
+        for (const Fine* o : B.of)
+            if (o->k == 1)
+                for (int v = 0; v < 2; ++v) one[bit_of[o->pos[0]]][v] = mul(one[bit_of[o->pos[0]]][v], o->m[v]);
+        f.m.resize(size_t(1) << f.k);
+        f.m[0] = 1.0;
+        for (int j = 0; j < f.k; ++j)
+            for (size_t c = 0; c < (size_t(1) << j); ++c) {
+                f.m[c | size_t(1) << j] = mul(f.m[c], one[j][1]);
+                f.m[c] = mul(f.m[c], one[j][0]);
+            }
         for (const Fine* o : B.of) {
-            int bit[kGroupDiagMax];
-            for (int j = 0; j < o->k; ++j) bit[j] = static_cast<int>(std::find(f.pos, f.pos + f.k, o->pos[j]) - f.pos);
+            if (o->k == 1) continue;
+            uint8_t part[kGroupDiagMax] = {}, at[1 << kGroupDiagMax] = {};   // index parts of f's bits, its indices
+            for (int j = 0; j < o->k; ++j) part[bit_of[o->pos[j]]] = static_cast<uint8_t>(1u << j);
             for (size_t c = 0; c < f.m.size(); ++c) {
-                size_t x = 0;
-                for (int j = 0; j < o->k; ++j) x |= ((c >> bit[j]) & 1) << j;
-                f.m[c] *= o->m[x];
+                if (c) at[c] = static_cast<uint8_t>(at[c & (c - 1)] | part[__builtin_ctzll(c)]);
+                f.m[c] = mul(f.m[c], o->m[at[c]]);
             }
         }
-        out.push_back(std::move(f));
+        out.push_back(&f);
     }
     return out;
 }
@@ -256,29 +283,30 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
     const int T = std::min(kGroupTileBits, n);
     const int max_high = kGroupTileBits - kGroupLowBits;
     std::vector<Fine> fine = split_operators(n, src);
-    std::vector<const Fine*> left(fine.size());
+    std::vector<Fine*> left(fine.size());
     for (size_t i = 0; i < fine.size(); ++i) left[i] = &fine[i];
     ModulusCarry carry;
+    const uint64_t all = n < 64 ? (1ull << n) - 1 : ~0ull;
     // What a pass may take, by the sizes before diagonal operators share tables and rotations share
     // entries; less of it where the program comes out too long after all.
     double room = 2.0 * kGroupProgBytes;
     while (!left.empty()) {
         // the operators of this pass
-        std::vector<Fine> take;
-        std::vector<const Fine*> later;
+        std::vector<Fine*> take, later;
         uint64_t tile = 0, held_dense = 0, held_diag = 0;
         double bytes = 0.0;
         size_t i = 0;
         for (; i < left.size(); ++i) {
             const Fine& f = *left[i];
-            if (later.size() >= kLookahead) break;
+            // nothing behind can be taken once every position is held
+            if (later.size() >= kLookahead || held_dense == all) break;
             const bool dg = f.kind == Fine::kDiag;
             const double b = op_bytes(f) + (dg && f.k < 3 ? 16.0 : 64.0);
             bool ok = !(f.mask & held_dense) && (dg || !(f.mask & held_diag));
             ok = ok && take.size() < kMaxOps && bytes + b <= room;
             if (ok && !dg && n > kGroupTileBits) ok = popc((tile | f.mask) >> kGroupLowBits) <= max_high;
             if (ok) {
-                take.push_back(f);
+                take.push_back(left[i]);
                 bytes += b;
                 if (!dg) tile |= f.mask;
             } else {
@@ -289,7 +317,7 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
         later.insert(later.end(), left.begin() + static_cast<long>(i), left.end());
 
         GroupPass p{};
-        p.only = take.size() == 1 ? take[0].src : -1;
+        p.only = take.size() == 1 ? take[0]->src : -1;
         // the tile: the positions of the dense operators, filled up from the lowest
         p.T = T;
         p.ntiles = 1ull << (n - T);
@@ -301,45 +329,46 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
         uint64_t tmask = (1ull << m) - 1;
         for (int e = 0; e < p.nx; ++e) tmask |= 1ull << p.xpos[e];
         // bit of (tile number, tile-local index) that holds position q
-        auto cbit = [&](int q) {
-            if (q < m) return q;
-            if ((tmask >> q) & 1) {
-                int e = 0;
-                while (p.xpos[e] != q) ++e;
-                return m + e;
-            }
-            return T + popc(~tmask & ((1ull << q) - 1));
-        };
+        int cbit[64];
+        for (int q = 0, e = 0; q < n; ++q)
+            cbit[q] = q < m ? q : (tmask >> q) & 1 ? m + e++ : T + popc(~tmask & ((1ull << q) - 1));
 
         // diagonal operators share tables of up to 2^6 entries (lanes read 512 bytes)
-        std::vector<Fine> ops = merge_diagonals(take, 6);
+        std::deque<Fine> made;
+        const std::vector<Fine*> ops = merge_diagonals(take, 6, &made);
 
         // inverted bits, as the operators in order leave them
         uint64_t flipped = 0;
-        for (Fine& f : ops) {
+        for (Fine* fp : ops) {
+            Fine& f = *fp;
+            f.inv = 0;
             for (int j = 0; j < f.k; ++j) f.inv |= static_cast<uint32_t>((flipped >> f.pos[j]) & 1) << j;
             if (f.flip) flipped ^= f.mask;
         }
         for (int q = 0; q < n; ++q)
-            if ((flipped >> q) & 1) p.flip |= 1u << cbit(q);
+            if ((flipped >> q) & 1) p.flip |= 1u << cbit[q];
 
         // rounds
         std::vector<GroupRound> rounds;
         std::vector<GroupOp> code;
         std::vector<unsigned char> par;
-        std::vector<const Fine*> rest(ops.size()), nextr;
-        for (size_t x = 0; x < ops.size(); ++x) rest[x] = &ops[x];
+        std::vector<const Fine*> rest(ops.begin(), ops.end()), nextr;
         while (!rest.empty()) {
             uint32_t reg = 0;
             uint64_t hd = 0, hg = 0;
             std::vector<const Fine*> now;
             nextr.clear();
-            for (const Fine* f : rest) {
+            for (size_t x = 0; x < rest.size(); ++x) {
+                const Fine* f = rest[x];
+                if (!(tile & ~hd) && tile) {   // every position that a dense operator acts on is held
+                    nextr.insert(nextr.end(), rest.begin() + static_cast<long>(x), rest.end());
+                    break;
+                }
                 const bool dg = f->kind == Fine::kDiag;
                 bool ok = !(f->mask & hd) && (dg || !(f->mask & hg));
                 uint32_t lm = 0;
                 if (!dg)
-                    for (int j = 0; j < f->k; ++j) lm |= 1u << cbit(f->pos[j]);
+                    for (int j = 0; j < f->k; ++j) lm |= 1u << cbit[f->pos[j]];
                 ok = ok && popc(reg | lm) <= 4;
                 if (ok) {
                     now.push_back(f);
@@ -375,7 +404,7 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                 GroupOp op{};
                 if (f->kind == Fine::kRot) {
                     // joins the last rotations when nothing after them acts on its position
-                    const int r = reg_of[cbit(f->pos[0])];
+                    const int r = reg_of[cbit[f->pos[0]]];
                     size_t x = masks.size();
                     bool joined = false;
                     while (x > 0 && !joined && !(masks[x - 1] & f->mask)) {
@@ -407,7 +436,7 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                     op.code = kGroupDiag;
                     int ord[kGroupDiagMax], key[kGroupDiagMax];
                     for (int j = 0; j < f->k; ++j) {
-                        const int c = cbit(f->pos[j]);
+                        const int c = cbit[f->pos[j]];
                         ord[j] = j;
                         key[j] = c >= kGroupTileBits ? 64 + c : (reg >> c) & 1 ? 32 + c
                                  : static_cast<int>(std::find(tb, tb + 8, c) - tb);
@@ -436,8 +465,9 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                         for (int j = 0; j < f->k; ++j) y |= ((x >> j) & 1) << ord[j];
                         const Cx z = f->m[y ^ f->inv];
                         const double m2 = std::norm(z);
-                        // rounded with error feedback on the modulus, relative to the entry's own
-                        const float2 e = m2 > 1e-30 && m2 < 1e30
+                        // small tables repeat over the state: rounded with error feedback on the modulus,
+                        // relative to the entry's own (in a large one the entries' errors average out)
+                        const float2 e = f->m.size() <= 8 && m2 > 1e-30 && m2 < 1e30
                                              ? f2_modulus(z, m2, share / m2, &carry)
                                              : make_float2(static_cast<float>(z.real()), static_cast<float>(z.imag()));
                         g[2 * x] = e.x;
@@ -448,7 +478,7 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                     float* g = reinterpret_cast<float*>(par.data() + op.off);
                     int rbit[4], ord[4];
                     for (int j = 0; j < f->k; ++j) {
-                        rbit[j] = reg_of[cbit(f->pos[j])];
+                        rbit[j] = reg_of[cbit[f->pos[j]]];
                         ord[j] = j;
                         op.code |= static_cast<uint8_t>(1u << rbit[j]);
                     }
