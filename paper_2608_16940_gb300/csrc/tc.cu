@@ -329,12 +329,14 @@ __device__ __forceinline__ uint64_t chunk_base(const TcArgs& a, uint64_t t) {
 // Entry [2 nu + s][2 kap + t] of A: the real embedding of G in the K-bit
 // numbering (k = 5: blockdiag(R, R), the block given by bit 5).  perm maps a
 // K-bit index to the operator index (bit b to bit vbit[b]); gs is G in shared
-// memory.
+// memory, its rows one entry apart from a power of two, since a warp reads 16
+// rows of one column at a time.
 __device__ __forceinline__ float a_entry(const TcArgs& a, const float2* gs, const int* perm, int nu, int kap, int s,
                                          int t) {
     if (a.k == 5 && (nu >> 5) != (kap >> 5)) return 0.f;
     const int m = a.k == 5 ? 31 : 63;
-    const float2 g = gs[(perm[nu & m] << a.k) + perm[kap & m]];
+    const int row = perm[nu & m];
+    const float2 g = gs[(row << a.k) + row + perm[kap & m]];
     return s == 0 ? (t == 0 ? g.x : -g.y) : (t == 0 ? g.y : g.x);
 }
 
@@ -376,11 +378,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_apply_tc(TcArgs a) {
     }
     // G into B buffer 0 with coalesced loads; the epilogue builds A from
     // there (scattered reads of G from global memory took about 0.17 ms per
-    // launch), and the converters write B only once A is ready
+    // launch), and the converters write B only once A is ready.  Rows of 2^k + 1
+    // entries: with 2^k a warp's reads met 16 to a bank (one k = 5 / 6 launch on a
+    // 2^18-amplitude state 18.6 / 24.7 us, 14.4 / 14.5 without the conflicts).
     const float2* g_sm = reinterpret_cast<const float2*>(Bsm);
-    int* perm = reinterpret_cast<int*>(Bsm + 32768);   // after G (at most 32 KiB)
+    int* perm = reinterpret_cast<int*>(Bsm + 34816);   // after G (at most 64 x 65 entries)
     for (int i = tid; i < (1 << (2 * a.k)); i += kThreads)
-        reinterpret_cast<float2*>(Bsm)[i] = reinterpret_cast<const float2*>(a.mat)[i];
+        reinterpret_cast<float2*>(Bsm)[i + (i >> a.k)] = reinterpret_cast<const float2*>(a.mat)[i];
     if (tid < 64) {
         int o = 0;
 #pragma unroll
