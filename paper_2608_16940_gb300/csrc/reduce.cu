@@ -665,10 +665,14 @@ __global__ void __launch_bounds__(256) k_draw_blocks(const uint64_t* __restrict_
     out[s] = ((t * nblocks + b) << kShotBits) | s;
 }
 
-// A warp takes `per` consecutive shots of the sorted list; for each block among
-// them it forms the prefix of the block's 1024 weights in shared memory (lanes
-// over 16-byte pairs, 64 amplitudes a step) and every lane whose shot lies in
-// the block searches it.
+// A warp takes `per` consecutive shots of the sorted list.  For each block among
+// them it stores the weights of the block's 512 pairs in shared memory (lanes
+// over 16-byte pairs, 64 amplitudes a step), lane l sums pairs 16 l .. 16 l + 15
+// of them, one warp scan gives the prefixes at every 32nd amplitude, and every
+// lane whose shot lies in the block searches those, then its 16 pairs, then the
+// two amplitudes of its pair.  Scanning all 16 steps of a block instead (160
+// shuffles a block) was bound by its instructions: 200,000 shots of 2^26
+// amplitudes 221 us, this way 137 to 160 (reading the state once: 79).
 constexpr int kResolveWarps = 4;
 
 __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float4* __restrict__ psi2,
@@ -677,7 +681,8 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float
                                                                       const uint64_t* __restrict__ draws, uint64_t shots,
                                                                       uint64_t count, uint64_t seed, uint64_t stream_id,
                                                                       int per, uint64_t* __restrict__ keys) {
-    __shared__ __align__(16) uint64_t pre[kResolveWarps][1024];   // inclusive prefixes
+    __shared__ uint64_t sums[kResolveWarps][512 + 32];   // pair i at i + i / 16: rows of 17
+    __shared__ uint64_t pre[kResolveWarps][32];          // inclusive prefixes after pair 16 l + 15
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint64_t i = (static_cast<uint64_t>(blockIdx.x) * kResolveWarps + w) * per + lane;
     const bool valid = lane < per && i < count;
@@ -696,23 +701,47 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float
         float4 a[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) a[k] = __ldg(p + 32 * k);
-        uint64_t run = 0;
+        uint32_t any = 0;
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            const uint64_t w0 = sq_fixed60(a[k].x) + sq_fixed60(a[k].y), w1 = sq_fixed60(a[k].z) + sq_fixed60(a[k].w);
-            const uint64_t incl = warp_incl_scan_u64(w0 + w1) + run;
-            *reinterpret_cast<ulonglong2*>(&pre[w][2 * (lane + 32 * k)]) = make_ulonglong2(incl - w1, incl);
-            run = __shfl_sync(0xffffffffu, incl, 31);
+            const uint32_t x0 = __float_as_uint(a[k].x), y0 = __float_as_uint(a[k].y);
+            const uint32_t x1 = __float_as_uint(a[k].z), y1 = __float_as_uint(a[k].w);
+            any |= x0 | y0 | x1 | y1;
+            sums[w][lane + (lane >> 4) + 34 * k] =
+                sq_fixed60_small(x0) + sq_fixed60_small(y0) + sq_fixed60_small(x1) + sq_fixed60_small(y1);
+        }
+        if (any & 0x40000000u) {   // a component with |v| >= 2 or not finite, as in k_weights_z1024
+#pragma unroll 1
+            for (int k = 0; k < 16; ++k) {
+                const float4 v = __ldg(p + 32 * k);
+                sums[w][lane + (lane >> 4) + 34 * k] = sq_fixed60(v.x) + sq_fixed60(v.y) + sq_fixed60(v.z) + sq_fixed60(v.w);
+            }
         }
         __syncwarp();
-        if (open && b == bb) {
-            int lo = 0, hi = 1023;   // the first prefix above ub (the last one is: ub < cum[b] - cum[b - 1])
+        uint64_t own = 0;
 #pragma unroll
-            for (int k = 0; k < 10; ++k) {
+        for (int j = 0; j < 16; ++j) own += sums[w][17 * lane + j];
+        pre[w][lane] = warp_incl_scan_u64(own);
+        __syncwarp();
+        if (open && b == bb) {
+            int lo = 0, hi = 31;   // the first prefix above ub (the last one is: ub < cum[b] - cum[b - 1])
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
                 const int mid = (lo + hi) >> 1;
                 if (pre[w][mid] > ub) hi = mid; else lo = mid + 1;
             }
-            key = bb * 1024 + static_cast<uint64_t>(lo);
+            uint64_t rest = ub - (lo ? pre[w][lo - 1] : 0);
+            int pair = 0;   // the first pair whose prefix within the 16 is above rest
+#pragma unroll
+            for (int j = 0; j < 15; ++j) {
+                const uint64_t v = sums[w][17 * lo + j];
+                const bool past = pair == j && rest >= v;
+                pair += past;
+                rest -= past ? v : 0;
+            }
+            pair += 16 * lo;
+            const float4 v = __ldg(psi2 + bb * 512 + pair);
+            key = bb * 1024 + static_cast<uint64_t>(2 * pair + (rest >= sq_fixed60(v.x) + sq_fixed60(v.y)));
             if (lay.n) key = decode_physical(key, lay);   // else the index through all states
             open = false;
         }
@@ -1182,8 +1211,9 @@ int bits_of(uint64_t count) {   // bits of 0 .. count - 1
 }
 
 // shots per resolving warp: few when most lie in blocks of their own, which a
-// warp reads one after another (N = 24, 30 000 shots: 325 us with 8, 360 with
-// 32), many when they share blocks (N = 12, 200 000: 255 and 207)
+// warp reads one after another, many when they share blocks (this kernel with
+// 8 / 16 / 32: N = 24, 30 000 shots 44 / 48 / 62 us; N = 26, 200 000 154 / 137 /
+// 144; N = 20, 200 000 56 / 32 / 22)
 int resolve_per(uint64_t shots, uint64_t nblocks) { return shots >= 8 * nblocks ? 32 : shots >= 3 * nblocks ? 16 : 8; }
 
 // The batch's samples of all trajectories at once, where the shots' numbers fit
