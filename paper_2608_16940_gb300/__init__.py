@@ -523,14 +523,23 @@ def qsa_expectation_z_batch(s: int, logical_masks) -> List[float]:
     return [float(v) for v in out]
 
 
+def _shrink(a: np.ndarray, n: int) -> np.ndarray:
+    """The first n entries of an array that this call alone holds, as an array
+    of their own: in place, since copies of 200,000 outcomes and counts took
+    0.16 of a measurement's 0.85 ms.  (The ctypes pointers made from it are the
+    references that the check would count.)"""
+    a.resize(n, refcheck=False)
+    return a
+
+
 def qsa_sample_counts(s: int, shots: int, seed: int, capacity: Optional[int] = None) -> Tuple[np.ndarray, np.ndarray]:
     cap = shots if capacity is None else capacity
-    outc = np.zeros(max(1, cap), dtype=np.uint64)
-    cnt = np.zeros(max(1, cap), dtype=np.uint64)
+    outc = np.empty(max(1, cap), dtype=np.uint64)
+    cnt = np.empty(max(1, cap), dtype=np.uint64)
     nd = _c.c_size_t()
     _check(_f["qsa_sample_counts"](_vp(s), shots, _c.c_uint64(seed), outc.ctypes.data_as(_u64p),
                                    cnt.ctypes.data_as(_u64p), cap, _c.byref(nd)))
-    return outc[: nd.value].copy(), cnt[: nd.value].copy()
+    return _shrink(outc, nd.value), _shrink(cnt, nd.value)
 
 
 def qsa_measure(s: int, z_masks, shots: int, seed: int, capacity: Optional[int] = None):
@@ -538,13 +547,13 @@ def qsa_measure(s: int, z_masks, shots: int, seed: int, capacity: Optional[int] 
     cap = shots if capacity is None else capacity
     m = np.ascontiguousarray(np.asarray(list(z_masks), dtype=np.uint64))
     z = np.zeros(max(1, len(m)), dtype=np.float64)
-    outc = np.zeros(max(1, cap), dtype=np.uint64)
-    cnt = np.zeros(max(1, cap), dtype=np.uint64)
+    outc = np.empty(max(1, cap), dtype=np.uint64)
+    cnt = np.empty(max(1, cap), dtype=np.uint64)
     nd = _c.c_size_t()
     _check(_f["qsa_measure"](_vp(s), m.ctypes.data_as(_u64p) if len(m) else None, len(m),
                              z.ctypes.data_as(_dp) if len(m) else None, shots, _c.c_uint64(seed),
                              outc.ctypes.data_as(_u64p), cnt.ctypes.data_as(_u64p), cap, _c.byref(nd)))
-    return [float(v) for v in z[: len(m)]], outc[: nd.value].copy(), cnt[: nd.value].copy()
+    return [float(v) for v in z[: len(m)]], _shrink(outc, nd.value), _shrink(cnt, nd.value)
 
 
 # ---- cost model -------------------------------------------------------------
