@@ -119,20 +119,29 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_z_multi(const float4* __
 }
 
 // Fixed-order sum of the partials (deterministic for a given grid); CTA m sums
-// partials[m n ..) into out[m].
-__global__ void k_finalize_sum(const double* __restrict__ partials, int n, double* __restrict__ out) {
-    __shared__ double sh[1024];
+// partials[m n ..) into out[m].  A launch between a pass and the caller's read:
+// its time is its serial chain, so each thread has four loads in flight and two
+// rounds of shuffles do the rest (3.4 us for 304 partials; a tree of 1024
+// threads in shared memory, a barrier a level, took 5.8).
+constexpr int kFinThreads = 256;
+__global__ void __launch_bounds__(kFinThreads) k_finalize_sum(const double* __restrict__ partials, int n,
+                                                              double* __restrict__ out) {
+    __shared__ double ws[kFinThreads / 32];
     partials += static_cast<size_t>(blockIdx.x) * n;
-    out += blockIdx.x;
     double v = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x >> 1; s > 0; s >>= 1) {
-        if (static_cast<int>(threadIdx.x) < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    for (int i = threadIdx.x; i < n; i += 4 * kFinThreads) {
+        double a[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = i + k * kFinThreads < n ? partials[i + k * kFinThreads] : 0.0;
+        v += (a[0] + a[1]) + (a[2] + a[3]);
     }
-    if (threadIdx.x == 0) *out = sh[0];
+    v = warp_sum_d(v);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = warp_sum_d(threadIdx.x < kFinThreads / 32 ? ws[threadIdx.x] : 0.0);
+        if (threadIdx.x == 0) out[blockIdx.x] = v;
+    }
 }
 
 
@@ -606,7 +615,8 @@ __device__ __forceinline__ uint64_t find_block(const uint64_t* __restrict__ cum,
     return lo;
 }
 
-// One warp per shot: draw u, find the block (first cum > u), then the amplitude.
+// One warp per shot on a state below one block of 1024 amplitudes: draw u, find
+// the block (first cum > u), then the amplitude.
 __global__ void k_draw(const float2* __restrict__ psi, const uint64_t* __restrict__ cum, uint64_t nblocks, int bsz,
                        Layout lay, uint64_t shots, uint64_t seed, uint64_t stream_id, uint64_t* __restrict__ keys) {
     const uint64_t s = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -665,6 +675,91 @@ __global__ void __launch_bounds__(256) k_draw_blocks(const uint64_t* __restrict_
     out[s] = ((t * nblocks + b) << kShotBits) | s;
 }
 
+// The pair weights of a block of 1024 amplitudes into sums (pair i at i + i / 16:
+// rows of 17), by one warp with the block's 8 KiB in flight; returns this
+// lane's inclusive prefix, through pair 16 lane + 15, and its own 16 pairs' sum.
+constexpr int kPairWords = 512 + 32;
+__device__ __forceinline__ uint64_t block_pairs(const float4* __restrict__ block, uint64_t* sums, int lane, uint64_t* own) {
+    const float4* p = block + lane;
+    float4 a[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) a[k] = __ldg(p + 32 * k);
+    uint32_t any = 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const uint32_t x0 = __float_as_uint(a[k].x), y0 = __float_as_uint(a[k].y);
+        const uint32_t x1 = __float_as_uint(a[k].z), y1 = __float_as_uint(a[k].w);
+        any |= x0 | y0 | x1 | y1;
+        sums[lane + (lane >> 4) + 34 * k] =
+            sq_fixed60_small(x0) + sq_fixed60_small(y0) + sq_fixed60_small(x1) + sq_fixed60_small(y1);
+    }
+    if (any & 0x40000000u) {   // a component with |v| >= 2 or not finite, as in k_weights_z1024
+#pragma unroll 1
+        for (int k = 0; k < 16; ++k) {
+            const float4 v = __ldg(p + 32 * k);
+            sums[lane + (lane >> 4) + 34 * k] = sq_fixed60(v.x) + sq_fixed60(v.y) + sq_fixed60(v.z) + sq_fixed60(v.w);
+        }
+    }
+    __syncwarp();
+    uint64_t s = 0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) s += sums[17 * lane + j];
+    *own = s;
+    return warp_incl_scan_u64(s);
+}
+
+constexpr int kResolveWarps = 4;
+
+// find_block by a warp: 32 probes a step, so 65536 blocks take 4 dependent reads
+// instead of 16.
+__device__ __forceinline__ uint64_t find_block_warp(const uint64_t* __restrict__ cum, uint64_t nblocks, uint64_t u, int lane) {
+    uint64_t lo = 0, hi = nblocks - 1;
+    while (lo < hi) {
+        const uint64_t step = (hi - lo) / 32 + 1;
+        const uint64_t at = min(lo + static_cast<uint64_t>(lane + 1) * step - 1, hi);
+        const int f = __ffs(__ballot_sync(0xffffffffu, cum[at] > u) | 0x80000000u) - 1;   // lane 31 reads cum[hi] > u
+        hi = min(lo + static_cast<uint64_t>(f + 1) * step - 1, hi);
+        lo = min(lo + static_cast<uint64_t>(f) * step, hi);
+    }
+    return lo;
+}
+
+// One warp per shot on blocks of 1024 amplitudes: the block, its pair sums as in
+// k_draw_resolve, then the 16 pairs and the two amplitudes.  A serial chain of
+// loads, so as few and as wide as they go: 1000 shots of 2^26 / 2^16 amplitudes
+// 10.2 / 7.5 us, 18.5 / 15.3 with a binary search and 32 strided reads a lane.
+__global__ void __launch_bounds__(32 * kResolveWarps) k_draw1024(const float4* __restrict__ psi2,
+                                                                  const uint64_t* __restrict__ cum, uint64_t nblocks,
+                                                                  const __grid_constant__ Layout lay, uint64_t shots,
+                                                                  uint64_t seed, uint64_t stream_id,
+                                                                  uint64_t* __restrict__ keys) {
+    __shared__ uint64_t sums[kResolveWarps][kPairWords];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint64_t s = static_cast<uint64_t>(blockIdx.x) * kResolveWarps + w;
+    if (s >= shots) return;
+    const uint64_t total = cum[nblocks - 1];
+    if (total == 0) {   // all-zero state: the host reports it
+        if (lane == 0) keys[s] = 0;
+        return;
+    }
+    const uint64_t u = draw_u(s, stream_id, seed, total);
+    const uint64_t b = find_block_warp(cum, nblocks, u, lane);
+    uint64_t rest = u - (b ? cum[b - 1] : 0), own;
+    const float4* block = psi2 + b * 512;
+    const uint64_t incl = block_pairs(block, sums[w], lane, &own);
+    // the first lane whose prefix is above rest (the last one's is)
+    const int row = __ffs(__ballot_sync(0xffffffffu, incl > rest) | 0x80000000u) - 1;
+    rest -= __shfl_sync(0xffffffffu, incl - own, row);
+    const uint64_t v = lane < 16 ? sums[w][17 * row + lane] : 0;
+    const uint64_t in16 = warp_incl_scan_u64(v);
+    const int col = __ffs(__ballot_sync(0xffffffffu, lane < 16 && in16 > rest) | 0x8000u) - 1;
+    if (lane == col) {
+        const float4 x = __ldg(block + 16 * row + col);
+        const bool second = rest - (in16 - v) >= sq_fixed60(x.x) + sq_fixed60(x.y);
+        keys[s] = decode_physical(b * 1024 + static_cast<uint64_t>(2 * (16 * row + col) + second), lay);
+    }
+}
+
 // A warp takes `per` consecutive shots of the sorted list.  For each block among
 // them it stores the weights of the block's 512 pairs in shared memory (lanes
 // over 16-byte pairs, 64 amplitudes a step), lane l sums pairs 16 l .. 16 l + 15
@@ -673,15 +768,13 @@ __global__ void __launch_bounds__(256) k_draw_blocks(const uint64_t* __restrict_
 // two amplitudes of its pair.  Scanning all 16 steps of a block instead (160
 // shuffles a block) was bound by its instructions: 200,000 shots of 2^26
 // amplitudes 221 us, this way 137 to 160 (reading the state once: 79).
-constexpr int kResolveWarps = 4;
-
 __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float4* __restrict__ psi2,
                                                                       const uint64_t* __restrict__ cum,
                                                                       uint64_t nblocks, const __grid_constant__ Layout lay,
                                                                       const uint64_t* __restrict__ draws, uint64_t shots,
                                                                       uint64_t count, uint64_t seed, uint64_t stream_id,
                                                                       int per, uint64_t* __restrict__ keys) {
-    __shared__ uint64_t sums[kResolveWarps][512 + 32];   // pair i at i + i / 16: rows of 17
+    __shared__ uint64_t sums[kResolveWarps][kPairWords];
     __shared__ uint64_t pre[kResolveWarps][32];          // inclusive prefixes after pair 16 l + 15
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint64_t i = (static_cast<uint64_t>(blockIdx.x) * kResolveWarps + w) * per + lane;
@@ -697,31 +790,8 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float
         const unsigned left = __ballot_sync(0xffffffffu, open);
         if (!left) break;
         const uint64_t bb = __shfl_sync(0xffffffffu, b, __ffs(left) - 1);
-        const float4* p = psi2 + bb * 512 + lane;
-        float4 a[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) a[k] = __ldg(p + 32 * k);
-        uint32_t any = 0;
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const uint32_t x0 = __float_as_uint(a[k].x), y0 = __float_as_uint(a[k].y);
-            const uint32_t x1 = __float_as_uint(a[k].z), y1 = __float_as_uint(a[k].w);
-            any |= x0 | y0 | x1 | y1;
-            sums[w][lane + (lane >> 4) + 34 * k] =
-                sq_fixed60_small(x0) + sq_fixed60_small(y0) + sq_fixed60_small(x1) + sq_fixed60_small(y1);
-        }
-        if (any & 0x40000000u) {   // a component with |v| >= 2 or not finite, as in k_weights_z1024
-#pragma unroll 1
-            for (int k = 0; k < 16; ++k) {
-                const float4 v = __ldg(p + 32 * k);
-                sums[w][lane + (lane >> 4) + 34 * k] = sq_fixed60(v.x) + sq_fixed60(v.y) + sq_fixed60(v.z) + sq_fixed60(v.w);
-            }
-        }
-        __syncwarp();
-        uint64_t own = 0;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) own += sums[w][17 * lane + j];
-        pre[w][lane] = warp_incl_scan_u64(own);
+        uint64_t own;
+        pre[w][lane] = block_pairs(psi2 + bb * 512, sums[w], lane, &own);
         __syncwarp();
         if (open && b == bb) {
             int lo = 0, hi = 31;   // the first prefix above ub (the last one is: ub < cum[b] - cum[b - 1])
@@ -925,66 +995,119 @@ __global__ void k_rle_counts(const uint64_t* __restrict__ starts, uint64_t n, co
     if (d < nd) counts[d] = (d + 1 < nd ? starts[d + 1] : n) - starts[d];
 }
 
-__global__ void k_fill_u64(uint64_t* a, uint64_t from, uint64_t to, uint64_t v) {
-    uint64_t i = from + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < to) a[i] = v;
+// Up to 4096 outcomes sorted and run-length encoded by one CTA: E keys a thread
+// in registers, key e B + t of thread t of B.  A bitonic step exchanges them by
+// shuffles below distance 32, through shared memory (two buffers in turn, one
+// barrier a step) below B, and within the thread above.  A serial chain of
+// steps: 1000 keys 8.8 us; with a barrier over all keys in shared memory for
+// every step and launches of their own for padding and runs, 18.2.
+// T holds an outcome (32 bits for N <= 32); the padding is the largest T, which
+// sorts behind every other key and beside equal ones.
+template <typename T>
+__device__ __forceinline__ void order(T& a, T& b, bool up) {
+    const T lo = a < b ? a : b, hi = a < b ? b : a;
+    a = up ? lo : hi;
+    b = up ? hi : lo;
 }
-
-// Bitonic sort of P = 2^p keys.  Small P: one CTA in shared memory.
-__global__ void __launch_bounds__(1024) k_bitonic_smem(uint64_t* keys, int P) {
-    extern __shared__ uint64_t sk[];
-    for (int i = threadIdx.x; i < P; i += blockDim.x) sk[i] = keys[i];
-    __syncthreads();
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < P; i += blockDim.x) {
-                int l = i ^ j;
-                if (l > i) {
-                    bool up = (i & k) == 0;
-                    uint64_t a = sk[i], c = sk[l];
-                    if ((a > c) == up) {
-                        sk[i] = c;
-                        sk[l] = a;
-                    }
+template <typename T, int E>
+__global__ void __launch_bounds__(1024) k_sort_rle(const uint64_t* __restrict__ in, uint32_t n,
+                                                   uint64_t* __restrict__ out_keys, uint64_t* __restrict__ out_counts,
+                                                   uint64_t* __restrict__ n_distinct) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    __shared__ uint32_t wsum[32];
+    const uint32_t B = blockDim.x, t = threadIdx.x, N = E * B;
+    T* cur = reinterpret_cast<T*>(sort_smem);
+    T* nxt = cur + N;
+    T v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = e * B + t < n ? static_cast<T>(in[e * B + t]) : static_cast<T>(~static_cast<T>(0));
+    for (uint32_t k = 2; k <= N; k <<= 1) {
+        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+            if (j >= B) {   // partner rows e ^ 1 or e ^ 2; k > j, so the direction is the row's
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const bool up = ((e * B) & k) == 0;
+                    if (E > 1 && !(e & 1) && j == B) order(v[e], v[(e + 1) % E], up);
+                    if (E > 2 && !(e & 2) && j != B) order(v[e], v[(e + 2) % E], up);
+                }
+            } else if (j >= 32) {
+#pragma unroll
+                for (int e = 0; e < E; ++e) cur[e * B + t] = v[e];
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const uint32_t i = e * B + t;
+                    const T c = cur[i ^ j];
+                    const bool low = ((i & j) == 0) == ((i & k) == 0);   // keeps the smaller
+                    v[e] = low ? (c < v[e] ? c : v[e]) : (c > v[e] ? c : v[e]);
+                }
+                T* x = cur;
+                cur = nxt;
+                nxt = x;
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const uint32_t i = e * B + t;
+                    const T c = __shfl_xor_sync(0xffffffffu, v[e], j);
+                    const bool low = ((i & j) == 0) == ((i & k) == 0);
+                    v[e] = low ? (c < v[e] ? c : v[e]) : (c > v[e] ? c : v[e]);
                 }
             }
-            __syncthreads();
         }
     }
-    for (int i = threadIdx.x; i < P; i += blockDim.x) keys[i] = sk[i];
+    // the runs: thread t takes keys E t ..; the run starts go to the other buffer
+#pragma unroll
+    for (int e = 0; e < E; ++e) cur[e * B + t] = v[e];
+    __syncthreads();
+    uint32_t* starts = reinterpret_cast<uint32_t*>(nxt);
+    uint32_t heads = 0, mask = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = E * t + e;
+        v[e] = cur[i];
+        const bool h = i < n && (i == 0 || v[e] != cur[i - 1]);
+        mask |= static_cast<uint32_t>(h) << e;
+        heads += h;
+    }
+    const uint32_t lane = t & 31, w = t >> 5;
+    uint32_t inc = heads;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    uint32_t pos = inc - heads, nd = 0;
+    for (uint32_t q = 0; q < B >> 5; ++q) {
+        const uint32_t x = wsum[q];
+        if (q < w) pos += x;
+        nd += x;
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if ((mask >> e) & 1u) {
+            out_keys[pos] = v[e];
+            starts[pos++] = E * t + e;
+        }
+    __syncthreads();
+    for (uint32_t d = t; d < nd; d += B) out_counts[d] = (d + 1 < nd ? starts[d + 1] : n) - starts[d];
+    if (t == 0) *n_distinct = nd;
 }
 
-// Run-length encode the sorted keys[0..n-1] with one CTA: distinct keys and
-// their counts, and the number of distinct keys.
-__global__ void __launch_bounds__(1024) k_rle(const uint64_t* __restrict__ keys, uint64_t n,
-                                              uint64_t* __restrict__ out_keys, uint64_t* __restrict__ starts,
-                                              uint64_t* __restrict__ out_counts, uint64_t* __restrict__ n_distinct) {
-    __shared__ uint64_t wsum[32];
-    __shared__ uint64_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (uint64_t base = 0; base < n; base += blockDim.x) {
-        const uint64_t i = base + threadIdx.x;
-        const uint64_t head = (i < n && (i == 0 || keys[i] != keys[i - 1])) ? 1 : 0;
-        uint64_t inc = warp_incl_scan_u64(head);
-        if (lane == 31) wsum[wid] = inc;
-        __syncthreads();
-        if (wid == 0) wsum[lane] = warp_incl_scan_u64(wsum[lane]);
-        __syncthreads();
-        const uint64_t pos = carry + (wid ? wsum[wid - 1] : 0) + inc - head;
-        if (head) {
-            out_keys[pos] = keys[i];
-            starts[pos] = i;
-        }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = pos + head;
-        __syncthreads();
+template <typename T>
+cudaError_t launch_sort_rle(const uint64_t* in, uint32_t n, uint32_t P, uint64_t* out_keys, uint64_t* out_counts,
+                            uint64_t* n_distinct, cudaStream_t st, uint64_t* launches) {
+    const uint32_t N = P < 32 ? 32 : P, B = N < 1024 ? N : 1024;   // N = E B, E = 1, 2 or 4
+    auto kern = N <= 1024 ? k_sort_rle<T, 1> : N == 2048 ? k_sort_rle<T, 2> : k_sort_rle<T, 4>;
+    const size_t smem = 2 * sizeof(T) * N;
+    if (smem > 48 * 1024) {
+        cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
     }
-    const uint64_t nd = carry;
-    for (uint64_t d = threadIdx.x; d < nd; d += blockDim.x)
-        out_counts[d] = (d + 1 < nd ? starts[d + 1] : n) - starts[d];
-    if (threadIdx.x == 0) *n_distinct = nd;
+    kern<<<1, B, smem, st>>>(in, n, out_keys, out_counts, n_distinct);
+    ++*launches;
+    return cudaGetLastError();
 }
 
 inline uint64_t next_pow2(uint64_t v) {
@@ -1315,7 +1438,7 @@ cudaError_t launch_zsums(const float2* psi, int n, const uint64_t* physmasks, in
     const uint64_t nb = std::min<uint64_t>((nblocks + 7) / 8, static_cast<uint64_t>(kZCtas) * num_sms());
     auto kern = nmasks == 1 ? k_zsums1024<1> : nmasks == 2 ? k_zsums1024<2> : nmasks == 3 ? k_zsums1024<3> : k_zsums1024<4>;
     kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, zm, d_partials);
-    k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_partials, static_cast<int>(nb), d_out);
+    k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_partials, static_cast<int>(nb), d_out);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -1332,7 +1455,7 @@ cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double*
     }
     if (n >= 10) return launch_zsums(psi, n, &physmask, 1, d_partials, d_out, st, launches);
     k_reduce_z<<<nb, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), npairs, physmask, d_partials);
-    k_finalize_sum<<<1, 1024, 0, st>>>(d_partials, nb, d_out);
+    k_finalize_sum<<<1, kFinThreads, 0, st>>>(d_partials, nb, d_out);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -1347,7 +1470,7 @@ cudaError_t launch_reduce_z_multi(const float2* psi, int n, const uint64_t* phys
     zm.n = nmasks;
     for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
     k_reduce_z_multi<<<nb, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), npairs, zm, d_partials);
-    k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_partials, nb, d_out);
+    k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_partials, nb, d_out);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -1359,7 +1482,7 @@ cudaError_t launch_dm_diag(const float2* psi, int n, const int32_t* layout_host,
     for (int q = 0; q < 2 * n; ++q) lay.L[q] = layout_host[q];
     const int nb = reduce_partials();
     k_dm_diag<<<nb, kRedThreads, 0, st>>>(psi, lay, n, mask, d_out, d_partials);
-    k_finalize_sum<<<1, 1024, 0, st>>>(d_partials, nb, d_sum);
+    k_finalize_sum<<<1, kFinThreads, 0, st>>>(d_partials, nb, d_sum);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -1426,7 +1549,7 @@ cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout
     k_probs_tile<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(a);
     ++*launches;
     if (d_norm) {
-        k_finalize_sum<<<1, 1024, 0, st>>>(d_partials, static_cast<int>(nb), d_norm);
+        k_finalize_sum<<<1, kFinThreads, 0, st>>>(d_partials, static_cast<int>(nb), d_norm);
         ++*launches;
     }
     return cudaGetLastError();
@@ -1479,7 +1602,7 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
         kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, cum,
                                                                  zm, d_zpartials);
         if (nmasks > 0) {
-            k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_zpartials, static_cast<int>(nb), d_zout);
+            k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_zpartials, static_cast<int>(nb), d_zout);
             ++*launches;
         }
     } else if (nmasks > 0) {
@@ -1488,7 +1611,7 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
         for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
         const int nb = reduce_partials();
         k_block_weights_z<<<nb, kRedThreads, 0, st>>>(psi, nblocks, bsz, cum, zm, d_zpartials);
-        k_finalize_sum<<<nmasks, 1024, 0, st>>>(d_zpartials, nb, d_zout);
+        k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_zpartials, nb, d_zout);
         ++*launches;
     } else {
         k_block_weights<<<static_cast<unsigned>((nblocks + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, nblocks, bsz,
@@ -1507,17 +1630,20 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
     } else {
         k_scan_inclusive<<<1, 1024, 0, st>>>(cum, nblocks);
     }
+    auto draw = [&](uint64_t* to) {
+        if (bsz == 1024)
+            k_draw1024<<<static_cast<unsigned>((shots + kResolveWarps - 1) / kResolveWarps), 32 * kResolveWarps, 0, st>>>(
+                reinterpret_cast<const float4*>(psi), cum, nblocks, lay, shots, seed, stream_id, to);
+        else
+            k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
+                                                                                         seed, stream_id, to);
+    };
     if (P <= kSortSmemMax) {
-        k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
-                                                                                     seed, stream_id, keys);
-        if (P > shots) {
-            k_fill_u64<<<static_cast<unsigned>((P - shots + 255) / 256), 256, 0, st>>>(keys, shots, P, ~0ull);
-            ++*launches;
-        }
-        k_bitonic_smem<<<1, 1024, sizeof(uint64_t) * P, st>>>(keys, static_cast<int>(P));
-        k_rle<<<1, 1024, 0, st>>>(keys, shots, d_out_keys, starts, d_out_counts, d_n_distinct);
-        *launches += 5;
-        return cudaGetLastError();
+        draw(keys);
+        *launches += 3;
+        const uint32_t m = static_cast<uint32_t>(shots), p2 = static_cast<uint32_t>(P);
+        return n <= 32 ? launch_sort_rle<uint32_t>(keys, m, p2, d_out_keys, d_out_counts, d_n_distinct, st, launches)
+                       : launch_sort_rle<uint64_t>(keys, m, p2, d_out_keys, d_out_counts, d_n_distinct, st, launches);
     }
     // Many shots: radix sorts between the arrays at hand (the digit counts go
     // where the outcome counts end up).  The outcomes must end in `keys`.
@@ -1543,8 +1669,7 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
             reinterpret_cast<const float4*>(psi), cum, nblocks, lay, d, shots, shots, seed, stream_id, per, first);
         *launches += 2;
     } else {
-        k_draw<<<static_cast<unsigned>((shots + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, cum, nblocks, bsz, lay, shots,
-                                                                                     seed, stream_id, first);
+        draw(first);
         ++*launches;
     }
     sort(first, second, 0, n);
