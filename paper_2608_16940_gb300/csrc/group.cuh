@@ -19,10 +19,13 @@
 // from small tables in the program instead of bit arithmetic.
 // Measured, one pass per block / group passes with complex 2 x 2 blocks / with
 // rotations: QFT + 3 random layers at N = 25, DP plan of k <= 4 blocks, 24.5 /
-// 4.58 / 3.30 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
+// 4.58 / 3.29 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
 // tile: one launch instead of about 250) with its probabilities and norm, 1.77
-// / 0.159 / 0.107 ms; 128 trajectories at N = 20 of 10..40 layers with their
-// samples, 295 / 45.9 / 28.4 ms.
+// / 0.159 / 0.100 ms; 128 trajectories at N = 20 of 10..40 layers with their
+// samples, 295 / 45.9 / 22.0 ms.
+// Dense 2- and 3-qubit blocks with scalar FMAs (3.63 ms at N = 25) and an
+// operator's head read ahead of it (3.53) were slower: what counts is the
+// number of instructions and registers.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -1116,8 +1116,8 @@ inline uint64_t next_pow2(uint64_t v) {
     return p;
 }
 
-// Sorts of up to this many keys run in one CTA's shared memory (a launch or
-// three cheaper than the radix sort's nine to fifteen).
+// Up to this many shots are sorted and counted by one CTA, more by radix sorts
+// and tiles (whole calls at N = 12: 3000 shots 122 us, 5000 139).
 constexpr uint64_t kSortSmemMax = 4096;
 
 // Run-length encoding of one CTA's sorted keys (any indexable), wsum and carry
@@ -1655,10 +1655,12 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
     const bool odd = ((n + 7) / 8) & 1;
     uint64_t* first = odd ? d_out_keys : keys;    // the unsorted outcomes
     uint64_t* second = odd ? keys : d_out_keys;
-    // Grouping by block costs a sort of the shots (about 40 us of launches) and saves about 4 ns a shot
-    // while blocks share shots: N = 26, 10 000 / 30 000 / 200 000 shots 350 / 440 / 790 us grouped,
-    // 324 / 441 / 1327 us shot by shot (whole calls); N = 28, 30 000 / 100 000: 697 / 930 and 671 / 1036.
-    if (bsz == 1024 && shots >= std::max<uint64_t>(16384, nblocks / 4)) {
+    // Grouping by block costs a sort of the shots (about 40 us of launches) and a read of every block met;
+    // shot by shot, each reads its block.  Where they meet grows with the root of the number of blocks
+    // (whole calls, grouped against shot by shot: N = 16, 16 384 shots 153 and 157 us, 30 000 155 and 185;
+    // N = 20, 16 384: 202 and 174, 60 000: 203 and 263; N = 26, 60 000: 420 and 382, 100 000: 445 and 460;
+    // N = 28, 100 000: 742 and 693, 200 000: 861 and 901).
+    if (bsz == 1024 && shots >= 16384 + (256ull << ((n - 10) / 2))) {
         uint64_t* d = starts;
         k_draw_blocks<<<static_cast<unsigned>((shots + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, shots, seed, stream_id,
                                                                                   d);
