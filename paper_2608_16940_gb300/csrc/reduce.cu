@@ -161,18 +161,39 @@ __global__ void k_probs_logical(const float2* __restrict__ psi, Layout lay, doub
 // issues two FP64 operations per clock and SM, so forming both squares in FP64
 // (two conversions and two products per amplitude) bounds the pass at several
 // times its memory traffic; the sum below is the only one left.
+__device__ __forceinline__ double square_normal(float v) {
+    const uint32_t b = __float_as_uint(v) & 0x7fffffffu;
+    const uint32_t M = (b & 0x7fffffu) | 0x800000u;
+    const uint64_t P = static_cast<uint64_t>(M) * M;   // in [2^46, 2^48)
+    const uint32_t top = static_cast<uint32_t>(P >> 47);
+    // value P 2^(2 e - 300): biased exponent 2 e + 769 + top; the leading bit adds one to it
+    return __longlong_as_double(static_cast<long long>(
+        (P << (6u - top)) + (static_cast<uint64_t>(((b >> 23) << 21) + ((768u + top) << 20)) << 32)));
+}
 __device__ __forceinline__ double square_exact(float v) {
     const uint32_t b = __float_as_uint(v) & 0x7fffffffu, e = b >> 23;
     if (e == 0u || e == 255u) {   // zero, subnormal, infinite or NaN
         if (b == 0u) return 0.0;
         return static_cast<double>(v) * static_cast<double>(v);
     }
-    const uint32_t M = (b & 0x7fffffu) | 0x800000u;
-    const uint64_t P = static_cast<uint64_t>(M) * M;   // in [2^46, 2^48)
-    const uint32_t top = static_cast<uint32_t>(P >> 47);
-    // value P 2^(2 e - 300): biased exponent 2 e + 769 + top; the leading bit adds one to it
-    return __longlong_as_double(static_cast<long long>((static_cast<uint64_t>(2u * e + 768u + top) << 52) +
-                                                       (P << (6u - top))));
+    return square_normal(v);
+}
+// A zero part leaves the other's square as it is (states with real amplitudes).
+__device__ __forceinline__ double probability_exact(float x, float y) {
+    if (y == 0.f) return square_exact(x);
+    return __dadd_rn(square_exact(x), square_exact(y));
+}
+// The two probabilities of a 16-byte unit.  One test tells whether its four
+// components are normal numbers (a sum that is not finite, if only by overflow,
+// takes the other way too), so that the usual unit runs without a branch per
+// component (2^27 amplitudes: 0.457 ms with one, 0.411 here; states with real
+// amplitudes, which take the other way, 0.421 and 0.404).
+__device__ __forceinline__ double2 probabilities(const float4& v) {
+    const float least = fminf(fminf(fabsf(v.x), fabsf(v.y)), fminf(fabsf(v.z), fabsf(v.w)));
+    const float sum = __fadd_rn(__fadd_rn(fabsf(v.x), fabsf(v.y)), __fadd_rn(fabsf(v.z), fabsf(v.w)));
+    if (!(least >= 0x1p-126f && sum <= 0x1.fffffep127f))
+        return make_double2(probability_exact(v.x, v.y), probability_exact(v.z, v.w));
+    return make_double2(__dadd_rn(square_normal(v.x), square_normal(v.y)), __dadd_rn(square_normal(v.z), square_normal(v.w)));
 }
 
 // Probabilities in logical order through tiles of 2^12 amplitudes: the tile's
@@ -184,8 +205,9 @@ __device__ __forceinline__ double square_exact(float v) {
 // the tile bits that the writing lanes vary (formed on the host).  With
 // partials the norm is taken in the same read (double-float per thread, as
 // k_reduce_z).  N = 27, random layout, probabilities and norm:
-// 2.01 ms by gather and a second pass, 0.458 ms here (0.317 ms at the copy rate;
-// 0.478 with four CTAs per SM and no loads in flight while a tile is written).
+// 2.01 ms by gather and a second pass, 0.411 ms here (0.317 ms at the copy rate;
+// before the test per unit, 0.457 with the three CTAs per SM, 0.524 with two and
+// 0.493 with four).
 constexpr int kProbT = 12, kProbCtas = 3;
 
 struct ProbArgs {
@@ -237,8 +259,7 @@ __global__ void __launch_bounds__(kRedThreads, kProbCtas) k_probs_tile(const __g
         for (int k = 0; k < 8; ++k) {
             const uint32_t s = sl ^ (k & 1 ? a.pslot[9] : 0u) ^ (k & 2 ? a.pslot[10] : 0u) ^ (k & 4 ? a.pslot[11] : 0u);
             *reinterpret_cast<double2*>(st + s) =
-                make_double2(__dadd_rn(square_exact(v[k].x), square_exact(v[k].y)),
-                             __dadd_rn(square_exact(v[k].z), square_exact(v[k].w)));
+                probabilities(v[k]);
             if (a.partials) {
                 acc_square(zs, zc, v[k].x, false);
                 acc_square(zs, zc, v[k].y, false);
