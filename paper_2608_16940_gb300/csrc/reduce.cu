@@ -845,9 +845,12 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_draw_resolve(const float
 // first): per-tile digit counts (hist[digit][tile]), their prefixes per digit,
 // and the scatter, where a warp ranks its keys by matching digits 32 at a time.
 // Three launches a digit against (log2 P)^2 / 2 for a whole bitonic network:
-// 200 000 26-bit outcomes 542 us in 171 global bitonic steps, 65 us in the 12
-// launches here; their run-length encoding 294 us in one CTA, 17 us in tiles.
-constexpr int kRadixThreads = 256, kRadixPer = 8, kRadixTile = kRadixThreads * kRadixPer;
+// 200 000 26-bit outcomes 542 us in 171 global bitonic steps, about 60 us in the
+// 12 launches here; their run-length encoding 294 us in one CTA, 17 us in tiles.
+// Four keys a thread: the kernels are chains of latencies, so smaller tiles are
+// faster until their number costs the scan more (whole calls with 2 / 4 / 8 keys:
+// N = 26, 200 000 shots 457 / 471 / 488 us, 5 000 000 4.83 / 4.67 / 4.72 ms).
+constexpr int kRadixThreads = 256, kRadixPer = 4, kRadixTile = kRadixThreads * kRadixPer;
 
 __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint64_t* __restrict__ keys, uint64_t n, int shift,
                                                                uint32_t ntiles, uint32_t* __restrict__ hist) {

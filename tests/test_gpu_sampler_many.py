@@ -1,5 +1,5 @@
 """Samplers with many shots (radix-sorted outcomes, shots grouped by block)
-bit for bit against the oracle: shot counts around the tile of 2048 keys and the
+bit for bit against the oracle: shot counts around the tile of 1024 keys and the
 4096-key limit of the one-CTA sort, states of one block and of many, more and
 fewer shots than blocks, permuted layouts, a state with empty bins, and
 outcomes that repeat often (a few large amplitudes)."""
