@@ -229,7 +229,9 @@ cudaError_t launch_permute(float2* psi, int n, const int* dest, cudaStream_t st,
 std::vector<std::vector<int>> plan_permutation(int n, const int* dest, int T);
 
 // FP64 sum of (-1)^{popcount(y & physmask)} |psi_y|^2 into *d_out (device).
-// d_partials must hold reduce_partials() doubles.
+// d_partials must hold reduce_partials() doubles, d_count a word that is zero
+// before the state's first pass (the passes count their CTAs in it and leave it
+// zero again).
 int reduce_partials();
 constexpr int kMaxZMasks = 4;
 struct ZMasks {
@@ -239,15 +241,16 @@ struct ZMasks {
 // Several <Z_mask> sums in one pass: d_partials holds nmasks * reduce_partials()
 // doubles, d_out nmasks doubles (device).  nmasks in 1..kMaxZMasks.
 cudaError_t launch_reduce_z_multi(const float2* psi, int n, const uint64_t* physmasks, int nmasks,
-                                  double* d_partials, double* d_out, cudaStream_t st, uint64_t* launches);
+                                  double* d_partials, double* d_out, unsigned* d_count, cudaStream_t st,
+                                  uint64_t* launches);
 cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double* d_partials, double* d_out,
-                            cudaStream_t st, uint64_t* launches);
+                            unsigned* d_count, cudaStream_t st, uint64_t* launches);
 
 // out[x] = |psi_{encode(x)}|^2 for logical x; layout_host = L[0..n-1].  With
 // d_norm, also the norm (FP64 sum) into *d_norm (device) via d_partials
 // (reduce_partials() doubles).
 cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout_host, double* out, double* d_partials,
-                                 double* d_norm, cudaStream_t st, uint64_t* launches);
+                                 double* d_norm, unsigned* d_count, cudaStream_t st, uint64_t* launches);
 
 // Sampler scratch sizes and launch (see qsa_sample_counts).
 uint64_t next_pow2_u64(uint64_t v);
@@ -261,6 +264,6 @@ cudaError_t launch_sample(const float2* psi, int n, const int32_t* d_layout, uin
 cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host, uint64_t shots, uint64_t seed,
                             uint64_t stream_id, void* d_scratch, uint64_t* d_out_keys, uint64_t* d_out_counts,
                             uint64_t* d_n_distinct, const uint64_t* physmasks, int nmasks, double* d_zpartials,
-                            double* d_zout, cudaStream_t st, uint64_t* launches);
+                            double* d_zout, unsigned* d_count, cudaStream_t st, uint64_t* launches);
 
 }  // namespace qsa

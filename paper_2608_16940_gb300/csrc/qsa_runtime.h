@@ -36,7 +36,7 @@ struct qsa_state_s {
     size_t dm_cap = 0;
     void* d_lrec = nullptr;           // per-tile records of layer passes
     size_t lrec_cap = 0;
-    int* d_err = nullptr;             // device error word written by bounded waits
+    int* d_err = nullptr;             // words 0-2: record of a bounded wait that gave up; word 3: pass_count
     qsa::CostModel cm;                // cost model attached to this state (qsa_costmodel_load), or null
     // CUDA-event timers
     struct Pending {
@@ -131,6 +131,9 @@ qsa_status fail(qsa_status st, const std::string& msg);
 qsa_status cuda_fail(qsa_state s, cudaError_t e, const char* where);
 qsa_status check_state(qsa_state s);
 qsa_status sync_and_check(qsa_state s, const char* where);
+// Word in which a reducing pass counts its finished CTAs: zero between passes.
+inline unsigned* pass_count(qsa_state s) { return reinterpret_cast<unsigned*>(s->d_err + 3); }
+
 qsa_status ensure_dev(qsa_state s, void** ptr, size_t* cap, size_t bytes);
 void to_float_matrix(const double* m, int k, float* out);
 // Running sum of the modulus errors left by the FP32 constants of one plan,

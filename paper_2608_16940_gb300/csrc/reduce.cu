@@ -118,30 +118,49 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_z_multi(const float4* __
     }
 }
 
-// Fixed-order sum of the partials (deterministic for a given grid); CTA m sums
-// partials[m n ..) into out[m].  A launch between a pass and the caller's read:
-// its time is its serial chain, so each thread has four loads in flight and two
-// rounds of shuffles do the rest (3.4 us for 304 partials; a tree of 1024
-// threads in shared memory, a barrier a level, took 5.8).
-constexpr int kFinThreads = 256;
-__global__ void __launch_bounds__(kFinThreads) k_finalize_sum(const double* __restrict__ partials, int n,
-                                                              double* __restrict__ out) {
-    __shared__ double ws[kFinThreads / 32];
-    partials += static_cast<size_t>(blockIdx.x) * n;
+// Fixed-order sum of n partials (deterministic for a given grid) by one CTA of
+// kRedThreads into *out: its time is a serial chain, so each thread has four
+// loads in flight and two rounds of shuffles do the rest.
+__device__ __forceinline__ void sum_partials(const double* partials, int n, double* out) {
+    __shared__ double ws[kRedThreads / 32];
     double v = 0.0;
-    for (int i = threadIdx.x; i < n; i += 4 * kFinThreads) {
+    for (int i = threadIdx.x; i < n; i += 4 * kRedThreads) {
         double a[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) a[k] = i + k * kFinThreads < n ? partials[i + k * kFinThreads] : 0.0;
+        for (int k = 0; k < 4; ++k) a[k] = i + k * kRedThreads < n ? __ldcg(partials + i + k * kRedThreads) : 0.0;
         v += (a[0] + a[1]) + (a[2] + a[3]);
     }
     v = warp_sum_d(v);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x < 32) {
-        v = warp_sum_d(threadIdx.x < kFinThreads / 32 ? ws[threadIdx.x] : 0.0);
-        if (threadIdx.x == 0) out[blockIdx.x] = v;
+        v = warp_sum_d(threadIdx.x < kRedThreads / 32 ? ws[threadIdx.x] : 0.0);
+        if (threadIdx.x == 0) *out = v;
     }
+    __syncthreads();
+}
+
+// As a launch of its own (3.4 us for 304 partials and the gap before it), for
+// passes whose CTAs outnumber the SMs many times: CTA m sums partials[m n ..).
+__global__ void __launch_bounds__(kRedThreads) k_finalize_sum(const double* __restrict__ partials, int n,
+                                                              double* __restrict__ out) {
+    sum_partials(partials + static_cast<size_t>(blockIdx.x) * n, n, out + blockIdx.x);
+}
+
+// In the pass itself: the CTA that finishes last sums every mask's partials
+// (thread 0 of each CTA has written its own).  The count wraps to zero for the
+// next pass on the stream.  A launch less: probabilities and norm at N = 12 37.2
+// -> 35.3 us a call, two <Z> sums 43.0 -> 40.8, 500 samples with them 106 -> 104.
+__device__ __forceinline__ void sum_by_last_cta(const double* partials, int nm, double* out, unsigned* count) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(count, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int m = 0; m < nm; ++m) sum_partials(partials + static_cast<size_t>(m) * gridDim.x, static_cast<int>(gridDim.x), out + m);
 }
 
 
@@ -214,6 +233,8 @@ struct ProbArgs {
     const float2* psi;
     double* out;
     double* partials;          // nullable
+    double* norm;              // with partials
+    unsigned* count;
     uint64_t ntiles;
     int nouter;                // n - 12
     uint8_t opos[24], oq[24];  // outer bit i: its physical position and its logical qubit
@@ -289,6 +310,7 @@ __global__ void __launch_bounds__(kRedThreads, kProbCtas) k_probs_tile(const __g
             x = warp_sum_d(x);
             if (tid == 0) a.partials[blockIdx.x] = x;
         }
+        sum_by_last_cta(a.partials, 1, a.norm, a.count);
     }
 }
 
@@ -410,7 +432,8 @@ __device__ __forceinline__ void add_scaled(float& s, float& c, float hi, float l
 template <int NM>
 __global__ void __launch_bounds__(kRedThreads, 2) k_weights_z1024(const float4* __restrict__ psi2, uint64_t nblocks,
                                                                   uint64_t* __restrict__ cum, ZMasks masks,
-                                                                  double* __restrict__ partials) {
+                                                                  double* partials, double* out,
+                                                                  unsigned* count) {
     constexpr int NA = NM > 0 ? NM : 1;
     const int lane = threadIdx.x & 31;
     const uint64_t warps = static_cast<uint64_t>(gridDim.x) * (blockDim.x >> 5);
@@ -489,6 +512,7 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_weights_z1024(const float4* 
             }
             __syncthreads();
         }
+        sum_by_last_cta(partials, NM, out, count);
     }
 }
 
@@ -502,7 +526,7 @@ constexpr int kZLoads = 4, kZCtas = 4;
 template <int NM>
 __global__ void __launch_bounds__(kRedThreads, NM <= 2 ? kZCtas : 1) k_zsums1024(const float4* __restrict__ psi2, uint64_t nblocks,
                                                            const __grid_constant__ ZMasks masks,
-                                                           double* __restrict__ partials) {
+                                                           double* partials, double* out, unsigned* count) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = static_cast<uint64_t>(gridDim.x) * (blockDim.x >> 5);
     float zs[NM] = {}, zc[NM] = {};
@@ -559,6 +583,7 @@ __global__ void __launch_bounds__(kRedThreads, NM <= 2 ? kZCtas : 1) k_zsums1024
         }
         __syncthreads();
     }
+    sum_by_last_cta(partials, NM, out, count);
 }
 
 // In-place inclusive scan of cum[0..n-1] by one CTA of 1024 threads.
@@ -1394,7 +1419,7 @@ cudaError_t launch_batch_sample(const float2* states, int n, int n_traj, uint32_
         uint32_t* hist = reinterpret_cast<uint32_t*>(y + total);
         const uint64_t nb = std::min<uint64_t>((all + 7) / 8, 2ull * num_sms());   // two CTAs of 8 warps fit an SM
         k_weights_z1024<0><<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(states), all,
-                                                                            cum, ZMasks{}, nullptr);
+                                                                            cum, ZMasks{}, nullptr, nullptr, nullptr);
         k_batch_scan<<<n_traj, 1024, 0, st>>>(cum, static_cast<int>(nblocks));
         k_draw_blocks<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, total, seed, 0, x);
         uint64_t* d = radix_sort(x, y, total, kShotBits, bits_of(all), hist, st, launches);
@@ -1453,7 +1478,7 @@ int reduce_partials() { return num_sms() * kRedBlocksPerSM; }
 namespace {
 
 cudaError_t launch_zsums(const float2* psi, int n, const uint64_t* physmasks, int nmasks, double* d_partials, double* d_out,
-                         cudaStream_t st, uint64_t* launches) {
+                         unsigned* d_count, cudaStream_t st, uint64_t* launches) {
     const uint64_t nblocks = 1ull << (n - 10);
     ZMasks zm{};
     zm.n = nmasks;
@@ -1461,40 +1486,41 @@ cudaError_t launch_zsums(const float2* psi, int n, const uint64_t* physmasks, in
     // the same grid for any number of masks: a mask's partial sums are the same in all of them
     const uint64_t nb = std::min<uint64_t>((nblocks + 7) / 8, static_cast<uint64_t>(kZCtas) * num_sms());
     auto kern = nmasks == 1 ? k_zsums1024<1> : nmasks == 2 ? k_zsums1024<2> : nmasks == 3 ? k_zsums1024<3> : k_zsums1024<4>;
-    kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, zm, d_partials);
-    k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_partials, static_cast<int>(nb), d_out);
-    *launches += 2;
+    kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, zm, d_partials,
+                                                             d_out, d_count);
+    ++*launches;
     return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_reduce_z(const float2* psi, int n, uint64_t physmask, double* d_partials, double* d_out,
-                            cudaStream_t st, uint64_t* launches) {
+                            unsigned* d_count, cudaStream_t st, uint64_t* launches) {
     const uint64_t npairs = (1ull << n) >> 1;
     const int nb = reduce_partials();
     if (npairs == 0) {
         // n = 1 is still >= one pair; n >= 1 always holds here
         return cudaErrorInvalidValue;
     }
-    if (n >= 10) return launch_zsums(psi, n, &physmask, 1, d_partials, d_out, st, launches);
+    if (n >= 10) return launch_zsums(psi, n, &physmask, 1, d_partials, d_out, d_count, st, launches);
     k_reduce_z<<<nb, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), npairs, physmask, d_partials);
-    k_finalize_sum<<<1, kFinThreads, 0, st>>>(d_partials, nb, d_out);
+    k_finalize_sum<<<1, kRedThreads, 0, st>>>(d_partials, nb, d_out);
     *launches += 2;
     return cudaGetLastError();
 }
 
 cudaError_t launch_reduce_z_multi(const float2* psi, int n, const uint64_t* physmasks, int nmasks,
-                                  double* d_partials, double* d_out, cudaStream_t st, uint64_t* launches) {
+                                  double* d_partials, double* d_out, unsigned* d_count, cudaStream_t st,
+                                  uint64_t* launches) {
     if (nmasks < 1 || nmasks > kMaxZMasks || n < 1) return cudaErrorInvalidValue;
-    if (n >= 10) return launch_zsums(psi, n, physmasks, nmasks, d_partials, d_out, st, launches);
+    if (n >= 10) return launch_zsums(psi, n, physmasks, nmasks, d_partials, d_out, d_count, st, launches);
     const uint64_t npairs = (1ull << n) >> 1;
     const int nb = reduce_partials();
     ZMasks zm{};
     zm.n = nmasks;
     for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
     k_reduce_z_multi<<<nb, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), npairs, zm, d_partials);
-    k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_partials, nb, d_out);
+    k_finalize_sum<<<nmasks, kRedThreads, 0, st>>>(d_partials, nb, d_out);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -1506,13 +1532,13 @@ cudaError_t launch_dm_diag(const float2* psi, int n, const int32_t* layout_host,
     for (int q = 0; q < 2 * n; ++q) lay.L[q] = layout_host[q];
     const int nb = reduce_partials();
     k_dm_diag<<<nb, kRedThreads, 0, st>>>(psi, lay, n, mask, d_out, d_partials);
-    k_finalize_sum<<<1, kFinThreads, 0, st>>>(d_partials, nb, d_sum);
+    k_finalize_sum<<<1, kRedThreads, 0, st>>>(d_partials, nb, d_sum);
     *launches += 2;
     return cudaGetLastError();
 }
 
 cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout_host, double* out, double* d_partials,
-                                 double* d_norm, cudaStream_t st, uint64_t* launches) {
+                                 double* d_norm, unsigned* d_count, cudaStream_t st, uint64_t* launches) {
     if (n < kProbT || reinterpret_cast<uintptr_t>(out) % 16) {   // small, or an output that takes no 16-byte stores
         Layout lay{};
         lay.n = n;
@@ -1522,7 +1548,7 @@ cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout
         ++*launches;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess || !d_norm) return e;
-        return launch_reduce_z(psi, n, 0, d_partials, d_norm, st, launches);
+        return launch_reduce_z(psi, n, 0, d_partials, d_norm, d_count, st, launches);
     }
     int inv[QSA_MAX_QUBITS];
     for (int q = 0; q < n; ++q) inv[layout_host[q]] = q;
@@ -1535,6 +1561,8 @@ cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout
     a.psi = psi;
     a.out = out;
     a.partials = d_norm ? d_partials : nullptr;
+    a.norm = d_norm;
+    a.count = d_count;
     a.ntiles = 1ull << (n - kProbT);
     int tb[QSA_MAX_QUBITS], nt = 0;   // tile bit of a position
     for (int p = 0; p < n; ++p) {
@@ -1572,10 +1600,6 @@ cudaError_t launch_probs_logical(const float2* psi, int n, const int32_t* layout
     const uint64_t nb = std::min<uint64_t>(a.ntiles, static_cast<uint64_t>(kProbCtas) * num_sms());
     k_probs_tile<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(a);
     ++*launches;
-    if (d_norm) {
-        k_finalize_sum<<<1, kFinThreads, 0, st>>>(d_partials, static_cast<int>(nb), d_norm);
-        ++*launches;
-    }
     return cudaGetLastError();
 }
 
@@ -1590,13 +1614,13 @@ cudaError_t launch_sample(const float2* psi, int n, const int32_t* layout_host, 
                           uint64_t stream_id, void* d_scratch, uint64_t* d_out_keys, uint64_t* d_out_counts,
                           uint64_t* d_n_distinct, cudaStream_t st, uint64_t* launches) {
     return launch_sample_z(psi, n, layout_host, shots, seed, stream_id, d_scratch, d_out_keys, d_out_counts,
-                           d_n_distinct, nullptr, 0, nullptr, nullptr, st, launches);
+                           d_n_distinct, nullptr, 0, nullptr, nullptr, nullptr, st, launches);
 }
 
 cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host, uint64_t shots, uint64_t seed,
                             uint64_t stream_id, void* d_scratch, uint64_t* d_out_keys, uint64_t* d_out_counts,
                             uint64_t* d_n_distinct, const uint64_t* physmasks, int nmasks, double* d_zpartials,
-                            double* d_zout, cudaStream_t st, uint64_t* launches) {
+                            double* d_zout, unsigned* d_count, cudaStream_t st, uint64_t* launches) {
     if (nmasks < 0 || nmasks > kMaxZMasks) return cudaErrorInvalidValue;
     Layout lay{};
     lay.n = n;
@@ -1624,18 +1648,14 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
         const uint64_t cap = static_cast<uint64_t>(num_sms()) * occ;
         if (nb > cap) nb = cap;
         kern<<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), nblocks, cum,
-                                                                 zm, d_zpartials);
-        if (nmasks > 0) {
-            k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_zpartials, static_cast<int>(nb), d_zout);
-            ++*launches;
-        }
+                                                                 zm, d_zpartials, d_zout, d_count);
     } else if (nmasks > 0) {
         ZMasks zm{};
         zm.n = nmasks;
         for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
         const int nb = reduce_partials();
         k_block_weights_z<<<nb, kRedThreads, 0, st>>>(psi, nblocks, bsz, cum, zm, d_zpartials);
-        k_finalize_sum<<<nmasks, kFinThreads, 0, st>>>(d_zpartials, nb, d_zout);
+        k_finalize_sum<<<nmasks, kRedThreads, 0, st>>>(d_zpartials, nb, d_zout);
         ++*launches;
     } else {
         k_block_weights<<<static_cast<unsigned>((nblocks + wpb - 1) / wpb), wpb * 32, 0, st>>>(psi, nblocks, bsz,

@@ -591,7 +591,7 @@ qsa_status qsa_expectation_z(qsa_state s, uint64_t logical_mask, double* out) {
     st = ensure_dev(s, reinterpret_cast<void**>(&s->d_red), &s->red_cap, sizeof(double) * (reduce_partials() + 8));
     if (st != QSA_OK) return st;
     double* d_out = s->d_red + reduce_partials();
-    cudaError_t e = launch_reduce_z(s->psi, s->n, pm, s->d_red, d_out, s->stream, &s->launches);
+    cudaError_t e = launch_reduce_z(s->psi, s->n, pm, s->d_red, d_out, pass_count(s), s->stream, &s->launches);
     if (e != cudaSuccess) return cuda_fail(s, e, "reduction kernel");
     e = cudaMemcpyAsync(out, d_out, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "reduction result");
@@ -615,7 +615,7 @@ qsa_status qsa_expectation_z_batch(qsa_state s, const uint64_t* logical_masks, i
                     sizeof(double) * (QSA_MAX_ZMASKS * nb + 8));
     if (st != QSA_OK) return st;
     double* d_out = s->d_red + QSA_MAX_ZMASKS * nb;
-    cudaError_t e = launch_reduce_z_multi(s->psi, s->n, pm, n_masks, s->d_red, d_out, s->stream, &s->launches);
+    cudaError_t e = launch_reduce_z_multi(s->psi, s->n, pm, n_masks, s->d_red, d_out, pass_count(s), s->stream, &s->launches);
     if (e != cudaSuccess) return cuda_fail(s, e, "reduction kernel");
     e = cudaMemcpyAsync(out, d_out, sizeof(double) * n_masks, cudaMemcpyDeviceToHost, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "reduction results");
@@ -643,7 +643,7 @@ qsa_status qsa_probabilities_device(qsa_state s, double* out_dev, double* norm_o
         if (st != QSA_OK) return st;
         d_norm = s->d_red + reduce_partials();
     }
-    cudaError_t e = launch_probs_logical(s->psi, s->n, s->L, out_dev, s->d_red, d_norm, s->stream, &s->launches);
+    cudaError_t e = launch_probs_logical(s->psi, s->n, s->L, out_dev, s->d_red, d_norm, pass_count(s), s->stream, &s->launches);
     if (e != cudaSuccess) return cuda_fail(s, e, "probability kernel");
     if (norm_out) {
         e = cudaMemcpyAsync(norm_out, d_norm, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
@@ -672,7 +672,7 @@ qsa_status qsa_probabilities(qsa_state s, double* out_host, double* norm_out) {
         cudaGetLastError();
         return fail(QSA_E_NOMEM, "cudaMalloc of the probability buffer failed");
     }
-    e = launch_probs_logical(s->psi, s->n, s->L, tmp, s->d_red, d_norm, s->stream, &s->launches);
+    e = launch_probs_logical(s->psi, s->n, s->L, tmp, s->d_red, d_norm, pass_count(s), s->stream, &s->launches);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, tmp, bytes, cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess && norm_out)
         e = cudaMemcpyAsync(norm_out, d_norm, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
@@ -720,7 +720,7 @@ qsa_status qsa_measure(qsa_state s, const uint64_t* z_masks, int n_masks, double
     uint64_t* d_nd = d_cnts + shots;
     double* d_zout = n_masks > 0 ? s->d_red + QSA_MAX_ZMASKS * nbp : nullptr;
     cudaError_t e = launch_sample_z(s->psi, s->n, s->L, shots, seed, 0, s->d_samp, d_keys, d_cnts, d_nd, pm, n_masks,
-                                    n_masks > 0 ? s->d_red : nullptr, d_zout, s->stream, &s->launches);
+                                    n_masks > 0 ? s->d_red : nullptr, d_zout, pass_count(s), s->stream, &s->launches);
     if (e != cudaSuccess) return cuda_fail(s, e, "sampler kernels");
     if (n_masks > 0) {
         e = cudaMemcpyAsync(z_out, d_zout, sizeof(double) * n_masks, cudaMemcpyDeviceToHost, s->stream);
