@@ -427,9 +427,11 @@ __device__ __forceinline__ void add_scaled(float& s, float& c, float hi, float l
 // frame of its own block-and-lane sign (the pair negated when that sign
 // changes between blocks; round-to-nearest is symmetric, so the values are
 // those of summing in the true signs, up to the sign of zeros), so the sign
-// left per amplitude, of its k and b bits, is the same across the warp.  Per
-// CTA partials of mask m at m * gridDim.x.
-template <int NM>
+// left per amplitude, of its k and b bits, is the same across the warp.  EVEN: no
+// mask holds the lowest position, so a pair's two squares are added once for all
+// masks (2^26 amplitudes, two masks: 126 us, 136 without).  Per CTA partials of
+// mask m at m * gridDim.x.
+template <int NM, bool EVEN>
 __global__ void __launch_bounds__(kRedThreads, 2) k_weights_z1024(const float4* __restrict__ psi2, uint64_t nblocks,
                                                                   uint64_t* __restrict__ cum, ZMasks masks,
                                                                   double* partials, double* out,
@@ -475,11 +477,21 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_weights_z1024(const float4* 
                 float h0, l0, h1, l1;
                 square_pair(a[k].x, a[k].y, h0, l0);
                 square_pair(a[k].z, a[k].w, h1, l1);
+                if constexpr (EVEN) {
+                    // both amplitudes of a pair enter every sum with the same sign: added once
+                    const float t = __fadd_rn(h0, h1), bp = __fsub_rn(t, h0);
+                    const float e = __fadd_rn(__fsub_rn(h0, __fsub_rn(t, bp)), __fsub_rn(h1, bp));
+                    const float l = __fadd_rn(e, __fadd_rn(l0, l1));
 #pragma unroll
-                for (int m = 0; m < NM; ++m) {
-                    const float g0 = __uint_as_float(0x3f800000u | (((kb[m] >> k) & 1u) << 31));
-                    add_scaled(zs[m], zc[m], h0, l0, g0);
-                    add_scaled(zs[m], zc[m], h1, l1, g0 * bf[m]);
+                    for (int m = 0; m < NM; ++m)
+                        add_scaled(zs[m], zc[m], t, l, __uint_as_float(0x3f800000u | (((kb[m] >> k) & 1u) << 31)));
+                } else {
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) {
+                        const float g0 = __uint_as_float(0x3f800000u | (((kb[m] >> k) & 1u) << 31));
+                        add_scaled(zs[m], zc[m], h0, l0, g0);
+                        add_scaled(zs[m], zc[m], h1, l1, g0 * bf[m]);
+                    }
                 }
             }
         }
@@ -1418,7 +1430,7 @@ cudaError_t launch_batch_sample(const float2* states, int n, int n_traj, uint32_
         uint64_t* y = x + total;
         uint32_t* hist = reinterpret_cast<uint32_t*>(y + total);
         const uint64_t nb = std::min<uint64_t>((all + 7) / 8, 2ull * num_sms());   // two CTAs of 8 warps fit an SM
-        k_weights_z1024<0><<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(states), all,
+        k_weights_z1024<0, true><<<static_cast<unsigned>(nb), kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(states), all,
                                                                             cum, ZMasks{}, nullptr, nullptr, nullptr);
         k_batch_scan<<<n_traj, 1024, 0, st>>>(cum, static_cast<int>(nblocks));
         k_draw_blocks<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(cum, nblocks, shots, total, seed, 0, x);
@@ -1637,8 +1649,13 @@ cudaError_t launch_sample_z(const float2* psi, int n, const int32_t* layout_host
         ZMasks zm{};
         zm.n = nmasks;
         for (int m = 0; m < nmasks; ++m) zm.m[m] = physmasks[m];
-        auto kern = nmasks == 0 ? k_weights_z1024<0> : nmasks == 1 ? k_weights_z1024<1>
-                  : nmasks == 2 ? k_weights_z1024<2> : nmasks == 3 ? k_weights_z1024<3> : k_weights_z1024<4>;
+        bool even = true;   // no mask holds the lowest position
+        for (int m = 0; m < nmasks; ++m) even = even && !(physmasks[m] & 1);
+        auto kern = nmasks == 0   ? k_weights_z1024<0, true>
+                    : nmasks == 1 ? (even ? k_weights_z1024<1, true> : k_weights_z1024<1, false>)
+                    : nmasks == 2 ? (even ? k_weights_z1024<2, true> : k_weights_z1024<2, false>)
+                    : nmasks == 3 ? (even ? k_weights_z1024<3, true> : k_weights_z1024<3, false>)
+                                  : (even ? k_weights_z1024<4, true> : k_weights_z1024<4, false>);
         // as many CTAs as stay resident (at most reduce_partials(), the partials' size)
         int occ = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kRedThreads, 0);
