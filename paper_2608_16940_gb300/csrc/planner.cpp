@@ -1058,8 +1058,9 @@ qsa_status run_block(qsa_state s, qsa_plan p, size_t i, qsa_run_stats* rs) {
     return apply_logical(s, b.t, b.k, p->d_mat + b.off, p->opts.lowering, p->opts.precision, rs);
 }
 
-// The blocks of a group in its passes; zero: the state is |0...0> and the first
-// pass writes it (nothing is read).
+// The blocks of a group in its passes (none, if its blocks multiply to the
+// identity); zero: the state is |0...0> and the first pass writes it (nothing is
+// read).
 qsa_status run_group(qsa_state s, qsa_plan p, const PlanGroup& g, bool zero, qsa_run_stats* rs) {
     for (size_t i = g.p0; i < g.p1; ++i) {
         const GroupPass& gp = p->gpasses[i];
@@ -1072,10 +1073,10 @@ qsa_status run_group(qsa_state s, qsa_plan p, const PlanGroup& g, bool zero, qsa
         cudaError_t e = launch_group(s->psi, s->n, gp, p->d_group, zero && i == g.p0, s->stream, &s->launches);
         tm.stop();
         if (e != cudaSuccess) return cuda_fail(s, e, "group kernel");
-        s->known_zero = false;
         rs->passes += 1;
         rs->hbm_bytes += 16.0 * static_cast<double>(1ull << s->n);
     }
+    s->known_zero = false;   // also of a group without passes: its blocks count as applied
     rs->blocks += g.blocks;
     rs->diag_blocks += g.diags;
     rs->prod_blocks += g.prods;
@@ -1133,7 +1134,8 @@ qsa_status qsa_plan_execute_from_zero(qsa_state s, qsa_plan p, qsa_run_stats* st
     // a plan whose first pass writes every amplitude (the zero_init preparation,
     // or a group pass) needs no clearing first: |0..0> in the plan's layout is relabelled
     const bool prep = !p->blocks.empty() && p->blocks[0].init && s->n >= QSA_LAYER_TILE_BITS;
-    const bool group = !p->groups.empty() && p->groups[0].b0 == 0 && p->gpasses[p->groups[0].p0].only < 0;
+    const PlanGroup* g0 = !p->groups.empty() && p->groups[0].b0 == 0 ? &p->groups[0] : nullptr;
+    const bool group = g0 && g0->p0 < g0->p1 && p->gpasses[g0->p0].only < 0;
     const bool writes = (prep || group) && !s->failed;
     if (!writes) {
         qsa_status st = qsa_state_reset(s);

@@ -86,7 +86,8 @@ struct PlanLayer {
     std::vector<LayerLaunch> launches;   // for the plan's layout (empty when N < 12)
 };
 
-// Consecutive blocks [b0, b1) that run as the group passes [p0, p1).
+// Consecutive blocks [b0, b1) that run as the group passes [p0, p1); none where
+// the blocks are one-qubit operators that multiply to the identity.
 struct PlanGroup {
     size_t b0, b1, p0, p1;
     uint64_t blocks = 0, diags = 0, prods = 0;   // of the passes with several blocks
