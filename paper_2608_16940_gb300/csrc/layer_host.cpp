@@ -41,7 +41,7 @@ bool split_rotation(const std::array<std::complex<double>, 4>& F, double* c, dou
     }
     const std::complex<double> rec[4] = {p[0] * ca * q[0], -p[0] * sb * q[1], p[1] * sb * q[0], p[1] * ca * q[1]};
     for (int i = 0; i < 4; ++i)
-        if (std::abs(rec[i] - F[i]) > 1e-10) return false;
+        if (!(std::abs(rec[i] - F[i]) <= 1e-10)) return false;   // also where either is not a number
     return true;
 }
 

@@ -1,5 +1,6 @@
 """Group passes at the edges of what they accept: groups that multiply to the
-identity and so have no pass.  Same tolerance as the other group tests (1e-5 on
+identity and so have no pass, and factors with entries that are not numbers
+(those also where products run as layers).  Same tolerance as the other group tests (1e-5 on
 fidelity and amplitudes, FP32 sums of at most 32 terms over a few blocks)."""
 import numpy as np
 import pytest
@@ -64,3 +65,76 @@ def test_identity_trajectory(q):
             check_close(oracle.run_circuit(n, ops), got)
     finally:
         q.qsa_batch_destroy(b)
+
+
+BAD = [(i, v) for i in range(4) for v in (np.nan, complex(0, np.nan))]
+
+
+def _with_bad(i, v, rng):
+    F = W.haar_unitary(2, rng) if i != 2 else np.diag([1.0, 1.0]).astype(np.complex128)
+    F.flat[i] = v
+    return F
+
+
+def _check_bad(ops, psi, got):
+    """Wherever the oracle's amplitude is not a number, neither is the library's."""
+    want = psi.astype(np.complex128)
+    with np.errstate(invalid="ignore"):
+        for o in ops:
+            oracle.apply(want, o.targets, o.matrix)
+    assert np.isnan(want).any()
+    assert np.isnan(got[np.isnan(want)]).all()
+
+
+@pytest.mark.parametrize("i,v", BAD)
+@pytest.mark.parametrize("n", [5, 13])
+@pytest.mark.parametrize("kind", ["one-qubit blocks", "product blocks", "layer"])
+def test_not_a_number_in_a_plan(q, n, kind, i, v):
+    rng = np.random.default_rng(10 * n + i)
+    ops = [W.Op((j,), W.haar_unitary(2, rng), False, "u") for j in range(n)]
+    ops[3] = W.Op((3,), _with_bad(i, v, rng), False, "bad")
+    opts = {"one-qubit blocks": dict(kmax=1), "product blocks": dict(kmax=1, kmax_prod=3),
+            "layer": dict(kmax=4, layer=1)}[kind]
+    psi = W.random_state(n, seed=i).astype(np.complex64)
+    st = GState(q, torch, n, init=psi)
+    try:
+        q.qsa_apply_circuit(st.h, ops, q.make_opts(planner=q.QSA_PLAN_DP, **opts))
+        _check_bad(ops, psi, st.logical())
+    finally:
+        st.close()
+
+
+@pytest.mark.parametrize("i,v", BAD)
+def test_not_a_number_in_a_batch(q, i, v):
+    n, rng = 5, np.random.default_rng(i)
+    ops = [W.Op((2,), W.haar_unitary(2, rng), False, "u"), W.Op((2,), _with_bad(i, v, rng), False, "bad"),
+           W.Op((2,), W.haar_unitary(2, rng), False, "u")]
+    b = q.qsa_batch_create(n, [ops], q.make_opts(planner=q.QSA_PLAN_DP, kmax=1, kmax_diag=1))
+    x = torch.zeros(1 << n, dtype=torch.complex64, device="cuda:0")
+    zero = np.zeros(1 << n, dtype=np.complex64)
+    zero[0] = 1
+    try:
+        q.qsa_batch_run(b, x.data_ptr(), x.numel() * 8, 1, 1)
+        _check_bad(ops, zero, x.cpu().numpy().astype(np.complex128))
+    finally:
+        q.qsa_batch_destroy(b)
+
+
+@pytest.mark.parametrize("i,v", BAD)
+@pytest.mark.parametrize("layer", [False, True])
+def test_not_a_number_in_a_large_product(q, layer, i, v):
+    """N = 24, where unitary products run as layers: the amplitudes whose qubit
+    selects the row of the entry (both rows of a state without zeros are read)."""
+    n, t, rng = 24, [2, 23], np.random.default_rng(i)
+    fac = [_with_bad(i, v, rng), W.haar_unitary(2, rng)]
+    st = GState(q, torch, n)
+    try:
+        st.buf.fill_(1.0)
+        if layer:
+            q.qsa_apply_layer(st.h, [], t, fac)
+        else:
+            q.qsa_apply_product(st.h, t, fac)
+        row = torch.isnan(st.buf.view(-1, 2, 4)[:, i >> 1])
+        assert bool(row.all())
+    finally:
+        st.close()
