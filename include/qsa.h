@@ -355,10 +355,11 @@ qsa_status qsa_plan_blocks(qsa_plan p, size_t* first_op, int32_t* widths, size_t
 
 /* qsa_state_reset + a relabel of |0..0> to the plan's layout (metadata only,
  * valid for |0..0>, §IV-D) + qsa_plan_execute, without the reset's clearing
- * pass when the plan begins with a zero-state preparation (opts.zero_init,
- * N >= 12), which writes every amplitude.  The
- * state's previous contents and layout are discarded.  Errors: as
- * qsa_plan_execute. */
+ * pass when the plan's first pass writes every amplitude: a zero-state
+ * preparation (opts.zero_init, N >= 12) or a group pass of several blocks
+ * (qsa_plan_execute).  The state's previous contents and layout are discarded.
+ * After a failed allocation (QSA_E_NOMEM) in a plan that needed no clearing
+ * the state is |0..0> in the plan's layout.  Errors: as qsa_plan_execute. */
 qsa_status qsa_plan_execute_from_zero(qsa_state s, qsa_plan p, qsa_run_stats* stats);
 
 /* Execution order of the input ops (order[i] = input index of the i-th op

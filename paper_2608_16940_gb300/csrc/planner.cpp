@@ -1144,7 +1144,13 @@ qsa_status qsa_plan_execute_from_zero(qsa_state s, qsa_plan p, qsa_run_stats* st
     for (int q = 0; q < s->n; ++q) s->L[q] = p->L0[q];   // relabelling |0..0> is free
     s->known_zero = true;
     const qsa_status st = execute(s, p, writes && group, stats);
-    if (st != QSA_OK && writes) s->known_zero = false;   // the amplitudes may be the old ones
+    if (st != QSA_OK && writes && !s->failed) {
+        // an allocation failed, perhaps before anything was written: the amplitudes may still be
+        // the old ones of another layout, so the state becomes what the reset would have left
+        const qsa_status rst = qsa_state_reset(s);
+        if (rst != QSA_OK) return rst;
+        for (int q = 0; q < s->n; ++q) s->L[q] = p->L0[q];
+    }
     return st;
 }
 

@@ -1,7 +1,8 @@
 """Group passes at the edges of what they accept: groups that multiply to the
-identity and so have no pass, and factors with entries that are not numbers
-(those also where products run as layers).  Same tolerance as the other group tests (1e-5 on
-fidelity and amplitudes, FP32 sums of at most 32 terms over a few blocks)."""
+identity and so have no pass, factors with entries that are not numbers (those
+also where products run as layers), and allocations that fail before the first
+pass.  Same tolerance as the other group tests (1e-5 on fidelity and amplitudes,
+FP32 sums of at most 32 terms over a few blocks)."""
 import numpy as np
 import pytest
 
@@ -138,3 +139,42 @@ def test_not_a_number_in_a_large_product(q, layer, i, v):
         assert bool(row.all())
     finally:
         st.close()
+
+
+@pytest.mark.parametrize("kind", ["group", "zero_init"])
+def test_from_zero_after_a_failed_allocation(q, kind):
+    """Every allocation of the call fails once, on a state that holds other
+    amplitudes in another layout: the state is then |0...0> in the plan's layout,
+    and the call works once memory is there."""
+    n = 13
+    rng = np.random.default_rng(3)
+    if kind == "group":
+        ops, opts = _identity_then(n, "dense", rng)[n + 1:], dict(planner=q.QSA_PLAN_DP, kmax=1)
+    else:
+        ops, _ = W.qaoa_circuit(n=14, p=1, seed=4)
+        n, opts = 14, dict(planner=q.QSA_PLAN_DP, kmax=6, kmax_diag=12, layer=1, zero_init=1)
+    L = [int(v) for v in rng.permutation(n)]
+    failures = 0
+    for nth in range(8):
+        plan = q.qsa_plan_create(ops, n, q.make_opts(**opts), layout=L)
+        st = GState(q, torch, n, init=W.random_state(n, seed=n).astype(np.complex64))
+        q.qsa_debug_fail_alloc(nth)
+        try:
+            try:
+                q.qsa_plan_execute_from_zero(st.h, plan)
+                break
+            except q.QsaError as e:
+                assert e.code == q.QSA_E_NOMEM
+            finally:
+                q.qsa_debug_fail_alloc(-1)
+            failures += 1
+            assert q.qsa_get_layout(st.h) == L
+            zero = np.zeros(1 << n, dtype=np.complex128)
+            zero[0] = 1
+            assert np.array_equal(st.logical(), zero)
+            q.qsa_plan_execute_from_zero(st.h, plan)
+            check_close(oracle.run_circuit(n, ops), st.logical())
+        finally:
+            st.close()
+            q.qsa_plan_destroy(plan)
+    assert failures >= 1
