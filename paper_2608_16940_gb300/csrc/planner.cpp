@@ -241,53 +241,76 @@ void build_next_use(qsa_plan_s* p) {
     }
 }
 
-// Runs of consecutive dense (k <= 4), diagonal and product blocks become group
-// passes (several blocks per pass over the state) for the plan's layout.
-// Per-gate plans keep one pass per op, and permuting plans one layout per block.
-// mat64: the blocks' matrices before rounding, at their offsets in host_mat.
-void build_groups(qsa_plan_s* p, const std::vector<double>& mat64) {
-    if (p->n > kGroupMaxQubits || p->opts.planner == QSA_PLAN_PER_GATE || p->opts.lowering == QSA_LOWER_PERMUTE) return;
+// Runs [i, e) of at least two consecutive dense (k <= 4), diagonal and product
+// blocks: they become group passes (several blocks per pass over the state) for
+// the plan's layout.  Per-gate plans keep one pass per op, and permuting plans
+// one layout per block.
+std::vector<std::pair<size_t, size_t>> group_runs(const qsa_plan_s* p) {
+    std::vector<std::pair<size_t, size_t>> runs;
+    if (p->n > kGroupMaxQubits || p->opts.planner == QSA_PLAN_PER_GATE || p->opts.lowering == QSA_LOWER_PERMUTE) return runs;
     auto takes = [](const PlanBlock& b) { return b.layer < 0 && (b.prod || group_takes(b.k, b.diag)); };
     const size_t nb = p->blocks.size();
     for (size_t i = 0; i < nb;) {
         size_t e = i;
         while (e < nb && takes(p->blocks[e])) ++e;
-        if (e - i >= 2) {
-            std::vector<GroupSrc> src;
-            std::vector<int> whole;   // the block an operator is all of, or -1 (a product's factor)
-            for (size_t x = i; x < e; ++x) {
-                const PlanBlock& b = p->blocks[x];
-                const double* mat = mat64.data() + b.off;
-                if (b.prod) {
-                    for (int j = 0; j < b.k; ++j) {
-                        src.push_back({1, false, {p->L0[b.t[j]]}, mat + 8 * j});
-                        whole.push_back(-1);
-                    }
-                } else {
-                    GroupSrc g{b.k, b.diag, {}, mat};
-                    for (int j = 0; j < b.k; ++j) g.pos[j] = p->L0[b.t[j]];
-                    src.push_back(g);
-                    whole.push_back(static_cast<int>(x));
-                }
-            }
-            PlanGroup gr{i, e, p->gpasses.size(), 0};
-            for (size_t x = i; x < e; ++x) {
-                gr.blocks += 1;
-                gr.diags += p->blocks[x].diag ? 1 : 0;
-                gr.prods += p->blocks[x].prod ? 1 : 0;
-            }
-            for (GroupPass& gp : group_build(p->n, src, &p->host_group)) {
-                if (gp.only >= 0) gp.only = whole[gp.only];
-                if (gp.only >= 0) {   // counted where it runs
-                    gr.blocks -= 1;
-                    gr.diags -= p->blocks[gp.only].diag ? 1 : 0;
-                }
-                p->gpasses.push_back(gp);
-            }
-            gr.p1 = p->gpasses.size();
-            p->groups.push_back(gr);
-        }
+        if (e - i >= 2) runs.push_back({i, e});
         i = std::max(e, i + 1);
+    }
+    return runs;
+}
+
+// Product blocks of unitary factors that no run holds become layers on large states.
+void build_prod_layers(qsa_plan_s* p, const std::vector<double>& mat64, const std::vector<std::pair<size_t, size_t>>& runs) {
+    if (p->n < kProdLayerQubits) return;
+    size_t r = 0;
+    for (size_t i = 0; i < p->blocks.size(); ++i) {
+        while (r < runs.size() && runs[r].second <= i) ++r;
+        PlanBlock& b = p->blocks[i];
+        if (!b.prod || (r < runs.size() && runs[r].first <= i)) continue;
+        PlanLayer pl;
+        if (!product_as_layer(b.t, b.k, mat64.data() + b.off, &pl.spec)) continue;
+        b.prod_layer = static_cast<int>(p->layers.size());
+        p->layers.push_back(std::move(pl));
+    }
+}
+
+// The passes of the runs.  mat64: the blocks' matrices before rounding, at their
+// offsets in host_mat.
+void build_groups(qsa_plan_s* p, const std::vector<double>& mat64, const std::vector<std::pair<size_t, size_t>>& runs) {
+    for (const auto& [i, e] : runs) {
+        std::vector<GroupSrc> src;
+        std::vector<int> whole;   // the block an operator is all of, or -1 (a product's factor)
+        for (size_t x = i; x < e; ++x) {
+            const PlanBlock& b = p->blocks[x];
+            const double* mat = mat64.data() + b.off;
+            if (b.prod) {
+                for (int j = 0; j < b.k; ++j) {
+                    src.push_back({1, false, {p->L0[b.t[j]]}, mat + 8 * j});
+                    whole.push_back(-1);
+                }
+            } else {
+                GroupSrc g{b.k, b.diag, {}, mat};
+                for (int j = 0; j < b.k; ++j) g.pos[j] = p->L0[b.t[j]];
+                src.push_back(g);
+                whole.push_back(static_cast<int>(x));
+            }
+        }
+        PlanGroup gr{i, e, p->gpasses.size(), 0};
+        for (size_t x = i; x < e; ++x) {
+            gr.blocks += 1;
+            gr.diags += p->blocks[x].diag ? 1 : 0;
+            gr.prods += p->blocks[x].prod ? 1 : 0;
+        }
+        for (GroupPass& gp : group_build(p->n, src, &p->host_group)) {
+            if (gp.only >= 0) gp.only = whole[gp.only];
+            if (gp.only >= 0) {   // counted where it runs
+                gr.blocks -= 1;
+                gr.diags -= p->blocks[gp.only].diag ? 1 : 0;
+            }
+            p->gpasses.push_back(gp);
+        }
+        gr.p1 = p->gpasses.size();
+        p->groups.push_back(gr);
     }
 }
 
@@ -771,11 +794,6 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
                 p->host_mat[b.off + 2 * c] = static_cast<float>(F[c].real());
                 p->host_mat[b.off + 2 * c + 1] = static_cast<float>(F[c].imag());
             }
-            PlanLayer pl;
-            if (n_qubits >= kProdLayerQubits && product_as_layer(b.t, t, mat64.data() + b.off, &pl.spec)) {
-                b.prod_layer = static_cast<int>(p->layers.size());
-                p->layers.push_back(std::move(pl));
-            }
         } else if (u.diag) {
             b.diag = true;
             st = fuse_diag_range(ops, u.s, u.e, b.t, &b.k, &M);
@@ -831,10 +849,12 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
     for (size_t i = 0; i + 1 < p->blocks.size(); ++i)
         if (p->blocks[i].layer >= 0 && p->blocks[i + 1].layer >= 0)
             layer_move_exit_phases(&p->layers[p->blocks[i].layer].spec, &p->layers[p->blocks[i + 1].layer].spec);
+    const auto runs = group_runs(p);
+    build_prod_layers(p, mat64, runs);
     for (PlanLayer& pl : p->layers)
         pl.launches = prepare_layer(n_qubits, p->L0.data(), pl.spec, &p->host_layer, &carry);
     build_next_use(p);
-    build_groups(p, mat64);
+    build_groups(p, mat64, runs);
     *out = p;
     return QSA_OK;
 }

@@ -1,7 +1,7 @@
 """Group passes at the edges of what they accept: groups that multiply to the
 identity and so have no pass, factors with entries that are not numbers (those
-also where products run as layers), and allocations that fail before the first
-pass.  Same tolerance as the other group tests (1e-5 on fidelity and amplitudes,
+also where products run as layers), allocations that fail before the first pass,
+and what a plan uploads for grouped products.  Same tolerance as the other group tests (1e-5 on fidelity and amplitudes,
 FP32 sums of at most 32 terms over a few blocks)."""
 import numpy as np
 import pytest
@@ -178,3 +178,22 @@ def test_from_zero_after_a_failed_allocation(q, kind):
             st.close()
             q.qsa_plan_destroy(plan)
     assert failures >= 1
+
+
+def test_grouped_products_upload_no_layers(q):
+    """Product blocks of a run go into group passes: on a state large enough for
+    products as layers the plan holds no layer tables for them, so its upload is
+    the one of a state below that size (the same targets, so the same programs)."""
+    rng = np.random.default_rng(8)
+    ops = [W.Op((j,), W.haar_unitary(2, rng), False, "u") for j in range(14)]
+    h2d = []
+    for n in (23, 24):
+        plan = q.qsa_plan_create(ops, n, q.make_opts(planner=q.QSA_PLAN_DP, kmax=1, kmax_prod=7))
+        assert list(q.qsa_plan_block_kinds(plan)[0]) == [2, 2]
+        st = GState(q, torch, n)
+        try:
+            h2d.append(q.qsa_plan_execute(st.h, plan)["h2d_bytes"])
+        finally:
+            st.close()
+            q.qsa_plan_destroy(plan)
+    assert h2d[0] == h2d[1] > 0
