@@ -486,16 +486,22 @@ cudaError_t launch_apply_k(float2* psi, int n, const int* phys, const float* d_m
 // issues every third cycle (84 FMAs per clock and SM with operands that change,
 // 95 with one held, measured), scalar ones reach 104.  The two half-warps of a
 // k = 6 team take neighbouring row pairs and read neighbouring 16-byte units.
-// Three teams per CTA, one CTA per SM, share the matrix; two stages per team
-// keep the next tile's copies under the arithmetic (with two teams 5 % slower,
-// four leave 128 registers a thread and spill).  The matrix's index bits are put
+// The teams of a CTA, one CTA per SM, share the matrix; two stages per team keep
+// the next tile's copies under the arithmetic.  k = 5 adds the products of the
+// real and of the imaginary parts in sums of their own (relative error of one
+// operator 1.09e-7, 1.47e-7 with one running sum): 128 accumulators, so two teams
+// with 255 registers a thread (N = 26: 381 us; three teams with 168 386, 428 with
+// a target on position 0).  k = 6 keeps one running sum and three teams (641 us;
+// two 686, four leave 128 registers and spill).  The matrix's index bits are put
 // in ascending position order, so a target on position 0 (P0) is column bit 0
 // and both columns of a pair come in one 16-byte load.  Outputs go back to the
 // stage in place and leave in address order.
-// N = 26, random targets, k = 5 / 6: 0.48 / 0.985 ms with one row of the matrix
-// read per group (the kernel above, 8 rows per thread), 0.360 / 0.647 ms here,
-// 0.59 / 0.66 of 128 FMAs per clock and SM.
-constexpr int kWideT = 12, kWideTeam = 128, kWideTeams = 3, kWideR = 8, kWideG = 4;
+// N = 26, four target sets, k = 5 / 6: 412..596 / 902..1224 us with one row of the
+// matrix read per group (the kernel above, 8 rows per thread), 381 / 623..648 us
+// here, 0.56 / 0.66 of 128 FMAs per clock and SM.
+constexpr int kWideT = 12, kWideTeam = 128, kWideR = 8, kWideG = 4;
+template <int K>
+constexpr int kWideTeams = K == 5 ? 2 : 3;
 constexpr int kWideChunks = (1 << (kWideT - 1)) / kWideTeam;   // 16-byte units per thread
 
 struct WideArgs {
@@ -515,17 +521,17 @@ struct WideArgs {
 
 template <int K>
 __host__ __device__ constexpr size_t wide_smem() {
-    return sizeof(float2) * 2 * kWideTeams * (1 << kWideT) + (8u << (2 * K));
+    return sizeof(float2) * 2 * kWideTeams<K> * (1 << kWideT) + (8u << (2 * K));
 }
 
 template <int K, bool P0>
-__global__ void __launch_bounds__(kWideTeam * kWideTeams, 1) k_apply_wide(const __grid_constant__ WideArgs a) {
+__global__ void __launch_bounds__(kWideTeam * kWideTeams<K>, 1) k_apply_wide(const __grid_constant__ WideArgs a) {
     constexpr int D = 1 << K, NRB = D / kWideR, NF = kWideT - K;
     static_assert((D / kWideR) * (1 << NF) / kWideG == kWideTeam, "a team covers the tile");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int team = threadIdx.x / kWideTeam, tid = threadIdx.x % kWideTeam;
     float2* stage = reinterpret_cast<float2*>(smem_raw) + team * 2 * (1 << kWideT);
-    float2* Mt = reinterpret_cast<float2*>(smem_raw + sizeof(float2) * 2 * kWideTeams * (1 << kWideT));   // [column][row]
+    float2* Mt = reinterpret_cast<float2*>(smem_raw + sizeof(float2) * 2 * kWideTeams<K> * (1 << kWideT));   // [column][row]
 
     const float2* gm = reinterpret_cast<const float2*>(a.mat);
     for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
@@ -561,7 +567,7 @@ __global__ void __launch_bounds__(kWideTeam * kWideTeams, 1) k_apply_wide(const 
     gs[3] = gs[1] ^ a.fslot[LB + 1];
     __syncthreads();
 
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kWideTeams;
+    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kWideTeams<K>;
     const uint64_t limit = a.ntiles << kWideT;
     auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kWideTeam) : "memory"); };
     auto tile_at = [&](uint64_t t) {
@@ -590,31 +596,29 @@ __global__ void __launch_bounds__(kWideTeam * kWideTeams, 1) k_apply_wide(const 
         next = tile_at(t + stride);
         if (t + stride < a.ntiles) load(next, stage + cur * (1 << kWideT));
         cp_async_commit();
-        float2 acc[kWideR][kWideG];
+        // k = 5: the products of the real and of the imaginary parts in sums of their own
+        constexpr bool TWO = K == 5;
+        float2 acc[kWideR][kWideG], acc2[kWideR][kWideG];
 #pragma unroll
         for (int r = 0; r < kWideR; ++r)
 #pragma unroll
-            for (int g = 0; g < kWideG; ++g) acc[r][g] = make_float2(0.f, 0.f);
+            for (int g = 0; g < kWideG; ++g) acc[r][g] = acc2[r][g] = make_float2(0.f, 0.f);
         auto column = [&](const float4* m, const float2 (&v)[kWideG]) {
+            auto row = [&](int r, float re, float im) {
+                float2 (&b)[kWideG] = TWO ? acc2[r] : acc[r];
+#pragma unroll
+                for (int g = 0; g < kWideG; ++g) {
+                    acc[r][g].x = fmaf(re, v[g].x, acc[r][g].x);
+                    acc[r][g].y = fmaf(re, v[g].y, acc[r][g].y);
+                    b[g].x = fmaf(-im, v[g].y, b[g].x);
+                    b[g].y = fmaf(im, v[g].x, b[g].y);
+                }
+            };
 #pragma unroll
             for (int r = 0; r < kWideR; r += 2) {
                 const float4 e = m[NRB * (r >> 1)];   // rows 2 (rb + NRB r / 2) and the next
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r][g].x = fmaf(e.x, v[g].x, acc[r][g].x);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r][g].y = fmaf(e.x, v[g].y, acc[r][g].y);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r][g].x = fmaf(-e.y, v[g].y, acc[r][g].x);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r][g].y = fmaf(e.y, v[g].x, acc[r][g].y);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].x = fmaf(e.z, v[g].x, acc[r + 1][g].x);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].y = fmaf(e.z, v[g].y, acc[r + 1][g].y);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].x = fmaf(-e.w, v[g].y, acc[r + 1][g].x);
-#pragma unroll
-                for (int g = 0; g < kWideG; ++g) acc[r + 1][g].y = fmaf(e.w, v[g].x, acc[r + 1][g].y);
+                row(r, e.x, e.y);
+                row(r + 1, e.z, e.w);
             }
         };
         // eight columns at a time: their low bits' slots enter from the parameter bank
@@ -646,7 +650,8 @@ __global__ void __launch_bounds__(kWideTeam * kWideTeams, 1) k_apply_wide(const 
         for (int r = 0; r < kWideR; ++r) {
             const int so = rslot ^ a.sloff[2 * NRB * (r >> 1) + (r & 1)];
 #pragma unroll
-            for (int g = 0; g < kWideG; ++g) st[gs[g] ^ so] = acc[r][g];
+            for (int g = 0; g < kWideG; ++g)
+                st[gs[g] ^ so] = TWO ? make_float2(acc[r][g].x + acc2[r][g].x, acc[r][g].y + acc2[r][g].y) : acc[r][g];
         }
         team_sync();
 #pragma unroll
@@ -694,7 +699,7 @@ cudaError_t launch_apply_wide(float2* psi, int n, const int* phys, const float* 
     cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(wide_smem<K>()));
     if (e != cudaSuccess) return e;
     const uint64_t grid = std::min<uint64_t>(g.ntiles, static_cast<uint64_t>(num_sms()));
-    kern<<<static_cast<unsigned>(grid), kWideTeam * kWideTeams, wide_smem<K>(), st>>>(a);
+    kern<<<static_cast<unsigned>(grid), kWideTeam * kWideTeams<K>, wide_smem<K>(), st>>>(a);
     ++*launches;
     return cudaGetLastError();
 }

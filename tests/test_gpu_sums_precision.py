@@ -1,0 +1,63 @@
+"""How an operator's products are added, by its error against 64 bits.
+
+An output of a dense operator on D = 2^k amplitudes is a sum of 2 D products
+per component.  With rounding errors of relative size d (2^-24 / sqrt(3) over a
+mantissa spread evenly in logarithm: d = 2.53e-8) and terms of equal variance,
+the sums of the D products of real and of the D products of imaginary parts,
+added at the end, have the relative error d sqrt((D + 1) / 2 + 2), with the
+rounding of the matrix and of the last addition; one running sum over all 2 D
+products d sqrt((2 D + 1) / 2 + 1), 1.10, 1.21 and 1.35 times as much at k = 2, 3
+and 5.  The bounds below lie at 1.05 times the first."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from gpu_helpers import GState  # noqa: E402
+
+D_ROUND = 2.0 ** -24 * np.sqrt(0.375 / np.log(2.0) / 3.0)
+
+
+@pytest.fixture(scope="module")
+def q():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2608_16940_gb300 as q
+    return q
+
+
+def _relative_error(q, n, ops, opts, seed):
+    psi = W.random_state(n, seed=seed).astype(np.complex64)
+    want = psi.astype(np.complex128)
+    for o in ops:
+        oracle.apply(want, o.targets, o.matrix)
+    st = GState(q, torch, n, init=psi)
+    try:
+        stats = q.qsa_apply_circuit(st.h, ops, opts)
+        return np.linalg.norm(st.logical() - want) / np.linalg.norm(want), stats
+    finally:
+        st.close()
+
+
+def _mean_error(q, n, k, count, opts):
+    errs = []
+    for seed in range(6):
+        rng = np.random.default_rng(100 * k + seed)
+        ops = [W.Op(tuple(int(t) for t in rng.permutation(n)[:k]), W.haar_unitary(1 << k, rng), False, "u")
+               for _ in range(count)]
+        e, stats = _relative_error(q, n, ops, opts, seed)
+        errs.append(e)
+    return np.sqrt(np.mean(np.square(errs))), stats
+
+
+def _bound(k, count):
+    return 1.05 * D_ROUND * np.sqrt(((1 << k) + 1) / 2 + 2) * np.sqrt(count)
+
+
+def test_five_qubit_operators(q):
+    e, _ = _mean_error(q, 14, 5, 4, q.make_opts(planner=q.QSA_PLAN_PER_GATE, kmax=5))
+    assert e <= _bound(5, 4)
