@@ -19,11 +19,11 @@
 // from small tables in the program instead of bit arithmetic.
 // Measured, one pass per block / group passes with complex 2 x 2 blocks / with
 // rotations: QFT + 3 random layers at N = 25, DP plan of k <= 4 blocks, 24.5 /
-// 4.58 / 3.29 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
+// 4.58 / 3.36 ms; the 12-qubit brick circuit of 20 layers from |0...0> (one
 // tile: one launch instead of about 250) with its probabilities and norm, 1.77
 // / 0.159 / 0.100 ms; 128 trajectories at N = 20 of 10..40 layers with their
-// samples, 295 / 45.9 / 22.0 ms.
-// Dense 2- and 3-qubit blocks with scalar FMAs (3.63 ms at N = 25) and an
+// samples, 295 / 45.9 / 22.8 ms.
+// Dense 2- and 3-qubit blocks with scalar FMAs (3.63 ms at N = 25 against 3.30) and an
 // operator's head read ahead of it (3.53) were slower: what counts is the
 // number of instructions and registers.
 #pragma once
@@ -83,10 +83,22 @@ __device__ __forceinline__ uint64_t cfma(const ulonglong2& g, uint64_t v, uint64
     return fma2(g.y, iv, fma2(g.x, v, acc));
 }
 
+// p + i q
+__device__ __forceinline__ uint64_t join(uint64_t p, uint64_t q) {
+    const float2 P = unpack2(p), Q = unpack2(q);
+    return pack2(P.x - Q.y, P.y + Q.x);
+}
+
 // The dense blocks on register bits B.. (ascending, as the matrix's index
 // bits).  An amplitude is one packed pair (Re, Im); a matrix entry is stored
-// as (Re, Re, Im, Im), so one complex multiply-add is two packed FMAs on
-// (v, i v) and the broadcast load of an entry is one 16-byte load.
+// as (Re, Re, Im, Im), so one complex multiply-add is two packed FMAs and the
+// broadcast load of an entry is one 16-byte load.  One-qubit blocks run on (v, i v)
+// in one sum of four products; wider ones sum the products with the real and
+// with the imaginary parts apart (p += Re v, q += Im v), as the kernels of single
+// blocks do: one sum of all had 1.10 / 1.21 times their error at k = 2 / 3, two
+// cost an addition per output (QFT and random layers at N = 25 3.29 -> 3.36 ms,
+// 128 trajectories at N = 20 22.5 -> 22.8 ms).  With two products a sum a
+// one-qubit block's error is the same either way.
 template <int B>
 __device__ __forceinline__ void dense1(uint64_t (&v)[16], const ulonglong2* __restrict__ g) {
     const ulonglong2 g00 = g[0], g01 = g[1], g10 = g[2], g11 = g[3];
@@ -117,48 +129,43 @@ template <int B0, int B1>
 __device__ __forceinline__ void dense2(uint64_t (&v)[16], const ulonglong2* __restrict__ g) {
 #pragma unroll
     for (int f0 = 0; f0 < 4; f0 += 2) {   // two groups at a time share the entries' loads
-        uint64_t x[2][4], ix[2][4];
+        uint64_t x[2][4];
 #pragma unroll
         for (int f = 0; f < 2; ++f)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                x[f][c] = v[reg_of<2, B0, B1, 0>(f0 + f, c)];
-                ix[f][c] = rot90(x[f][c]);
-            }
+            for (int c = 0; c < 4; ++c) x[f][c] = v[reg_of<2, B0, B1, 0>(f0 + f, c)];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const ulonglong2 e0 = g[4 * r], e1 = g[4 * r + 1], e2 = g[4 * r + 2], e3 = g[4 * r + 3];
 #pragma unroll
             for (int f = 0; f < 2; ++f)
                 v[reg_of<2, B0, B1, 0>(f0 + f, r)] =
-                    cfma(e3, x[f][3], ix[f][3],
-                         cfma(e2, x[f][2], ix[f][2],
-                              cfma(e1, x[f][1], ix[f][1], fma2(e0.y, ix[f][0], mul2(e0.x, x[f][0])))));
+                    join(fma2(e3.x, x[f][3], fma2(e2.x, x[f][2], fma2(e1.x, x[f][1], mul2(e0.x, x[f][0])))),
+                         fma2(e3.y, x[f][3], fma2(e2.y, x[f][2], fma2(e1.y, x[f][1], mul2(e0.y, x[f][0])))));
         }
     }
 }
 
 template <int B0, int B1, int B2>
 __device__ __forceinline__ void dense3(uint64_t (&v)[16], const ulonglong2* __restrict__ g) {
-    uint64_t x[2][8], ix[2][8];
+    uint64_t x[2][8];
 #pragma unroll
     for (int f = 0; f < 2; ++f)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            x[f][c] = v[reg_of<3, B0, B1, B2>(f, c)];
-            ix[f][c] = rot90(x[f][c]);
-        }
+        for (int c = 0; c < 8; ++c) x[f][c] = v[reg_of<3, B0, B1, B2>(f, c)];
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-        uint64_t a0 = 0, a1 = 0;
+        uint64_t p0 = 0, q0 = 0, p1 = 0, q1 = 0;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const ulonglong2 e = g[8 * r + c];
-            a0 = cfma(e, x[0][c], ix[0][c], a0);
-            a1 = cfma(e, x[1][c], ix[1][c], a1);
+            p0 = fma2(e.x, x[0][c], p0);
+            q0 = fma2(e.y, x[0][c], q0);
+            p1 = fma2(e.x, x[1][c], p1);
+            q1 = fma2(e.y, x[1][c], q1);
         }
-        v[reg_of<3, B0, B1, B2>(0, r)] = a0;
-        v[reg_of<3, B0, B1, B2>(1, r)] = a1;
+        v[reg_of<3, B0, B1, B2>(0, r)] = join(p0, q0);
+        v[reg_of<3, B0, B1, B2>(1, r)] = join(p1, q1);
     }
 }
 
@@ -183,8 +190,7 @@ __device__ __forceinline__ void dense4(uint64_t (&v)[16], const ulonglong2* __re
             p = fma2(x2[c + 1], e.y, p);
             q = fma2(y2[c + 1], e.y, q);
         }
-        const float2 P = unpack2(p), Q = unpack2(q);
-        v[r] = pack2(P.x - Q.y, P.y + Q.x);
+        v[r] = join(p, q);
     }
 }
 

@@ -61,3 +61,11 @@ def _bound(k, count):
 def test_five_qubit_operators(q):
     e, _ = _mean_error(q, 14, 5, 4, q.make_opts(planner=q.QSA_PLAN_PER_GATE, kmax=5))
     assert e <= _bound(5, 4)
+
+
+@pytest.mark.parametrize("k", [2, 3])
+def test_grouped_operators(q, k):
+    """Twelve operators, several to a pass."""
+    e, stats = _mean_error(q, 14, k, 12, q.make_opts(planner=q.QSA_PLAN_GREEDY, kmax=k))
+    assert stats["blocks"] == 12 and stats["passes"] < 12
+    assert e <= _bound(k, 12)
