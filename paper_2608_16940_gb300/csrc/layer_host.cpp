@@ -200,30 +200,58 @@ bool prepare_pass(int n, const int32_t* L, const LayerSpec& spec, const std::vec
                 qph[2 * b + 1] =
                     f2_modulus(rq[b][1], std::norm(rq[b][1]) * scale, 0.5, static_tables ? nullptr : carry);
             }
-        for (int r = 0; r < 3; ++r)
+        // One table of 16 entries z, of squared modulus m2 once rounded.  A product block's round to
+        // nearest, for the least error of one pass (plans of layers, which repeat their angles many
+        // times, keep the modulus: f2_modulus); what a table loses of the modulus the next one makes up,
+        // since entries of one modulus (equal angles) would add it up.
+        using Table = std::array<std::complex<double>, 16>;
+        double before = 1.0;
+        auto round_table = [&](const Table& z, const std::array<double, 16>& m2, bool used, float2* out) {
+            double exact = 0.0, got = 0.0;
+            for (int i = 0; i < 16; ++i) {
+                if (!spec.nearest) {
+                    out[i] = f2_modulus(z[i], m2[i], 1.0 / 16, carry);
+                    continue;
+                }
+                const double n2 = std::norm(z[i]);
+                const std::complex<double> w = z[i] * (used && n2 > 0.0 ? before * std::sqrt(m2[i] / n2) : 1.0);
+                out[i] = f2(w);
+                exact += std::norm(w);
+                got += static_cast<double>(out[i].x) * out[i].x + static_cast<double>(out[i].y) * out[i].y;
+            }
+            if (spec.nearest && used && got > 0.0) before = std::sqrt(exact / got);
+        };
+        for (int r = 0; r < 3; ++r) {
+            Table z;
+            std::array<double, 16> m2;
             for (int i = 0; i < 16; ++i) {
                 // the amplitude in place i of the round has the local index i ^ (exchanged bits)
                 const int li = i ^ static_cast<int>((p.rswap >> (4 * r)) & 15u);
-                std::complex<double> z = 1.0;
+                z[i] = 1.0;
                 for (int lb = 0; lb < 4; ++lb)
-                    if ((p.active >> (4 * r + lb)) & 1u) z *= rp[4 * r + lb][(li >> lb) & 1];
-                rpt[16 * r + i] = f2m(z, 1.0 / 16, carry);
-                if (std::abs(z - 1.0) > 1e-15) p.rpmask |= 1u << r;
+                    if ((p.active >> (4 * r + lb)) & 1u) z[i] *= rp[4 * r + lb][(li >> lb) & 1];
+                m2[i] = std::norm(z[i]);
+                if (std::abs(z[i] - 1.0) > 1e-15) p.rpmask |= 1u << r;
             }
+            round_table(z, m2, (p.rpmask >> r) & 1u, &rpt[16 * r]);
+        }
         if (static_tables)
-            for (int r = 0; r < 3; ++r)
+            for (int r = 0; r < 3; ++r) {
+                Table z;
+                std::array<double, 16> m2;
                 for (int i = 0; i < 16; ++i) {
-                    std::complex<double> z = 1.0;
-                    double m2 = 1.0;
+                    z[i] = 1.0;
+                    m2[i] = 1.0;
                     for (int lb = 0; lb < 4; ++lb) {
                         const int b = 4 * r + lb, v = (i >> lb) & 1;
                         if (!((p.pmask >> b) & 1u)) continue;
                         const double tf = static_cast<float>(rcoef[b]);
-                        z *= rq[b][v];
-                        m2 *= std::norm(rq[b][v]) * (1.0 + rcoef[b] * rcoef[b]) / (1.0 + tf * tf);
+                        z[i] *= rq[b][v];
+                        m2[i] *= std::norm(rq[b][v]) * (1.0 + rcoef[b] * rcoef[b]) / (1.0 + tf * tf);
                     }
-                    sph[16 * r + i] = f2_modulus(z, m2, 1.0 / 16, carry);
                 }
+                round_table(z, m2, (p.pmask >> (4 * r)) & 15u, &sph[16 * r]);
+            }
     }
     std::stable_sort(cross.begin(), cross.end(), [](const LayerGate& x, const LayerGate& y) { return x.a < y.a; });
     p.ncross = static_cast<int>(cross.size());
@@ -438,6 +466,8 @@ qsa_status run_layer_launches(qsa_state s, const std::vector<LayerLaunch>& ls, c
 }
 
 bool product_as_layer(const int32_t* targets, int k, const double* factors, LayerSpec* spec) {
+    if (k < kProdLayerFactors) return false;
+    spec->nearest = true;
     for (int j = 0; j < k; ++j) {
         std::array<std::complex<double>, 4> F;
         double big = 0.0;

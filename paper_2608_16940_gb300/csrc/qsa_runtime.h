@@ -56,6 +56,7 @@ struct LayerDiagOp {
 };
 struct LayerSpec {
     bool generate = false;                                  // write-only on a state taken as all ones
+    bool nearest = false;                                   // constants rounded to nearest (a product block)
     std::vector<LayerDiagOp> diag;
     std::vector<int32_t> t;                                 // factor qubits
     std::vector<std::array<std::complex<double>, 4>> f;     // factor j on t[j], row-major
@@ -185,13 +186,20 @@ std::vector<LayerLaunch> prepare_layer(int n, const int32_t* L, const LayerSpec&
                                        std::vector<unsigned char>* bytes, ModulusCarry* carry = nullptr);
 qsa_status run_layer_launches(qsa_state s, const std::vector<LayerLaunch>& ls, const unsigned char* d_base,
                               qsa_run_stats* rs, bool product = false);
-// Smallest state on which a product of unitary factors runs as a layer: the layer
-// kernel takes 0.36 ms for seven factors on random targets at N = 27 where the
-// product kernel's complex butterflies take 0.64, but forming its tables costs
-// the host about 10 us, which a smaller state's pass does not hide.
+// Smallest state and fewest factors with which a product of unitary factors runs
+// as a layer.  The layer kernel takes 0.36 ms for seven factors on random targets
+// at N = 27 where the product kernel's complex butterflies take 0.63, but forming
+// its tables costs the host about 10 us, which a smaller state's pass does not
+// hide.  Its phase tables cost up to six complex products per amplitude whatever
+// the number of factors, a butterfly four roundings per factor: the error against
+// 64 bits (Haar factors, N = 26, product kernel / layer) is 4.9e-8 / 5.6e-8 for
+// one, 7.9e-8 / 7.9e-8 for three, 9.4e-8 / 8.5e-8 for four and 1.39e-7 / 1.22e-7
+// for nine, so fewer than four factors stay with the butterflies (0.34..0.41 ms at
+// N = 27, 0.33 as a layer).
 constexpr int kProdLayerQubits = 24;
-// A product block as a layer without diagonal ops (8 doubles per factor), if
-// every factor is unitary.
+constexpr int kProdLayerFactors = 4;
+// A product block as a layer without diagonal ops (8 doubles per factor), if it
+// has enough factors and every one is unitary.
 bool product_as_layer(const int32_t* targets, int k, const double* factors, LayerSpec* spec);
 // Prepare for the state's current layout, upload to scratch and run (N < 12:
 // the diagonal and product kernels, op by op).

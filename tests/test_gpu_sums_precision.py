@@ -69,3 +69,30 @@ def test_grouped_operators(q, k):
     e, stats = _mean_error(q, 14, k, 12, q.make_opts(planner=q.QSA_PLAN_GREEDY, kmax=k))
     assert stats["blocks"] == 12 and stats["passes"] < 12
     assert e <= _bound(k, 12)
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5, 7, 9, 11])
+def test_large_products(q, k):
+    """N = 24, where some products run as layers: no further from 64 bits than the
+    complex butterflies, whose factors have sums of four products each (relative
+    error d sqrt(3.5) a factor; a tenth more for the spread over the factors drawn)."""
+    n, errs = 24, []
+    for seed in range(8):
+        rng = np.random.default_rng(1000 * k + seed)
+        t = [int(v) for v in rng.permutation(n)[:k]]
+        fac = [W.haar_unitary(2, rng) for _ in range(k)]
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        x = torch.view_as_complex(torch.randn(1 << n, 2, device="cuda", generator=g)) / 2 ** 12.5
+        want = x.to(torch.complex128)
+        for p, f in zip(t, fac):
+            m = torch.from_numpy(np.ascontiguousarray(f)).cuda()
+            want = torch.einsum("rc,acb->arb", m, want.view(-1, 2, 1 << p)).reshape(-1)
+        st = GState(q, torch, n)
+        try:
+            st.buf.copy_(x)
+            q.qsa_apply_product(st.h, t, fac)
+            d = torch.linalg.vector_norm(st.buf.to(torch.complex128) - want)
+            errs.append(float(d / torch.linalg.vector_norm(want)))
+        finally:
+            st.close()
+    assert np.sqrt(np.mean(np.square(errs))) <= 1.1 * D_ROUND * np.sqrt(3.5 * k)
