@@ -285,7 +285,12 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
     std::vector<Fine> fine = split_operators(n, src);
     std::vector<Fine*> left(fine.size());
     for (size_t i = 0; i < fine.size(); ++i) left[i] = &fine[i];
+    // Small tables round to nearest until the plan's constants would change the norm by 5e-8, then with
+    // error feedback.  Feedback alone takes entries up to an ulp and a half away: two one-qubit
+    // operators (a plan of blocks of one qubit) 8.8e-8 from 64 bits, 6.5e-8 this way, 6.7e-8 as passes
+    // of their own; a slack of 2e-8 left 7.0e-8.
     ModulusCarry carry;
+    carry.slack = 1e-7;
     const uint64_t all = n < 64 ? (1ull << n) - 1 : ~0ull;
     // What a pass may take, by the sizes before diagonal operators share tables and rotations share
     // entries; less of it where the program comes out too long after all.
@@ -465,7 +470,7 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                         for (int j = 0; j < f->k; ++j) y |= ((x >> j) & 1) << ord[j];
                         const Cx z = f->m[y ^ f->inv];
                         const double m2 = std::norm(z);
-                        // small tables repeat over the state: rounded with error feedback on the modulus,
+                        // small tables repeat over the state: the carry bounds what they do to the modulus,
                         // relative to the entry's own (in a large one the entries' errors average out)
                         const float2 e = f->m.size() <= 8 && m2 > 1e-30 && m2 < 1e30
                                              ? f2_modulus(z, m2, share / m2, &carry)

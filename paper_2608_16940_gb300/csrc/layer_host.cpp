@@ -341,6 +341,14 @@ float2 f2_modulus(std::complex<double> z, double m2, double weight, ModulusCarry
         rr[a] = static_cast<double>(rs[a]) * rs[a];
         ii[a] = static_cast<double>(is[a]) * is[a];
     }
+    // with slack: the nearest candidate while the carry stays within it
+    if (carry && carry->slack > 0.0) {
+        const double e = rr[1] + ii[1] - m2;
+        if (std::fabs(acc + weight * e) <= carry->slack) {
+            carry->acc += weight * e;
+            return make_float2(r0, i0);
+        }
+    }
     auto dist = [&](int a, int b) {
         return (rs[a] - zr) * (rs[a] - zr) + (is[b] - zi) * (is[b] - zi);
     };

@@ -142,6 +142,7 @@ void to_float_matrix(const double* m, int k, float* out);
 // each weighted by the share of the state it multiplies (see f2_modulus).
 struct ModulusCarry {
     double acc = 0.0;
+    double slack = 0.0;   // a carry up to this is left as it is: constants are rounded to nearest
 };
 // FP32 complex number within a few ulps of z whose squared modulus, weighted
 // by `weight` and added to the carry, leaves the carry nearest zero (with no

@@ -96,3 +96,18 @@ def test_large_products(q, k):
         finally:
             st.close()
     assert np.sqrt(np.mean(np.square(errs))) <= 1.1 * D_ROUND * np.sqrt(3.5 * k)
+
+
+@pytest.mark.parametrize("n", [13, 20])
+def test_two_grouped_one_qubit_operators(q, n):
+    """The shortest group: its phases and rotations cost no more than the two
+    operators as complex 2 x 2 passes (sums of two and two products, relative error
+    d sqrt(3.5) each; a tenth more for the spread over the operators drawn)."""
+    errs = []
+    for seed in range(12):
+        rng = np.random.default_rng(seed)
+        ops = [W.Op((t,), W.haar_unitary(2, rng), False, "u") for t in (3, 7)]
+        e, stats = _relative_error(q, n, ops, q.make_opts(planner=q.QSA_PLAN_GREEDY, kmax=1), seed)
+        assert stats["blocks"] == 2 and stats["passes"] == 1
+        errs.append(e)
+    assert np.sqrt(np.mean(np.square(errs))) <= 1.1 * D_ROUND * np.sqrt(3.5 * 2)
