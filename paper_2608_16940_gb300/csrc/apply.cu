@@ -880,12 +880,20 @@ __global__ void __launch_bounds__(kThreads) k_apply_prod(ProdArgs a) {
 // A permutation of the tile's bits, in place: the tile (2^T amplitudes, 16-byte
 // copies) is in shared memory before any of it is written.  Bound by HBM; what
 // counts is the number of passes a permutation of the state's positions takes,
-// so tiles are wide (2^13 amplitudes, runs of at least 64 bytes): ten positions
-// above the lowest three can move in one pass (plan_permutation).  One stage
-// per CTA, three CTAs of 512 threads per SM hide each other's latency.
-// N = 28, two random layouts and five bit swaps: 22 passes of 0.71 ms in
-// 2^11-amplitude tiles with up to six swaps each (14.5 ms), 7 of 0.69 ms here.
-constexpr int kPermT = 13, kPermThreads = 512, kPermLow = 3;
+// so tiles are wide (up to 2^13 amplitudes, runs of at least 64 bytes): ten
+// positions above the lowest three can move in one pass (plan_permutation).  One
+// stage per CTA; the CTAs of an SM, 128 KiB of stages, hide each other's latency
+// (192 KiB was slower: 40 registers a thread, with spills).  Up to nine such
+// positions: tiles of 2^12 and CTAs of 256 threads, whose shorter steps leave
+// less of the last wave empty.  Beyond the L2 a CTA per tile: the loads of one
+// start while the stores of another drain, which CTAs that walk tiles in step do
+// not reach; in the L2 starting CTAs costs more than that.
+// One pair at N = 22 / 23 / 24 / 28: 10.3 / 15.2 / 43.2 / 607 us here; in 2^13 tiles
+// with three walking CTAs per SM 12.4 / 18.7 / 48.0 / 684; in 2^11 tiles with three
+// stages and up to six positions (before) 10.3 / 17.6 / 46.1 / 708.  Two random
+// layouts and five bit swaps at N = 28: 22 passes of that kind, 14.5 ms; 7 passes
+// here, 4.5 ms.
+constexpr int kPermT = 13, kPermLow = 3;
 
 struct PermArgs {
     float2* psi;
@@ -897,11 +905,11 @@ struct PermArgs {
     uint16_t sslot[kPermT];   // slot of the tile bit whose content tile bit b receives
 };
 
-__global__ void __launch_bounds__(kPermThreads, 3) k_permute(const __grid_constant__ PermArgs a) {
+// LT: thread bits, CTAS: CTAs of an SM
+template <int LT, int CTAS>
+__global__ void __launch_bounds__(1 << LT, CTAS) k_permute(const __grid_constant__ PermArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* st = reinterpret_cast<float2*>(smem_raw);
-    constexpr int LT = 9;   // thread bits
-    static_assert(1 << LT == kPermThreads, "thread bits");
     const int tid = threadIdx.x;
     uint64_t g0 = 0;
     uint32_t sl = 0, ss = 0;
@@ -913,7 +921,7 @@ __global__ void __launch_bounds__(kPermThreads, 3) k_permute(const __grid_consta
             ss ^= a.sslot[b + 1];
         }
     const uint32_t chunks = 1u << (a.T - 1);
-    const int nk = chunks > kPermThreads ? static_cast<int>(chunks / kPermThreads) : 1;
+    const int nk = chunks > (1u << LT) ? static_cast<int>(chunks >> LT) : 1;
     const bool copies = static_cast<uint32_t>(tid) < chunks;
     const uint64_t limit = a.ntiles << a.T;
     const uint32_t s0 = a.sslot[0];
@@ -1170,54 +1178,76 @@ std::vector<std::vector<int>> plan_permutation(int n, const int* dest, int T) {
     }
 }
 
+namespace {
+
+// One pass: the content of position p moves to dest[p], at most kPermT - kPermLow
+// positions at kPermLow or above move.
+cudaError_t permute_pass(float2* psi, int n, const int* dest, cudaStream_t st) {
+    uint64_t moved = 0;
+    for (int p = 0; p < n; ++p)
+        if (dest[p] != p) moved |= 1ull << p;
+    const bool wide = __builtin_popcountll(moved >> kPermLow) > kPermT - 1 - kPermLow;
+    const int T = std::min(wide ? kPermT : kPermT - 1, n);
+    PermArgs a{};
+    a.psi = psi;
+    a.T = T;
+    a.ntiles = 1ull << (n - T);
+    int m = T;
+    while (m + __builtin_popcountll(moved >> m) > T) --m;
+    if (m < 1) return cudaErrorInvalidValue;
+    a.m = m;
+    for (int p = m; p < n; ++p)
+        if ((moved >> p) & 1) a.xpos[a.nx++] = p;
+    auto position = [&](int b) { return b < m ? b : a.xpos[b - m]; };
+    int bit_of[QSA_MAX_QUBITS] = {}, from[kPermT] = {};
+    for (int b = 0; b < T; ++b) bit_of[position(b)] = b;
+    for (int b = 0; b < T; ++b) from[bit_of[dest[position(b)]]] = b;
+    // The reading lanes vary the destination's bits 1..4: their source bits at 4 or above take slot
+    // bits 1..3 that no other of them has.
+    uint32_t used = 0, vec[kPermT] = {};
+    for (int b = 1; b <= 4 && b < T; ++b)
+        if (from[b] >= 1 && from[b] <= 3) used |= 1u << from[b];
+    for (int b = 1; b <= 4 && b < T; ++b)
+        if (from[b] >= 4)
+            for (int j = 1; j <= 3; ++j)
+                if (!((used >> j) & 1)) {
+                    used |= 1u << j;
+                    vec[from[b]] = 1u << j;
+                    break;
+                }
+    for (int b = 0; b < T; ++b) {
+        a.poff[b] = 1ull << position(b);
+        a.pslot[b] = static_cast<uint16_t>((1u << b) ^ vec[b]);
+    }
+    for (int b = 0; b < T; ++b) a.sslot[b] = a.pslot[from[b]];
+    const size_t smem = sizeof(float2) << T;
+    auto kern = wide ? k_permute<9, 2> : k_permute<8, 4>;
+    if (wide) {
+        cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+    }
+    const uint64_t grid = n >= kBeyondL2 ? a.ntiles : std::min<uint64_t>(a.ntiles, num_sms() * (wide ? 2ull : 4ull));
+    kern<<<static_cast<unsigned>(grid), wide ? 512 : 256, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_permute(float2* psi, int n, const int* dest, cudaStream_t st, uint64_t* launches) {
-    const int T = std::min(kPermT, n);
-    for (const std::vector<int>& pass : plan_permutation(n, dest, kPermT)) {
-        PermArgs a{};
-        a.psi = psi;
-        a.T = T;
-        a.ntiles = 1ull << (n - T);
-        uint64_t moved = 0;
-        for (int p = 0; p < n; ++p)
-            if (pass[p] != p) moved |= 1ull << p;
-        int m = T;
-        while (m + __builtin_popcountll(moved >> m) > T) --m;
-        if (m < 1) return cudaErrorInvalidValue;
-        a.m = m;
-        for (int p = m; p < n; ++p)
-            if ((moved >> p) & 1) a.xpos[a.nx++] = p;
-        auto position = [&](int b) { return b < m ? b : a.xpos[b - m]; };
-        int bit_of[QSA_MAX_QUBITS] = {}, from[kPermT] = {};
-        for (int b = 0; b < T; ++b) bit_of[position(b)] = b;
-        for (int b = 0; b < T; ++b) from[bit_of[pass[position(b)]]] = b;
-        // The reading lanes vary the destination's bits 1..4: their source bits at 4 or above take slot
-        // bits 1..3 that no other of them has.
-        uint32_t used = 0, vec[kPermT] = {};
-        for (int b = 1; b <= 4 && b < T; ++b)
-            if (from[b] >= 1 && from[b] <= 3) used |= 1u << from[b];
-        for (int b = 1; b <= 4 && b < T; ++b)
-            if (from[b] >= 4)
-                for (int j = 1; j <= 3; ++j)
-                    if (!((used >> j) & 1)) {
-                        used |= 1u << j;
-                        vec[from[b]] = 1u << j;
-                        break;
-                    }
-        for (int b = 0; b < T; ++b) {
-            a.poff[b] = 1ull << position(b);
-            a.pslot[b] = static_cast<uint16_t>((1u << b) ^ vec[b]);
-        }
-        for (int b = 0; b < T; ++b) a.sslot[b] = a.pslot[from[b]];
-        const size_t smem = sizeof(float2) << T;
-        cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(k_permute), static_cast<int>(sizeof(float2) << kPermT));
-        if (e != cudaSuccess) return e;
-        int occ = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_permute, kPermThreads, smem);
-        if (e != cudaSuccess) return e;
-        const uint64_t grid = std::min<uint64_t>(a.ntiles, static_cast<uint64_t>(num_sms()) * std::max(occ, 1));
-        k_permute<<<static_cast<unsigned>(grid), kPermThreads, smem, st>>>(a);
+    auto run = [&](const int* pass) {
         ++*launches;
-        e = cudaGetLastError();
+        return permute_pass(psi, n, pass, st);
+    };
+    int moved = 0, high = 0;
+    for (int p = 0; p < n; ++p)
+        if (dest[p] != p) {
+            ++moved;
+            high += p >= kPermLow ? 1 : 0;
+        }
+    if (moved == 0) return cudaSuccess;
+    if (high <= kPermT - kPermLow) return run(dest);   // what plan_permutation would find
+    for (const std::vector<int>& pass : plan_permutation(n, dest, kPermT)) {
+        cudaError_t e = run(pass.data());
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
