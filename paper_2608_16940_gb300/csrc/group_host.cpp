@@ -61,18 +61,26 @@ struct Fine {
     int pos[kGroupDiagMax];
     float t = 0.f;           // rotation: tangent, and whether the bit is inverted after it
     bool flip = false;
-    std::vector<Cx> m;       // dense: row-major; diagonal: entries
+    // dense: row-major; diagonal: entries.  In m, or the source operator's as they are (own), or the
+    // two of a diagonal on one position (two): most operators need no memory of their own
+    std::vector<Cx> m;
+    const double* own = nullptr;
+    Cx two[2];
+    Cx entry(size_t i) const { return own ? Cx(own[2 * i], own[2 * i + 1]) : m.empty() ? two[i] : m[i]; }
+    Fine* next = nullptr;    // in the block of diagonal operators that it is part of
     int src = -1;            // the source operator it is all of, unchanged
     uint32_t inv = 0;        // index bits on positions that are inverted when it runs
 };
 
 std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
     std::vector<Fine> out;
+    out.reserve(2 * src.size() + static_cast<size_t>(n));
     std::vector<std::array<Cx, 2>> wait(n, {1.0, 1.0});   // phases that wait on a position
     auto waiting = [&](int q) { return wait[q][0] != 1.0 || wait[q][1] != 1.0; };
     auto diag1 = [&](int q, Cx d0, Cx d1) {
         Fine f{Fine::kDiag, 1ull << q, 1, {q}};
-        f.m = {d0, d1};
+        f.two[0] = d0;
+        f.two[1] = d1;
         out.push_back(std::move(f));
     };
     for (size_t i = 0; i < src.size(); ++i) {
@@ -84,21 +92,21 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
             f.mask |= 1ull << s.pos[j];
         }
         const size_t D = size_t(1) << s.k, cnt = s.diag ? D : D * D;
-        f.m.resize(cnt);
-        for (size_t e = 0; e < cnt; ++e) f.m[e] = Cx(s.mat[2 * e], s.mat[2 * e + 1]);
+        f.own = s.mat;
         if (!s.diag && s.k == 1) {
             const int at = s.pos[0];
             // the phases that wait join the operator, their moduli (the factors of a rotation's rows) stay
             // with the diagonal before it, so that it is still unitary
             const double m0 = modulus(wait[at][0]), m1 = modulus(wait[at][1]);
             const Cx w0 = wait[at][0] / m0, w1 = wait[at][1] / m1;
+            const Cx e[4] = {f.entry(0), f.entry(1), f.entry(2), f.entry(3)};
             double scale = 0.0;
-            for (const Cx& z : f.m) scale = std::max(scale, modulus(z));
+            for (const Cx& z : e) scale = std::max(scale, modulus(z));
             double c = 0.0, sn = 0.0;
             Cx p[2], q[2];
             if (m0 > 0.0 && m1 > 0.0 && scale > 0.0 && scale < 1e30 &&
-                split_rotation({mul(f.m[0], w0) / scale, mul(f.m[1], w1) / scale, mul(f.m[2], w0) / scale,
-                                mul(f.m[3], w1) / scale}, &c, &sn, p, q)) {
+                split_rotation({mul(e[0], w0) / scale, mul(e[1], w1) / scale, mul(e[2], w0) / scale,
+                                mul(e[3], w1) / scale}, &c, &sn, p, q)) {
                 if (sn == 0.0) {   // diagonal after all
                     wait[at] = {scale * c * p[0] * m0, scale * c * p[1] * m1};
                     continue;
@@ -113,7 +121,7 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
                 f.kind = Fine::kRot;
                 f.flip = flip;
                 f.src = -1;
-                f.m.clear();
+                f.own = nullptr;
                 out.push_back(std::move(f));
                 continue;
             }
@@ -121,6 +129,11 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
         if (!s.diag)
             for (int j = 0; j < s.k; ++j) {
                 if (!waiting(s.pos[j])) continue;
+                if (f.own) {
+                    f.m.resize(cnt);
+                    for (size_t e = 0; e < cnt; ++e) f.m[e] = f.entry(e);
+                    f.own = nullptr;
+                }
                 for (size_t r = 0; r < D; ++r)
                     for (size_t c = 0; c < D; ++c) f.m[r * D + c] *= wait[s.pos[j]][(c >> j) & 1];
                 wait[s.pos[j]] = {1.0, 1.0};
@@ -140,14 +153,20 @@ std::vector<Fine> split_operators(int n, const std::vector<GroupSrc>& src) {
 // has touched since where it stands.
 // New blocks are kept in *made.
 std::vector<Fine*> merge_diagonals(const std::vector<Fine*>& ops, int cap, std::deque<Fine>* made) {
+    int diagonal = 0;
+    for (const Fine* f : ops) diagonal += f->kind == Fine::kDiag ? 1 : 0;
+    if (diagonal < 2) return ops;
     struct Block {
         uint64_t mask = 0, closed = 0;
         int64_t place = -1;          // index in seq, -1: not placed yet
-        std::vector<Fine*> of;
+        Fine *first = nullptr, *last = nullptr;
     };
     std::vector<Block> blocks;
     std::vector<std::pair<Fine*, int>> seq;         // an operator, or a block's index
-    std::vector<int64_t> last(64, -1);              // per position: the last operator that is not diagonal
+    blocks.reserve(static_cast<size_t>(diagonal));
+    seq.reserve(ops.size());
+    int64_t last[64];                               // per position: the last operator that is not diagonal
+    std::fill(last, last + 64, int64_t(-1));
     size_t open = 0;   // blocks before this one are closed on every position
     for (Fine* fp : ops) {
         Fine& f = *fp;
@@ -181,19 +200,23 @@ std::vector<Fine*> merge_diagonals(const std::vector<Fine*>& ops, int cap, std::
             blocks.emplace_back();
         }
         blocks[best].mask |= f.mask;
-        blocks[best].of.push_back(fp);
+        Block& B = blocks[best];
+        (B.last ? B.last->next : B.first) = fp;
+        B.last = fp;
+        fp->next = nullptr;
     }
     for (size_t b = 0; b < blocks.size(); ++b)
         if (blocks[b].place < 0) seq.push_back({nullptr, static_cast<int>(b)});
     std::vector<Fine*> out;
+    out.reserve(seq.size());
     for (const auto& it : seq) {
         if (it.first) {
             out.push_back(it.first);
             continue;
         }
         const Block& B = blocks[it.second];
-        if (B.of.size() == 1) {
-            out.push_back(B.of[0]);
+        if (B.first == B.last) {
+            out.push_back(B.first);
             continue;
         }
         made->push_back(Fine{Fine::kDiag, B.mask, 0, {}});
@@ -207,9 +230,9 @@ std::vector<Fine*> merge_diagonals(const std::vector<Fine*>& ops, int cap, std::
         // one-qubit members as an outer product, then the others
         std::array<std::array<Cx, 2>, kGroupDiagMax> one;
         one.fill({1.0, 1.0});
-        for (const Fine* o : B.of)
+        for (const Fine* o = B.first; o; o = o->next)
             if (o->k == 1)
-                for (int v = 0; v < 2; ++v) one[bit_of[o->pos[0]]][v] = mul(one[bit_of[o->pos[0]]][v], o->m[v]);
+                for (int v = 0; v < 2; ++v) one[bit_of[o->pos[0]]][v] = mul(one[bit_of[o->pos[0]]][v], o->entry(v));
         f.m.resize(size_t(1) << f.k);
         f.m[0] = 1.0;
         for (int j = 0; j < f.k; ++j)
@@ -217,13 +240,13 @@ std::vector<Fine*> merge_diagonals(const std::vector<Fine*>& ops, int cap, std::
                 f.m[c | size_t(1) << j] = mul(f.m[c], one[j][1]);
                 f.m[c] = mul(f.m[c], one[j][0]);
             }
-        for (const Fine* o : B.of) {
+        for (const Fine* o = B.first; o; o = o->next) {
             if (o->k == 1) continue;
             uint8_t part[kGroupDiagMax] = {}, at[1 << kGroupDiagMax] = {};   // index parts of f's bits, its indices
             for (int j = 0; j < o->k; ++j) part[bit_of[o->pos[j]]] = static_cast<uint8_t>(1u << j);
             for (size_t c = 0; c < f.m.size(); ++c) {
                 if (c) at[c] = static_cast<uint8_t>(at[c & (c - 1)] | part[__builtin_ctzll(c)]);
-                f.m[c] = mul(f.m[c], o->m[at[c]]);
+                f.m[c] = mul(f.m[c], o->entry(at[c]));
             }
         }
         out.push_back(&f);
@@ -294,7 +317,8 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
     const uint64_t all = n < 64 ? (1ull << n) - 1 : ~0ull;
     // What a pass may take, by the sizes before diagonal operators share tables and rotations share
     // entries; less of it where the program comes out too long after all.
-    double room = 2.0 * kGroupProgBytes;
+    constexpr double kRoom = 2.0 * kGroupProgBytes;
+    double room = kRoom;
     while (!left.empty()) {
         // the operators of this pass
         std::vector<Fine*> take, later;
@@ -464,15 +488,16 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                         }
                     }
                     float* g = reinterpret_cast<float*>(par.data() + op.off);
-                    const double share = 1.0 / static_cast<double>(f->m.size());
-                    for (size_t x = 0; x < f->m.size(); ++x) {
-                        size_t y = 0;
-                        for (int j = 0; j < f->k; ++j) y |= ((x >> j) & 1) << ord[j];
-                        const Cx z = f->m[y ^ f->inv];
+                    const size_t entries = size_t(1) << f->k;
+                    const double share = 1.0 / static_cast<double>(entries);
+                    uint8_t own[1 << kGroupDiagMax] = {static_cast<uint8_t>(f->inv)};   // the operator's own index
+                    for (size_t x = 0; x < entries; ++x) {
+                        if (x) own[x] = static_cast<uint8_t>(own[x & (x - 1)] ^ 1u << ord[__builtin_ctzll(x)]);
+                        const Cx z = f->entry(own[x]);
                         const double m2 = std::norm(z);
                         // small tables repeat over the state: the carry bounds what they do to the modulus,
                         // relative to the entry's own (in a large one the entries' errors average out)
-                        const float2 e = f->m.size() <= 8 && m2 > 1e-30 && m2 < 1e30
+                        const float2 e = entries <= 8 && m2 > 1e-30 && m2 < 1e30
                                              ? f2_modulus(z, m2, share / m2, &carry)
                                              : make_float2(static_cast<float>(z.real()), static_cast<float>(z.imag()));
                         g[2 * x] = e.x;
@@ -489,15 +514,15 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
                     }
                     std::sort(ord, ord + f->k, [&](int x, int y) { return rbit[x] < rbit[y]; });
                     const int D = 1 << f->k;
-                    auto from = [&](int x) {   // sorted index -> the operator's own
-                        int y = 0;
+                    int from[16];   // sorted index -> the operator's own
+                    for (int x = 0; x < D; ++x) {
+                        from[x] = static_cast<int>(f->inv);
                         for (int j = 0; j < f->k; ++j)
-                            if ((x >> j) & 1) y |= 1 << ord[j];
-                        return y ^ static_cast<int>(f->inv);
-                    };
+                            if ((x >> j) & 1) from[x] ^= 1 << ord[j];
+                    }
                     for (int r = 0; r < D; ++r)
                         for (int c = 0; c < D; ++c) {
-                            const Cx e = f->m[static_cast<size_t>(from(r)) * D + from(c)];
+                            const Cx e = f->entry(static_cast<size_t>(from[r]) * D + from[c]);
                             const float re = static_cast<float>(e.real()), im = static_cast<float>(e.imag());
                             *g++ = re;
                             if (f->k < 4) *g++ = re;
@@ -517,11 +542,12 @@ std::vector<GroupPass> group_build(int n, const std::vector<GroupSrc>& src, std:
         p.ops_off = up16(rounds.size() * sizeof(GroupRound));
         p.par_off = up16(p.ops_off + code.size() * sizeof(GroupOp));
         p.bytes = up16(p.par_off + par.size());
-        if (p.bytes > kGroupProgBytes) {
-            room *= 0.7;   // the same operators again, fewer of them
+        if (p.bytes > kGroupProgBytes) {   // the same operators again, as many fewer as it was too long
+            room = std::min(bytes, room) * std::min(0.95, 0.98 * kGroupProgBytes / p.bytes);
             continue;
         }
-        room = 2.0 * kGroupProgBytes;
+        // the operators to come are much like these: as much again, or more where the program is short
+        if (p.bytes < 0.9 * kGroupProgBytes) room = std::min(kRoom, room * 0.95 * kGroupProgBytes / p.bytes);
         left.swap(later);
         p.prog = static_cast<uint32_t>(progs->size());
         progs->resize(p.prog + p.bytes);

@@ -17,18 +17,24 @@
 namespace qsa {
 
 // F = diag(p) [[c, -s], [s, c]] diag(q) with q[0] = 1, c = |F00|, s = |F01|;
-// false unless the product reproduces F to 1e-10 (a unitary F does).
+// false unless the product reproduces F to 1e-10 (a unitary F does).  Plain moduli
+// and products: a plan splits every one-qubit operator of its groups, and the
+// library's guarded ones took most of that time.
 bool split_rotation(const std::array<std::complex<double>, 4>& F, double* c, double* s, std::complex<double>* p,
                     std::complex<double>* q) {
-    const std::complex<double> a = F[0], b = F[1], cc = F[2], d = F[3];
-    const double ca = std::abs(a), sb = std::abs(b);
+    using Cx = std::complex<double>;
+    auto mul = [](Cx a, Cx b) {
+        return Cx(a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real());
+    };
+    const Cx a = F[0], b = F[1], cc = F[2], d = F[3];
+    const double ca = std::sqrt(std::norm(a)), sb = std::sqrt(std::norm(b));
     if (ca == 0.0 && sb == 0.0) return false;
     *c = ca;
     *s = sb;
     q[0] = 1.0;
     if (ca > 0.0 && sb > 0.0) {
         p[0] = a / ca;
-        q[1] = -b / (p[0] * sb);
+        q[1] = mul(-b, std::conj(p[0])) / sb;   // |p0| = 1
         p[1] = cc / sb;
     } else if (sb == 0.0) {
         p[0] = a / ca;
@@ -39,9 +45,9 @@ bool split_rotation(const std::array<std::complex<double>, 4>& F, double* c, dou
         p[0] = -b / sb;
         p[1] = cc / sb;
     }
-    const std::complex<double> rec[4] = {p[0] * ca * q[0], -p[0] * sb * q[1], p[1] * sb * q[0], p[1] * ca * q[1]};
+    const Cx rec[4] = {p[0] * ca, mul(p[0], q[1]) * -sb, p[1] * sb, mul(p[1], q[1]) * ca};
     for (int i = 0; i < 4; ++i)
-        if (!(std::abs(rec[i] - F[i]) <= 1e-10)) return false;   // also where either is not a number
+        if (!(std::norm(rec[i] - F[i]) <= 1e-20)) return false;   // also where either is not a number
     return true;
 }
 
@@ -332,6 +338,13 @@ inline float step_float(float x, bool up) {
 
 float2 f2_modulus(std::complex<double> z, double m2, double weight, ModulusCarry* carry) {
     const float r0 = static_cast<float>(z.real()), i0 = static_cast<float>(z.imag());
+    if (carry && carry->slack > 0.0) {   // the nearest candidate while the carry stays within it
+        const double e = static_cast<double>(r0) * r0 + static_cast<double>(i0) * i0 - m2;
+        if (std::fabs(carry->acc + weight * e) <= carry->slack) {
+            carry->acc += weight * e;
+            return make_float2(r0, i0);
+        }
+    }
     const float rs[3] = {step_float(r0, false), r0, step_float(r0, true)};
     const float is[3] = {step_float(i0, false), i0, step_float(i0, true)};
     const double acc = carry ? carry->acc : 0.0;
@@ -340,14 +353,6 @@ float2 f2_modulus(std::complex<double> z, double m2, double weight, ModulusCarry
     for (int a = 0; a < 3; ++a) {
         rr[a] = static_cast<double>(rs[a]) * rs[a];
         ii[a] = static_cast<double>(is[a]) * is[a];
-    }
-    // with slack: the nearest candidate while the carry stays within it
-    if (carry && carry->slack > 0.0) {
-        const double e = rr[1] + ii[1] - m2;
-        if (std::fabs(acc + weight * e) <= carry->slack) {
-            carry->acc += weight * e;
-            return make_float2(r0, i0);
-        }
     }
     auto dist = [&](int a, int b) {
         return (rs[a] - zr) * (rs[a] - zr) + (is[b] - zi) * (is[b] - zi);

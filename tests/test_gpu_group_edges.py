@@ -197,3 +197,25 @@ def test_grouped_products_upload_no_layers(q):
             st.close()
             q.qsa_plan_destroy(plan)
     assert h2d[0] == h2d[1] > 0
+
+
+@pytest.mark.parametrize("n,k,count", [(4, 4, 40), (5, 4, 60), (12, 4, 60), (13, 4, 45), (12, 3, 200), (12, 1, 700)])
+def test_long_programs(q, n, k, count):
+    """More operators on one tile than a pass's program holds: several passes, each
+    filled as far as it goes (the errors of so many operators stay below 1e-5)."""
+    rng = np.random.default_rng(1000 * n + count)
+    ops = [W.Op(tuple(int(t) for t in rng.permutation(n)[:k]), W.haar_unitary(1 << k, rng), False, "u")
+           for _ in range(count)]
+    psi = W.random_state(n, seed=n).astype(np.complex64)
+    plan = q.qsa_plan_create(ops, n, q.make_opts(planner=q.QSA_PLAN_GREEDY, kmax=k if n > 4 else 1))
+    st = GState(q, torch, n, init=psi)
+    try:
+        stats = q.qsa_plan_execute(st.h, plan)
+        assert 1 < stats["passes"] < stats["blocks"]
+        want = psi.astype(np.complex128)
+        for o in ops:
+            oracle.apply(want, o.targets, o.matrix)
+        check_close(want, st.logical())
+    finally:
+        st.close()
+        q.qsa_plan_destroy(plan)
