@@ -277,6 +277,7 @@ void build_prod_layers(qsa_plan_s* p, const std::vector<double>& mat64, const st
 // The passes of the runs.  mat64: the blocks' matrices before rounding, at their
 // offsets in host_mat.
 void build_groups(qsa_plan_s* p, const std::vector<double>& mat64, const std::vector<std::pair<size_t, size_t>>& runs) {
+    std::vector<unsigned char> progs;
     for (const auto& [i, e] : runs) {
         std::vector<GroupSrc> src;
         std::vector<int> whole;   // the block an operator is all of, or -1 (a product's factor)
@@ -301,7 +302,7 @@ void build_groups(qsa_plan_s* p, const std::vector<double>& mat64, const std::ve
             gr.diags += p->blocks[x].diag ? 1 : 0;
             gr.prods += p->blocks[x].prod ? 1 : 0;
         }
-        for (GroupPass& gp : group_build(p->n, src, &p->host_group)) {
+        for (GroupPass& gp : group_build(p->n, src, &progs)) {
             if (gp.only >= 0) gp.only = whole[gp.only];
             if (gp.only >= 0) {   // counted where it runs
                 gr.blocks -= 1;
@@ -312,6 +313,9 @@ void build_groups(qsa_plan_s* p, const std::vector<double>& mat64, const std::ve
         gr.p1 = p->gpasses.size();
         p->groups.push_back(gr);
     }
+    p->group_off = p->host_mat.size();
+    p->host_mat.resize(p->group_off + progs.size() / sizeof(float));   // lengths are multiples of 16
+    if (!progs.empty()) std::memcpy(p->host_mat.data() + p->group_off, progs.data(), progs.size());
 }
 
 uint64_t op_mask(const qsa_op& op) {
@@ -959,7 +963,7 @@ qsa_status qsa_plan_info(qsa_plan p, size_t* n_blocks, size_t* n_ops, int* max_w
     if (n_blocks) *n_blocks = p->blocks.size();
     if (n_ops) *n_ops = p->n_ops;
     if (max_width) *max_width = p->max_width;
-    if (matrix_bytes) *matrix_bytes = p->host_mat.size() * sizeof(float);
+    if (matrix_bytes) *matrix_bytes = p->group_off * sizeof(float);
     return QSA_OK;
 }
 
@@ -996,17 +1000,15 @@ namespace {
 void plan_free_device(qsa_plan p) {
     if (p->d_mat) dev_free(p->d_mat);
     if (p->d_layer) dev_free(p->d_layer);
-    if (p->d_group) dev_free(p->d_group);
     p->d_mat = nullptr;
     p->d_layer = nullptr;
-    p->d_group = nullptr;
 }
 
 }  // namespace
 
 qsa_status qsa_plan_destroy(qsa_plan p) {
     if (!p) return fail(QSA_E_ARG, "plan is NULL");
-    if (p->d_mat || p->d_layer || p->d_group) cudaDeviceSynchronize();
+    if (p->d_mat || p->d_layer) cudaDeviceSynchronize();
     plan_free_device(p);
     delete p;
     return QSA_OK;
@@ -1014,19 +1016,18 @@ qsa_status qsa_plan_destroy(qsa_plan p) {
 
 namespace {
 
-// First execution on a device: the fused matrices, the layer payloads and the
-// group programs are uploaded once.
+// First execution on a device: the fused matrices with the group programs, and
+// the layer payloads are uploaded once.
 qsa_status plan_upload(qsa_state s, qsa_plan p, qsa_run_stats* rs) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (p->dev == dev) return QSA_OK;
-    if (p->d_mat || p->d_layer || p->d_group) cudaStreamSynchronize(s->stream);
+    if (p->d_mat || p->d_layer) cudaStreamSynchronize(s->stream);
     plan_free_device(p);
     const size_t bytes = p->host_mat.size() * sizeof(float);
-    const size_t lbytes = p->host_layer.size(), gbytes = p->host_group.size();
+    const size_t lbytes = p->host_layer.size();
     cudaError_t e = bytes ? dev_malloc(&p->d_mat, bytes) : cudaSuccess;
     if (e == cudaSuccess && lbytes) e = dev_malloc(&p->d_layer, lbytes);
-    if (e == cudaSuccess && gbytes) e = dev_malloc(&p->d_group, gbytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         plan_free_device(p);
@@ -1040,12 +1041,8 @@ qsa_status plan_upload(qsa_state s, qsa_plan p, qsa_run_stats* rs) {
         e = cudaMemcpyAsync(p->d_layer, p->host_layer.data(), lbytes, cudaMemcpyHostToDevice, s->stream);
         if (e != cudaSuccess) return cuda_fail(s, e, "plan layer upload");
     }
-    if (gbytes) {
-        e = cudaMemcpyAsync(p->d_group, p->host_group.data(), gbytes, cudaMemcpyHostToDevice, s->stream);
-        if (e != cudaSuccess) return cuda_fail(s, e, "plan group upload");
-    }
     p->dev = dev;
-    rs->h2d_bytes = static_cast<double>(bytes + lbytes + gbytes);
+    rs->h2d_bytes = static_cast<double>(bytes + lbytes);
     return QSA_OK;
 }
 
@@ -1090,7 +1087,8 @@ qsa_status run_group(qsa_state s, qsa_plan p, const PlanGroup& g, bool zero, qsa
             continue;
         }
         Timer tm(s, &rs->apply_seconds);
-        cudaError_t e = launch_group(s->psi, s->n, gp, p->d_group, zero && i == g.p0, s->stream, &s->launches);
+        cudaError_t e = launch_group(s->psi, s->n, gp, reinterpret_cast<const unsigned char*>(p->d_mat + p->group_off),
+                                     zero && i == g.p0, s->stream, &s->launches);
         tm.stop();
         if (e != cudaSuccess) return cuda_fail(s, e, "group kernel");
         rs->passes += 1;
@@ -1182,7 +1180,7 @@ qsa_status qsa_apply_circuit(qsa_state s, const qsa_op* ops, size_t n_ops, const
     st = plan_create(ops, n_ops, s->n, opts, s->L, s->cm ? s->cm : costmodel_global(), &p);
     if (st != QSA_OK) return st;
     st = qsa_plan_execute(s, p, stats);
-    if (p->d_mat || p->d_layer || p->d_group) {
+    if (p->d_mat || p->d_layer) {
         // free after the stream has consumed the matrices
         cudaStreamSynchronize(s->stream);
         plan_free_device(p);

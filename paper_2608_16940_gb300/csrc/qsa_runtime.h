@@ -100,7 +100,7 @@ struct qsa_plan_s {
     size_t n_ops = 0;
     int max_width = 0;
     std::vector<PlanBlock> blocks;
-    std::vector<float> host_mat;   // all fused matrices, FP32, 16-byte aligned
+    std::vector<float> host_mat;   // all fused matrices, FP32, 16-byte aligned; then the group programs
     float* d_mat = nullptr;        // device copy (uploaded on first execution)
     std::vector<int32_t> next_use; // per block, per logical qubit: next dense block targeting it
     int dev = -1;
@@ -112,8 +112,9 @@ struct qsa_plan_s {
     // group passes for the layout L0 (GroupPass::only: a block index)
     std::vector<PlanGroup> groups;
     std::vector<qsa::GroupPass> gpasses;
-    std::vector<unsigned char> host_group;   // their programs
-    unsigned char* d_group = nullptr;
+    // Their programs, from float group_off of host_mat and d_mat on: one allocation and one copy for
+    // both, whose cost a circuit that is planned, run and dropped pays every time (about 8 us).
+    size_t group_off = 0;
 };
 
 namespace qsa {
