@@ -19,6 +19,7 @@
 #include <cstdint>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -154,7 +155,7 @@ __device__ __forceinline__ void store_tile_swz(const TileArgs& a, const uint64_t
 // item writes its outputs in place and the tile goes back in address order
 // (16-byte units of 2^TB-amplitude tiles), for target sets whose direct
 // stores would give every lane its own sector.
-template <int K, int R, int S, bool SWZ = false, bool WB = false, int TB = 11, bool PO = false, int NG = 1, int TH = kThreads>
+template <int K, int R, int S, bool SWZ = false, bool WB = false, int TB = 11, bool PO = false, int NG = 1, int TH = kThreads, bool SC = false>
 __device__ __forceinline__ void apply_tiles(const ApplyArgs& a, float2* stage, const float2* Ms,
                                             const uint64_t* runoff, const int* loff, uint64_t t0, uint64_t stride,
                                             const uint8_t* htab = nullptr, const int* sloff = nullptr) {
@@ -212,7 +213,7 @@ __device__ __forceinline__ void apply_tiles(const ApplyArgs& a, float2* stage, c
                     if (dbg::in_bounds(gj, 1, a.t.ntiles << a.t.T, 4)) __stcs(a.t.psi + gj, make_float2(re, im));
                 }
             };
-            if constexpr (K != 3) {
+            if constexpr (!SC) {
                 // Packed FP32 pairs: with x2_c = (Re v_c, Re v_c), y2_c = (Im v_c, Im v_c)
                 // and g = (Re G, Im G), p = sum x2_c * g and q = sum y2_c * g give
                 // Re = p.x - q.y and Im = p.y + q.x; one 16-byte load of two G entries
@@ -307,7 +308,7 @@ __device__ __forceinline__ void build_loff(const int* tl, int* loff) {
     }
 }
 
-template <int K, int R, int S, bool SWZ, bool WB, int TB, int NG, int TH>
+template <int K, int R, int S, bool SWZ, bool WB, int TB, int NG, int TH, bool SC>
 __global__ void __launch_bounds__(TH) k_apply_fp32(ApplyArgs a) {
     constexpr int D = 1 << K;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(TH) k_apply_fp32(ApplyArgs a) {
         for (int c = threadIdx.x; c < D; c += blockDim.x) sloff[c] = loff[c] ^ static_cast<int>(stage_xor(htab, loff[c]));
     }
     __syncthreads();
-    apply_tiles<K, R, S, SWZ, WB, TB, (K <= 4), NG, TH>(a, stage, Ms, runoff, loff, blockIdx.x, gridDim.x, htab, sloff);
+    apply_tiles<K, R, S, SWZ, WB, TB, (K <= 4), NG, TH, SC>(a, stage, Ms, runoff, loff, blockIdx.x, gridDim.x, htab, sloff);
 }
 
 template <int K>
@@ -339,7 +340,8 @@ struct ApplyCfg;
 template <> struct ApplyCfg<1> { static constexpr int NG = 1, TH = kThreads, T = 11, R = 2, S = 2; static constexpr bool SWZ = true; };
 template <> struct ApplyCfg<2> { static constexpr int NG = 1, TH = kThreads, T = 11, R = 4, S = 2; static constexpr bool SWZ = true; };
 template <> struct ApplyCfg<3> { static constexpr int NG = 1, TH = kThreads, T = 11, R = 8, S = 2; static constexpr bool SWZ = true; };
-// k = 3: scalar FMAs (N = 27: 0.349 ms, packed ones 0.367).  k = 4: CTAs of 128
+// k = 3: scalar FMAs beyond the L2 (N = 27: 0.349 ms, packed ones 0.367; N = 23:
+// 28.3 us, packed 26.7).  k = 4: CTAs of 128
 // threads with two groups per thread, which share the matrix's broadcast loads
 // (N = 27: 0.406 ms; one group, 256 threads: 0.422; scalar FMAs 0.452 / 0.499 with
 // one / two groups); 2^12-amplitude tiles, two stages so that three CTAs fit an SM
@@ -449,10 +451,17 @@ cudaError_t launch_apply_k(float2* psi, int n, const int* phys, const float* d_m
     const size_t smem = sizeof(float2) * (static_cast<size_t>(C::S) << g.T) + sizeof(float2) * D * D + tables;
     // several groups per item on full tiles only
     const bool whole = g.T == C::T;
-    auto kern = form == 2   ? k_apply_fp32<K, C::R, C::S, C::SWZ, C::SWZ, C::T, C::NG, C::TH>
-                : form == 1 ? k_apply_fp32<K, C::R, C::S, C::SWZ, false, C::T, C::NG, C::TH>
-                : whole     ? k_apply_fp32<K, C::R, C::S, false, false, C::T, C::NG, C::TH>
-                            : k_apply_fp32<K, C::R, C::S, false, false, C::T, 1, C::TH>;
+    auto of_form = [&](auto scalar) {
+        constexpr bool SC = decltype(scalar)::value;
+        return form == 2   ? k_apply_fp32<K, C::R, C::S, C::SWZ, C::SWZ, C::T, C::NG, C::TH, SC>
+               : form == 1 ? k_apply_fp32<K, C::R, C::S, C::SWZ, false, C::T, C::NG, C::TH, SC>
+               : whole     ? k_apply_fp32<K, C::R, C::S, false, false, C::T, C::NG, C::TH, SC>
+                           : k_apply_fp32<K, C::R, C::S, false, false, C::T, 1, C::TH, SC>;
+    };
+    auto kern = of_form(std::false_type{});
+    if constexpr (K == 3) {
+        if (n >= kBeyondL2) kern = of_form(std::true_type{});
+    }
     {
         const size_t full = sizeof(float2) * (static_cast<size_t>(C::S) << C::T) + sizeof(float2) * D * D + tables;
         cudaError_t e = set_smem_attr(reinterpret_cast<const void*>(kern), static_cast<int>(full));

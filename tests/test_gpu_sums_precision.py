@@ -111,3 +111,28 @@ def test_two_grouped_one_qubit_operators(q, n):
         assert stats["blocks"] == 2 and stats["passes"] == 1
         errs.append(e)
     assert np.sqrt(np.mean(np.square(errs))) <= 1.1 * D_ROUND * np.sqrt(3.5 * 2)
+
+
+@pytest.mark.parametrize("n", [23, 24])
+def test_three_qubit_operators_in_and_beyond_the_l2(q, n):
+    """Packed and scalar FMAs, both with two sums: the same bound."""
+    errs = []
+    for seed in range(4):
+        rng = np.random.default_rng(seed)
+        t = sorted(int(v) for v in rng.permutation(n)[:3])
+        m = W.haar_unitary(8, rng)
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        x = torch.view_as_complex(torch.randn(1 << n, 2, device="cuda", generator=g)) / 2 ** 12
+        # axes: bits above t[2], t[2], between, t[1], between, t[0], below
+        v = x.to(torch.complex128).view(1 << (n - 1 - t[2]), 2, 1 << (t[2] - t[1] - 1), 2, 1 << (t[1] - t[0] - 1), 2,
+                                        1 << t[0])
+        want = torch.einsum("cbafed,ufvewdx->ucvbwax", torch.from_numpy(m.reshape([2] * 6)).cuda(), v).reshape(-1)
+        st = GState(q, torch, n)
+        try:
+            st.buf.copy_(x)
+            q.qsa_apply_fused(st.h, t, m)
+            d = torch.linalg.vector_norm(st.buf.to(torch.complex128) - want)
+            errs.append(float(d / torch.linalg.vector_norm(want)))
+        finally:
+            st.close()
+    assert np.sqrt(np.mean(np.square(errs))) <= _bound(3, 1)
