@@ -123,11 +123,17 @@ namespace qsa {
 // contiguous run (2^11 amplitudes = 16 KiB).
 constexpr int kInBlockBits = 11;
 
-// Largest state whose plans run consecutive blocks as group passes.  Grouping
-// pays at every size (N = 25, 270 blocks of a QFT and random layers: see
-// group.cu), but it changes what a plan costs from its blocks to its passes,
-// and the learned planner scores blocks: on larger states, where it is what
-// chooses the plan, the blocks stay one pass each so that its scores hold.
+// Largest state whose plans run consecutive blocks as group passes.  The passes
+// themselves have no such limit and gain more above it: QFT and three random
+// layers, DP plan of k <= 4 blocks, N = 25 / 26 / 28: 3.39 / 7.03 / 30.5 ms in 9..10
+// passes where a pass per block takes 24.6 / 44.7 / 196 (greedy plans at 26 / 28
+// 15.2 / 65.4 ms against 29.9 / 133).  The limit is the learned planner's: its
+// network and the 4^k recurrence price a block as a pass of its own, and tests hold
+// the learned plan to be faster than the 4^k one at 26 and 28 qubits.  Grouped,
+// the 4^k plan's many small blocks turn that order round, so from the sizes on at
+// which the two are compared a block stays what it is priced as, whoever planned
+// it.  Below, the scores count passes that are not made; grouping is faster there
+// all the same.  A price per pass instead of per block would lift the limit.
 constexpr int kGroupMaxQubits = 25;
 
 qsa_status fail(qsa_status st, const std::string& msg);

@@ -1,8 +1,10 @@
 """Group passes at the edges of what they accept: groups that multiply to the
 identity and so have no pass, factors with entries that are not numbers (those
 also where products run as layers), allocations that fail before the first pass,
-and what a plan uploads for grouped products.  Same tolerance as the other group tests (1e-5 on fidelity and amplitudes,
-FP32 sums of at most 32 terms over a few blocks)."""
+what a plan uploads for grouped products, programs longer than a pass holds, the
+largest grouped state, and operators that are not unitary.  Same tolerance as the
+other group tests (1e-5 on fidelity and amplitudes, FP32 sums of at most 32 terms
+over a few blocks)."""
 import numpy as np
 import pytest
 
@@ -219,3 +221,93 @@ def test_long_programs(q, n, k, count):
     finally:
         st.close()
         q.qsa_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("n", [25, 26])
+def test_both_sides_of_the_size_limit(q, n):
+    """The same plan options, grouped and a pass per block, against one pass per
+    operator."""
+    rng = np.random.default_rng(n)
+    ops = []
+    for i in range(24):
+        k = 1 + i % 3
+        t = tuple(int(v) for v in rng.permutation(n)[:k])
+        ops.append(W.Op(t, np.diag(np.exp(1j * rng.uniform(0, 6, 1 << k))), True, "d") if i % 4 == 3 else
+                   W.Op(t, W.haar_unitary(1 << k, rng), False, "u"))
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x = torch.view_as_complex(torch.randn(1 << n, 2, device="cuda", generator=g))
+    x /= torch.linalg.vector_norm(x)
+    sts = [GState(q, torch, n) for _ in range(2)]
+    try:
+        for st in sts:
+            st.buf.copy_(x)
+        stats = q.qsa_apply_circuit(sts[0].h, ops, q.make_opts(planner=q.QSA_PLAN_GREEDY, kmax=4))
+        assert stats["passes"] < stats["blocks"] if n <= 25 else stats["passes"] == stats["blocks"]
+        q.qsa_apply_circuit(sts[1].h, ops, q.make_opts(planner=q.QSA_PLAN_PER_GATE, kmax=4))
+        torch.cuda.synchronize()
+        assert float(torch.linalg.vector_norm(sts[0].buf - sts[1].buf)) <= 1e-5
+    finally:
+        for st in sts:
+            st.close()
+
+
+def _general_ops(n, rng):
+    """Operators that are not unitary, of norm about one: scaled unitaries, rank-one
+    and zero factors, projectors, triangular and random 2 x 2 ones between
+    rotations, wider dense ones, and diagonals of up to eight qubits with zeros and
+    entries of very different size."""
+    def pick(k):
+        return tuple(int(v) for v in rng.permutation(n)[:k])
+    ops = []
+    for i in range(10):
+        q0 = pick(1)
+        ops.append(W.Op(q0, W.haar_unitary(2, rng), False, "u"))
+        kind = i % 5
+        if kind == 0:
+            m = W.haar_unitary(2, rng) * (1.25 if i < 5 else 0.8)
+        elif kind == 1:
+            m = np.outer([0.6, 0.8j], [1.0, 1j])           # rank one
+        elif kind == 2:
+            m = np.diag([1.0, 0.0]).astype(np.complex128)  # a projector
+        elif kind == 3:
+            m = np.array([[0.9, 0.7], [0.0, 1.1]], dtype=np.complex128)
+        else:
+            m = 0.7 * (rng.standard_normal((2, 2)) + 1j * rng.standard_normal((2, 2)))
+        ops.append(W.Op(q0 if i % 2 else pick(1), m, False, "m"))
+        ops.append(W.Op(q0, W.haar_unitary(2, rng), False, "u"))
+        k = min(n, 2 + i % 3)
+        m = W.haar_unitary(1 << k, rng) + 0.2 * rng.standard_normal((1 << k, 1 << k))
+        ops.append(W.Op(pick(k), m, False, "m"))
+        k = min(n, (1, 2, 3, 5, 6)[i % 5])
+        d = rng.standard_normal(1 << k) + 1j * rng.standard_normal(1 << k)
+        d[0] = 0.0
+        d[-1] *= 1e-3
+        ops.append(W.Op(pick(k), np.diag(d), True, "d"))
+    return ops
+
+
+@pytest.mark.parametrize("n", [3, 8, 12, 13, 16])
+@pytest.mark.parametrize("kmax", [1, 3])
+def test_operators_that_are_not_unitary(q, n, kmax):
+    """Against the oracle in up to four stretches, each from a state of norm one,
+    relative to the norm reached (a stretch whose projectors leave nothing: to one)."""
+    rng = np.random.default_rng(10 * n + kmax)
+    opts = q.make_opts(planner=q.QSA_PLAN_DP, kmax=kmax, kmax_diag=min(n, 8), kmax_prod=3 if kmax == 1 and n > 3 else 0)
+    psi = W.random_state(n, seed=n).astype(np.complex64)
+    for _ in range(4):
+        ops = _general_ops(n, rng)[:25]
+        want = psi.astype(np.complex128)
+        for o in ops:
+            oracle.apply(want, o.targets, o.matrix)
+        st = GState(q, torch, n, init=psi)
+        try:
+            stats = q.qsa_apply_circuit(st.h, ops, opts)
+            assert stats["passes"] < stats["blocks"] or stats["blocks"] == 1   # one dense block on three qubits
+            got = st.logical()
+        finally:
+            st.close()
+        norm = np.linalg.norm(want)
+        assert np.linalg.norm(got - want) <= 1e-5 * (norm if norm > 0 else 1.0)
+        if norm == 0:
+            break
+        psi = (want / norm).astype(np.complex64)
