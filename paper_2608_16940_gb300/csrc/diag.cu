@@ -6,7 +6,8 @@
 // A CTA walks tiles of 1024 pairs of amplitudes (16 bytes, physical indices y and
 // y + 1), four per thread in flight; three 256-thread CTAs per SM put 48 KiB in
 // flight: the memory's latency takes no more, and more turn its bus around more
-// often (N = 26, k = 4: 187 us with 96 KiB, 181 with 72, 173 with 48).  The entry
+// often (N = 26, k = 4: 183 / 166 / 171 / 172 us with 2 / 3 / 4 / 5 CTAs; in the L2 the
+// last three are alike, N = 20 9.7..10.1, N = 23 18.8 / 17.9 / 18.2).  The entry
 // index c(y) (bit j = bit p_j of y) is the OR of a part per thread, per tile and
 // per place in the tile; shared tables over the bits of y, 18 KiB formed by every
 // CTA, cost a small state most of its launch (N = 20, k = 4: 20.5 us, 6.1 here;

@@ -1395,9 +1395,11 @@ int bits_of(uint64_t count) {   // bits of 0 .. count - 1
 }
 
 // shots per resolving warp: few when most lie in blocks of their own, which a
-// warp reads one after another, many when they share blocks (this kernel with
-// 8 / 16 / 32: N = 24, 30 000 shots 44 / 48 / 62 us; N = 26, 200 000 154 / 137 /
-// 144; N = 20, 200 000 56 / 32 / 22)
+// warp reads one after another, many when they share blocks.  Whole calls with
+// 8 / 16 / 32 at so many shots a block: N = 26, 1.5: 413 / 421 / 447 us, 2.5: 458 / 457
+// / 475, 4: 501 / 485 / 492, 6: 552 / 524 / 509, 12: 721 / 633 / 600; N = 24, 3: 261 /
+// 269 / 295, 4: 270 / 271 / 280, 8: 282 / 272 / 274, 30: 438 / 380 / 352; N = 22, 8: 202 /
+// 195 / 201, 12: 203 / 197 / 197, 30: 232 / 212 / 206.
 int resolve_per(uint64_t shots, uint64_t nblocks) { return shots >= 8 * nblocks ? 32 : shots >= 3 * nblocks ? 16 : 8; }
 
 // The batch's samples of all trajectories at once, where the shots' numbers fit
