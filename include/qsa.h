@@ -67,7 +67,9 @@ typedef struct qsa_state_s* qsa_state;
 /* Widest product block (qsa_apply_product, product plan blocks): one-qubit
  * factors on distinct qubits, applied in one pass of the FP32 tile engine
  * (2^11-amplitude tiles) when at most 6 of them lie above the tile's
- * contiguous low bits, else in several passes. */
+ * contiguous low bits, else in several passes.  From N = 24 on four or more
+ * unitary factors run as a layer (below): nine positions at 3 or above to a
+ * pass. */
 #define QSA_MAX_PROD 11
 /* Layer blocks (qsa_apply_layer, layer plan blocks): tiles of 2^12
  * amplitudes whose 3 lowest bits are the state's 3 lowest positions, so at
@@ -489,12 +491,16 @@ qsa_status qsa_sample_counts(qsa_state s, uint64_t shots, uint64_t seed, uint64_
  * Many independent small states (noisy trajectories: the per-gate Pauli
  * channels of §IV-A sampled into explicit Pauli branches, so every trajectory
  * is a unitary circuit) evolved in ONE persistent kernel launch: each
- * thread-block cluster (up to four CTAs) pops a trajectory from an atomic queue
- * (longest first) and applies all of its fused blocks to |0..0> in group
- * passes (several blocks per pass), the CTAs splitting every pass's tiles and
- * meeting at a cluster barrier between passes; a second kernel samples every state (one CTA per
- * trajectory, Philox stream id = trajectory index, identity layout), and both
- * can be replayed as one captured CUDA graph. */
+ * thread-block cluster (up to eight CTAs, by the size of the states and the
+ * number of trajectories) pops a trajectory from an atomic queue (longest
+ * first) and applies all of its fused blocks to |0..0> in group passes (several
+ * blocks per pass), the CTAs splitting every pass's tiles and meeting at a
+ * cluster barrier between passes.  Then every state is sampled (Philox stream
+ * id = trajectory index, identity layout): from N = 10 on the shots of all
+ * trajectories (at most 2^26) are drawn and sorted together in a few launches,
+ * in device scratch that the batch allocates beside its outputs; below, with
+ * more shots, or where that scratch does not fit, by one CTA per trajectory.
+ * All of it can be replayed as one captured CUDA graph. */
 typedef struct qsa_batch_s* qsa_batch;
 
 /* Host planning + one-time upload: trajectory t is ops[op_offsets[t] ..
