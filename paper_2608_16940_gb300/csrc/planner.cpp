@@ -241,13 +241,18 @@ void build_next_use(qsa_plan_s* p) {
     }
 }
 
+// Whether a plan's blocks may share passes: per-gate plans keep one pass per op,
+// and permuting plans one layout per block.
+bool plan_groups(const qsa_plan_s* p) {
+    return p->n <= kGroupMaxQubits && p->opts.planner != QSA_PLAN_PER_GATE && p->opts.lowering != QSA_LOWER_PERMUTE;
+}
+
 // Runs [i, e) of at least two consecutive dense (k <= 4), diagonal and product
 // blocks: they become group passes (several blocks per pass over the state) for
-// the plan's layout.  Per-gate plans keep one pass per op, and permuting plans
-// one layout per block.
+// the plan's layout.
 std::vector<std::pair<size_t, size_t>> group_runs(const qsa_plan_s* p) {
     std::vector<std::pair<size_t, size_t>> runs;
-    if (p->n > kGroupMaxQubits || p->opts.planner == QSA_PLAN_PER_GATE || p->opts.lowering == QSA_LOWER_PERMUTE) return runs;
+    if (!plan_groups(p)) return runs;
     auto takes = [](const PlanBlock& b) { return b.layer < 0 && (b.prod || group_takes(b.k, b.diag)); };
     const size_t nb = p->blocks.size();
     for (size_t i = 0; i < nb;) {
@@ -268,14 +273,13 @@ void build_prod_layers(qsa_plan_s* p, const std::vector<double>& mat64, const st
         PlanBlock& b = p->blocks[i];
         if (!b.prod || (r < runs.size() && runs[r].first <= i)) continue;
         PlanLayer pl;
-        if (!product_as_layer(b.t, b.k, mat64.data() + b.off, &pl.spec)) continue;
+        if (!product_as_layer(b.t, b.k, mat64.data() + b.off64, &pl.spec)) continue;
         b.prod_layer = static_cast<int>(p->layers.size());
         p->layers.push_back(std::move(pl));
     }
 }
 
-// The passes of the runs.  mat64: the blocks' matrices before rounding, at their
-// offsets in host_mat.
+// The passes of the runs.  mat64: the blocks' matrices before rounding, at off64.
 void build_groups(qsa_plan_s* p, const std::vector<double>& mat64, const std::vector<std::pair<size_t, size_t>>& runs) {
     std::vector<unsigned char> progs;
     for (const auto& [i, e] : runs) {
@@ -283,7 +287,7 @@ void build_groups(qsa_plan_s* p, const std::vector<double>& mat64, const std::ve
         std::vector<int> whole;   // the block an operator is all of, or -1 (a product's factor)
         for (size_t x = i; x < e; ++x) {
             const PlanBlock& b = p->blocks[x];
-            const double* mat = mat64.data() + b.off;
+            const double* mat = mat64.data() + b.off64;
             if (b.prod) {
                 for (int j = 0; j < b.k; ++j) {
                     src.push_back({1, false, {p->L0[b.t[j]]}, mat + 8 * j});
@@ -681,7 +685,13 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
     p->blocks.resize(blocks.size());
     std::vector<double> M;
     ModulusCarry carry;   // modulus errors of the plan's FP32 constants (error feedback)
-    std::vector<double> mat64;   // host_mat before rounding
+    // the matrices of blocks that may be grouped, and product factors, before rounding
+    std::vector<double> mat64;
+    auto keep = [&](PlanBlock& b, const double* m, size_t count) {
+        if (!b.prod && !(plan_groups(p) && group_takes(b.k, b.diag))) return;
+        b.off64 = mat64.size();
+        mat64.insert(mat64.end(), m, m + count);
+    };
     for (size_t i = 0; i < blocks.size(); ++i) {
         const Unit& u = blocks[i];
         PlanBlock& b = p->blocks[i];
@@ -791,10 +801,8 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
                 F[4 * j + 3] = h[2] * f[1] + h[3] * f[3];
             }
             p->host_mat.resize(b.off + 8 * t);
-            mat64.resize(b.off + 8 * t);
+            keep(b, reinterpret_cast<const double*>(F.data()), 8 * static_cast<size_t>(t));
             for (int c = 0; c < 4 * t; ++c) {
-                mat64[b.off + 2 * c] = F[c].real();
-                mat64[b.off + 2 * c + 1] = F[c].imag();
                 p->host_mat[b.off + 2 * c] = static_cast<float>(F[c].real());
                 p->host_mat[b.off + 2 * c + 1] = static_cast<float>(F[c].imag());
             }
@@ -808,7 +816,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
             p->host_mat.resize(b.off + M.size());
             to_float_moduli(M.data(), M.size() / 2, p->host_mat.data() + b.off, 1.0 / static_cast<double>(M.size() / 2),
                             &carry);
-            mat64.insert(mat64.end(), M.begin(), M.end());
+            keep(b, M.data(), M.size());
         } else if (u.e - u.s == 1) {
             const qsa_op& op = ops[u.s];
             b.k = op.k;
@@ -816,7 +824,7 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
             const size_t cnt = 2ull << (2 * op.k);
             p->host_mat.resize(b.off + cnt);
             to_float_matrix(op.matrix, op.k, p->host_mat.data() + b.off);
-            mat64.insert(mat64.end(), op.matrix, op.matrix + cnt);
+            keep(b, op.matrix, cnt);
         } else {
             st = fuse_range(ops, u.s, u.e, b.t, &b.k, &M);
             if (st != QSA_OK) {
@@ -825,11 +833,10 @@ qsa_status plan_create(const qsa_op* ops, size_t n_ops, int n_qubits, const qsa_
             }
             p->host_mat.resize(b.off + M.size());
             for (size_t j = 0; j < M.size(); ++j) p->host_mat[b.off + j] = static_cast<float>(M[j]);
-            mat64.insert(mat64.end(), M.begin(), M.end());
+            keep(b, M.data(), M.size());
         }
         p->max_width = std::max(p->max_width, b.k);
         while (p->host_mat.size() % 4) p->host_mat.push_back(0.f);  // 16-byte aligned matrices
-        mat64.resize(p->host_mat.size());
     }
     // the zero-state block takes over the layer block after it: the generated
     // product state passes through that block's diagonal part and factors in

@@ -79,6 +79,7 @@ struct PlanBlock {
     bool init = false;         // zero-state preparation (a write-only layer block)
     int n_diag = 0;            // layer block: ops of its diagonal part
     size_t off = 0;            // float offset of its matrix / diagonal in host_mat / d_mat
+    size_t off64 = 0;          // of its matrix before rounding, while the plan is formed
     size_t first_op = 0;       // in execution order
 };
 
