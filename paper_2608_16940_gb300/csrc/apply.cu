@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_prod(ProdArgs a) {
 // with three walking CTAs per SM 12.4 / 18.7 / 48.0 / 684; in 2^11 tiles with three
 // stages and up to six positions (before) 10.3 / 17.6 / 46.1 / 708.  Two random
 // layouts and five bit swaps at N = 28: 22 passes of that kind, 14.5 ms; 7 passes
-// here, 4.5 ms.
+// here, 4.4 ms.
 constexpr int kPermT = 13, kPermLow = 3;
 
 struct PermArgs {
